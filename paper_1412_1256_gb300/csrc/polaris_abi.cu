@@ -620,9 +620,11 @@ extern "C" int spectrometer_create(const polaris_config* cfg, polaris_spec** out
   cudaError_t e = cudaMemcpy(s->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && c.window != POLARIS_WIN_RECT) {
     std::vector<float> taps(N);
+    const TapOrder order = tap_order(logn);
     for (int64_t n = 0; n < N; ++n)
-      taps[n] = c.window == POLARIS_WIN_HANN ? (float)(0.5 - 0.5 * std::cos(2.0 * M_PI * (double)n / (double)N))
-                                             : c.taps[n];
+      taps[order.slot(n)] = c.window == POLARIS_WIN_HANN
+                                    ? (float)(0.5 - 0.5 * std::cos(2.0 * M_PI * (double)n / (double)N))
+                                    : c.taps[n];
     e = cudaMemcpy(s->d_taps, taps.data(), N * 4, cudaMemcpyHostToDevice);
   }
   if (e == cudaSuccess) e = cudaMemset(s->d_acc, 0, acc_bytes);
@@ -1149,11 +1151,16 @@ __global__ void k_noalloc_twiddles(float2* tw, int N2, int UPS, long long N) {
   tw[i] = make_float2((float)c, (float)s);
 }
 
-// periodic Hann taps 0.5 - 0.5 cos(2 pi n / N)
-__global__ void k_noalloc_hann(float* taps, long long N) {
+// periodic Hann taps 0.5 - 0.5 cos(2 pi n / N), in tap_order
+__global__ void k_noalloc_hann(float* taps, long long N, TapOrder order) {
   const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= N) return;
-  taps[n] = (float)(0.5 - 0.5 * cospi(2.0 * (double)n / (double)N));
+  taps[order.slot(n)] = (float)(0.5 - 0.5 * cospi(2.0 * (double)n / (double)N));
+}
+// custom taps from sample order into tap_order
+__global__ void k_noalloc_taps(const float* __restrict__ src, float* __restrict__ taps, long long N, TapOrder order) {
+  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (n < N) taps[order.slot(n)] = src[n];
 }
 
 static size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -1296,10 +1303,16 @@ extern "C" int spectrometer_run_noalloc(const polaris_config* cfg, const void* c
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && c.window == POLARIS_WIN_HANN) {
-    k_noalloc_hann<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(taps, N);
+    k_noalloc_hann<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(taps, N, tap_order(logn));
     e = cudaGetLastError();
   } else if (e == cudaSuccess && c.window == POLARIS_WIN_CUSTOM) {
-    e = cudaMemcpyAsync(taps, c.taps, (size_t)N * 4, cudaMemcpyHostToDevice, st);
+    // sample order first into the slab (at least N float2, not yet in use), then into tap_order
+    float* raw = reinterpret_cast<float*>(slab);
+    e = cudaMemcpyAsync(raw, c.taps, (size_t)N * 4, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) {
+      k_noalloc_taps<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(raw, taps, N, tap_order(logn));
+      e = cudaGetLastError();
+    }
   }
   if (e != cudaSuccess) return set_err(nullptr, POLARIS_ECUDA, "no-alloc set-up: %s", cudaGetErrorString(e));
   const int64_t nseg = (n_samples_per_if - N) / hop + 1;

@@ -235,6 +235,30 @@ constexpr int plan_log_n2(int logn) {
   // 4:2 5:3 6:3 7:4 8:4 9:5 10:5 11:6 12:6 13:7 14:7 15:8 16:8 17:9 18:9 19:9 20:9
   return logn >= 17 ? 9 : (logn + 1) / 2;
 }
+// Order of the window taps in device memory from N = 2^13 up: the order in which phase 1's lanes
+// take them.  Lane q1 CW + cw of the warp that owns columns gb CW .. gb CW + CW - 1 needs the taps
+// of rows q1 + Q1 t; with four consecutive t of a lane side by side and the 32 lanes after one
+// another, a warp's request is 512 contiguous bytes (one 16-byte load per lane).  In sample
+// order it was one 4-byte load per point over 32 / CW rows of 4 CW bytes: at 2^20 (CW = 1) 32
+// sectors of 32 bytes for 128 bytes used.  Measured with a Hann window, whole passes, before and
+// after: 15 x 2^20 int8 223 -> 160 us, 610 x 2^18 int8 1162 -> 884 us, 1953 half-overlapped 2^14
+// int8 segments of four IFs 379 -> 332 us.  Smaller N loads its taps per lane in sample order (a
+// lane's rows are adjacent columns there).
+constexpr int kTapsOrderedMin = 13;
+struct TapOrder {
+  int ln2, lq1, lcw, lt4;  // log2 of N2, Q1, CW and P1/4 (ln2 < 0: sample order)
+  __host__ __device__ constexpr long long slot(long long n) const {
+    if (ln2 < 0) return n;
+    const long long row = n >> ln2, b = n & ((1LL << ln2) - 1), t = row >> lq1;
+    const long long lane = ((row & ((1LL << lq1) - 1)) << lcw) | (b & ((1LL << lcw) - 1));
+    return (((((b >> lcw) << lt4) + (t >> 2)) * 32 + lane) << 2) + (t & 3);
+  }
+};
+__host__ __device__ constexpr TapOrder tap_order(int logn) {
+  if (logn < kTapsOrderedMin) return TapOrder{-1, 0, 0, 0};
+  const int ln2 = plan_log_n2(logn), n1 = 1 << (logn - ln2), p1 = plan_p1(logn, n1), lq1 = ct::ilog2(n1 / p1);
+  return TapOrder{ln2, lq1, 5 - lq1, ct::ilog2(p1 / 4)};
+}
 // ----------------------------------------------------------------------------------------
 // shared-memory layouts of the warp-local transposes.  The strides below were chosen by an
 // offline simulation of the bank conflicts of each transpose's write and read patterns.

@@ -72,7 +72,7 @@ struct BatchArgs {
   int n_fpair;
   int seg0;             // first feed segment of this batch
   int nseg;             // segments in this batch
-  const float* taps;    // window taps (N) or nullptr for the rectangular window
+  const float* taps;    // window taps (N, in tap_order) or nullptr for the rectangular window
   float2* scratch;      // slab [nseg * n_fpair][N1][N2]: row c (phase-1 output index), b contiguous
   const float2* tw;     // [UPS + 1][N2]: W_N^{b u} (unit-major)
   void* acc;            // native accumulators [acc_copies][n_fpair][N/2 + 1] of float4 (double4 if fp64)
@@ -283,7 +283,7 @@ __device__ __forceinline__ void p1_load(const BatchArgs& a, int g, int b, int q1
     float x = decode_level<BITS>(ok ? __ldg(pa + word_i) : 0u, shift);
     float y = pb ? decode_level<BITS>(ok ? __ldg(pb + word_i) : 0u, shift) : 0.0f;
     if (taps) {
-      const float wv = __ldg(taps + n);
+      const float wv = __ldg(taps + tap_order(LOGN).slot(n));
       x *= wv;
       y *= wv;
     }
@@ -710,12 +710,16 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
         // window (TP) are uniform per tile
         auto decode = [&](auto tl_, auto hb_, auto tp_) {
           constexpr bool TL = decltype(tl_)::value, HB = decltype(hb_)::value, TP = decltype(tp_)::value;
+          [[maybe_unused]] const float4* tp =
+              reinterpret_cast<const float4*>(a.taps) + (size_t)((b - cw) / CW) * (P / 4) * 32 + lane;
+          [[maybe_unused]] float4 w4;
           sfor<0, P>([&](auto t_) {
             constexpr int t = decltype(t_)::value;
             const int row = q1 + Q1 * t;
             float2 z = p1_stage_decode<BITS, TL, HB, N1, WPR, RS>(sb, row, wd, rot);
-            if constexpr (TP) {
-              const float tv = __ldg(a.taps + row * N2 + b);
+            if constexpr (TP) {  // (four consecutive t per load: tap_order)
+              if constexpr (t % 4 == 0) w4 = __ldg(tp + (t / 4) * 32);
+              const float tv = t % 4 == 0 ? w4.x : t % 4 == 1 ? w4.y : t % 4 == 2 ? w4.z : w4.w;
               z.x *= tv;
               z.y *= tv;
             }
