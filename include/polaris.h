@@ -81,7 +81,8 @@ typedef struct polaris_spec polaris_spec; /* opaque, library-owned */
  *   device      CUDA device ordinal.
  *   max_batch_segments  segments processed per kernel pass (bounds the device
  *               scratch: 2 * max_batch_segments * n_fft * 8 bytes per pair);
- *               0 selects the default (passes of at least 64 segments).
+ *               0 selects the default (passes of at least 64 segments).  n_fft of
+ *               1024 to 4096 run in one kernel without scratch, whatever the value.
  *   code_stats  1: also count, per IF, how often each b-bit code occurs in the
  *               segments that feed() integrates (the bit distribution used for
  *               total-power measurement, Sec. 2 and Sec. 3.2.2); read with
@@ -223,8 +224,8 @@ const char* spectrometer_last_error(const polaris_spec* s);
  * every later launch with CUDA events on its stream; spectrometer_kernel_times then
  * waits for those events and returns, per kind, the summed device time in ms and the
  * launch count since profiling began or since the previous query (kinds: 0 = phase 1,
- * decode/window/row DFT; 1 = phase 2, column DFT/correlate/accumulate; 2 = readout and
- * Stokes; 3 = code histogram).  n is the length of both arrays and must be >= 3; kinds
+ * decode/window/row DFT; 1 = phase 2, column DFT/correlate/accumulate (and the one kernel that
+ * does both phases at n_fft of 1024 to 4096); 2 = readout and Stokes; 3 = code histogram).  n is the length of both arrays and must be >= 3; kinds
  * >= n are not reported. */
 int64_t spectrometer_kernel_launches(const polaris_spec* s);
 int spectrometer_set_profiling(polaris_spec* s, int on);
@@ -381,7 +382,7 @@ void polaris_set_wait_limit(int64_t polls);
  * word, and the next synchronising call returns POLARIS_EBOUNDS.  Nothing traps.
  * polaris_checked_build: 1 in such a build, 0 otherwise.
  * polaris_set_check_understate (test hook, checked build only): on != 0 makes later feeds
- * tell the kernels half the slab they have, so that the checks fire while every access
+ * tell the kernels half the slab (n_fft of 1024 to 4096: half the input) they have, so that the checks fire while every access
  * stays inside its buffer; POLARIS_EINVAL in a build without checks. */
 int polaris_checked_build(void);
 int polaris_set_check_understate(int on);

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/polaris.h"
+#include "polaris_fused.cuh"
 #include "polaris_kernels.cuh"
 #include "polaris_tuning.h"
 
@@ -28,9 +29,6 @@ POLARIS_DECLARE(6)
 POLARIS_DECLARE(7)
 POLARIS_DECLARE(8)
 POLARIS_DECLARE(9)
-POLARIS_DECLARE(10)
-POLARIS_DECLARE(11)
-POLARIS_DECLARE(12)
 POLARIS_DECLARE(13)
 POLARIS_DECLARE(14)
 POLARIS_DECLARE(15)
@@ -40,6 +38,10 @@ POLARIS_DECLARE(18)
 POLARIS_DECLARE(19)
 POLARIS_DECLARE(20)
 #undef POLARIS_DECLARE
+// the one-kernel path of the small sizes (polaris_f<LOGN>.cu)
+extern template cudaError_t run_fused<10>(const BatchArgs&, cudaStream_t, bool);
+extern template cudaError_t run_fused<11>(const BatchArgs&, cudaStream_t, bool);
+extern template cudaError_t run_fused<12>(const BatchArgs&, cudaStream_t, bool);
 
 // (args, stream, programmatic dependent launch on the predecessor in `stream`)
 typedef cudaError_t (*phase_fn)(const BatchArgs&, cudaStream_t, bool);
@@ -51,12 +53,14 @@ bool phase1_staged(int logn, int bits);
 cudaError_t launch_unpack_staged(int logn, int bits, const uint32_t* pa, const uint32_t* pb, long long nseg, int dense,
                                  float* oa, float* ob, cudaStream_t st);
 #define POLARIS_ROW(LOGN) {run_phase1<LOGN>, run_phase2<LOGN>}
+#define POLARIS_FUSED_ROW(LOGN) {run_fused<LOGN>, nullptr}  // both phases in one kernel
 static const phase_fn kPhases[21][2] = {
     {nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr},
     POLARIS_ROW(4),  POLARIS_ROW(5),  POLARIS_ROW(6),  POLARIS_ROW(7),  POLARIS_ROW(8),  POLARIS_ROW(9),
-    POLARIS_ROW(10), POLARIS_ROW(11), POLARIS_ROW(12), POLARIS_ROW(13), POLARIS_ROW(14), POLARIS_ROW(15),
+    POLARIS_FUSED_ROW(10), POLARIS_FUSED_ROW(11), POLARIS_FUSED_ROW(12), POLARIS_ROW(13), POLARIS_ROW(14), POLARIS_ROW(15),
     POLARIS_ROW(16), POLARIS_ROW(17), POLARIS_ROW(18), POLARIS_ROW(19), POLARIS_ROW(20)};
 #undef POLARIS_ROW
+#undef POLARIS_FUSED_ROW
 
 // ---------------------------------------------------------------------------------------
 // data translation alone
@@ -83,6 +87,7 @@ struct ReadoutArgs {
   int copies;             // accumulator copies summed per slot (0 or 1: one)
   long long copy_stride;  // slots per copy
   int fp64;
+  int fused;  // bins in natural order (k_readout_bins)
   int N1, N2, UPS, nbin, native;
   int fa[kMaxIF], fb[kMaxIF], fcorr[kMaxIF];
   float* autos;
@@ -93,6 +98,59 @@ struct ReadoutArgs {
   float inv_ga2[kMaxIF], inv_gb2[kMaxIF], ig_re[kMaxIF], ig_im[kMaxIF];  // 1/|Ga|^2, 1/|Gb|^2, 1/(Ga conj Gb)
   const int* err;  // nonzero: a phase kernel gave up a wait; every output is NaN
   long long acc_slots;  // accumulator slots over all copies (read by the checked build)
+};
+
+// where the outputs of FFT pair f go, and one bin's outputs from its sums (xx, yy, Re xy, Im xy)
+struct BinOut {
+  bool failed;
+  float *autos_a, *autos_b, *stokes;
+  float2* cross;
+  float inv_ga2 = 0.f, inv_gb2 = 0.f, ig_re = 0.f, ig_im = 0.f;
+  __device__ __forceinline__ BinOut(const ReadoutArgs& a, int f) {
+    failed = a.err && *a.err != 0;
+    const int p = a.fcorr[f];
+    autos_a = a.autos ? a.autos + (size_t)a.fa[f] * a.nbin : nullptr;
+    autos_b = (a.autos && a.fb[f] >= 0) ? a.autos + (size_t)a.fb[f] * a.nbin : nullptr;
+    cross = (a.cross && p >= 0) ? reinterpret_cast<float2*>(a.cross) + (size_t)p * a.nbin : nullptr;
+    stokes = (a.stokes && p >= 0) ? a.stokes + (size_t)p * 4 * a.nbin : nullptr;
+    if (p >= 0) {
+      inv_ga2 = a.inv_ga2[p];
+      inv_gb2 = a.inv_gb2[p];
+      ig_re = a.ig_re[p];
+      ig_im = a.ig_im[p];
+    }
+  }
+  __device__ __forceinline__ void write(const ReadoutArgs& a, int k, float4 v) const {
+    if (failed) {
+      const float qnan = __int_as_float(0x7fc00000);
+      v = make_float4(qnan, qnan, qnan, qnan);
+    }
+    const float xx = v.x, yy = v.y, xr = v.z, xi = v.w;
+    if (autos_a) autos_a[k] = xx;
+    if (autos_b) autos_b[k] = yy;
+    if (cross) cross[k] = make_float2(xr, xi);
+    if (stokes) {
+      const float x = xx * inv_ga2, y = yy * inv_gb2;
+      const float cr = xr * ig_re - xi * ig_im;
+      const float ci = xr * ig_im + xi * ig_re;
+      float I, Q, Uq, V;
+      if (a.feed == POLARIS_FEED_LINEAR) {
+        I = 0.5f * (x + y);
+        Q = 0.5f * (a.c2 * (x - y) - a.s2 * 2.0f * cr);
+        Uq = 0.5f * (a.s2 * (x - y) + a.c2 * 2.0f * cr);
+        V = ci;
+      } else {
+        I = 0.5f * (x + y);
+        V = 0.5f * (x - y);
+        Q = a.c2 * cr - a.s2 * ci;
+        Uq = a.s2 * cr + a.c2 * ci;
+      }
+      stokes[k] = I;
+      stokes[a.nbin + k] = Q;
+      stokes[2 * (size_t)a.nbin + k] = Uq;
+      stokes[3 * (size_t)a.nbin + k] = V;
+    }
+  }
 };
 
 // Readout of one block: a tile of CT consecutive columns c times DT consecutive values of d,
@@ -174,55 +232,47 @@ __global__ void __launch_bounds__(kReadoutThreads) k_readout(ReadoutArgs a) {
     tile[sidx[i]] = v[i];
   }
   __syncthreads();
-  const bool failed = a.err && *a.err != 0;
-  const int p = a.fcorr[f];
-  float* autos_a = a.autos ? a.autos + (size_t)a.fa[f] * a.nbin : nullptr;
-  float* autos_b = (a.autos && a.fb[f] >= 0) ? a.autos + (size_t)a.fb[f] * a.nbin : nullptr;
-  float2* cross = (a.cross && p >= 0) ? reinterpret_cast<float2*>(a.cross) + (size_t)p * a.nbin : nullptr;
-  float* stokes = (a.stokes && p >= 0) ? a.stokes + (size_t)p * 4 * a.nbin : nullptr;
-  float inv_ga2 = 0.f, inv_gb2 = 0.f, ig_re = 0.f, ig_im = 0.f;
-  if (p >= 0) {
-    inv_ga2 = a.inv_ga2[p];
-    inv_gb2 = a.inv_gb2[p];
-    ig_re = a.ig_re[p];
-    ig_im = a.ig_im[p];
-  }
+  const BinOut out(a, f);
   // consecutive threads take consecutive c of one d (consecutive bins)
   for (int e = threadIdx.x; e < kReadoutTile; e += kReadoutThreads) {
     const int cc = e % CT, dd = e / CT;
     const int k = c0 + cc + N1 * (d0 + dd);
     if (k >= a.nbin) continue;
-    float4 v = tile[dd * (CT + 1) + cc];
-    if (failed) {
-      const float qnan = __int_as_float(0x7fc00000);
-      v = make_float4(qnan, qnan, qnan, qnan);
-    }
-    const float xx = v.x, yy = v.y, xr = v.z, xi = v.w;
-    if (autos_a) autos_a[k] = xx;
-    if (autos_b) autos_b[k] = yy;
-    if (cross) cross[k] = make_float2(xr, xi);
-    if (stokes) {
-      const float x = xx * inv_ga2, y = yy * inv_gb2;
-      const float cr = xr * ig_re - xi * ig_im;
-      const float ci = xr * ig_im + xi * ig_re;
-      float I, Q, Uq, V;
-      if (a.feed == POLARIS_FEED_LINEAR) {
-        I = 0.5f * (x + y);
-        Q = 0.5f * (a.c2 * (x - y) - a.s2 * 2.0f * cr);
-        Uq = 0.5f * (a.s2 * (x - y) + a.c2 * 2.0f * cr);
-        V = ci;
-      } else {
-        I = 0.5f * (x + y);
-        V = 0.5f * (x - y);
-        Q = a.c2 * cr - a.s2 * ci;
-        Uq = a.s2 * cr + a.c2 * ci;
-      }
-      stokes[k] = I;
-      stokes[a.nbin + k] = Q;
-      stokes[2 * (size_t)a.nbin + k] = Uq;
-      stokes[3 * (size_t)a.nbin + k] = V;
-    }
+    out.write(a, k, tile[dd * (CT + 1) + cc]);
   }
+}
+
+// Readout of the sizes that run in one kernel (k_fused), whose accumulators hold the bins in
+// natural order: one thread per bin, every access along consecutive bins.
+__global__ void __launch_bounds__(kReadoutThreads) k_readout_bins(ReadoutArgs a) {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");  // accumulators complete (dependent launch)
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  const int f = blockIdx.y, k = blockIdx.x * kReadoutThreads + threadIdx.x;
+  if (k >= a.nbin) return;
+  const size_t o = (size_t)f * a.nbin + k;
+  const int copies = a.copies > 1 ? a.copies : 1;
+  if (!in_bounds(const_cast<int*>(a.err), (long long)(copies - 1) * a.copy_stride + o, a.acc_slots)) return;
+  float4 v;
+  if (a.fp64) {
+    double4* acc = reinterpret_cast<double4*>(a.acc) + o;
+    double4 w = acc[0];
+    for (int c = 1; c < copies; ++c) {
+      const double4 x = acc[(size_t)c * a.copy_stride];
+      w = make_double4(w.x + x.x, w.y + x.y, w.z + x.z, w.w + x.w);
+    }
+    for (int c = 0; c < copies; ++c) acc[(size_t)c * a.copy_stride] = make_double4(0.0, 0.0, 0.0, 0.0);
+    v = make_float4((float)(0.25 * w.x), (float)(0.25 * w.y), (float)(0.25 * w.z), (float)(0.25 * w.w));
+  } else {
+    float4* acc = reinterpret_cast<float4*>(a.acc) + o;
+    float4 w = acc[0];
+    for (int c = 1; c < copies; ++c) {
+      const float4 x = acc[(size_t)c * a.copy_stride];
+      w = make_float4(w.x + x.x, w.y + x.y, w.z + x.z, w.w + x.w);
+    }
+    for (int c = 0; c < copies; ++c) acc[(size_t)c * a.copy_stride] = make_float4(0.f, 0.f, 0.f, 0.f);
+    v = make_float4(0.25f * w.x, 0.25f * w.y, 0.25f * w.z, 0.25f * w.w);
+  }
+  BinOut(a, f).write(a, k, v);
 }
 
 static dim3 readout_grid(int N1, int N2, int n_fpair) {
@@ -240,6 +290,10 @@ static cudaError_t launch_readout(const ReadoutArgs& r, int n_fpair, cudaStream_
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
+  if (r.fused) {
+    cfg.gridDim = dim3((unsigned)((r.nbin + kReadoutThreads - 1) / kReadoutThreads), (unsigned)n_fpair);
+    return cudaLaunchKernelEx(&cfg, k_readout_bins, r);
+  }
   switch (r.N1) {
 #define POLARIS_RO(LN1)                                       \
   case 1 << LN1:                                              \
@@ -251,7 +305,16 @@ static cudaError_t launch_readout(const ReadoutArgs& r, int n_fpair, cudaStream_
   }
 }
 
-static int host_plan_n2(int logn) { return 1 << plan_log_n2(logn); }
+// columns of a size's plan (b runs over them; N / columns rows)
+static int host_plan_n2(int logn) { return 1 << (is_fused(logn) ? fused_log_b(logn) : plan_log_n2(logn)); }
+// entries of the twiddle table W_N^{b u}, b < N2: u <= N1/2 (the units of phase 2), or, where one
+// kernel does both phases, every u < N1
+static int host_tw_rows(int logn, int n1) { return is_fused(logn) ? n1 : n1 / 2 + 1; }
+// Accumulator copies K.  At small N many warps (or, in the one-kernel path, CTAs) add into the
+// same few slots, and adds to one address are served one after another: each adds into copy
+// (its range or CTA) mod K instead, about 64 adds per copy, and the readout sums the copies.
+// adders: how many add into a slot in one pass.
+static int copies_for(long long adders) { return (int)(adders / 64 < 1 ? 1 : (adders / 64 > 16 ? 16 : adders / 64)); }
 
 }  // namespace polaris
 
@@ -508,7 +571,7 @@ extern "C" int spectrometer_create(const polaris_config* cfg, polaris_spec** out
   s->N2 = host_plan_n2(logn);
   s->N1 = (int)(N / s->N2);
   s->UPS = s->N1 / 2;
-  s->native = s->UPS * s->N2 + 1;
+  s->native = s->UPS * s->N2 + 1;  // (= N/2 + 1; natural bin order in the one-kernel path)
   s->n_pair = n_pair;
   // FFT pairs: correlation pairs first, then the remaining IFs two at a time
   int nf = 0;
@@ -563,21 +626,19 @@ extern "C" int spectrometer_create(const polaris_config* cfg, polaris_spec** out
   s->slab_half = (size_t)s->max_batch * nf * N;
   s->carry_words_cap = N / spw;               // carried samples < N
   s->stage_words_cap = 2 * N / spw;           // staging < carry + N samples
-  // Accumulator copies.  Phase 2 gives each warp one range of segments of one (pair, unit
-  // group) and adds the range's sums into every slot of the group once; at small N (few
-  // groups, ranges of a few segments) a slot would take ~1200 atomic adds per pass, which
-  // serialise per address.  Range r adds into copy r % K (about 64 adds per copy); the
-  // readout sums the copies.
-  {
+  if (is_fused(logn)) {
+    s->acc_copies = copies_for(2LL * s->num_sms / nf);  // CTAs per FFT pair
+  } else {
+    // phase 2: every resident warp has one range of segments of one (pair, unit group)
     const int P = plan_p(logn), Q2 = s->N2 / P, UPW = 16 / Q2;
     const int UGW = UPW > s->UPS ? 1 : s->UPS / UPW;
     const long long warps = (s->cap2 == 1 ? 1LL : 2LL) * s->num_sms * 8;  // phase-2 warps resident (8-warp CTAs)
-    const long long nrg = warps / ((long long)nf * UGW);
-    s->acc_copies = (int)(nrg / 64 < 1 ? 1 : (nrg / 64 > 16 ? 16 : nrg / 64));
+    s->acc_copies = copies_for(warps / ((long long)nf * UGW));
   }
   const size_t acc_bytes = (size_t)s->acc_copies * nf * s->native * 4 * (s->accum_fp64 ? 8 : 4);
-  const size_t bytes_tw = (size_t)s->N2 * (s->UPS + 1) * sizeof(float2);
-  const size_t bytes_scratch = 2 * (size_t)s->max_batch * nf * N * sizeof(float2);
+  const size_t bytes_tw = (size_t)s->N2 * host_tw_rows(logn, s->N1) * sizeof(float2);
+  // (the one-kernel path of the small sizes has no slab)
+  const size_t bytes_scratch = is_fused(logn) ? 0 : 2 * (size_t)s->max_batch * nf * N * sizeof(float2);
   const size_t bytes_carry = (size_t)c.n_if * s->carry_words_cap * 4;
   const size_t bytes_stage = (size_t)c.n_if * s->stage_words_cap * 4;
   const size_t bytes_out = (size_t)s->nbin * 4 * (c.n_if + 2 * n_pair + 4 * n_pair);
@@ -608,11 +669,11 @@ extern "C" int spectrometer_create(const polaris_config* cfg, polaris_spec** out
     delete s;
     return set_err(nullptr, POLARIS_ENOMEM, "cudaMalloc failed");
   }
-  // twiddles W_N^{b u} for b < N2, u <= N1/2, in FP64 then rounded; unit-major ([u][b]), so
-  // that the lanes of a phase-2 item (consecutive b of one unit) read one contiguous run
-  std::vector<float2> tw((size_t)s->N2 * (s->UPS + 1));
+  // twiddles W_N^{b u} for b < N2 (u: host_tw_rows), in FP64 then rounded; unit-major ([u][b]),
+  // so that the lanes that take one (consecutive b of one unit) read one contiguous run
+  std::vector<float2> tw((size_t)s->N2 * host_tw_rows(logn, s->N1));
   for (int b = 0; b < s->N2; ++b)
-    for (int u = 0; u <= s->UPS; ++u) {
+    for (int u = 0; u < host_tw_rows(logn, s->N1); ++u) {
       const int64_t e = ((int64_t)b * u) % N;
       const double ang = -2.0 * M_PI * (double)e / (double)N;
       tw[(size_t)u * s->N2 + b] = make_float2((float)std::cos(ang), (float)std::sin(ang));
@@ -801,8 +862,11 @@ extern "C" int spectrometer_feed(polaris_spec* s, const void* const* packed, int
   a.wait_limit = g_wait_limit;
   a.slab_elems = (long long)s->slab_half;
   // (test hook: half of what the pass writes and reads)
+  // (the one-kernel path has no slab: half of its input there)
   auto understate = [&](BatchArgs& x) {
-    if (g_check_understate) x.slab_elems = (long long)x.nseg * s->n_fpair * s->N / 2;
+    if (!g_check_understate) return;
+    x.slab_elems = (long long)x.nseg * s->n_fpair * s->N / 2;
+    if (is_fused(s->logn)) x.in.in_words0 /= 2, x.in.in_words1 /= 2;
   };
   a.acc_slots = (long long)s->acc_copies * s->n_fpair * s->native;
   const phase_fn f1 = kPhases[s->logn][0], f2 = kPhases[s->logn][1];
@@ -812,7 +876,13 @@ extern "C" int spectrometer_feed(polaris_spec* s, const void* const* packed, int
     });
     if (e != cudaSuccess) return set_err(s, POLARIS_ECUDA, "code-histogram launch: %s", cudaGetErrorString(e));
   }
-  if (nseg > 0 && nseg <= s->max_batch) {
+  if (nseg > 0 && is_fused(s->logn)) {
+    a.seg0 = 0;
+    a.nseg = (int)nseg;
+    understate(a);
+    cudaError_t e = counted_launch(s, 1, st, [&]() { return f1(a, st, st != nullptr && !s->profiling); });
+    if (e != cudaSuccess) return set_err(s, POLARIS_ECUDA, "FFT-correlator launch: %s", cudaGetErrorString(e));
+  } else if (nseg > 0 && nseg <= s->max_batch) {
     // one pass: both phases on the caller's stream, each a programmatic dependent launch
     // (its CTAs set up while the previous kernel drains, then wait for it) unless launches
     // are being timed
@@ -887,6 +957,7 @@ static int fill_readout(polaris_spec* s, const polaris_stokes_params* prm, Reado
   r.UPS = s->UPS;
   r.nbin = (int)s->nbin;
   r.native = s->native;
+  r.fused = is_fused(s->logn);
   for (int f = 0; f < kMaxIF; ++f) {
     r.fa[f] = s->fa[f];
     r.fb[f] = s->fb[f];
@@ -1139,10 +1210,10 @@ static const int kNoallocMaxDevices = 64;
 static void* g_noalloc_ptr[kNoallocMaxDevices] = {nullptr};
 static std::mutex g_noalloc_mu;
 
-// twiddles W_N^{b u} (b < N2, u <= N1/2) in FP64, rounded once to f32, unit-major ([u][b])
-__global__ void k_noalloc_twiddles(float2* tw, int N2, int UPS, long long N) {
+// twiddles W_N^{b u} (b < N2, u < rows) in FP64, rounded once to f32, unit-major ([u][b])
+__global__ void k_noalloc_twiddles(float2* tw, int N2, int rows, long long N) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long total = (long long)N2 * (UPS + 1);
+  const long long total = (long long)N2 * rows;
   if (i >= total) return;
   const long long u = i / N2, b = i % N2;
   const long long e = (b * u) % N;
@@ -1259,7 +1330,8 @@ extern "C" int spectrometer_run_noalloc(const polaris_config* cfg, const void* c
   const int N2 = host_plan_n2(logn), N1 = (int)(N / N2), UPS = N1 / 2, native = UPS * N2 + 1;
   // carve the static array: accumulators | twiddles | taps | slab
   const size_t acc_bytes = align256((size_t)nf * native * 4 * (c.accum_fp64 ? 8 : 4));
-  const size_t tw_bytes = align256((size_t)N2 * (UPS + 1) * sizeof(float2));
+  const int tw_rows = host_tw_rows(logn, N1);
+  const size_t tw_bytes = align256((size_t)N2 * tw_rows * sizeof(float2));
   const size_t taps_bytes = c.window == POLARIS_WIN_RECT ? 0 : align256((size_t)N * 4);
   const size_t err_bytes = 256;  // the phase kernels' status word
   const size_t per_seg = (size_t)nf * N * sizeof(float2);
@@ -1298,8 +1370,8 @@ extern "C" int spectrometer_run_noalloc(const polaris_config* cfg, const void* c
   cudaError_t e = cudaMemsetAsync(acc, 0, acc_bytes, st);  // accumulators start at zero
   if (e == cudaSuccess) e = cudaMemsetAsync(d_err, 0, sizeof(int), st);
   if (e == cudaSuccess) {
-    const long long ntw = (long long)N2 * (UPS + 1);
-    k_noalloc_twiddles<<<(unsigned)((ntw + 255) / 256), 256, 0, st>>>(tw, N2, UPS, N);
+    const long long ntw = (long long)N2 * tw_rows;
+    k_noalloc_twiddles<<<(unsigned)((ntw + 255) / 256), 256, 0, st>>>(tw, N2, tw_rows, N);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && c.window == POLARIS_WIN_HANN) {
@@ -1342,10 +1414,11 @@ extern "C" int spectrometer_run_noalloc(const polaris_config* cfg, const void* c
   a.fp64 = c.accum_fp64 ? 1 : 0;
   a.bits = c.bits;
   a.num_sms = num_sms;
-  for (int64_t s0 = 0; s0 < nseg; s0 += batch) {
+  const int64_t pass = is_fused(logn) ? nseg : batch;  // (no slab in the one-kernel path)
+  for (int64_t s0 = 0; s0 < nseg; s0 += pass) {
     a.seg0 = (int)s0;
-    a.nseg = (int)(nseg - s0 < batch ? nseg - s0 : batch);
-    for (int ph = 0; ph < 2 && e == cudaSuccess; ++ph) e = kPhases[logn][ph](a, st, st != nullptr);
+    a.nseg = (int)(nseg - s0 < pass ? nseg - s0 : pass);
+    for (int ph = 0; ph < (is_fused(logn) ? 1 : 2) && e == cudaSuccess; ++ph) e = kPhases[logn][ph](a, st, st != nullptr);
     if (e != cudaSuccess) return set_err(nullptr, POLARIS_ECUDA, "no-alloc FFT-correlator: %s", cudaGetErrorString(e));
   }
   // readout (same kernel as spectrometer_integrate_device)
@@ -1362,6 +1435,7 @@ extern "C" int spectrometer_run_noalloc(const polaris_config* cfg, const void* c
   r.UPS = UPS;
   r.nbin = (int)(N / 2 + 1);
   r.native = native;
+  r.fused = is_fused(logn);
   for (int f = 0; f < kMaxIF; ++f) {
     r.fa[f] = fa[f];
     r.fb[f] = fb[f];

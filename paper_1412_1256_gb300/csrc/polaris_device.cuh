@@ -242,19 +242,25 @@ constexpr int plan_log_n2(int logn) {
 // order it was one 4-byte load per point over 32 / CW rows of 4 CW bytes: at 2^20 (CW = 1) 32
 // sectors of 32 bytes for 128 bytes used.  Measured with a Hann window, whole passes, before and
 // after: 15 x 2^20 int8 223 -> 160 us, 610 x 2^18 int8 1162 -> 884 us, 1953 half-overlapped 2^14
-// int8 segments of four IFs 379 -> 332 us.  Smaller N loads its taps per lane in sample order (a
-// lane's rows are adjacent columns there).
+// int8 segments of four IFs 379 -> 332 us.  Below
+// 2^10 the taps stay in sample order.
+// The sizes that run in one kernel (2^10 to 2^12) take them the same way: lane b of its team owns
+// column b of the N/R columns of R rows, four rows per load.
+constexpr int kFusedMin = 10, kFusedMax = 12;
+constexpr bool is_fused(int logn) { return logn >= kFusedMin && logn <= kFusedMax; }
+constexpr int fused_log_b(int logn) { return logn == 10 ? 5 : 6; }  // columns of their plan: 32, 64, 64
 constexpr int kTapsOrderedMin = 13;
 struct TapOrder {
-  int ln2, lq1, lcw, lt4;  // log2 of N2, Q1, CW and P1/4 (ln2 < 0: sample order)
+  int ln2, lq1, lcw, lt4;  // log2 of the columns, Q1, CW and P1/4 (ln2 < 0: sample order)
   __host__ __device__ constexpr long long slot(long long n) const {
     if (ln2 < 0) return n;
     const long long row = n >> ln2, b = n & ((1LL << ln2) - 1), t = row >> lq1;
     const long long lane = ((row & ((1LL << lq1) - 1)) << lcw) | (b & ((1LL << lcw) - 1));
-    return (((((b >> lcw) << lt4) + (t >> 2)) * 32 + lane) << 2) + (t & 3);
+    return ((((((b >> lcw) << lt4) + (t >> 2)) << (lq1 + lcw)) + lane) << 2) + (t & 3);
   }
 };
 __host__ __device__ constexpr TapOrder tap_order(int logn) {
+  if (is_fused(logn)) return TapOrder{fused_log_b(logn), 0, fused_log_b(logn), logn - fused_log_b(logn) - 2};
   if (logn < kTapsOrderedMin) return TapOrder{-1, 0, 0, 0};
   const int ln2 = plan_log_n2(logn), n1 = 1 << (logn - ln2), p1 = plan_p1(logn, n1), lq1 = ct::ilog2(n1 / p1);
   return TapOrder{ln2, lq1, 5 - lq1, ct::ilog2(p1 / 4)};
