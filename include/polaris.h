@@ -198,14 +198,14 @@ int spectrometer_debug_unpack(polaris_spec* s, const void* packed, int64_t n, fl
 
 /* The data-translation step as the FFT kernel runs it from N = 2^13 up (Fig. 2 caption:
  * integer codes to floats; Sec. 2: two IF streams enter one transform): that kernel stages
- * each tile's packed words in shared memory and decodes every column at a per-column
- * rotation, both IFs of a pair in one packed subtraction.  This call stages and decodes
- * through that same device code, for bit-exact checks of the levels the transform sees.
+ * each tile's packed words in shared memory, transposes their codes so that the rows of one
+ * column share a word, and decodes both IFs of a pair together.  This call stages, transposes
+ * and decodes through that same device code, for bit-exact checks of the levels the transform
+ * sees.
  *   packed_a, packed_b  host words of IF a and IF b of one FFT pair (packed_b NULL: a pair
  *               without an IF b, decoded by the single-IF variant), n samples each;
  *   n           a positive multiple of n_fft (whole segments, hop = n_fft);
- *   layout      0: the interleaved stage of cp.async staging; 1: the dense [IF][row][word]
- *               stage of TMA staging;
+ *   layout      0: transposed into a second buffer; 1: transposed in place;
  *   out_a, out_b  host floats, n each (out_b unused when packed_b is NULL).
  * POLARIS_EINVAL when the FFT kernel does not stage at this handle's size and width (below
  * 2^13, and 1-bit samples at 2^19 and 2^20: there it decodes as spectrometer_debug_unpack). */
@@ -225,8 +225,8 @@ const char* spectrometer_last_error(const polaris_spec* s);
  * waits for those events and returns, per kind, the summed device time in ms and the
  * launch count since profiling began or since the previous query (kinds: 0 = phase 1,
  * decode/window/row DFT; 1 = phase 2, column DFT/correlate/accumulate (and the one kernel that
- * does both phases at n_fft of 1024 to 4096); 2 = readout and Stokes; 3 = code histogram).  n is the length of both arrays and must be >= 3; kinds
- * >= n are not reported. */
+ * does both phases at n_fft of 1024 to 4096); 2 = readout and Stokes; 3 = code histogram).
+ * n is the length of both arrays and must be >= 3; kinds >= n are not reported. */
 int64_t spectrometer_kernel_launches(const polaris_spec* s);
 int spectrometer_set_profiling(polaris_spec* s, int on);
 int spectrometer_kernel_times(polaris_spec* s, double* ms, int64_t* launches, int n);
@@ -382,8 +382,8 @@ void polaris_set_wait_limit(int64_t polls);
  * word, and the next synchronising call returns POLARIS_EBOUNDS.  Nothing traps.
  * polaris_checked_build: 1 in such a build, 0 otherwise.
  * polaris_set_check_understate (test hook, checked build only): on != 0 makes later feeds
- * tell the kernels half the slab (n_fft of 1024 to 4096: half the input) they have, so that the checks fire while every access
- * stays inside its buffer; POLARIS_EINVAL in a build without checks. */
+ * tell the kernels half the slab (n_fft of 1024 to 4096: half the input) they have, so that
+ * the checks fire while every access stays inside its buffer; POLARIS_EINVAL in a build without checks. */
 int polaris_checked_build(void);
 int polaris_set_check_understate(int on);
 

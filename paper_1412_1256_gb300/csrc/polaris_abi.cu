@@ -1097,7 +1097,7 @@ extern "C" int spectrometer_debug_unpack_staged(polaris_spec* s, const void* pac
   if (rc) return rc;
   if (!packed_a || !out_a || (packed_b && !out_b)) return set_err(s, POLARIS_EINVAL, "null pointer");
   if (n <= 0 || n % s->N) return set_err(s, POLARIS_EINVAL, "n must be a positive multiple of n_fft");
-  if (layout != 0 && layout != 1) return set_err(s, POLARIS_EINVAL, "layout must be 0 (interleaved) or 1 (dense)");
+  if (layout != 0 && layout != 1) return set_err(s, POLARIS_EINVAL, "layout must be 0 (transposed apart) or 1 (in place)");
   if (!phase1_staged(s->logn, s->bits))
     return set_err(s, POLARIS_EINVAL, "phase 1 does not stage its input at this size and width");
   DeviceGuard dg(s->device);

@@ -168,55 +168,14 @@ __device__ __forceinline__ float decode_level(uint32_t word, uint32_t shift) {
   }
 }
 
-// (a & b) | c and (a & b) ^ c as one three-input logic operation each (truth tables 0xEA and
-// 0x6A over the operand patterns 0xF0, 0xCC, 0xAA).  Written out because with two constant
-// operands the compiler spends two logic operations on each.
+// (a & b) | c as one three-input logic operation (truth table 0xEA over the operand patterns
+// 0xF0, 0xCC, 0xAA).  Written out because with two constant operands the compiler spends two
+// logic operations on it.
 __device__ __forceinline__ uint32_t and_or(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
   asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
   return d;
 }
-__device__ __forceinline__ uint32_t and_xor(uint32_t a, uint32_t b, uint32_t c) {
-  uint32_t d;
-  asm("lop3.b32 %0, %1, %2, %3, 0x6A;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-  return d;
-}
-
-// The same decode from a rotation of the word, for a lane that decodes the same bit
-// offset of many words: with rot = decode_rot<BITS>(shift) computed once, a code sits at
-// bits [1, BITS] (b < 8) or [0, 8) (b = 8) of rotr(word, rot), so one funnel shift, one
-// three-input logic op and one add give the level.
-template <int BITS>
-__host__ __device__ constexpr uint32_t decode_rot(uint32_t shift) {
-  return BITS == 8 ? shift : ((shift + 31u) & 31u);
-}
-template <int BITS>
-__device__ __forceinline__ float decode_level_rot(uint32_t word, uint32_t rot) {
-  const uint32_t r = __funnelshift_r(word, word, rot);
-  if constexpr (BITS == 8) {
-    return __uint_as_float(and_xor(r, 0xFFu, 0x4B000080u)) - 8388736.0f;  // 2^23 + (c ^ 0x80) - 2^23 - 128
-  } else {
-    return __uint_as_float(and_or(r, ((1u << BITS) - 1u) << 1, 0x4B000000u)) - (8388608.0f + (float)((1 << BITS) - 1));
-  }
-}
-
-// Both IFs' codes at one rotation into one complex sample, the two final subtractions as
-// one packed add (each component rounds as the scalar subtraction; exact here).
-template <int BITS>
-__device__ __forceinline__ float2 decode_pair_rot(uint32_t wa, uint32_t wb, uint32_t rot) {
-  const uint32_t ra = __funnelshift_r(wa, wa, rot), rb = __funnelshift_r(wb, wb, rot);
-  if constexpr (BITS == 8) {
-    return __fadd2_rn(make_float2(__uint_as_float(and_xor(ra, 0xFFu, 0x4B000080u)),
-                                  __uint_as_float(and_xor(rb, 0xFFu, 0x4B000080u))),
-                      make_float2(-8388736.0f, -8388736.0f));
-  } else {
-    constexpr uint32_t m = ((1u << BITS) - 1u) << 1;
-    constexpr float c = -(8388608.0f + (float)((1 << BITS) - 1));
-    return __fadd2_rn(make_float2(__uint_as_float(and_or(ra, m, 0x4B000000u)), __uint_as_float(and_or(rb, m, 0x4B000000u))),
-                      make_float2(c, c));
-  }
-}
-
 // ----------------------------------------------------------------------------------------
 // two-phase plan: N = N1 * N2, n = N2 a + b (a row, b column), k = c + N1 d
 //   phase 1: for each column b, DFT-N1 over a (P points per thread, Q1 = N1/P threads)
@@ -338,48 +297,71 @@ struct Plan {
   static constexpr int MINB1 = P1 <= 16 ? 3 : (P1 <= 32 ? 2 : 1);  // phase-1 CTAs per SM the registers aim at
   static constexpr int TCOLS1 = pow2_at_least((WARPS / 4) * TW1, 32);
   // CTA tiles of IPT * WARPS * CW columns inside one segment (Stage1<BITS>): the CTA stages
-  // the tile's packed words (both IFs) in shared memory; otherwise (small N) every lane loads
-  // its own words.  IPT column groups per warp per tile: two where the tile divides N2 and two
-  // stage buffers still leave room for two CTAs per SM (fewer CTA barriers and less staging
-  // work per column).  Four measured slower at 2^17: too few tiles per SM to balance.
+  // the tile's packed words (both IFs) in shared memory and transposes their codes there;
+  // otherwise (small N) every lane loads its own words.  IPT column groups per warp per tile:
+  // two where the tile divides N2 and the staged and the transposed words still leave room for
+  // two CTAs per SM (fewer CTA barriers and less staging work per column).  Four measured slower
+  // at 2^17: too few tiles per SM to balance.
   static constexpr size_t kSmemPerCta2 = (233472 - MINB1 * 1024) / MINB1;  // MINB1 CTAs per SM
   static constexpr size_t REGIONS1 = sizeof(float2) * (size_t)WARPS * REGION1;
   template <int BITS>
   struct Stage1 {
     static constexpr int tile_of(int ipt) { return ipt * WARPS * CW; }
-    static constexpr int wpr_of(int ipt) { return tile_of(ipt) * BITS / 32; }
-    // staged row: the tile's words of the two IFs interleaved (word w of IF a, of IF b, ...)
-    // so that one 8-byte load fetches both, padded to an odd number of 8-byte pairs (rows of
-    // distinct q1 then fall on distinct bank pairs)
-    static constexpr int row_words(int ipt) { return 2 * wpr_of(ipt) + (wpr_of(ipt) % 2 ? 0 : 2); }
-    static constexpr bool fits(int ipt, int bufs) {
-      return REGIONS1 + 4 * (size_t)bufs * N1 * row_words(ipt) + 32 <= kSmemPerCta2;
+    static constexpr int SPW = 32 / BITS;  // codes per word
+    // Transposed words (p1_transpose): SPW rows of one column in one word, BR words per column
+    // and lane q1 (both IFs; IF a's codes first), VL of them side by side.  Vector (q1, col) sits
+    // at q1 s_of + col + (col / SPW) PADW: PADW and the stride put the 8 vectors of 16 bytes (16
+    // of 8) that a warp's request takes at once on distinct banks, and spread the writers' words
+    // (bank simulation: the reads at the minimum, the writes at 1 to 4 times theirs)
+    static constexpr int BR = 2 * P1 / SPW, VL = BR < 4 ? BR : 4;
+    static constexpr int KB = BITS == 8 ? 4 : BITS == 4 ? 2 : 1;  // blocks a thread takes (words it stores at once)
+    static constexpr int PADW = CW >= 4 ? 1 : 0;
+    static constexpr int s_of(int ipt) {
+      int s = tile_of(ipt) + tile_of(ipt) / SPW * PADW;
+      while (CW < 8 && s % 8 != CW) ++s;
+      return s;
+    }
+    static constexpr size_t raw_bytes(int ipt) { return 2 * (size_t)N1 * tile_of(ipt) * BITS / 8; }
+    static constexpr size_t tr_bytes(int ipt) { return 4 * (size_t)Q1 * s_of(ipt) * BR; }
+    static constexpr bool fits(int ipt, bool in_place) {
+      const size_t r = raw_bytes(ipt), t = tr_bytes(ipt);
+      return REGIONS1 + (in_place ? (r > t ? r : t) : r + t) + 32 <= kSmemPerCta2;
     }
     // a tile of whole words that divides N2
     static constexpr bool aligned(int ipt) {
       return N2 % tile_of(ipt) == 0 && (tile_of(ipt) * BITS) % 32 == 0 && tile_of(ipt) * BITS >= 32;
     }
-    static constexpr bool ok(int ipt) { return aligned(ipt) && tile_of(ipt) % 32 == 0 && fits(ipt, 2); }
-    // Column groups per tile, 0 = not staged.  Tiles of 32 or more columns first; for
-    // N1 >= 512 (warps of one or two columns, whose unstaged loads would each touch 32
-    // sectors) any tile of whole words, preferring two stage buffers, then more columns.
+    static constexpr bool ok(int ipt) { return aligned(ipt) && tile_of(ipt) % 32 == 0 && fits(ipt, false); }
+    // Column groups per tile, 0 = not staged; + 10: transposed in place (one buffer, the next
+    // tile in flight only once the last column group has been decoded).  Tiles of 32 or more
+    // columns first; for N1 >= 512 (warps of one or two columns, whose unstaged loads would each
+    // touch 32 sectors) any tile of whole words, with two groups in place before one group apart
+    // at N1 >= 1024 (8-bit: 16 bytes per row and IF instead of 8, half the copies).
     static constexpr int pick() {
-      return ok(2)                                                 ? 2
-             : (N2 % tile_of(1) == 0 && tile_of(1) % 32 == 0)     ? 1
-             : N1 < 512                                           ? 0
-             : (aligned(2) && fits(2, 2))                         ? 2
-             : (aligned(1) && fits(1, 2))                         ? 1
-             : (aligned(2) && fits(2, 1))                         ? 2
-             : (aligned(1) && fits(1, 1))                         ? 1
-                                                                  : 0;
+      return ok(2)                                                                ? 2
+             : (N2 % tile_of(1) == 0 && tile_of(1) % 32 == 0 && fits(1, false))  ? 1
+             : N1 < 512                                                          ? 0
+             : (aligned(2) && fits(2, false))                                    ? 2
+             : (N1 >= 1024 && aligned(2) && fits(2, true))                       ? 12
+             : (aligned(1) && fits(1, false))                                    ? 1
+             : (aligned(2) && fits(2, true))                                     ? 12
+             : (aligned(1) && fits(1, true))                                     ? 11
+                                                                                 : 0;
     }
-    static constexpr int IPT = pick() > 0 ? pick() : 1;
+    // (1 bit at 2^19 and 2^20 stays unstaged)
+    static constexpr bool STAGED = pick() > 0 && !(BITS == 1 && LOGN >= 19);
+    static constexpr bool INPLACE = pick() >= 10;
+    static constexpr int IPT = STAGED ? pick() % 10 : 1;
     static constexpr int TILE = IPT * WARPS * CW;
-    static constexpr bool STAGED = pick() > 0;
     static constexpr int WPR = TILE * BITS / 32;  // words per IF per staged row
-    static constexpr int RS = row_words(IPT);
-    static constexpr int NB = fits(IPT, 2) ? 2 : 1;  // 2: the next tile in flight
-    static constexpr int WORDS = STAGED ? NB * N1 * RS : 0;
+    static constexpr int SQ = s_of(IPT);          // vectors between lanes q1
+    static constexpr int RAWW = STAGED ? (int)(raw_bytes(IPT) / 4) : 0, TRW = STAGED ? (int)(tr_bytes(IPT) / 4) : 0;
+    static constexpr int TR0 = INPLACE ? 0 : RAWW;  // where the transposed words start
+    static constexpr int WORDS = INPLACE ? (RAWW > TRW ? RAWW : TRW) : RAWW + TRW;
+    static constexpr int UNITS = WPR * Q1 * (BR / KB);  // transposing work units of a tile
+    static constexpr int VEC = WPR >= 4 ? 4 : WPR;      // words per cp.async of an aligned input
+    static_assert(!STAGED || (BR % VL == 0 && VL % KB == 0 && RAWW % 4 == 0 && (WPR & (WPR - 1)) == 0), "staged words");
+    static_assert(!INPLACE || UNITS % THREADS == 0, "whole units per thread");
     // TMA boxes are at most 256 rows: larger N1 moves by N1 / BOXR boxes per copy
     static constexpr int BOXR = N1 < 256 ? N1 : 256;
     // N1 <= 256: the warp's [N1][CW] output block leaves by one TMA store (rows of 32 bytes
@@ -392,10 +374,9 @@ struct Plan {
     static constexpr bool JOINT_OUT = STAGED && Q1 > 1 && N1 >= 512 && (JC * 8 == 64 || JC * 8 == 128) &&
                                       (size_t)N1 * JC * 8 <= REGIONS1;
     static constexpr int JSW = JC * 8 == 128 ? 7 : 3;  // swizzle mask: 128-byte (SW128) or 64-byte (SW64) rows
-    // the tile's input may be staged by TMA (two buffers, 16-byte box rows, one box of all
-    // N1 rows: at N1 = 512 two boxes of 256 rows measured slower than cp.async staging)
-    static constexpr bool TMA_IN = STAGED && NB == 2 && (WPR * 4) % 16 == 0 && N1 <= 256;
-    static constexpr size_t SMEM = REGIONS1 + 4 * (size_t)WORDS + 16 + 16;  // + 2 mbarriers + TMEM slot
+    // the tile's input may be staged by TMA (16-byte box rows, one box of all N1 rows)
+    static constexpr bool TMA_IN = STAGED && (WPR * 4) % 16 == 0 && N1 <= 256;
+    static constexpr size_t SMEM = REGIONS1 + 4 * (size_t)WORDS + 16 + 16;  // + mbarrier + TMEM slot
   };
 
   // phase 2: a warp owns UPW units; lane = (uw * 2 + e) * Q2 + q2 holds rows q2 + Q2 t

@@ -23,6 +23,7 @@
 #include <type_traits>
 #include <cudaTypedefs.h>
 
+#include "polaris_codes.cuh"
 #include "polaris_device.cuh"
 
 namespace polaris {
@@ -110,7 +111,9 @@ __device__ __forceinline__ long long seg_word0(const SegSrc& in, int s) {
 
 // Tensor maps of the packed input for phase 1's TMA staging: m[0][i] views IF i's staged
 // segments [0, n0) and m[1][i] its segments from n0 on, each as words x rows x segments.
-// use = 0: the kernel stages with cp.async instead (layouts a tensor map cannot describe).
+// use = 0: the kernel stages with 4-byte cp.async instead (layouts a tensor map cannot describe).
+// Where phase 1 has no tensor-map path (N1 >= 512), use = 1 says that rows are aligned for its
+// widest cp.async and no map is encoded.
 struct InMaps {
   CUtensorMap m[2][kMaxIF];
   int use;
@@ -123,6 +126,11 @@ __device__ __forceinline__ const uint32_t* seg_ptr(const SegSrc& in, int ifx, in
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
+}
+template <int BYTES>  // 4, 8 or 16, both addresses aligned to it
+__device__ __forceinline__ void cp_async(uint32_t dst, const void* src) {
+  if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(dst), "l"(src), "n"(BYTES) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
@@ -291,35 +299,6 @@ __device__ __forceinline__ void p1_load(const BatchArgs& a, int g, int b, int q1
   });
 }
 
-// Data translation of the staged phase 1 (N >= 2^13), shared with the bit-exactness check
-// (k_unpack_staged): column `col` of a tile starts at word p1_col_word(col) of each staged row,
-// and its code sits at rotation p1_col_rot(col) of that word.
-template <int BITS>
-__device__ __forceinline__ int p1_col_word(int col) { return (col * BITS) >> 5; }
-template <int BITS>
-__device__ __forceinline__ uint32_t p1_col_rot(int col) { return decode_rot<BITS>((uint32_t)((col * BITS) & 31)); }
-// The codes of staged row `row` at word wd, decoded at rotation rot, before the window:
-// (level of IF a, level of IF b) for a pair with an IF b (HB), else (level of IF a, 0).
-// Interleaved stage (cp.async, TL false): word w of IF a at 2w, of IF b at 2w + 1 of the
-// row's RS words.  Dense stage (TMA, TL true): [IF][row][WPR].
-template <int BITS, bool TL, bool HB, int N1, int WPR, int RS>
-__device__ __forceinline__ float2 p1_stage_decode(const uint32_t* sb, int row, int wd, uint32_t rot) {
-  uint32_t wa, wb = 0;
-  if constexpr (TL) {
-    wa = sb[row * WPR + wd];
-    if constexpr (HB) wb = sb[N1 * WPR + row * WPR + wd];
-  } else {
-    const uint2 w = *reinterpret_cast<const uint2*>(sb + row * RS + 2 * wd);  // IF a, IF b
-    wa = w.x;
-    wb = w.y;
-  }
-  if constexpr (HB) {
-    return decode_pair_rot<BITS>(wa, wb, rot);
-  } else {
-    return make_float2(decode_level_rot<BITS>(wa, rot), 0.0f);
-  }
-}
-
 __device__ __forceinline__ void corr_acc(float (&acc)[4], float2 U, float2 V) {
   // S = 2X, D = 2iY;  |S|^2, |D|^2, Re/Im of i S conj(D) (= 4 X conj(Y)).  S and D by packed
   // operations (each component rounds once, as the scalar sum and difference would)
@@ -392,17 +371,16 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
   }
   const int q1 = lane / CW, cw = lane % CW;
   float2* region = sm1 + warp * PL::REGION1;
-  uint32_t* stage = reinterpret_cast<uint32_t*>(sm1 + PL::WARPS * PL::REGION1);  // stage buffers
-  const uint32_t bar0 = smem_addr(stage + ST::WORDS);  // two mbarriers (TMA staging), then the TMEM slot
+  uint32_t* stage = reinterpret_cast<uint32_t*>(sm1 + PL::WARPS * PL::REGION1);  // staged, transposed words
+  const uint32_t bar0 = smem_addr(stage + ST::WORDS);  // mbarrier (TMA staging), then the TMEM slot
   uint32_t* tslot = stage + ST::WORDS + 4;
-  // TMA staging of the input: possible for this plan (two buffers, 16-byte box rows) and
-  // chosen by the host for this launch
+  // TMA staging of the input: possible for this plan (16-byte box rows) and chosen by the host
+  // for this launch
   constexpr bool TIN = ST::TMA_IN;
   static_assert(!TIN || (N1 % BOXR == 0 && (BOXR * WPR * 4) % 128 == 0), "TMA input boxes");
   const bool tin = TIN && in_maps.use != 0;
   if (TIN && tin && tid == 0) {
     mbar_init(bar0, 1);
-    mbar_init(bar0 + 8, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     fence_async_shared();
   }
@@ -574,76 +552,78 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
     }
   } else {
     // CTA tiles of TILE columns of one pair-segment.  The packed words of a tile (both IFs)
-    // are staged in shared memory with cp.async, double-buffered so that the next tile's
-    // words are in flight while the warps work on this one; every warp decodes its CW
-    // columns from the stage.
-    constexpr int RS = ST::RS;   // words per staged row
-    constexpr int SB = N1 * RS;  // words per stage buffer
-    constexpr int NB = ST::NB;   // 2: next tile in flight
+    // arrive in shared memory as dense rows ([IF][row][word]) while the warps work on the tile
+    // before; the CTA transposes their codes (polaris_codes.cuh), and every lane then takes its
+    // rows with a few vector loads.  (Decoding from the staged words themselves, a 4-byte load,
+    // a funnel shift and a logic operation per sample, bound this kernel: shared-memory pipe 77%
+    // busy at 2^14 and 8 bits, the loads up to four-way bank-conflicted; at N1 >= 512 the words
+    // came in 4-byte copies.  Kernel times before and after, beside the others of a pass: 15 x 2^20
+    // int8 Hann 113 -> 68 us, 122 x 2^18 int8 Hann 172 -> 109 us (of which the taps' order 27 us),
+    // 122 x 2^17 4-bit 30.2 -> 27.3 us; 2^17 2-bit unchanged alone, 1% in a three-handle pipeline.)
     const long long n_tiles = total_cols / TILE;
-    const uint32_t stage_a = smem_addr(stage);
-    // this thread's share of a tile's words: source offsets (words from the tile's first word
-    // of its row 0) and stage offsets (bytes), the same for every tile
-    constexpr int KW = N1 * WPR, KPT = (KW + PL::THREADS - 1) / PL::THREADS;
-    uint32_t soff[KPT], doff[KPT];
-    sfor<0, KPT>([&](auto i_) {
-      constexpr int i = decltype(i_)::value;
-      const int k = (int)threadIdx.x + i * PL::THREADS;
-      const int row = k / WPR, wd = k % WPR;
-      soff[i] = (uint32_t)(row * (N2 * BITS / 32) + wd);
-      doff[i] = 4u * (uint32_t)(row * RS + 2 * wd);
-    });
-    auto issue = [&](long long tile, int buf) {
+    uint32_t* tr = stage + ST::TR0;
+    const uint32_t raw_a = smem_addr(stage);
+    constexpr int ROWW = N2 * BITS / 32;  // words per row of a segment
+    auto issue_words = [&](long long tile, auto vec_) {
+      constexpr int V = decltype(vec_)::value;  // words per copy
       const int g = (int)(tile / (N2 / TILE)), b0 = (int)(tile % (N2 / TILE)) * TILE;
       const int s_local = g / a.n_fpair, f = g - s_local * a.n_fpair;
       const int sg = a.seg0 + s_local;
       const int ia = a.fa[f], ib = a.fb[f];
       const uint32_t* pa = seg_ptr(a.in, ia, sg) + (b0 * BITS) / 32;
       const uint32_t* pb = ib >= 0 ? seg_ptr(a.in, ib, sg) + (b0 * BITS) / 32 : pa;
-      const uint32_t dst0 = stage_a + 4u * (uint32_t)(buf * SB);
       const long long w0 = seg_word0(a.in, sg) + (b0 * BITS) / 32;
       const long long wext = sg < a.in.n0 ? a.in.in_words0 : a.in.in_words1;
-      sfor<0, KPT>([&](auto i_) {
-        constexpr int i = decltype(i_)::value;
-        if (KW % PL::THREADS == 0 || (int)threadIdx.x + i * PL::THREADS < KW) {
-          if (in_bounds(a.err, w0 + soff[i], wext)) {
-            cp_async4(dst0 + doff[i], pa + soff[i]);
-            cp_async4(dst0 + doff[i] + 4u, pb + soff[i]);  // (IF a again when the pair has no IF b)
-          }
+      constexpr int K = N1 * WPR / V;  // copies per IF
+#pragma unroll 4
+      for (int k = tid; k < K; k += PL::THREADS) {
+        const uint32_t so = (uint32_t)((k / (WPR / V)) * ROWW + (k % (WPR / V)) * V);
+        if (in_bounds(a.err, w0 + so + V - 1, wext)) {
+          cp_async<4 * V>(raw_a + 4u * (uint32_t)(k * V), pa + so);
+          cp_async<4 * V>(raw_a + 4u * (uint32_t)(N1 * WPR + k * V), pb + so);  // (IF a again without an IF b)
         }
-      });
+      }
       cp_async_commit();
     };
-    // TMA staging: one thread loads the tile's words of each IF (N1 rows x WPR words, in
-    // boxes of BOXR rows) into a dense [IF][row][word] stage and the CTA waits on that
-    // buffer's mbarrier (bounded)
-    auto issue_tma = [&](long long tile, int buf) {
+    auto issue = [&](long long tile) {
+      if (ST::VEC > 1 && !TIN && in_maps.use) issue_words(tile, std::integral_constant<int, ST::VEC>{});
+      else issue_words(tile, std::integral_constant<int, 1>{});
+    };
+    // TMA staging: one thread loads the tile's words of each IF (N1 rows x WPR words) and the
+    // CTA waits on the mbarrier (bounded)
+    auto issue_tma = [&](long long tile) {
       const int g = (int)(tile / (N2 / TILE)), b0 = (int)(tile % (N2 / TILE)) * TILE;
       const int s_local = g / a.n_fpair, f = g - s_local * a.n_fpair;
       const int sg = a.seg0 + s_local;
       const int ia = a.fa[f], ib = a.fb[f];
       const int src = sg < a.in.n0 ? 0 : 1, z = sg < a.in.n0 ? sg : sg - a.in.n0;
-      const uint32_t bar = bar0 + 8u * (uint32_t)buf, dst = stage_a + 4u * (uint32_t)(buf * SB);
-      const uint32_t box = (uint32_t)(N1 * WPR * 4), sub = (uint32_t)(BOXR * WPR * 4);  // bytes per IF, per box
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar),
+      const uint32_t box = (uint32_t)(N1 * WPR * 4);  // bytes per IF
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar0),
                    "r"(ib >= 0 ? 2 * box : box)
                    : "memory");
       const int x = (b0 * BITS) / 32;
       const uint64_t pol_in = l2_evict_first();
-      sfor<0, N1 / BOXR>([&](auto h_) {
-        constexpr int h = decltype(h_)::value;
+      asm volatile(
+          "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, "
+          "{%2, %3, %4}], [%5], %6;\n" ::"r"(raw_a),
+          "l"(&in_maps.m[src][ia]), "r"(x), "r"(0), "r"(z), "r"(bar0), "l"(pol_in)
+          : "memory");
+      if (ib >= 0)
         asm volatile(
             "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, "
-            "{%2, %3, %4}], [%5], %6;\n" ::"r"(dst + h * sub),
-            "l"(&in_maps.m[src][ia]), "r"(x), "r"(h * BOXR), "r"(z), "r"(bar), "l"(pol_in)
+            "{%2, %3, %4}], [%5], %6;\n" ::"r"(raw_a + box),
+            "l"(&in_maps.m[src][ib]), "r"(x), "r"(0), "r"(z), "r"(bar0), "l"(pol_in)
             : "memory");
-        if (ib >= 0)
-          asm volatile(
-              "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, "
-              "{%2, %3, %4}], [%5], %6;\n" ::"r"(dst + box + h * sub),
-              "l"(&in_maps.m[src][ib]), "r"(x), "r"(h * BOXR), "r"(z), "r"(bar), "l"(pol_in)
-              : "memory");
-      });
+    };
+    auto issue_next = [&](long long tile) {
+      if (tin) {
+        if (tid == 0) {
+          fence_async_shared();  // the CTA's reads of the staged words come before the copy
+          issue_tma(tile);
+        }
+      } else {
+        issue(tile);
+      }
     };
     // Work units: whole tiles for the complete rounds over the grid, then, for the last,
     // partial round, half tiles (one column group per warp; the whole tile is staged), so
@@ -653,44 +633,46 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
     if (IPT == 2 && n_tiles % G != 0) F = (n_tiles / G) * G;
     const long long n_units = F + (n_tiles - F) * (IPT == 2 ? 2 : 1);
     auto unit_tile = [&](long long u) { return u < F ? u : F + (u - F) / 2; };
-    uint32_t par[2] = {0u, 0u};
+    uint32_t par = 0;
     long long unit = blockIdx.x;
-    if (unit < n_units) {
-      if (tin) {
-        if (tid == 0) issue_tma(unit_tile(unit), 0);
-      } else {
-        issue(unit_tile(unit), 0);
-      }
-    }
-    for (int buf = 0; unit < n_units; unit += G, buf = (NB == 2) ? buf ^ 1 : 0) {
+    if (unit < n_units) issue_next(unit_tile(unit));
+    for (; unit < n_units; unit += G) {
       const long long tile = unit_tile(unit);
       const int it_begin = unit < F ? 0 : (int)((unit - F) & 1), it_end = unit < F ? IPT : it_begin + 1;
       int timed_out = 0;
       if (tin) {
-        const uint32_t bar = bar0 + 8u * (uint32_t)buf;
-        if (!mbar_wait_bounded(bar, par[buf], a.wait_limit)) {
+        if (!mbar_wait_bounded(bar0, par, a.wait_limit)) {
           timed_out = 1;
           if (lane == 0 && a.err) atomicExch(a.err, 1);
-          mbar_wait_bounded(bar, par[buf], kWaitAfterTimeout);  // the copy in flight lands first
+          mbar_wait_bounded(bar0, par, kWaitAfterTimeout);  // the copy in flight lands first
         }
-        par[buf] ^= 1u;
+        par ^= 1u;
       } else {
         cp_async_wait_all();
       }
-      // this tile's words are staged; every warp is done with the other buffer
+      // this tile's words are staged; every warp has decoded the tile before
       if (__syncthreads_or(timed_out)) break;
       const long long next = unit + G;
-      if constexpr (NB == 2) {
-        if (next < n_units) {
-          if (tin) {
-            if (tid == 0) {
-              fence_async_shared();  // the CTA's reads of that buffer come before the copy
-              issue_tma(unit_tile(next), buf ^ 1);
-            }
-          } else {
-            issue(unit_tile(next), buf ^ 1);
-          }
+      if constexpr (ST::INPLACE) {
+        constexpr int UPT = ST::UNITS / PL::THREADS;
+        uint32_t x[UPT][ST::KB][32 / BITS];
+        sfor<0, UPT>([&](auto i_) {
+          p1_unit_load<PL, ST, BITS>(stage, tid + decltype(i_)::value * PL::THREADS, x[decltype(i_)::value]);
+        });
+        __syncthreads();
+        sfor<0, UPT>([&](auto i_) {
+          p1_unit_store<PL, ST, BITS>(tr, tid + decltype(i_)::value * PL::THREADS, x[decltype(i_)::value]);
+        });
+        __syncthreads();
+      } else {
+#pragma unroll 1
+        for (int u = tid; u < ST::UNITS; u += PL::THREADS) {
+          uint32_t x[ST::KB][32 / BITS];
+          p1_unit_load<PL, ST, BITS>(stage, u, x);
+          p1_unit_store<PL, ST, BITS>(tr, u, x);
         }
+        __syncthreads();
+        if (next < n_units) issue_next(unit_tile(next));
       }
       if (next >= n_units) pdl_trigger();  // this CTA's last unit: phase 2 may be scheduled
       const int g = (int)(tile / (N2 / TILE)), b0 = (int)(tile % (N2 / TILE)) * TILE;
@@ -702,51 +684,39 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
       for (int it = it_begin; it < it_end; ++it) {
         const int col = (it * PL::WARPS + warp) * CW + cw;  // column inside the tile
         const long long b = b0 + col;
-        const int wd = p1_col_word<BITS>(col);
-        const uint32_t rot = p1_col_rot<BITS>(col);
-        const uint32_t* sb = stage + buf * SB;
         float2 v[P];
-        // decode the lane's rows; the stage layout (TL), the pair's shape (HB) and the
-        // window (TP) are uniform per tile
-        auto decode = [&](auto tl_, auto hb_, auto tp_) {
-          constexpr bool TL = decltype(tl_)::value, HB = decltype(hb_)::value, TP = decltype(tp_)::value;
+        uint32_t codes[ST::BR];
+        p1_lane_codes<PL, ST>(tr, q1, col, codes);
+        // decode the lane's rows; the pair's shape (HB) and the window (TP) are uniform per tile
+        auto decode = [&](auto hb_, auto tp_) {
+          constexpr bool HB = decltype(hb_)::value, TP = decltype(tp_)::value;
           [[maybe_unused]] const float4* tp =
               reinterpret_cast<const float4*>(a.taps) + (size_t)((b - cw) / CW) * (P / 4) * 32 + lane;
           [[maybe_unused]] float4 w4;
           sfor<0, P>([&](auto t_) {
             constexpr int t = decltype(t_)::value;
-            const int row = q1 + Q1 * t;
-            float2 z = p1_stage_decode<BITS, TL, HB, N1, WPR, RS>(sb, row, wd, rot);
+            float2 z = p1_level<PL, ST, BITS, HB, t>(codes);
             if constexpr (TP) {  // (four consecutive t per load: tap_order)
               if constexpr (t % 4 == 0) w4 = __ldg(tp + (t / 4) * 32);
               const float tv = t % 4 == 0 ? w4.x : t % 4 == 1 ? w4.y : t % 4 == 2 ? w4.z : w4.w;
-              z.x *= tv;
-              z.y *= tv;
+              z = __fmul2_rn(z, make_float2(tv, tv));
             }
             v[ct::bitrev(t, P)] = z;
           });
         };
         using T_ = std::true_type;
         using F_ = std::false_type;
-        auto decode_tl = [&](auto tl) {
-          if (a.taps) {
-            if (has_b) decode(tl, T_{}, T_{});
-            else decode(tl, F_{}, T_{});
-          } else {
-            if (has_b) decode(tl, T_{}, F_{});
-            else decode(tl, F_{}, F_{});
-          }
-        };
-        if constexpr (TIN) {
-          if (tin) decode_tl(T_{});
-          else decode_tl(F_{});
+        if (a.taps) {
+          if (has_b) decode(T_{}, T_{});
+          else decode(F_{}, T_{});
         } else {
-          decode_tl(F_{});
+          if (has_b) decode(T_{}, F_{});
+          else decode(F_{}, F_{});
         }
-        if constexpr (NB == 1) {
+        if constexpr (ST::INPLACE) {
           if (it == it_end - 1) {
-            __syncthreads();  // every warp has decoded the tile: the single buffer is free
-            if (next < n_units) issue(unit_tile(next), 0);
+            __syncthreads();  // every warp has decoded the tile: the buffer is free
+            if (next < n_units) issue_next(unit_tile(next));
           }
         }
         finish(v, true, g, b, b0 + (it * PL::WARPS + warp) * CW);
@@ -1283,6 +1253,18 @@ static cudaError_t launch_phase1(const BatchArgs& a, cudaStream_t st, bool pdl) 
             ok = encode_input_map(&ms->in.m[src][ifx], base, PL::N2 * BITS / 32, PL::N1, ST::BOXR, nseg_src,
                                   row_bytes, seg_bytes, ST::WPR) == cudaSuccess;
           }
+        }
+      ms->in.use = ok ? 1 : 0;
+    } else if constexpr (ST::STAGED && ST::VEC > 1) {
+      // rows of VEC words aligned for the widest cp.async?
+      constexpr uintptr_t m = 4 * ST::VEC - 1;
+      bool ok = (a.in.hop_w * 4 & (long long)m) == 0;
+      for (int f = 0; f < a.n_fpair && ok; ++f)
+        for (int k = 0; k < 2 && ok; ++k) {
+          const int ifx = k == 0 ? a.fa[f] : a.fb[f];
+          if (ifx < 0) continue;
+          if (key.nsrc[0][ifx] > 0) ok = (reinterpret_cast<uintptr_t>(a.in.src0[ifx]) & m) == 0;
+          if (key.nsrc[1][ifx] > 0) ok = ok && (reinterpret_cast<uintptr_t>(a.in.src1[ifx]) & m) == 0;
         }
       ms->in.use = ok ? 1 : 0;
     }
