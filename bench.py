@@ -95,8 +95,8 @@ def fp32_peak_tflops(num_sms: int, sm_mhz: float) -> float:
 
 KERNEL_SOURCES = {
     # files whose contents define each timed kernel (a traffic record is valid for these only)
-    "phase1_decode_rowdft": ("polaris_device.cuh", "polaris_kernels.cuh", "polaris_n17.cu"),
-    "phase2_coldft_correlate": ("polaris_device.cuh", "polaris_kernels.cuh", "polaris_n17.cu"),
+    "phase1_decode_rowdft": ("polaris_device.cuh", "polaris_codes.cuh", "polaris_kernels.cuh", "polaris_n17.cu"),
+    "phase2_coldft_correlate": ("polaris_device.cuh", "polaris_codes.cuh", "polaris_kernels.cuh", "polaris_n17.cu"),
     "readout_stokes": ("polaris_abi.cu",),
 }
 
