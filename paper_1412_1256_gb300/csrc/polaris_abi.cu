@@ -74,6 +74,55 @@ __global__ void k_unpack(const uint32_t* __restrict__ w, long long n, float* __r
 }
 
 // ---------------------------------------------------------------------------------------
+// carried samples: the copies between feeds (carry and new samples into the staging buffer of
+// the segments that straddle two feeds, the tail of the stream into the next carry), all of a
+// feed's in one launch.  As one cudaMemcpyAsync each (up to three per IF) they cost about 3 us
+// of host time and 1.4 us of device time apiece: seven feeds of three IFs at 2^12 took 269 us.
+// ---------------------------------------------------------------------------------------
+constexpr int kMaxCopies = 4 * kMaxIF;
+struct CopyArgs {
+  uint32_t* dst[kMaxCopies];
+  const uint32_t* src[kMaxCopies];
+  long long words[kMaxCopies];
+};
+constexpr int kCopyThreads = 256;
+
+// blockIdx.y: the copy; 16 bytes per load where both ends are aligned to it, else 4
+__global__ void __launch_bounds__(kCopyThreads) k_feed_copies(CopyArgs a) {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");  // the buffers' last readers have ended
+  uint32_t* dst = a.dst[blockIdx.y];
+  const uint32_t* src = a.src[blockIdx.y];
+  const long long n = a.words[blockIdx.y], step = (long long)gridDim.x * kCopyThreads;
+  const long long t = (long long)blockIdx.x * kCopyThreads + threadIdx.x;
+  long long done = 0;
+  if (((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15) == 0) {
+    done = n & ~3LL;
+    for (long long i = t; i < done / 4; i += step)
+      reinterpret_cast<uint4*>(dst)[i] = __ldcs(reinterpret_cast<const uint4*>(src) + i);
+  }
+  for (long long i = done + t; i < n; i += step) dst[i] = __ldcs(src + i);
+}
+
+static cudaError_t launch_feed_copies(const CopyArgs& a, int n, int num_sms, cudaStream_t st, bool pdl) {
+  long long most = 0;
+  for (int i = 0; i < n; ++i) most = a.words[i] > most ? a.words[i] : most;
+  long long bx = (most + 4 * kCopyThreads - 1) / (4 * kCopyThreads);  // four words per thread, one wave at most
+  const long long cap = (8LL * num_sms + n - 1) / n;
+  if (bx > cap) bx = cap;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(bx < 1 ? 1 : bx), (unsigned)n);
+  cfg.blockDim = dim3(kCopyThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_feed_copies, a);
+}
+
+// ---------------------------------------------------------------------------------------
 // readout + Stokes (Eq. 2).  One thread per output bin k and FFT pair f.
 // Native accumulator order of FFT pair f (k = c + N1 d):
 //   c = 0         : slot d              (d = 0 .. N2/2)
@@ -821,16 +870,38 @@ extern "C" int spectrometer_feed(polaris_spec* s, const void* const* packed, int
   const int64_t total = carry + n;
   const int64_t nseg = total >= N ? (total - N) / hop + 1 : 0;
   const int64_t n0 = nseg < (carry + hop - 1) / hop ? nseg : (carry + hop - 1) / hop;
-  uint32_t* cur_carry = s->d_carry[s->carry_sel];
-  if (n0 > 0) {
-    const int64_t stage_len = (n0 - 1) * hop + N;  // samples: carry + (stage_len - carry) new ones
+  // the segments that start in the carried samples are assembled in the staging buffer; the
+  // samples after the last whole segment, stream positions [nseg*hop, total), are carried on
+  const int64_t keep0 = nseg * hop, keep = total - keep0;
+  {
+    CopyArgs c;
+    int nc = 0;
+    auto copy = [&](uint32_t* dst, const uint32_t* from, int64_t samples) {
+      if (samples <= 0) return;
+      c.dst[nc] = dst;
+      c.src[nc] = from;
+      c.words[nc++] = samples / spw;
+    };
     for (int i = 0; i < s->n_if; ++i) {
-      uint32_t* dst = s->d_stage + (size_t)i * s->stage_words_cap;
-      if (carry)
-        CUDA_OR_FAIL(s, cudaMemcpyAsync(dst, cur_carry + (size_t)i * s->carry_words_cap, (size_t)(carry / spw) * 4,
-                                        cudaMemcpyDeviceToDevice, st));
-      CUDA_OR_FAIL(s, cudaMemcpyAsync(dst + carry / spw, src[i], (size_t)((stage_len - carry) / spw) * 4,
-                                      cudaMemcpyDeviceToDevice, st));
+      const uint32_t* cur = s->d_carry[s->carry_sel] + (size_t)i * s->carry_words_cap;
+      uint32_t* nxt = s->d_carry[s->carry_sel ^ 1] + (size_t)i * s->carry_words_cap;
+      if (n0 > 0) {
+        uint32_t* dst = s->d_stage + (size_t)i * s->stage_words_cap;
+        copy(dst, cur, carry);
+        copy(dst + carry / spw, src[i], (n0 - 1) * hop + N - carry);
+      }
+      if (keep0 >= carry) {
+        copy(nxt, src[i] + (keep0 - carry) / spw, keep);
+      } else {
+        copy(nxt, cur + keep0 / spw, carry - keep0);
+        copy(nxt + (carry - keep0) / spw, src[i], n);
+      }
+    }
+    if (nc > 0) {
+      const cudaError_t e = counted_launch(s, 4, st, [&]() {
+        return launch_feed_copies(c, nc, s->num_sms, st, !s->profiling);
+      });
+      if (e != cudaSuccess) return set_err(s, POLARIS_ECUDA, "carry copies: %s", cudaGetErrorString(e));
     }
   }
   BatchArgs a;
@@ -922,21 +993,6 @@ extern "C" int spectrometer_feed(polaris_spec* s, const void* const* packed, int
     // join: phase 2 of the last batch follows every phase 1, so waiting on st_p2 suffices
     CUDA_OR_FAIL(s, cudaEventRecord(s->ev_join, s->st_p2));
     CUDA_OR_FAIL(s, cudaStreamWaitEvent(st, s->ev_join, 0));
-  }
-  // carry the samples after the last whole segment: stream positions [nseg*hop, total)
-  const int64_t keep0 = nseg * hop, keep = total - keep0;
-  uint32_t* nxt = s->d_carry[s->carry_sel ^ 1];
-  for (int i = 0; i < s->n_if && keep > 0; ++i) {
-    uint32_t* dst = nxt + (size_t)i * s->carry_words_cap;
-    if (keep0 >= carry) {
-      CUDA_OR_FAIL(s, cudaMemcpyAsync(dst, src[i] + (keep0 - carry) / spw, (size_t)(keep / spw) * 4,
-                                      cudaMemcpyDeviceToDevice, st));
-    } else {
-      const int64_t from_old = carry - keep0;
-      CUDA_OR_FAIL(s, cudaMemcpyAsync(dst, cur_carry + (size_t)i * s->carry_words_cap + keep0 / spw,
-                                      (size_t)(from_old / spw) * 4, cudaMemcpyDeviceToDevice, st));
-      CUDA_OR_FAIL(s, cudaMemcpyAsync(dst + from_old / spw, src[i], (size_t)(n / spw) * 4, cudaMemcpyDeviceToDevice, st));
-    }
   }
   s->carry_sel ^= 1;
   s->carry_len = keep;
