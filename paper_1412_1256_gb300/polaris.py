@@ -9,6 +9,7 @@ no fallback: if the library is missing or cannot be loaded, every call raises.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import threading
 
@@ -449,6 +450,15 @@ class Adjoint:
     def run(self, packed, n_samples: int, window, gains, leak, target=None, grads: bool = False, stream=None):
         """dict(stokes [4, nb], loss (float64, 1 element) and, with grads=True, grad_window [N],
         grad_gains [4], grad_leak [2, nb, 2]).  packed: two CUDA tensors of packed words."""
+        return self._run(packed, n_samples, window, gains, leak, target, grads, stream)[0]
+
+    def _split(self, flat):
+        """grad_window, grad_gains and grad_leak as they lie in one buffer."""
+        n, nb = self.n_fft, self.n_bins
+        return flat[:n], flat[n:n + 4], flat[n + 4:].view(2, nb, 2)
+
+    def _run(self, packed, n_samples: int, window, gains, leak, target, grads: bool, stream):
+        """run()'s outputs, and the buffer that holds the three gradients."""
         import torch
 
         dev = window.device
@@ -456,10 +466,10 @@ class Adjoint:
         out = {"stokes": torch.empty((4, nb), dtype=torch.float32, device=dev)}
         if target is not None:
             out["loss"] = torch.empty((1,), dtype=torch.float64, device=dev)
+        flat = None
         if grads:
-            out["grad_window"] = torch.empty((self.n_fft,), dtype=torch.float32, device=dev)
-            out["grad_gains"] = torch.empty((4,), dtype=torch.float32, device=dev)
-            out["grad_leak"] = torch.empty((2, nb, 2), dtype=torch.float32, device=dev)
+            flat = torch.empty((self.n_fft + 4 + 4 * nb,), dtype=torch.float32, device=dev)
+            out["grad_window"], out["grad_gains"], out["grad_leak"] = self._split(flat)
         arr = (ctypes.c_void_p * 2)(*[_ptr(p) for p in packed])
         ins = [t.contiguous() for t in (window, gains, leak)]
         tgt = None if target is None else target.contiguous()
@@ -471,31 +481,38 @@ class Adjoint:
                                     _ptr(out["grad_leak"]) if grads else None, _stream_ptr(stream))
         if rc != OK:
             raise PolarisError(rc, load().polaris_adj_last_error(self._h).decode())
-        return out
+        return out, flat
+
+
+@functools.lru_cache(maxsize=None)
+def _leakage_function():
+    """The autograd function of leakage_loss (made once: a class made per call cost about 100 us)."""
+    import torch
+
+    class _LeakageLoss(torch.autograd.Function):
+        @staticmethod
+        def forward(ctx, w, g, d, data):
+            adj, packed, n_samples, target = data  # (in a tuple: not part of the graph)
+            need = any(ctx.needs_input_grad)
+            r, flat = adj._run(packed, n_samples, w.detach(), g.detach(), d.detach(), target, need,
+                               torch.cuda.current_stream(w.device))
+            if need:
+                ctx.adj = adj
+                ctx.save_for_backward(flat)
+            return r["loss"][0]
+
+        @staticmethod
+        def backward(ctx, gout):
+            (flat,) = ctx.saved_tensors
+            return (*ctx.adj._split(flat * gout), None)  # (gout is one value: float32 stays)
+
+    return _LeakageLoss
 
 
 def leakage_loss(adj: "Adjoint", packed, n_samples: int, window, gains, leak, target):
     """The calibration loss as a differentiable function of window, gains and leak
     (torch.autograd), its gradient from the library's adjoint."""
-    import torch
-
-    class _LeakageLoss(torch.autograd.Function):
-        @staticmethod
-        def forward(ctx, w, g, d):
-            need = any(ctx.needs_input_grad)
-            r = adj.run(packed, n_samples, w.detach(), g.detach(), d.detach(), target, grads=need,
-                        stream=torch.cuda.current_stream(w.device))
-            if need:
-                ctx.save_for_backward(r["grad_window"], r["grad_gains"], r["grad_leak"])
-            return r["loss"][0]
-
-        @staticmethod
-        def backward(ctx, gout):
-            gw, gg, gd = ctx.saved_tensors
-            s = gout.to(torch.float32)
-            return s * gw, s * gg, s * gd
-
-    return _LeakageLoss.apply(window, gains, leak)
+    return _leakage_function().apply(window, gains, leak, (adj, packed, n_samples, target))
 
 
 class TensorCoreSpectrometer:
@@ -552,14 +569,14 @@ class TensorCoreSpectrometer:
         """dict(autos [2, nb], cross [nb] complex128, stokes [4, nb], n_segments) on the host."""
         import torch
 
+        # one device buffer and one copy for the three outputs; the cross spectrum's (re, im) pairs
+        # are complex values as they lie
         nb = self.n_bins
-        dev = torch.device("cuda", self.device)
-        autos = torch.empty((2, nb), dtype=torch.float64, device=dev)
-        cross = torch.empty((nb, 2), dtype=torch.float64, device=dev)
-        stokes = torch.empty((4, nb), dtype=torch.float64, device=dev)
+        buf = torch.empty((8, nb), dtype=torch.float64, device=torch.device("cuda", self.device))
+        p = buf.data_ptr()
         nseg = ctypes.c_int64()
-        self._check(load().polaris_tc_integrate(self._h, _ptr(autos), _ptr(cross), _ptr(stokes), ctypes.byref(nseg),
+        self._check(load().polaris_tc_integrate(self._h, p, p + 16 * nb, p + 32 * nb, ctypes.byref(nseg),
                                                 _stream_ptr(stream)))
-        c = cross.cpu().numpy()
-        return {"autos": autos.cpu().numpy(), "cross": c[:, 0] + 1j * c[:, 1], "stokes": stokes.cpu().numpy(),
+        host = buf.cpu().numpy()
+        return {"autos": host[:2], "cross": host[2:4].reshape(-1).view(np.complex128), "stokes": host[4:],
                 "n_segments": nseg.value}
