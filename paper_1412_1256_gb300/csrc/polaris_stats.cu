@@ -19,7 +19,23 @@ struct HistArgs {
   int* err;                  // status word (the bounds-checked build records a bad index)
 };
 
-// counts of each code value in one 32-bit word (codes are the word's bits / BITS fields)
+// 4-bit words: one indicator bit per nibble and code, from the products of the codes' low and
+// high bit pairs, added nibble by nibble (up to 15 words) and summed by fold_nibbles.  A population
+// count per code and word instead (16 per word, a quarter-rate instruction) bound this kernel.
+__device__ __forceinline__ void mark_nibbles(uint32_t w, uint32_t (&n)[16]) {
+  const uint32_t m = 0x11111111u, w1 = w >> 1, w2 = w >> 2, w3 = w >> 3;
+  const uint32_t lo[4] = {~w & ~w1 & m, w & ~w1 & m, ~w & w1 & m, w & w1 & m};
+  const uint32_t hi[4] = {~w2 & ~w3 & m, w2 & ~w3 & m, ~w2 & w3 & m, w2 & w3 & m};
+#pragma unroll
+  for (int v = 0; v < 16; ++v) n[v] += lo[v & 3] & hi[v >> 2];
+}
+__device__ __forceinline__ void fold_nibbles(const uint32_t (&n)[16], uint32_t (&c)[16]) {
+#pragma unroll
+  for (int v = 0; v < 16; ++v)
+    c[v] = __dp4a((n[v] & 0x0F0F0F0Fu) + ((n[v] >> 4) & 0x0F0F0F0Fu), 0x01010101u, c[v]);
+}
+
+// counts of each code value in one 32-bit word (codes are the word's bits / BITS fields; 1, 2 and 8 bits)
 template <int BITS>
 __device__ __forceinline__ void count_word(uint32_t w, uint32_t (&c)[(BITS <= 4) ? (1 << BITS) : 1],
                                            uint32_t* sh) {
@@ -34,14 +50,6 @@ __device__ __forceinline__ void count_word(uint32_t w, uint32_t (&c)[(BITS <= 4)
     c[2] += n2;
     c[1] += n1;
     c[0] += 16u - n1 - n2 - n3;
-  } else if constexpr (BITS == 4) {
-    const uint32_t m = 0x11111111u;
-    const uint32_t b0 = w & m, b1 = (w >> 1) & m, b2 = (w >> 2) & m, b3 = (w >> 3) & m;
-#pragma unroll
-    for (int v = 0; v < 16; ++v) {
-      const uint32_t x = ((v & 1) ? b0 : ~b0) & ((v & 2) ? b1 : ~b1) & ((v & 4) ? b2 : ~b2) & ((v & 8) ? b3 : ~b3) & m;
-      c[v] += __popc(x);
-    }
   } else {
 #pragma unroll
     for (int j = 0; j < 4; ++j) atomicAdd(sh + ((w >> (8 * j)) & 0xFFu), 1u);
@@ -52,10 +60,13 @@ __device__ __forceinline__ void count_word(uint32_t w, uint32_t (&c)[(BITS <= 4)
 // summed in registers, then over the block in shared memory, so that each block adds
 // one value per code to the global histogram (few, wide blocks per IF: the global
 // atomics all hit the same 2^b addresses).
-constexpr int kHistThreads = 512, kHistWords = 16;  // words per thread per pass, all loads in flight
+constexpr int kHistThreads = 512;
+// words per thread per pass, all loads in flight (4 bits: what a nibble can count)
+constexpr int hist_words(int bits) { return bits == 4 ? 15 : 16; }
 
 template <int BITS>
 __global__ void __launch_bounds__(kHistThreads, 2) k_code_hist(HistArgs a) {
+  constexpr int kHistWords = hist_words(BITS);
   constexpr int NC = 1 << BITS, NR = (BITS <= 4) ? NC : 1, NW = kHistThreads / 32;
   __shared__ uint32_t sh[NC * (BITS == 8 ? 1 : NW)];  // 8-bit: the block's bins; else [warp][code]
   const int ifx = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -87,18 +98,25 @@ __global__ void __launch_bounds__(kHistThreads, 2) k_code_hist(HistArgs a) {
           w[j] = __ldg((s < n0 ? src0 : src1) + o);
       }
     }
+    if constexpr (BITS == 4) {
+      uint32_t n[16];
 #pragma unroll
-    for (int j = 0; j < kHistWords; ++j) {
-      if (base + (long long)j * kHistThreads + threadIdx.x < total) count_word<BITS>(w[j], c, sh);
+      for (int v = 0; v < 16; ++v) n[v] = 0;
+#pragma unroll
+      for (int j = 0; j < kHistWords; ++j)
+        if (base + (long long)j * kHistThreads + threadIdx.x < total) mark_nibbles(w[j], n);
+      fold_nibbles(n, c);
+    } else {
+#pragma unroll
+      for (int j = 0; j < kHistWords; ++j)
+        if (base + (long long)j * kHistThreads + threadIdx.x < total) count_word<BITS>(w[j], c, sh);
     }
   }
   unsigned long long* h = a.hist + (size_t)ifx * NC;
   if constexpr (BITS <= 4) {
 #pragma unroll
     for (int v = 0; v < NC; ++v) {
-      uint32_t x = c[v];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      const uint32_t x = __reduce_add_sync(0xffffffffu, c[v]);
       if (lane == 0) sh[warp * NC + v] = x;
     }
     __syncthreads();
@@ -126,7 +144,7 @@ cudaError_t launch_code_hist(const SegSrc& in, int n_if, int bits, int nseg, int
   a.hist = hist;
   a.err = err;
   const long long total = (long long)nseg << wl;
-  const long long chunk = (long long)kHistThreads * kHistWords;
+  const long long chunk = (long long)kHistThreads * hist_words(bits);
   long long bx = (total + chunk - 1) / chunk;                 // one pass per block where possible
   const long long cap = (2LL * num_sms + n_if - 1) / n_if;  // at most two blocks per SM over all IFs
   if (bx > cap) bx = cap;
