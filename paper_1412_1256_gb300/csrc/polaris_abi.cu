@@ -372,6 +372,8 @@ using namespace polaris;
 // ---------------------------------------------------------------------------------------
 // handle
 // ---------------------------------------------------------------------------------------
+constexpr size_t kStatusBytes = 256;
+
 struct polaris_spec {
   int n_if = 0, bits = 0, window = 0, accum_fp64 = 0, device = 0, num_sms = 0;
   int logn = 0;
@@ -397,8 +399,8 @@ struct polaris_spec {
   float* d_out_cross = nullptr;
   float* d_out_stokes = nullptr;
   int code_stats = 0;
-  unsigned long long* d_hist = nullptr;  // [n_if][2^bits] code counts (code_stats only)
   int* d_err = nullptr;                  // device status word written by the phase kernels
+  unsigned long long* d_hist = nullptr;  // [n_if][2^bits] code counts (code_stats only), kStatusBytes after d_err
   cudaEvent_t ev_h2d = nullptr;
   // two internal streams: phase 1 of batch b+1 runs beside phase 2 of batch b; the
   // slab is split into two halves used by alternate batches
@@ -523,7 +525,6 @@ static void free_all(polaris_spec* s) {
   cudaFree(s->d_out_autos);
   cudaFree(s->d_out_cross);
   cudaFree(s->d_out_stokes);
-  cudaFree(s->d_hist);
   cudaFree(s->d_err);
   if (s->ev_h2d) cudaEventDestroy(s->ev_h2d);
 }
@@ -710,8 +711,9 @@ extern "C" int spectrometer_create(const polaris_config* cfg, polaris_spec** out
             alloc((void**)&s->d_out_cross, (size_t)s->nbin * 8 * (n_pair ? n_pair : 1)) &&
             alloc((void**)&s->d_out_stokes, (size_t)s->nbin * 16 * (n_pair ? n_pair : 1));
   if (ok && c.window != POLARIS_WIN_RECT) ok = alloc((void**)&s->d_taps, N * 4);
-  if (ok && c.code_stats) ok = alloc((void**)&s->d_hist, bytes_hist);
-  if (ok) ok = alloc((void**)&s->d_err, 256);
+  if (ok) ok = alloc((void**)&s->d_err, kStatusBytes + bytes_hist);
+  if (ok && c.code_stats)
+    s->d_hist = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(s->d_err) + kStatusBytes);
   if (!ok) {
     cudaGetLastError();
     free_all(s);
@@ -738,8 +740,7 @@ extern "C" int spectrometer_create(const polaris_config* cfg, polaris_spec** out
     e = cudaMemcpy(s->d_taps, taps.data(), N * 4, cudaMemcpyHostToDevice);
   }
   if (e == cudaSuccess) e = cudaMemset(s->d_acc, 0, acc_bytes);
-  if (e == cudaSuccess && c.code_stats) e = cudaMemset(s->d_hist, 0, bytes_hist);
-  if (e == cudaSuccess) e = cudaMemset(s->d_err, 0, 256);
+  if (e == cudaSuccess) e = cudaMemset(s->d_err, 0, kStatusBytes + bytes_hist);
   s->code_stats = c.code_stats;
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->ev_h2d, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->st_p1, cudaStreamNonBlocking);
@@ -780,15 +781,9 @@ static int check_usable(polaris_spec* s) {
   return POLARIS_OK;
 }
 
-// After a synchronisation: a phase kernel that gave up a bounded wait has set the status
-// word (its outputs are NaN); the handle becomes unusable.
-static int check_device_status(polaris_spec* s) {
-  int st = 0;
-  const cudaError_t e = cudaMemcpy(&st, s->d_err, sizeof st, cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) {
-    s->broken = true;
-    return set_err(s, POLARIS_ECUDA, "status read: %s", cudaGetErrorString(e));
-  }
+// The status word read after a synchronisation: a phase kernel that gave up a bounded wait has
+// set it (its outputs are NaN); the handle becomes unusable.
+static int check_device_status(polaris_spec* s, int st) {
   if (st == kErrBounds) {
     set_err(s, POLARIS_EBOUNDS, "an index check of the bounds-checked build failed; outputs are NaN");
     s->broken = true;
@@ -800,6 +795,53 @@ static int check_device_status(polaris_spec* s) {
     return POLARIS_ETIMEOUT;
   }
   return POLARIS_OK;
+}
+
+// A synchronous host feed goes over in pieces of 8 MB or more, four at most.  Whole passes of
+// four IFs (copy in, kernels, spectra back) with one / two / three / four pieces: 122 x 2^17 int8
+// (64 MB) 488 / 435 / 422 / 416 us, 976 x 2^14 int8 Hann (64 MB) 473 / 419 / 407 / 400 us; 61 x
+// 2^17 4-bit with code statistics (16 MB) 243 / 227 / 246 / 246 us (each piece costs about 20 us of
+// host time in launches); 8 MB and less: no gain.
+constexpr int64_t kPieceBytes = 8 << 20;
+constexpr int kMaxPieces = 4;
+
+// words [w0, w1) of every IF's nw host words into the handle's input buffer
+static cudaError_t copy_input(polaris_spec* s, const void* const* packed, int64_t w0, int64_t w1, int64_t nw,
+                              cudaStream_t st) {
+  // IF streams at one constant stride (rows of one host array, say) go over in one
+  // pitched copy: one API call instead of one per IF (each costs host time).  The CUDA driver
+  // refuses (at the call, queueing nothing) a pitched copy whose rows lie in different
+  // pinned allocations; then the streams go one by one.
+  const long long stride = s->n_if > 1 ? (long long)((const char*)packed[1] - (const char*)packed[0]) : 0;
+  bool uniform = s->n_if > 1 && stride >= nw * 4;
+  for (int i = 2; i < s->n_if && uniform; ++i)
+    uniform = (long long)((const char*)packed[i] - (const char*)packed[i - 1]) == stride;
+  const size_t bytes = (size_t)(w1 - w0) * 4;
+  const char* first = (const char*)packed[0] + w0 * 4;
+  if (uniform) {
+    // contiguous on both sides (no gap between rows): one linear copy, the cheapest call
+    const bool linear = stride == (long long)bytes && s->in_words_cap * 4 == (int64_t)bytes;
+    const cudaError_t ec =
+        linear ? cudaMemcpyAsync(s->d_in, first, bytes * s->n_if, cudaMemcpyHostToDevice, st)
+               : cudaMemcpy2DAsync(s->d_in + w0, (size_t)s->in_words_cap * 4, first, (size_t)stride, bytes,
+                                   (size_t)s->n_if, cudaMemcpyHostToDevice, st);
+    if (ec == cudaSuccess) return ec;
+    cudaGetLastError();
+  }
+  for (int i = 0; i < s->n_if; ++i) {
+    const cudaError_t e = cudaMemcpyAsync(s->d_in + (size_t)i * s->in_words_cap + w0, (const char*)packed[i] + w0 * 4,
+                                          bytes, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+// pieces of a synchronous host feed of `bytes` that completes nseg segments
+static int feed_pieces(int64_t bytes, int64_t nseg) {
+  int64_t k = bytes / kPieceBytes;
+  if (k > kMaxPieces) k = kMaxPieces;
+  if (k > nseg / 8) k = nseg / 8;
+  return k < 1 ? 1 : (int)k;
 }
 
 extern "C" int spectrometer_feed(polaris_spec* s, const void* const* packed, int64_t n, int on_device,
@@ -821,7 +863,19 @@ extern "C" int spectrometer_feed(polaris_spec* s, const void* const* packed, int
   DeviceGuard dg(s->device);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   const int64_t nw = n / s->spw;
+  const int64_t N = s->N, hop = s->hop, spw = s->spw;
+  const int64_t carry = s->carry_len;
+  const int64_t total = carry + n;
+  const int64_t nseg = total >= N ? (total - N) / hop + 1 : 0;
+  const int64_t n0 = nseg < (carry + hop - 1) / hop ? nseg : (carry + hop - 1) / hop;
   const uint32_t* src[kMaxIF] = {nullptr};
+  // A large synchronous host feed goes over in pieces on an internal stream, and the kernels of
+  // a piece run beside the copy of the next.  (Asynchronous feeds do not: their callers keep
+  // several handles in flight, which overlaps whole feeds without the extra launches.)
+  int pieces = 1;
+  if (on_device == POLARIS_INPUT_HOST && carry == 0 && (is_fused(s->logn) || nseg <= s->max_batch))
+    pieces = feed_pieces(nw * 4 * s->n_if, nseg);
+  cudaStream_t st_in = pieces > 1 ? s->st_p1 : st;  // where the input is copied
   if (host_in) {
     if (nw > s->in_words_cap) {
       CUDA_OR_FAIL(s, cudaStreamSynchronize(st));
@@ -835,45 +889,21 @@ extern "C" int spectrometer_feed(polaris_spec* s, const void* const* packed, int
       }
       s->in_words_cap = nw;
     }
-    // IF streams at one constant stride (rows of one host array, say) go over in one
-    // pitched copy: one API call instead of one per IF (each costs host time).  The CUDA driver
-    // refuses (at the call, queueing nothing) a pitched copy whose rows lie in different
-    // pinned allocations; then the streams go one by one.
-    const long long stride = s->n_if > 1 ? (long long)((const char*)packed[1] - (const char*)packed[0]) : 0;
-    bool uniform = s->n_if > 1 && stride >= nw * 4;
-    for (int i = 2; i < s->n_if && uniform; ++i)
-      uniform = (long long)((const char*)packed[i] - (const char*)packed[i - 1]) == stride;
-    if (uniform) {
-      // contiguous on both sides (no gap between rows): one linear copy, the cheapest call
-      const bool linear = stride == nw * 4 && s->in_words_cap == nw;
-      const cudaError_t ec =
-          linear ? cudaMemcpyAsync(s->d_in, packed[0], (size_t)nw * 4 * s->n_if, cudaMemcpyHostToDevice, st)
-                 : cudaMemcpy2DAsync(s->d_in, (size_t)s->in_words_cap * 4, packed[0], (size_t)stride, (size_t)nw * 4,
-                                     (size_t)s->n_if, cudaMemcpyHostToDevice, st);
-      if (ec != cudaSuccess) {
-        cudaGetLastError();
-        uniform = false;
-      }
-    }
-    if (!uniform) {
-      for (int i = 0; i < s->n_if; ++i)
-        CUDA_OR_FAIL(s, cudaMemcpyAsync(s->d_in + (size_t)i * s->in_words_cap, packed[i], (size_t)nw * 4,
-                                        cudaMemcpyHostToDevice, st));
-    }
     for (int i = 0; i < s->n_if; ++i) src[i] = s->d_in + (size_t)i * s->in_words_cap;
-    CUDA_OR_FAIL(s, cudaEventRecord(s->ev_h2d, st));
+    if (pieces > 1) {  // everything queued so far may still read the input buffer
+      CUDA_OR_FAIL(s, cudaEventRecord(s->ev_fork, st));
+      CUDA_OR_FAIL(s, cudaStreamWaitEvent(st_in, s->ev_fork, 0));
+    } else {
+      CUDA_OR_FAIL(s, copy_input(s, packed, 0, nw, nw, st));
+      CUDA_OR_FAIL(s, cudaEventRecord(s->ev_h2d, st));
+    }
   } else {
     for (int i = 0; i < s->n_if; ++i) src[i] = static_cast<const uint32_t*>(packed[i]);
   }
-  const int64_t N = s->N, hop = s->hop, spw = s->spw;
-  const int64_t carry = s->carry_len;
-  const int64_t total = carry + n;
-  const int64_t nseg = total >= N ? (total - N) / hop + 1 : 0;
-  const int64_t n0 = nseg < (carry + hop - 1) / hop ? nseg : (carry + hop - 1) / hop;
   // the segments that start in the carried samples are assembled in the staging buffer; the
   // samples after the last whole segment, stream positions [nseg*hop, total), are carried on
   const int64_t keep0 = nseg * hop, keep = total - keep0;
-  {
+  auto carry_copies = [&]() -> int {
     CopyArgs c;
     int nc = 0;
     auto copy = [&](uint32_t* dst, const uint32_t* from, int64_t samples) {
@@ -903,6 +933,11 @@ extern "C" int spectrometer_feed(polaris_spec* s, const void* const* packed, int
       });
       if (e != cudaSuccess) return set_err(s, POLARIS_ECUDA, "carry copies: %s", cudaGetErrorString(e));
     }
+    return POLARIS_OK;
+  };
+  if (pieces == 1) {
+    const int rc1 = carry_copies();
+    if (rc1) return rc1;
   }
   BatchArgs a;
   memset(&a, 0, sizeof a);
@@ -941,35 +976,62 @@ extern "C" int spectrometer_feed(polaris_spec* s, const void* const* packed, int
   };
   a.acc_slots = (long long)s->acc_copies * s->n_fpair * s->native;
   const phase_fn f1 = kPhases[s->logn][0], f2 = kPhases[s->logn][1];
-  if (nseg > 0 && s->code_stats) {
-    cudaError_t e = counted_launch(s, 3, st, [&]() {
-      return launch_code_hist(a.in, s->n_if, s->bits, (int)nseg, N, s->d_hist, s->d_err, s->num_sms, st);
-    });
-    if (e != cudaSuccess) return set_err(s, POLARIS_ECUDA, "code-histogram launch: %s", cudaGetErrorString(e));
-  }
-  if (nseg > 0 && is_fused(s->logn)) {
-    a.seg0 = 0;
-    a.nseg = (int)nseg;
-    understate(a);
-    cudaError_t e = counted_launch(s, 1, st, [&]() { return f1(a, st, !s->profiling); });
-    if (e != cudaSuccess) return set_err(s, POLARIS_ECUDA, "FFT-correlator launch: %s", cudaGetErrorString(e));
-  } else if (nseg > 0 && nseg <= s->max_batch) {
-    // one pass: both phases on the caller's stream, each a programmatic dependent launch
-    // (its CTAs set up while the previous kernel drains, then wait for it) unless launches
-    // are being timed.  The legacy default stream takes dependent launches too: without them a
-    // 61 x 2^17 2-bit pass took 69.2 us there instead of 57.7, 15 x 2^20 int8 158.7 instead of 144.6
-    a.seg0 = 0;
-    a.nseg = (int)nseg;
-    a.scratch = s->d_scratch;
-    understate(a);
+  // The kernels of segments [s0, s1) of `a` in one pass on the caller's stream: programmatic
+  // dependent launches (a kernel's CTAs set up while its predecessor drains, then wait for it)
+  // unless launches are being timed.  The legacy default stream takes dependent launches too:
+  // without them a 61 x 2^17 2-bit pass took 69.2 us there instead of 57.7, 15 x 2^20 int8 158.7
+  // instead of 144.6
+  auto one_pass = [&](int64_t s0, int64_t s1) -> int {
+    BatchArgs b = a;
+    for (int i = 0; i < s->n_if && s0 > 0; ++i) b.in.src1[i] += s0 * (hop / spw);  // (pieces: nothing carried)
+    b.in.in_words1 -= s0 * (hop / spw);
+    b.nseg = (int)(s1 - s0);
+    cudaError_t e = cudaSuccess;
+    if (s->code_stats) {
+      e = counted_launch(s, 3, st, [&]() {
+        return launch_code_hist(b.in, s->n_if, s->bits, b.nseg, N, s->d_hist, s->d_err, s->num_sms, st);
+      });
+      if (e != cudaSuccess) return set_err(s, POLARIS_ECUDA, "code-histogram launch: %s", cudaGetErrorString(e));
+    }
+    understate(b);
     const bool pdl = !s->profiling;
-    cudaError_t e = counted_launch(s, 0, st, [&]() { return f1(a, st, pdl); });
+    if (is_fused(s->logn)) {
+      e = counted_launch(s, 1, st, [&]() { return f1(b, st, pdl); });
+      if (e != cudaSuccess) return set_err(s, POLARIS_ECUDA, "FFT-correlator launch: %s", cudaGetErrorString(e));
+      return POLARIS_OK;
+    }
+    e = counted_launch(s, 0, st, [&]() { return f1(b, st, pdl); });
     if (e != cudaSuccess) return set_err(s, POLARIS_ECUDA, "phase-1 launch: %s", cudaGetErrorString(e));
-    e = counted_launch(s, 1, st, [&]() { return f2(a, st, pdl); });
+    e = counted_launch(s, 1, st, [&]() { return f2(b, st, pdl); });
     if (e != cudaSuccess) return set_err(s, POLARIS_ECUDA, "phase-2 launch: %s", cudaGetErrorString(e));
+    return POLARIS_OK;
+  };
+  if (pieces > 1) {
+    int64_t w0 = 0;
+    for (int k = 0; k < pieces; ++k) {
+      const int64_t s0 = nseg * k / pieces, s1 = nseg * (k + 1) / pieces;
+      const int64_t w1 = k + 1 < pieces ? ((s1 - 1) * hop + N) / spw : nw;  // the words its segments need
+      CUDA_OR_FAIL(s, copy_input(s, packed, w0, w1, nw, st_in));
+      w0 = w1;
+      CUDA_OR_FAIL(s, cudaEventRecord(s->ev_h2d, st_in));
+      CUDA_OR_FAIL(s, cudaStreamWaitEvent(st, s->ev_h2d, 0));
+      const int rc1 = one_pass(s0, s1);
+      if (rc1) return rc1;
+    }
+    const int rc1 = carry_copies();
+    if (rc1) return rc1;
+  } else if (nseg > 0 && (is_fused(s->logn) || nseg <= s->max_batch)) {
+    const int rc1 = one_pass(0, nseg);
+    if (rc1) return rc1;
   } else if (nseg > 0) {
     // several passes: phase 1 and phase 2 on two internal streams, pass b + 1's phase 1
     // overlapping pass b's phase 2 (alternate slab halves).
+    if (s->code_stats) {
+      const cudaError_t e = counted_launch(s, 3, st, [&]() {
+        return launch_code_hist(a.in, s->n_if, s->bits, (int)nseg, N, s->d_hist, s->d_err, s->num_sms, st);
+      });
+      if (e != cudaSuccess) return set_err(s, POLARIS_ECUDA, "code-histogram launch: %s", cudaGetErrorString(e));
+    }
     // fork: both internal streams start after everything queued so far on the caller's stream
     CUDA_OR_FAIL(s, cudaEventRecord(s->ev_fork, st));
     CUDA_OR_FAIL(s, cudaStreamWaitEvent(s->st_p1, s->ev_fork, 0));
@@ -1109,8 +1171,10 @@ extern "C" int spectrometer_integrate(polaris_spec* s, const polaris_stokes_para
   if (stokes && s->n_pair)
     CUDA_OR_FAIL(s, cudaMemcpyAsync(stokes, s->d_out_stokes, (size_t)s->nbin * 16 * s->n_pair,
                                     cudaMemcpyDeviceToHost, nullptr));
+  int status = 0;  // (a copy of its own after a synchronisation cost another 8 us)
+  CUDA_OR_FAIL(s, cudaMemcpyAsync(&status, s->d_err, sizeof status, cudaMemcpyDeviceToHost, nullptr));
   CUDA_OR_FAIL(s, cudaStreamSynchronize(nullptr));
-  return check_device_status(s);
+  return check_device_status(s, status);
 }
 
 extern "C" int spectrometer_debug_unpack(polaris_spec* s, const void* packed, int64_t n, float* out) {
@@ -1240,9 +1304,14 @@ extern "C" int spectrometer_code_histogram(polaris_spec* s, uint64_t* counts, in
   DeviceGuard dg(s->device);
   const size_t bytes = (size_t)s->n_if * ((size_t)1 << s->bits) * 8;
   CUDA_OR_FAIL(s, cudaDeviceSynchronize());  // the counts of everything queued so far
-  rc = check_device_status(s);
+  // the status word and the counts, which lie side by side, in one copy
+  unsigned char buf[kStatusBytes + kMaxIF * 256 * 8];
+  CUDA_OR_FAIL(s, cudaMemcpy(buf, s->d_err, kStatusBytes + bytes, cudaMemcpyDeviceToHost));
+  int status = 0;
+  memcpy(&status, buf, sizeof status);
+  rc = check_device_status(s, status);
   if (rc) return rc;
-  CUDA_OR_FAIL(s, cudaMemcpy(counts, s->d_hist, bytes, cudaMemcpyDeviceToHost));
+  memcpy(counts, buf + kStatusBytes, bytes);
   if (reset) CUDA_OR_FAIL(s, cudaMemset(s->d_hist, 0, bytes));
   return POLARIS_OK;
 }

@@ -1189,8 +1189,8 @@ static cudaError_t launch_phase1(const BatchArgs& a, cudaStream_t st, bool pdl) 
   }
   using ST = typename PL::template Stage1<BITS>;
   // The tensor maps (slab output, packed input) depend only on the pointers and sizes below;
-  // the last four sets per instance are kept, so that steady streaming (one or a few
-  // handles feeding equal chunks) encodes none of them again.
+  // the last eight sets per instance are kept, so that steady streaming (one or a few
+  // handles feeding equal chunks, or a host feed in pieces) encodes none of them again.
   struct MapKey {
     const void* scratch;
     long long slab_rows, hop_w;
@@ -1203,7 +1203,7 @@ static cudaError_t launch_phase1(const BatchArgs& a, cudaStream_t st, bool pdl) 
     InMaps in;
     bool valid;
   };
-  static thread_local MapSet cache[4];
+  static thread_local MapSet cache[8];
   static thread_local int cache_next = 0;
   MapKey key;
   memset(&key, 0, sizeof key);
@@ -1225,7 +1225,7 @@ static cudaError_t launch_phase1(const BatchArgs& a, cudaStream_t st, bool pdl) 
     if (c.valid && memcmp(&c.key, &key, sizeof key) == 0) ms = &c;
   if (!ms) {
     ms = &cache[cache_next];
-    cache_next = (cache_next + 1) % 4;
+    cache_next = (cache_next + 1) % 8;
     ms->valid = false;
     memset(&ms->slab, 0, sizeof ms->slab);
     if constexpr (ST::TMA_OUT || ST::JOINT_OUT) {  // the kernel's TMA output paths
