@@ -82,7 +82,7 @@ typedef struct polaris_spec polaris_spec; /* opaque, library-owned */
  *   max_batch_segments  segments processed per kernel pass (bounds the device
  *               scratch: 2 * max_batch_segments * n_fft * 8 bytes per pair);
  *               0 selects the default (passes of at least 64 segments).  n_fft of
- *               1024 to 4096 run in one kernel without scratch, whatever the value.
+ *               1024 to 16384 run in one kernel without scratch, whatever the value.
  *   code_stats  1: also count, per IF, how often each b-bit code occurs in the
  *               segments that feed() integrates (the bit distribution used for
  *               total-power measurement, Sec. 2 and Sec. 3.2.2); read with
@@ -196,8 +196,8 @@ int spectrometer_n_pairs(const polaris_spec* s);
  * host floats `out`, on the GPU.  n must be a multiple of 32/bits. */
 int spectrometer_debug_unpack(polaris_spec* s, const void* packed, int64_t n, float* out);
 
-/* The data-translation step as the FFT kernel runs it from N = 2^13 up (Fig. 2 caption:
- * integer codes to floats; Sec. 2: two IF streams enter one transform): that kernel stages
+/* The data-translation step as the FFT kernel runs it on staged input, N = 2^13 and up (Fig. 2
+ * caption: integer codes to floats; Sec. 2: two IF streams enter one transform): that kernel stages
  * each tile's packed words in shared memory, transposes their codes so that the rows of one
  * column share a word, and decodes both IFs of a pair together.  This call stages, transposes
  * and decodes through that same device code, for bit-exact checks of the levels the transform
@@ -225,7 +225,7 @@ const char* spectrometer_last_error(const polaris_spec* s);
  * waits for those events and returns, per kind, the summed device time in ms and the
  * launch count since profiling began or since the previous query (kinds: 0 = phase 1,
  * decode/window/row DFT; 1 = phase 2, column DFT/correlate/accumulate (and the one kernel that
- * does both phases at n_fft of 1024 to 4096); 2 = readout and Stokes; 3 = code histogram).
+ * does both phases at n_fft of 1024 to 16384); 2 = readout and Stokes; 3 = code histogram).
  * n is the length of both arrays and must be >= 3; kinds >= n are not reported. */
 int64_t spectrometer_kernel_launches(const polaris_spec* s);
 int spectrometer_set_profiling(polaris_spec* s, int on);
@@ -382,7 +382,7 @@ void polaris_set_wait_limit(int64_t polls);
  * word, and the next synchronising call returns POLARIS_EBOUNDS.  Nothing traps.
  * polaris_checked_build: 1 in such a build, 0 otherwise.
  * polaris_set_check_understate (test hook, checked build only): on != 0 makes later feeds
- * tell the kernels half the slab (n_fft of 1024 to 4096: half the input) they have, so that
+ * tell the kernels half the slab (n_fft of 1024 to 16384: half the input) they have, so that
  * the checks fire while every access stays inside its buffer; POLARIS_EINVAL in a build without checks. */
 int polaris_checked_build(void);
 int polaris_set_check_understate(int on);

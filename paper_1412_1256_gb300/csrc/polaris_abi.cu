@@ -29,8 +29,6 @@ POLARIS_DECLARE(6)
 POLARIS_DECLARE(7)
 POLARIS_DECLARE(8)
 POLARIS_DECLARE(9)
-POLARIS_DECLARE(13)
-POLARIS_DECLARE(14)
 POLARIS_DECLARE(15)
 POLARIS_DECLARE(16)
 POLARIS_DECLARE(17)
@@ -42,6 +40,8 @@ POLARIS_DECLARE(20)
 extern template cudaError_t run_fused<10>(const BatchArgs&, cudaStream_t, bool);
 extern template cudaError_t run_fused<11>(const BatchArgs&, cudaStream_t, bool);
 extern template cudaError_t run_fused<12>(const BatchArgs&, cudaStream_t, bool);
+extern template cudaError_t run_fused<13>(const BatchArgs&, cudaStream_t, bool);
+extern template cudaError_t run_fused<14>(const BatchArgs&, cudaStream_t, bool);
 
 // (args, stream, programmatic dependent launch on the predecessor in `stream`)
 typedef cudaError_t (*phase_fn)(const BatchArgs&, cudaStream_t, bool);
@@ -57,7 +57,7 @@ cudaError_t launch_unpack_staged(int logn, int bits, const uint32_t* pa, const u
 static const phase_fn kPhases[21][2] = {
     {nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr},
     POLARIS_ROW(4),  POLARIS_ROW(5),  POLARIS_ROW(6),  POLARIS_ROW(7),  POLARIS_ROW(8),  POLARIS_ROW(9),
-    POLARIS_FUSED_ROW(10), POLARIS_FUSED_ROW(11), POLARIS_FUSED_ROW(12), POLARIS_ROW(13), POLARIS_ROW(14), POLARIS_ROW(15),
+    POLARIS_FUSED_ROW(10), POLARIS_FUSED_ROW(11), POLARIS_FUSED_ROW(12), POLARIS_FUSED_ROW(13), POLARIS_FUSED_ROW(14), POLARIS_ROW(15),
     POLARIS_ROW(16), POLARIS_ROW(17), POLARIS_ROW(18), POLARIS_ROW(19), POLARIS_ROW(20)};
 #undef POLARIS_ROW
 #undef POLARIS_FUSED_ROW
@@ -677,7 +677,7 @@ extern "C" int spectrometer_create(const polaris_config* cfg, polaris_spec** out
   s->carry_words_cap = N / spw;               // carried samples < N
   s->stage_words_cap = 2 * N / spw;           // staging < carry + N samples
   if (is_fused(logn)) {
-    s->acc_copies = copies_for(2LL * s->num_sms / nf);  // CTAs per FFT pair
+    s->acc_copies = copies_for((logn == kFusedMax ? 1LL : 2LL) * s->num_sms / nf);  // CTAs per FFT pair
   } else {
     // phase 2: every resident warp has one range of segments of one (pair, unit group)
     const int P = plan_p(logn), Q2 = s->N2 / P, UPW = 16 / Q2;

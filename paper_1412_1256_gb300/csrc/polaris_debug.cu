@@ -3,7 +3,8 @@
 // their codes there and decodes each lane's rows from the transposed words (polaris_codes.cuh).
 // k_unpack_staged stages tile by tile and transposes and decodes through those same device
 // functions, so the levels phase 1 transforms can be compared with the oracle's decode bit for
-// bit, transposed apart (layout 0) or in place (layout 1).
+// bit, transposed apart (layout 0) or in place (layout 1).  (2^13 and 2^14 run in k_fused, which
+// transposes and decodes through the same transpose_codes and code_pair; here they stage phase 1's tiles.)
 #include "polaris_kernels.cuh"
 
 namespace polaris {

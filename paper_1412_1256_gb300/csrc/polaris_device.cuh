@@ -203,11 +203,11 @@ constexpr int plan_log_n2(int logn) {
 // after: 15 x 2^20 int8 223 -> 160 us, 610 x 2^18 int8 1162 -> 884 us, 1953 half-overlapped 2^14
 // int8 segments of four IFs 379 -> 332 us.  Below
 // 2^10 the taps stay in sample order.
-// The sizes that run in one kernel (2^10 to 2^12) take them the same way: lane b of its team owns
-// column b of the N/R columns of R rows, four rows per load.
-constexpr int kFusedMin = 10, kFusedMax = 12;
+// The sizes that run in one kernel (2^10 to 2^14) take them the same way: lane b of its team owns
+// column b of the N/32 columns of 32 rows, four rows per load.
+constexpr int kFusedMin = 10, kFusedMax = 14;
 constexpr bool is_fused(int logn) { return logn >= kFusedMin && logn <= kFusedMax; }
-constexpr int fused_log_b(int logn) { return logn == 10 ? 5 : 6; }  // columns of their plan: 32, 64, 64
+constexpr int fused_log_b(int logn) { return logn - 5; }  // columns of their plan (32 rows)
 constexpr int kTapsOrderedMin = 13;
 struct TapOrder {
   int ln2, lq1, lcw, lt4;  // log2 of the columns, Q1, CW and P1/4 (ln2 < 0: sample order)

@@ -1,0 +1,3 @@
+#include "polaris_fused.cuh"
+
+POLARIS_INSTANTIATE_FUSED(14)

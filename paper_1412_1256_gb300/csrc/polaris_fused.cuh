@@ -1,28 +1,31 @@
-// The whole hot path of the small transforms (N = 2^10 .. 2^12) in one kernel: data translation,
+// The whole hot path of the small transforms (N = 2^10 .. 2^14) in one kernel: data translation,
 // window, segment FFT, correlation and integration (Fig. 2 caption), with the pair-segment in
 // registers and shared memory from its packed words to its accumulators.
 //
 //   k_fused  a team of W = N/1024 warps takes a range of segments of one FFT pair, one segment
-//            at a time, 32 points per lane.  N = R B (row a, column b, n = B a + b; bin
-//            k = c + R d): lane b runs the R-point DFT over its column's rows, multiplies by
-//            W_N^{b c} (tensor memory), the team exchanges [c][b] through shared memory once,
-//            and lane c runs the B-point DFT.  R and B are 32 or 64: a 64-point DFT is split over
-//            two lanes by the parity of the output index (x_i +- x_{i+32}, the odd half turned by
-//            W_64^i), so that every lane holds 32 points throughout.
-//            Lane c's bin c + R d and its mirror (in the lane of column R - c, which sits in the
-//            same warp) meet by one shuffle per component; |X|^2, |Y|^2 and X conj(Y) (as in
-//            k_phase2) accumulate in tensor memory over the range.  At the end the CTA's teams
-//            are summed in shared memory and added once to the integration accumulators, which
-//            hold the bins in natural order.
+//            at a time, 32 points per lane.  N = 32 B (row a, column b, n = B a + b; bin
+//            k = c + 32 d): lane b runs the 32-point DFT over its column's rows, multiplies by
+//            W_N^{b c} (tensor memory) and the team exchanges [c][b] through shared memory; the
+//            B-point DFTs of the 32 columns c follow within warps:
+//              2^10  lane c, 32 points
+//              2^11  64 points over two lanes by the parity of the output index (x_i +- x_{i+32},
+//                    the odd half turned by W_64^i)
+//              2^12+ B = 16 P1: P1-point DFTs over b1 (b = 16 b1 + b0), W_B^{b0 d1}, an exchange
+//                    among the P1/2 lanes of the column, 16-point DFTs over b0 (d = d1 + P1 d0)
+//            A bin and its mirror (column 32 - c, in the same warp) meet by one shuffle per
+//            component; |X|^2, |Y|^2 and X conj(Y) (as in k_phase2) accumulate in tensor memory
+//            over the range.  At the end the CTA's teams are summed in shared memory and added
+//            once to the integration accumulators, which hold the bins in natural order.
 //
-// What bounds it: about 40 (1024, 2048 points) and 46 (4096) instructions per complex point, against
-// 64 of the two-phase path of the larger sizes, which these sizes took before and which sends
-// every point through a slab in L2.  Measured against that path (GB300): 4 pairs of 1-bit IFs,
-// 2441 segments of 2048 points, 41 instead of 31 + 54 us of kernel time (2.05 us per million
-// complex points); 64 int8 Hann segments of 1024 points, a whole pass 14.4 (host-bound) instead of
-// 28.7 us; at 4096 points 86 segments of two 4-bit pairs take 10.3 instead of 5.8 + 10.3 us.
-// Sizes: 2^13 and up would split a transform over more than two lanes per output column (or keep
-// more than 32 points per lane) and stay with the two phases; below 2^10 likewise.
+// What bounds it: instruction issue, about 40 to 43 instructions per complex point, of which 14
+// packed FP32, at 45 to 50% of the issue slots with 16 warps per SM (registers), against 64 of the
+// two-phase path of the larger sizes, which these sizes took before and which sends every point
+// through a slab in L2.  Measured against that path (GB300, four 2-bit IFs of 8 M samples, whole
+// passes, Msample/s before and after): 2^10 313k, 1114k; 2^11 435k, 926k; 2^12 393k, 770k; 2^13
+// 480k, 697k; 2^14 478k, 638k; 64 int8 Hann segments of 1024 points 28.7 and 13.2 us (host-bound);
+// one 2^14 segment 23 and 17 us.  (2^12 with both transforms split by parity like 2^11's second one,
+// 64 x 64 points, ran at 727k.)  The line: 2^15 points do not fit an SM's registers, and below 2^10
+// a warp would hold several segments.
 #pragma once
 #include "polaris_codes.cuh"
 #include "polaris_kernels.cuh"
@@ -32,11 +35,18 @@ namespace polaris {
 template <int LOGN>
 struct FusedPlan {
   static constexpr int N = 1 << LOGN, W = N / 1024;     // warps per team
-  static constexpr int THREADS = 256, WARPS = THREADS / 32, T = WARPS / W;  // teams per CTA
-  static constexpr int B = 1 << fused_log_b(LOGN), R = N / B;
-  static constexpr int HA = R / 32, HB = B / 32;        // lanes per R-point, B-point DFT
-  static constexpr int PITCH = B + 1;                   // [c][b] rows: consecutive c on distinct bank pairs
+  static constexpr int WARPS = W > 8 ? W : 8, THREADS = 32 * WARPS, T = WARPS / W;  // teams per CTA
+  static constexpr int MINB = WARPS > 8 ? 1 : 2;        // CTAs per SM (16 warps either way)
+  static constexpr int R = 32, B = 1 << fused_log_b(LOGN);  // rows, columns
+  static constexpr int HB = B == 64 ? 2 : 1;            // lanes per column (2^10, 2^11)
+  static constexpr bool THREE = B > 64;                 // the B-point DFT in two steps
+  static constexpr int P1 = THREE ? B / 16 : 1;
+  static constexpr int LC = THREE ? P1 / 2 : 1;         // lanes per column
+  // [c][b] rows.  Two steps: an odd pitch puts consecutive c on distinct bank pairs.  Three: rows
+  // also take [d1][b0] at 17 d1 + b0, and the columns of a half-warp lie an odd multiple of LC bank pairs apart
+  static constexpr int PITCH = !THREE ? B + 1 : B == 128 ? 140 : B == 256 ? 280 : 544;
   static constexpr int REGION = R * PITCH;              // float2 per team
+  static constexpr int TW2 = THREE ? B : 0;             // W_B^{b0 d1} at 16 d1 + b0
   static constexpr int TCOLS = (WARPS / 4) * 128;       // 64 accumulator and 64 twiddle columns per lane
   template <int BITS>
   struct In {
@@ -56,11 +66,12 @@ struct FusedPlan {
     static constexpr int VW = BR, VL = VW < 4 ? VW : 4;
     static constexpr int SLAB = (B + WPR) * VL, TR = (VW / VL) * SLAB;
     static constexpr size_t TEAM = sizeof(float2) * REGION + 4 * (size_t)G * (RAW + TR);
-    static constexpr size_t SMEM = T * TEAM + 16 * T + 16;  // + extra bin per team, TMEM slot
+    static constexpr size_t SMEM = T * TEAM + 16 * T + 8 * TW2 + 16;  // + extra bin per team, W_B, TMEM slot
     static_assert((G * RAW) % 4 == 0 && SLAB % VL == 0 && TR % VL == 0 && TEAM % 16 == 0, "vector loads aligned");
-    static_assert(2 * (SMEM + 1024) <= 233472, "two CTAs per SM");
+    static_assert(MINB * (SMEM + 1024) <= 233472, "CTAs per SM");
   };
   static_assert(REGION * sizeof(float2) % 16 == 0 && REGION * 8 >= 16 * (N / 2), "region holds the team's sums");
+  static_assert(!THREE || (PITCH >= 17 * P1 && (LC == 16 || (PITCH % LC == 0 && PITCH / LC % 2 == 1))), "column rows");
 };
 
 template <int W>
@@ -88,10 +99,11 @@ __device__ __forceinline__ float2 turn64(float2 x) {
 }
 
 template <int LOGN, int BITS>
-__global__ void __launch_bounds__(256, 2) k_fused(BatchArgs a) {
+__global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MINB) k_fused(BatchArgs a) {
   using PL = FusedPlan<LOGN>;
   using IN = typename PL::template In<BITS>;
-  constexpr int W = PL::W, T = PL::T, B = PL::B, R = PL::R, HA = PL::HA, HB = PL::HB, PITCH = PL::PITCH;
+  constexpr int W = PL::W, T = PL::T, B = PL::B, R = PL::R, HB = PL::HB, PITCH = PL::PITCH, P1 = PL::P1, LC = PL::LC;
+  constexpr bool THREE = PL::THREE;
   constexpr int SPW = IN::SPW, WPR = IN::WPR, VL = IN::VL, G = IN::G, TL = 32 * W;
   extern __shared__ __align__(16) unsigned char smf[];
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -101,19 +113,29 @@ __global__ void __launch_bounds__(256, 2) k_fused(BatchArgs a) {
   uint32_t* raw = reinterpret_cast<uint32_t*>(mine + sizeof(float2) * PL::REGION);
   uint32_t* tr = raw + G * IN::RAW;
   float4* xbin = reinterpret_cast<float4*>(smf + T * IN::TEAM);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(xbin + T);
+  float2* tw2 = reinterpret_cast<float2*>(xbin + T);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(tw2 + PL::TW2);
 
-  // lane roles: step A column ba and output parity ha (the same for a whole warp); step B column
-  // cb (unit u: column u, or its mirror R - u; unit 0: columns 0 and R/2) and output parity hb
-  const int ba = tl % B, ha = __shfl_sync(0xffffffffu, tl / B, 0);
-  const int hb = HB == 2 ? (lane >> 3) & 1 : 0, mir = lane >> 4;
-  const int u = HB == 2 ? 8 * wt + (lane & 7) : lane & 15;
-  const int cb = u == 0 ? (mir ? R / 2 : 0) : (mir ? R - u : u);
-  // the lane whose output 31 - i is the mirror of this lane's output i; column 0's even outputs
-  // mirror onto themselves (output (32 - i) mod 32 of the lane itself)
-  const int partner = u == 0 ? (mir == 0 || HB == 1 ? lane : lane ^ 8) : (HB == 2 ? lane ^ 24 : lane ^ 16);
-  const bool self = cb == 0 && hb == 0;
+  // lane roles: step A column tl.  Afterwards column cb (unit u: column u in lanes 0-15, its mirror
+  // 32 - u in lanes 16-31; unit 0: columns 0 and 16), output parity hb (2^11) or lane l of the
+  // column's LC (2^12 and up)
+  const int mir = lane >> 4;
+  const int hb = HB == 2 ? (lane >> 3) & 1 : 0, l = THREE ? lane % LC : 0;
+  const int u = THREE ? (16 / LC) * wt + (lane & 15) / LC : HB == 2 ? 8 * wt + (lane & 7) : lane & 15;
+  const int cb = u == 0 ? (mir ? 16 : 0) : (mir ? 32 - u : u);
+  // the lanes that hold this lane's mirror bins.  Two steps: output 31 - i of `partner` mirrors output
+  // i; column 0's even outputs mirror onto themselves (output (32 - i) mod 32 of the lane itself).
+  // Three: a lane holds d1 = l (slot 0) and P1 - 1 - l (slot 1); the mirror of (slot, d0) is the other
+  // slot's 15 - d0 in the same lane of column 32 - c; in column 0 it is slot 1 of lane l - 1 (for slot
+  // 0) and slot 0 of lane l + 1 (for slot 1), except d1 = 0 and P1/2, which mirror onto themselves
+  const int partner = u == 0 ? (THREE || HB == 1 || mir == 0 ? lane : lane ^ 8) : (HB == 2 ? lane ^ 24 : lane ^ 16);
+  const int partner0 = THREE && cb == 0 && l > 0 ? lane - 1 : partner;
+  const int partner1 = THREE && cb == 0 && l < LC - 1 ? lane + 1 : partner;
+  const bool self = cb == 0 && hb == 0 && l == 0, self1 = THREE && cb == 0 && l == LC - 1;
 
+  if constexpr (THREE) {
+    for (int i = tid; i < B; i += PL::THREADS) tw2[i] = tw_small<B>((i & 15) * (i >> 4));
+  }
   const uint32_t tbase = __shfl_sync(0xffffffffu, cta_tmem_begin<PL::TCOLS>(tslot, warp), 0);
   const uint32_t t_acc = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * 128);
   const uint32_t t_tw = t_acc + 64;
@@ -122,9 +144,9 @@ __global__ void __launch_bounds__(256, 2) k_fused(BatchArgs a) {
     float z16[16], w16[16];
     sfor<0, 16>([&](auto k_) { z16[decltype(k_)::value] = 0.f; });
     tmem_st16(t_acc + 16 * cc, z16);
-    sfor<0, 8>([&](auto k_) {  // W_N^{ba c}, c = HA c' + ha
+    sfor<0, 8>([&](auto k_) {  // W_N^{b c}, b = tl
       constexpr int k = decltype(k_)::value;
-      const float2 w = __ldg(a.tw + (HA * (8 * cc + k) + ha) * B + ba);
+      const float2 w = __ldg(a.tw + (8 * cc + k) * B + tl);
       w16[2 * k] = w.x;
       w16[2 * k + 1] = w.y;
     });
@@ -158,7 +180,7 @@ __global__ void __launch_bounds__(256, 2) k_fused(BatchArgs a) {
   };
 
   float extra[4] = {0.f, 0.f, 0.f, 0.f};
-  const float sgn_b = hb ? -1.f : 1.f;
+  [[maybe_unused]] const float sgn_b = hb ? -1.f : 1.f;
   if (s_begin < s_end) issue(s_begin);
 #pragma unroll 1
   for (int s0 = s_begin; s0 < s_end; s0 += G) {
@@ -180,10 +202,10 @@ __global__ void __launch_bounds__(256, 2) k_fused(BatchArgs a) {
     if (s0 + G < s_end) issue(s0 + G);
 #pragma unroll 1
     for (int g = 0; g < cnt; ++g) {
-      // step A: decode column ba, window, R-point DFT
+      // step A: decode column tl, window, 32-point DFT
       float2 v[32];
       uint32_t cw[IN::VW];
-      const uint32_t* col = tr + g * IN::TR + ((ba % SPW) * WPR + ba / SPW) * VL;
+      const uint32_t* col = tr + g * IN::TR + ((tl % SPW) * WPR + tl / SPW) * VL;
       sfor<0, IN::VW / VL>([&](auto q_) {
         constexpr int q = decltype(q_)::value;
         if constexpr (VL == 4) {
@@ -200,29 +222,18 @@ __global__ void __launch_bounds__(256, 2) k_fused(BatchArgs a) {
       });
       auto rows = [&](auto hb_, auto tp_) {
         constexpr bool HBP = decltype(hb_)::value, TP = decltype(tp_)::value;
-        const float4* tp = reinterpret_cast<const float4*>(a.taps) + ba;
-        float4 w4[HA];
-        auto sample = [&](auto t_, auto h_) {
-          constexpr int t = decltype(t_)::value, h = decltype(h_)::value;
-          float2 z = code_pair<BITS, t % SPW>(cw[t / SPW], cw[IN::VW / 2 + t / SPW]);
-          if constexpr (!HBP) z.y = 0.f;
-          if constexpr (TP) {
-            if constexpr (t % 4 == 0) w4[h] = __ldg(tp + (t / 4) * B);
-            const float x = t % 4 == 0 ? w4[h].x : t % 4 == 1 ? w4[h].y : t % 4 == 2 ? w4[h].z : w4[h].w;
-            z = __fmul2_rn(z, make_float2(x, x));
-          }
-          return z;
-        };
+        [[maybe_unused]] const float4* tp = reinterpret_cast<const float4*>(a.taps) + tl;
+        [[maybe_unused]] float4 w4;
         sfor<0, 32>([&](auto t_) {
           constexpr int t = decltype(t_)::value;
-          const float2 z = sample(t_, std::integral_constant<int, 0>{});
-          if constexpr (HA == 1) {
-            v[ct::bitrev(t, 32)] = z;
-          } else {
-            const float2 y = sample(std::integral_constant<int, t + 32>{}, std::integral_constant<int, 1>{});
-            const float sg = ha ? -1.f : 1.f;
-            v[ct::bitrev(t, 32)] = __ffma2_rn(y, make_float2(sg, sg), z);
+          float2 z = code_pair<BITS, t % SPW>(cw[t / SPW], cw[IN::VW / 2 + t / SPW]);
+          if constexpr (!HBP) z.y = 0.f;
+          if constexpr (TP) {  // (four consecutive t per load: tap_order)
+            if constexpr (t % 4 == 0) w4 = __ldg(tp + (t / 4) * B);
+            const float x = t % 4 == 0 ? w4.x : t % 4 == 1 ? w4.y : t % 4 == 2 ? w4.z : w4.w;
+            z = __fmul2_rn(z, make_float2(x, x));
           }
+          v[ct::bitrev(t, 32)] = z;
         });
       };
       using T_ = std::true_type;
@@ -234,14 +245,6 @@ __global__ void __launch_bounds__(256, 2) k_fused(BatchArgs a) {
         if (ib >= 0) rows(T_{}, F_{});
         else rows(F_{}, F_{});
       }
-      if constexpr (HA == 2) {
-        if (ha) {
-          sfor<0, 32>([&](auto t_) {
-            constexpr int t = decltype(t_)::value;
-            v[ct::bitrev(t, 32)] = turn64<t>(v[ct::bitrev(t, 32)]);
-          });
-        }
-      }
       dit<32>(v);
       sfor<0, 4>([&](auto c_) {
         constexpr int cc = decltype(c_)::value;
@@ -250,50 +253,94 @@ __global__ void __launch_bounds__(256, 2) k_fused(BatchArgs a) {
         tmem_wait_ld();
         sfor<0, 8>([&](auto k_) {
           constexpr int k = decltype(k_)::value, i = 8 * cc + k;
-          if constexpr (HA == 2 || i > 0) v[i] = cmul(v[i], make_float2(w16[2 * k], w16[2 * k + 1]));
+          if constexpr (i > 0) v[i] = cmul(v[i], make_float2(w16[2 * k], w16[2 * k + 1]));
         });
       });
       team_sync<W>(team);  // the previous segment's exchange has been read
       sfor<0, 32>([&](auto i_) {
         constexpr int i = decltype(i_)::value;
-        region[(HA * i + ha) * PITCH + ba] = v[i];
+        region[i * PITCH + tl] = v[i];
       });
       team_sync<W>(team);
-      // step B: B-point DFT of column cb
-      const float2* src = region + cb * PITCH;
-      sfor<0, 32>([&](auto i_) {
-        constexpr int i = decltype(i_)::value;
-        if constexpr (HB == 1) {
-          v[ct::bitrev(i, 32)] = src[i];
-        } else {
-          float2 z = __ffma2_rn(src[i + 32], make_float2(sgn_b, sgn_b), src[i]);
-          const float2 zt = turn64<i>(z);
-          z.x = hb ? zt.x : z.x;
-          z.y = hb ? zt.y : z.y;
-          v[ct::bitrev(i, 32)] = z;
-        }
-      });
-      dit<32>(v);
-      // correlate: this lane's bins are outputs i < 16 (d = HB i + hb), k = cb + R d < N/2
-      sfor<0, 4>([&](auto c_) {
-        constexpr int cc = decltype(c_)::value;
-        float a16[16];
-        tmem_ld16(t_acc + 16 * cc, a16);
-        tmem_wait_ld();
-        sfor<0, 4>([&](auto k_) {
-          constexpr int k = decltype(k_)::value, i = 4 * cc + k;
-          const float2 own = v[(32 - i) % 32];
-          float2 z = make_float2(__shfl_sync(0xffffffffu, v[31 - i].x, partner),
-                                 __shfl_sync(0xffffffffu, v[31 - i].y, partner));
-          z.x = self ? own.x : z.x;
-          z.y = self ? own.y : z.y;
-          float(&q)[4] = *reinterpret_cast<float(*)[4]>(a16 + 4 * k);
-          corr_acc(q, v[i], make_float2(z.x, -z.y));
+      // B-point DFT of column cb
+      float2* row = region + cb * PITCH;
+      if constexpr (THREE) {
+        sfor<0, 32 / P1>([&](auto j_) {
+          constexpr int j = decltype(j_)::value;
+          sfor<0, P1>([&](auto i_) {
+            constexpr int i = decltype(i_)::value;
+            v[j * P1 + ct::bitrev(i, P1)] = row[16 * i + l + LC * j];
+          });
+          dit<P1, j * P1>(v);
+          sfor<1, P1>([&](auto i_) {
+            constexpr int i = decltype(i_)::value;
+            v[j * P1 + i] = cmul(v[j * P1 + i], tw2[16 * i + l + LC * j]);
+          });
         });
-        tmem_st16(t_acc + 16 * cc, a16);
-      });
+        __syncwarp();  // the column's row has been read
+        sfor<0, 32>([&](auto i_) {
+          constexpr int i = decltype(i_)::value;
+          row[17 * (i % P1) + l + LC * (i / P1)] = v[i];
+        });
+        __syncwarp();
+        sfor<0, 2>([&](auto s_) {
+          constexpr int sl = decltype(s_)::value;
+          const float2* src = row + 17 * (sl ? P1 - 1 - l : l);
+          sfor<0, 16>([&](auto i_) {
+            constexpr int i = decltype(i_)::value;
+            v[16 * sl + ct::bitrev(i, 16)] = src[i];
+          });
+          dit<16, 16 * sl>(v);
+        });
+      } else {
+        sfor<0, 32>([&](auto i_) {
+          constexpr int i = decltype(i_)::value;
+          if constexpr (HB == 1) {
+            v[ct::bitrev(i, 32)] = row[i];
+          } else {
+            float2 z = __ffma2_rn(row[i + 32], make_float2(sgn_b, sgn_b), row[i]);
+            const float2 zt = turn64<i>(z);
+            z.x = hb ? zt.x : z.x;
+            z.y = hb ? zt.y : z.y;
+            v[ct::bitrev(i, 32)] = z;
+          }
+        });
+        dit<32>(v);
+      }
+      // correlate this lane's 16 bins k < N/2: k = cb + 32 d, d = HB i + hb, i < 16, or
+      // d = d1 + P1 d0, d0 < 8, for the lane's two d1 (i = 8 slot + d0)
+      auto correlate = [&](auto sp_) {
+        constexpr bool SP = decltype(sp_)::value;  // the warp holds column 0
+        sfor<0, 4>([&](auto c_) {
+          constexpr int cc = decltype(c_)::value;
+          float a16[16];
+          tmem_ld16(t_acc + 16 * cc, a16);
+          tmem_wait_ld();
+          sfor<0, 4>([&](auto k_) {
+            constexpr int k = decltype(k_)::value, i = 4 * cc + k;
+            constexpr int sl = THREE ? i / 8 : 0, d0 = i % 8;
+            constexpr int own = THREE ? 16 * sl + d0 : i, far = THREE ? 16 * (sl ^ 1) + 15 - d0 : 31 - i;
+            const int from = !THREE ? partner : sl ? partner1 : partner0;
+            float2 z = make_float2(__shfl_sync(0xffffffffu, v[far].x, from), __shfl_sync(0xffffffffu, v[far].y, from));
+            if constexpr (SP) {  // the bins that mirror onto their own lane's outputs
+              constexpr int near = THREE ? (sl ? 16 + 15 - d0 : (16 - d0) % 16) : (32 - i) % 32;
+              const bool me = sl ? self1 : self;
+              z.x = me ? v[near].x : z.x;
+              z.y = me ? v[near].y : z.y;
+            }
+            float(&q)[4] = *reinterpret_cast<float(*)[4]>(a16 + 4 * k);
+            corr_acc(q, v[own], make_float2(z.x, -z.y));
+          });
+          tmem_st16(t_acc + 16 * cc, a16);
+        });
+      };
+      if (W == 1 || wt == 0) correlate(std::true_type{});
+      else correlate(std::false_type{});
       tmem_wait_st();
-      if (self) corr_acc(extra, v[16], make_float2(v[16].x, -v[16].y));  // bin N/2, its own mirror
+      if (self) {  // bin N/2, its own mirror
+        constexpr int i = THREE ? 8 : 16;
+        corr_acc(extra, v[i], make_float2(v[i].x, -v[i].y));
+      }
     }
   }
   pdl_trigger();
@@ -307,7 +354,8 @@ __global__ void __launch_bounds__(256, 2) k_fused(BatchArgs a) {
     tmem_wait_ld();
     sfor<0, 4>([&](auto k_) {
       constexpr int k = decltype(k_)::value, i = 4 * cc + k;
-      sums[cb + R * (HB * i + hb)] = make_float4(a16[4 * k], a16[4 * k + 1], a16[4 * k + 2], a16[4 * k + 3]);
+      const int d = THREE ? (i / 8 ? P1 - 1 - l : l) + P1 * (i % 8) : HB * i + hb;
+      sums[cb + 32 * d] = make_float4(a16[4 * k], a16[4 * k + 1], a16[4 * k + 2], a16[4 * k + 3]);
     });
   });
   if (self) xbin[team] = make_float4(extra[0], extra[1], extra[2], extra[3]);

@@ -1,4 +1,4 @@
-"""The sizes whose whole path runs in one kernel (2^10 to 2^12) against the FP64 oracle, at its
+"""The sizes whose whole path runs in one kernel (2^10 to 2^14) against the FP64 oracle, at its
 edges: fewer segments than one team takes, uneven ranges over the teams, groups of staged
 segments that end early, one to eight IFs (pairs with and without a second IF, CTAs shared
 unevenly between pairs), segments split between staged and new input, launch caps, FP64 sums.
@@ -14,7 +14,7 @@ from tests.helpers import assert_close
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("logn", [10, 11, 12])
+@pytest.mark.parametrize("logn", [10, 11, 12, 13, 14])
 @pytest.mark.parametrize("bits,n_if,n_seg,hop_half,window,kw", [
     (1, 2, 1, False, "rect", {}),
     (1, 5, 37, False, "hann", {"pairs": [(3, 1)]}),
