@@ -58,13 +58,16 @@ struct FusedPlan {
     // segments staged at once: as many as give each lane of the team a block (at most 8, for
     // shared memory; a block's transpose is 100 to 260 instructions however many lanes have one)
     static constexpr int G = (32 * W / NB < 1) ? 1 : (32 * W / NB > 8 ? 8 : 32 * W / NB);
-    // packed words as they arrive, WPR words of padding per block row: the lanes' (word, block
-    // row) then fall on consecutive banks
-    static constexpr int RAWBLK = (SPW + 1) * WPR, RAW = BR * RAWBLK;
-    // transposed words: BR words per column, VL of them side by side for one vector load;
-    // column b = w SPW + c at place c WPR + w, so that the writers' lanes are consecutive
+    // A warp's lanes take WL consecutive words of consecutive block rows.  Packed words as they
+    // arrive: WL words of padding per block row put those on distinct banks
+    static constexpr int WL = WPR < 8 ? WPR : 8;
+    static constexpr int RAWBLK = SPW * WPR + WL, RAW = BR * RAWBLK;
+    // transposed words: BR words per column, VL of them side by side for one vector load, column b
+    // at place b + b / PADC: the readers' eight lanes are consecutive vectors, the writers' WL
+    // columns SPW apart fall on distinct ones of eight (sixteen of 8 bytes at 1 bit)
     static constexpr int VW = BR, VL = VW < 4 ? VW : 4;
-    static constexpr int SLAB = (B + WPR) * VL, TR = (VW / VL) * SLAB;
+    static constexpr int PADC = SPW < 8 ? 8 : SPW;
+    static constexpr int SLAB = (B + B / PADC) * VL, TR = (VW / VL) * SLAB;
     static constexpr size_t TEAM = sizeof(float2) * REGION + 4 * (size_t)G * (RAW + TR);
     static constexpr size_t SMEM = T * TEAM + 16 * T + 8 * TW2 + 16;  // + extra bin per team, W_B, TMEM slot
     static_assert((G * RAW) % 4 == 0 && SLAB % VL == 0 && TR % VL == 0 && TEAM % 16 == 0, "vector loads aligned");
@@ -104,7 +107,7 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
   using IN = typename PL::template In<BITS>;
   constexpr int W = PL::W, T = PL::T, B = PL::B, R = PL::R, HB = PL::HB, PITCH = PL::PITCH, P1 = PL::P1, LC = PL::LC;
   constexpr bool THREE = PL::THREE;
-  constexpr int SPW = IN::SPW, WPR = IN::WPR, VL = IN::VL, G = IN::G, TL = 32 * W;
+  constexpr int SPW = IN::SPW, WPR = IN::WPR, WL = IN::WL, VL = IN::VL, G = IN::G, TL = 32 * W;
   extern __shared__ __align__(16) unsigned char smf[];
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int team = warp / W, wt = warp % W, tl = wt * 32 + lane;  // team, warp and lane inside it
@@ -169,7 +172,7 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
       const uint32_t dst = smem_addr(raw + g * IN::RAW);
       sfor<0, IN::NW / TL>([&](auto i_) {
         const int j = tl + decltype(i_)::value * TL;
-        const uint32_t o = 4u * (uint32_t)(j + (j / (SPW * WPR)) * WPR);
+        const uint32_t o = 4u * (uint32_t)(j + (j / (SPW * WPR)) * WL);
         if (in_bounds(a.err, w0 + j, wext)) {
           cp_async4(dst + o, pa + j);
           cp_async4(dst + o + 4u * (uint32_t)(IN::RAW / 2), pb + j);
@@ -181,167 +184,179 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
 
   float extra[4] = {0.f, 0.f, 0.f, 0.f};
   [[maybe_unused]] const float sgn_b = hb ? -1.f : 1.f;
-  if (s_begin < s_end) issue(s_begin);
-#pragma unroll 1
-  for (int s0 = s_begin; s0 < s_end; s0 += G) {
-    const int cnt = min(G, s_end - s0);
-    cp_async_wait_all();
-    team_sync<W>(team);  // the words are staged; the last group's transposed words have been read
-    // codes transposed, block by block: SPW words down a word column of one block row
+  // codes of the cnt staged segments transposed, block by block: SPW words down a word column of one
+  // block row
+  auto transpose = [&](int cnt) {
 #pragma unroll 1
     for (int k = tl; k < cnt * IN::NB; k += TL) {
-      const int w = k % WPR, br = (k / WPR) % IN::BR, g = k / IN::NB;
+      const int br = (k / WL) % IN::BR, w = k % WL + (k / (WL * IN::BR)) % (WPR / WL) * WL, g = k / IN::NB;
       const uint32_t* src = raw + g * IN::RAW + br * IN::RAWBLK + w;
       uint32_t x[SPW];
       sfor<0, SPW>([&](auto i_) { x[decltype(i_)::value] = src[decltype(i_)::value * WPR]; });
       transpose_codes<BITS>(x);
-      uint32_t* dst = tr + g * IN::TR + (br / VL) * IN::SLAB + w * VL + br % VL;
-      sfor<0, SPW>([&](auto c_) { dst[decltype(c_)::value * WPR * VL] = stored_codes<BITS>(x[decltype(c_)::value]); });
+      // (columns w SPW + c, c < SPW, share one PADC group)
+      uint32_t* dst = tr + g * IN::TR + (br / VL) * IN::SLAB + (w * SPW + w * SPW / IN::PADC) * VL + br % VL;
+      sfor<0, SPW>([&](auto c_) { dst[decltype(c_)::value * VL] = stored_codes<BITS>(x[decltype(c_)::value]); });
     }
+  };
+  // Segments come in groups of G.  The next group's words are copied during a group and transposed in
+  // its last segment, between the two barriers of the exchange, which order those steps too: two
+  // barriers per segment (with a pass of its own over each group, four per segment at 4 and 8 bits)
+  if (s_begin < s_end) {
+    issue(s_begin);
+    cp_async_wait_all();
     team_sync<W>(team);
-    if (s0 + G < s_end) issue(s0 + G);
+    transpose(min(G, s_end - s_begin));
+    team_sync<W>(team);
+    if (s_begin + G < s_end) issue(s_begin + G);
+  }
+  int g = 0;
 #pragma unroll 1
-    for (int g = 0; g < cnt; ++g) {
-      // step A: decode column tl, window, 32-point DFT
-      float2 v[32];
-      uint32_t cw[IN::VW];
-      const uint32_t* col = tr + g * IN::TR + ((tl % SPW) * WPR + tl / SPW) * VL;
-      sfor<0, IN::VW / VL>([&](auto q_) {
-        constexpr int q = decltype(q_)::value;
-        if constexpr (VL == 4) {
-          const uint4 x = *reinterpret_cast<const uint4*>(col + q * IN::SLAB);
-          cw[4 * q] = x.x;
-          cw[4 * q + 1] = x.y;
-          cw[4 * q + 2] = x.z;
-          cw[4 * q + 3] = x.w;
-        } else {
-          const uint2 x = *reinterpret_cast<const uint2*>(col + q * IN::SLAB);
-          cw[2 * q] = x.x;
-          cw[2 * q + 1] = x.y;
-        }
-      });
-      auto rows = [&](auto hb_, auto tp_) {
-        constexpr bool HBP = decltype(hb_)::value, TP = decltype(tp_)::value;
-        [[maybe_unused]] const float4* tp = reinterpret_cast<const float4*>(a.taps) + tl;
-        [[maybe_unused]] float4 w4;
-        sfor<0, 32>([&](auto t_) {
-          constexpr int t = decltype(t_)::value;
-          float2 z = code_pair<BITS, t % SPW>(cw[t / SPW], cw[IN::VW / 2 + t / SPW]);
-          if constexpr (!HBP) z.y = 0.f;
-          if constexpr (TP) {  // (four consecutive t per load: tap_order)
-            if constexpr (t % 4 == 0) w4 = __ldg(tp + (t / 4) * B);
-            const float x = t % 4 == 0 ? w4.x : t % 4 == 1 ? w4.y : t % 4 == 2 ? w4.z : w4.w;
-            z = __fmul2_rn(z, make_float2(x, x));
-          }
-          v[ct::bitrev(t, 32)] = z;
-        });
-      };
-      using T_ = std::true_type;
-      using F_ = std::false_type;
-      if (a.taps) {
-        if (ib >= 0) rows(T_{}, T_{});
-        else rows(F_{}, T_{});
+  for (int s = s_begin; s < s_end; ++s) {
+    const bool turn = g == G - 1 && s + 1 < s_end;  // the next segment starts a group
+    // step A: decode column tl, window, 32-point DFT
+    float2 v[32];
+    uint32_t cw[IN::VW];
+    const uint32_t* col = tr + g * IN::TR + (tl + tl / IN::PADC) * VL;
+    sfor<0, IN::VW / VL>([&](auto q_) {
+      constexpr int q = decltype(q_)::value;
+      if constexpr (VL == 4) {
+        const uint4 x = *reinterpret_cast<const uint4*>(col + q * IN::SLAB);
+        cw[4 * q] = x.x;
+        cw[4 * q + 1] = x.y;
+        cw[4 * q + 2] = x.z;
+        cw[4 * q + 3] = x.w;
       } else {
-        if (ib >= 0) rows(T_{}, F_{});
-        else rows(F_{}, F_{});
+        const uint2 x = *reinterpret_cast<const uint2*>(col + q * IN::SLAB);
+        cw[2 * q] = x.x;
+        cw[2 * q + 1] = x.y;
       }
-      dit<32>(v);
-      sfor<0, 4>([&](auto c_) {
-        constexpr int cc = decltype(c_)::value;
-        float w16[16];
-        tmem_ld16(t_tw + 16 * cc, w16);
-        tmem_wait_ld();
-        sfor<0, 8>([&](auto k_) {
-          constexpr int k = decltype(k_)::value, i = 8 * cc + k;
-          if constexpr (i > 0) v[i] = cmul(v[i], make_float2(w16[2 * k], w16[2 * k + 1]));
+    });
+    auto rows = [&](auto hb_, auto tp_) {
+      constexpr bool HBP = decltype(hb_)::value, TP = decltype(tp_)::value;
+      [[maybe_unused]] const float4* tp = reinterpret_cast<const float4*>(a.taps) + tl;
+      [[maybe_unused]] float4 w4;
+      sfor<0, 32>([&](auto t_) {
+        constexpr int t = decltype(t_)::value;
+        float2 z = code_pair<BITS, t % SPW>(cw[t / SPW], cw[IN::VW / 2 + t / SPW]);
+        if constexpr (!HBP) z.y = 0.f;
+        if constexpr (TP) {  // (four consecutive t per load: tap_order)
+          if constexpr (t % 4 == 0) w4 = __ldg(tp + (t / 4) * B);
+          const float x = t % 4 == 0 ? w4.x : t % 4 == 1 ? w4.y : t % 4 == 2 ? w4.z : w4.w;
+          z = __fmul2_rn(z, make_float2(x, x));
+        }
+        v[ct::bitrev(t, 32)] = z;
+      });
+    };
+    using T_ = std::true_type;
+    using F_ = std::false_type;
+    if (a.taps) {
+      if (ib >= 0) rows(T_{}, T_{});
+      else rows(F_{}, T_{});
+    } else {
+      if (ib >= 0) rows(T_{}, F_{});
+      else rows(F_{}, F_{});
+    }
+    dit<32>(v);
+    sfor<0, 4>([&](auto c_) {
+      constexpr int cc = decltype(c_)::value;
+      float w16[16];
+      tmem_ld16(t_tw + 16 * cc, w16);
+      tmem_wait_ld();
+      sfor<0, 8>([&](auto k_) {
+        constexpr int k = decltype(k_)::value, i = 8 * cc + k;
+        if constexpr (i > 0) v[i] = cmul(v[i], make_float2(w16[2 * k], w16[2 * k + 1]));
+      });
+    });
+    if (turn) cp_async_wait_all();
+    team_sync<W>(team);  // the previous exchange and this group's codes have been read; the next group is staged
+    sfor<0, 32>([&](auto i_) {
+      constexpr int i = decltype(i_)::value;
+      region[i * PITCH + tl] = v[i];
+    });
+    if (turn) transpose(min(G, s_end - s - 1));
+    team_sync<W>(team);
+    if (turn && s + 1 + G < s_end) issue(s + 1 + G);
+    // B-point DFT of column cb
+    float2* row = region + cb * PITCH;
+    if constexpr (THREE) {
+      sfor<0, 32 / P1>([&](auto j_) {
+        constexpr int j = decltype(j_)::value;
+        sfor<0, P1>([&](auto i_) {
+          constexpr int i = decltype(i_)::value;
+          v[j * P1 + ct::bitrev(i, P1)] = row[16 * i + l + LC * j];
+        });
+        dit<P1, j * P1>(v);
+        sfor<1, P1>([&](auto i_) {
+          constexpr int i = decltype(i_)::value;
+          v[j * P1 + i] = cmul(v[j * P1 + i], tw2[16 * i + l + LC * j]);
         });
       });
-      team_sync<W>(team);  // the previous segment's exchange has been read
+      __syncwarp();  // the column's row has been read
       sfor<0, 32>([&](auto i_) {
         constexpr int i = decltype(i_)::value;
-        region[i * PITCH + tl] = v[i];
+        row[17 * (i % P1) + l + LC * (i / P1)] = v[i];
       });
-      team_sync<W>(team);
-      // B-point DFT of column cb
-      float2* row = region + cb * PITCH;
-      if constexpr (THREE) {
-        sfor<0, 32 / P1>([&](auto j_) {
-          constexpr int j = decltype(j_)::value;
-          sfor<0, P1>([&](auto i_) {
-            constexpr int i = decltype(i_)::value;
-            v[j * P1 + ct::bitrev(i, P1)] = row[16 * i + l + LC * j];
-          });
-          dit<P1, j * P1>(v);
-          sfor<1, P1>([&](auto i_) {
-            constexpr int i = decltype(i_)::value;
-            v[j * P1 + i] = cmul(v[j * P1 + i], tw2[16 * i + l + LC * j]);
-          });
-        });
-        __syncwarp();  // the column's row has been read
-        sfor<0, 32>([&](auto i_) {
+      __syncwarp();
+      sfor<0, 2>([&](auto s_) {
+        constexpr int sl = decltype(s_)::value;
+        const float2* src = row + 17 * (sl ? P1 - 1 - l : l);
+        sfor<0, 16>([&](auto i_) {
           constexpr int i = decltype(i_)::value;
-          row[17 * (i % P1) + l + LC * (i / P1)] = v[i];
+          v[16 * sl + ct::bitrev(i, 16)] = src[i];
         });
-        __syncwarp();
-        sfor<0, 2>([&](auto s_) {
-          constexpr int sl = decltype(s_)::value;
-          const float2* src = row + 17 * (sl ? P1 - 1 - l : l);
-          sfor<0, 16>([&](auto i_) {
-            constexpr int i = decltype(i_)::value;
-            v[16 * sl + ct::bitrev(i, 16)] = src[i];
-          });
-          dit<16, 16 * sl>(v);
-        });
-      } else {
-        sfor<0, 32>([&](auto i_) {
-          constexpr int i = decltype(i_)::value;
-          if constexpr (HB == 1) {
-            v[ct::bitrev(i, 32)] = row[i];
-          } else {
-            float2 z = __ffma2_rn(row[i + 32], make_float2(sgn_b, sgn_b), row[i]);
-            const float2 zt = turn64<i>(z);
-            z.x = hb ? zt.x : z.x;
-            z.y = hb ? zt.y : z.y;
-            v[ct::bitrev(i, 32)] = z;
-          }
-        });
-        dit<32>(v);
-      }
-      // correlate this lane's 16 bins k < N/2: k = cb + 32 d, d = HB i + hb, i < 16, or
-      // d = d1 + P1 d0, d0 < 8, for the lane's two d1 (i = 8 slot + d0)
-      auto correlate = [&](auto sp_) {
-        constexpr bool SP = decltype(sp_)::value;  // the warp holds column 0
-        sfor<0, 4>([&](auto c_) {
-          constexpr int cc = decltype(c_)::value;
-          float a16[16];
-          tmem_ld16(t_acc + 16 * cc, a16);
-          tmem_wait_ld();
-          sfor<0, 4>([&](auto k_) {
-            constexpr int k = decltype(k_)::value, i = 4 * cc + k;
-            constexpr int sl = THREE ? i / 8 : 0, d0 = i % 8;
-            constexpr int own = THREE ? 16 * sl + d0 : i, far = THREE ? 16 * (sl ^ 1) + 15 - d0 : 31 - i;
-            const int from = !THREE ? partner : sl ? partner1 : partner0;
-            float2 z = make_float2(__shfl_sync(0xffffffffu, v[far].x, from), __shfl_sync(0xffffffffu, v[far].y, from));
-            if constexpr (SP) {  // the bins that mirror onto their own lane's outputs
-              constexpr int near = THREE ? (sl ? 16 + 15 - d0 : (16 - d0) % 16) : (32 - i) % 32;
-              const bool me = sl ? self1 : self;
-              z.x = me ? v[near].x : z.x;
-              z.y = me ? v[near].y : z.y;
-            }
-            float(&q)[4] = *reinterpret_cast<float(*)[4]>(a16 + 4 * k);
-            corr_acc(q, v[own], make_float2(z.x, -z.y));
-          });
-          tmem_st16(t_acc + 16 * cc, a16);
-        });
-      };
-      if (W == 1 || wt == 0) correlate(std::true_type{});
-      else correlate(std::false_type{});
-      tmem_wait_st();
-      if (self) {  // bin N/2, its own mirror
-        constexpr int i = THREE ? 8 : 16;
-        corr_acc(extra, v[i], make_float2(v[i].x, -v[i].y));
-      }
+        dit<16, 16 * sl>(v);
+      });
+    } else {
+      sfor<0, 32>([&](auto i_) {
+        constexpr int i = decltype(i_)::value;
+        if constexpr (HB == 1) {
+          v[ct::bitrev(i, 32)] = row[i];
+        } else {
+          float2 z = __ffma2_rn(row[i + 32], make_float2(sgn_b, sgn_b), row[i]);
+          const float2 zt = turn64<i>(z);
+          z.x = hb ? zt.x : z.x;
+          z.y = hb ? zt.y : z.y;
+          v[ct::bitrev(i, 32)] = z;
+        }
+      });
+      dit<32>(v);
     }
+    // correlate this lane's 16 bins k < N/2: k = cb + 32 d, d = HB i + hb, i < 16, or
+    // d = d1 + P1 d0, d0 < 8, for the lane's two d1 (i = 8 slot + d0)
+    auto correlate = [&](auto sp_) {
+      constexpr bool SP = decltype(sp_)::value;  // the warp holds column 0
+      sfor<0, 4>([&](auto c_) {
+        constexpr int cc = decltype(c_)::value;
+        float a16[16];
+        tmem_ld16(t_acc + 16 * cc, a16);
+        tmem_wait_ld();
+        sfor<0, 4>([&](auto k_) {
+          constexpr int k = decltype(k_)::value, i = 4 * cc + k;
+          constexpr int sl = THREE ? i / 8 : 0, d0 = i % 8;
+          constexpr int own = THREE ? 16 * sl + d0 : i, far = THREE ? 16 * (sl ^ 1) + 15 - d0 : 31 - i;
+          const int from = !THREE ? partner : sl ? partner1 : partner0;
+          float2 z = make_float2(__shfl_sync(0xffffffffu, v[far].x, from), __shfl_sync(0xffffffffu, v[far].y, from));
+          if constexpr (SP) {  // the bins that mirror onto their own lane's outputs
+            constexpr int near = THREE ? (sl ? 16 + 15 - d0 : (16 - d0) % 16) : (32 - i) % 32;
+            const bool me = sl ? self1 : self;
+            z.x = me ? v[near].x : z.x;
+            z.y = me ? v[near].y : z.y;
+          }
+          float(&q)[4] = *reinterpret_cast<float(*)[4]>(a16 + 4 * k);
+          corr_acc(q, v[own], make_float2(z.x, -z.y));
+        });
+        tmem_st16(t_acc + 16 * cc, a16);
+      });
+    };
+    if (W == 1 || wt == 0) correlate(std::true_type{});
+    else correlate(std::false_type{});
+    tmem_wait_st();
+    if (self) {  // bin N/2, its own mirror
+      constexpr int i = THREE ? 8 : 16;
+      corr_acc(extra, v[i], make_float2(v[i].x, -v[i].y));
+    }
+    g = turn ? 0 : g + 1;
   }
   pdl_trigger();
   // the CTA's teams summed in shared memory, then one add per bin (natural order; copy by CTA)
