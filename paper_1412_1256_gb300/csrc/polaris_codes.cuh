@@ -84,23 +84,23 @@ __device__ __forceinline__ float2 code_pair(uint32_t wa, uint32_t wb) {
 }
 
 // ------------------------------------------------------------------------------------------
-// phase 1's staged tiles (Plan<LOGN>::Stage1<BITS>): N1 rows of WPR words per IF, dense
-// ([IF][row][word]), transposed so that lane q1 of column col finds its rows q1 + Q1 t, t < P1, of
+// phase 1's staged tiles (Plan<LOGN>::Stage1<BITS>, WidePlan<LOGN>::Stage<BITS>): N1 rows of WPR words per IF, RP
+// words apart ([IF][row][word]), transposed so that lane q1 of column col finds its rows q1 + Q1 t, t < P1, of
 // both IFs in BR words: code t of IF a is code t % SPW of word t / SPW, IF b's follow IF a's.
 // ------------------------------------------------------------------------------------------
 // unit u of a tile: KB blocks of SPW words, from the staged words into x (transposed)
 template <typename PL, typename ST, int BITS>
 __device__ __forceinline__ void p1_unit_load(const uint32_t* raw, int u, uint32_t (&x)[ST::KB][32 / BITS]) {
-  constexpr int SPW = ST::SPW, P = PL::P1, Q1 = PL::Q1, N1 = PL::N1, WPR = ST::WPR, KB = ST::KB;
+  constexpr int SPW = ST::SPW, P = PL::P1, Q1 = PL::Q1, N1 = PL::N1, WPR = ST::WPR, RP = ST::RP, KB = ST::KB;
   const int w = u % WPR, q1 = (u / WPR) % Q1, vb = (u / (WPR * Q1)) * KB;
   // codes vb SPW .. of the lane: of one IF where P >= SPW (P codes per IF), else of both
   constexpr int BPI = P >= SPW ? P / SPW : 1;  // blocks per IF
-  const uint32_t* src = raw + (P >= SPW ? (vb / BPI) * N1 * WPR + (vb % BPI) * SPW * Q1 * WPR : 0) + q1 * WPR + w;
+  const uint32_t* src = raw + (P >= SPW ? (vb / BPI) * N1 * RP + (vb % BPI) * SPW * Q1 * RP : 0) + q1 * RP + w;
   sfor<0, KB>([&](auto k_) {
     constexpr int k = decltype(k_)::value;
     sfor<0, SPW>([&](auto i_) {
       constexpr int i = decltype(i_)::value, j = k * SPW + i;
-      constexpr int off = P >= SPW ? j * Q1 * WPR : (j / P) * N1 * WPR + (j % P) * Q1 * WPR;
+      constexpr int off = P >= SPW ? j * Q1 * RP : (j / P) * N1 * RP + (j % P) * Q1 * RP;
       x[k][i] = src[off];
     });
     transpose_codes<BITS>(x[k]);

@@ -9,14 +9,28 @@
 
 namespace polaris {
 
+template <int LOGN, int BITS, bool WIDE>
+struct StagedPlan {
+  using PL = Plan<LOGN>;
+  using ST = typename PL::template Stage1<BITS>;
+  static constexpr bool STAGED = ST::STAGED;
+};
+template <int LOGN, int BITS>
+struct StagedPlan<LOGN, BITS, true> {
+  using PL = WidePlan<LOGN>;
+  using ST = typename PL::template Stage<BITS>;
+  static constexpr bool STAGED = !(BITS == 1 && LOGN >= 19);  // (what this check has always answered)
+};
+
 // One CTA per tile (segment s, first column b0): stage the tile's N1 rows x WPR words of IF a
 // (and IF b), transpose, then decode lane q1's rows t of column col -> sample
 // n = s N + (q1 + Q1 t) N2 + b0 + col.
 template <int LOGN, int BITS>
 __global__ void __launch_bounds__(256) k_unpack_staged(const uint32_t* __restrict__ pa, const uint32_t* __restrict__ pb,
                                                        int in_place, float* __restrict__ oa, float* __restrict__ ob) {
-  using PL = Plan<LOGN>;
-  using ST = typename PL::template Stage1<BITS>;
+  using SP = StagedPlan<LOGN, BITS, (LOGN >= kWideMin)>;
+  using PL = typename SP::PL;
+  using ST = typename SP::ST;
   constexpr int N = PL::N, N1 = PL::N1, N2 = PL::N2, Q1 = PL::Q1, P = PL::P1, TILE = ST::TILE, WPR = ST::WPR;
   constexpr int SEGW = N * BITS / 32, ROWW = N2 * BITS / 32;  // words per segment, per row
   constexpr int UPT = (ST::UNITS + 255) / 256;
@@ -26,9 +40,9 @@ __global__ void __launch_bounds__(256) k_unpack_staged(const uint32_t* __restric
   const uint32_t* sa = pa + (size_t)s * SEGW + (b0 * BITS) / 32;
   const uint32_t* sbp = pb ? pb + (size_t)s * SEGW + (b0 * BITS) / 32 : nullptr;
   for (int k = threadIdx.x; k < N1 * WPR; k += blockDim.x) {
-    const int row = k / WPR, w = k % WPR;
-    stg[k] = sa[row * ROWW + w];
-    stg[N1 * WPR + k] = sbp ? sbp[row * ROWW + w] : stg[k];  // (IF a again without an IF b, as phase 1 stages it)
+    const int row = k / WPR, w = k % WPR, o = row * ST::RP + w;
+    stg[o] = sa[row * ROWW + w];
+    stg[N1 * ST::RP + o] = sbp ? sbp[row * ROWW + w] : stg[o];  // (IF a again without an IF b, as phase 1 stages it)
   }
   __syncthreads();
   uint32_t* tr = in_place ? stg : stg + ST::RAWW;
@@ -58,12 +72,13 @@ __global__ void __launch_bounds__(256) k_unpack_staged(const uint32_t* __restric
 template <int LOGN, int BITS>
 static cudaError_t launch_unpack_staged_t(const uint32_t* pa, const uint32_t* pb, long long nseg, int in_place, float* oa,
                                           float* ob, cudaStream_t st) {
-  using PL = Plan<LOGN>;
-  using ST = typename PL::template Stage1<BITS>;
-  if constexpr (!ST::STAGED) {
+  using SP = StagedPlan<LOGN, BITS, (LOGN >= kWideMin)>;
+  using PL = typename SP::PL;
+  using ST = typename SP::ST;
+  if constexpr (!SP::STAGED) {
     return cudaErrorInvalidValue;
   } else {
-    const size_t smem = 4 * (size_t)(ST::RAWW + ST::TRW);
+    const size_t smem = 4 * (size_t)(ST::RAWW + ST::TRW);  // (in place: the larger of the two would do)
     cudaError_t e = cudaFuncSetAttribute(k_unpack_staged<LOGN, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
@@ -87,7 +102,7 @@ static cudaError_t launch_unpack_staged_n(int bits, const uint32_t* pa, const ui
 
 template <int LOGN, int BITS>
 static constexpr bool staged_t() {
-  return Plan<LOGN>::template Stage1<BITS>::STAGED;
+  return StagedPlan<LOGN, BITS, (LOGN >= kWideMin)>::STAGED;
 }
 template <int LOGN>
 static constexpr bool staged_n(int bits) {

@@ -151,6 +151,24 @@ __device__ __forceinline__ void dit(A& x) {
   }
 }
 
+// x e^{-2 pi i J / 64}, J compile-time (the butterflies' cosine-factored form)
+template <int J>
+__device__ __forceinline__ float2 turn64(float2 x) {
+  constexpr ct::CS cs = ct::cossin2pi(J, 64);
+  constexpr double wr = cs.c, wi = -cs.s;
+  if constexpr (J == 0) return x;
+  else if constexpr (J == 16) return make_float2(x.y, -x.x);
+  else if constexpr (ct::dabs(wr) >= ct::dabs(wi)) {
+    constexpr float r = (float)(wi / wr), sc = (float)wr;
+    const float2 u = __ffma2_rn(make_float2(x.y, x.x), make_float2(-r, r), x);
+    return __fmul2_rn(u, make_float2(sc, sc));
+  } else {
+    constexpr float r = (float)(wr / wi), sc = (float)wi;
+    const float2 v = __ffma2_rn(x, make_float2(-r, r), make_float2(x.y, x.x));
+    return __fmul2_rn(v, make_float2(-sc, sc));
+  }
+}
+
 // ----------------------------------------------------------------------------------------
 // data translation (Fig. 2 caption): b-bit code -> level, exactly, without I2F
 //   b < 8 : level = 2c - (2^b - 1);   b = 8 : two's complement int8
@@ -187,30 +205,32 @@ constexpr int plan_p(int logn) { return logn >= 10 ? 32 : (logn >= 8 ? 16 : (log
 // phase-1 points per lane: 16 at N1 = 128 (half the registers of 32, so three CTAs per SM,
 // with the same FFT work per point and warps still four columns = 32 bytes wide).  At
 // N1 = 256 sixteen would leave two-column warps whose 16-byte output rows split sectors;
-// that measured slower than 32 points per lane at two CTAs per SM.  N1 = 2048 (N = 2^20):
-// 64 points per lane, so that one warp still holds a whole column (one CTA per SM).
-constexpr int plan_p1(int logn, int n1) { return n1 == 128 ? 16 : (n1 == 2048 ? 64 : plan_p(logn)); }
+// that measured slower than 32 points per lane at two CTAs per SM.
+constexpr int plan_p1(int logn, int n1) { return n1 == 128 ? 16 : plan_p(logn); }
 constexpr int plan_log_n2(int logn) {
   // 4:2 5:3 6:3 7:4 8:4 9:5 10:5 11:6 12:6 13:7 14:7 15:8 16:8 17:9 18:9 19:9 20:9
   return logn >= 17 ? 9 : (logn + 1) / 2;
 }
-// Order of the window taps in device memory from N = 2^13 up: the order in which phase 1's lanes
-// take them.  Lane q1 CW + cw of the warp that owns columns gb CW .. gb CW + CW - 1 needs the taps
-// of rows q1 + Q1 t; with four consecutive t of a lane side by side and the 32 lanes after one
-// another, a warp's request is 512 contiguous bytes (one 16-byte load per lane).  In sample
-// order it was one 4-byte load per point over 32 / CW rows of 4 CW bytes: at 2^20 (CW = 1) 32
-// sectors of 32 bytes for 128 bytes used.  Measured with a Hann window, whole passes, before and
-// after: 15 x 2^20 int8 223 -> 160 us, 610 x 2^18 int8 1162 -> 884 us, 1953 half-overlapped 2^14
-// int8 segments of four IFs 379 -> 332 us.  Below
-// 2^10 the taps stay in sample order.
-// The sizes that run in one kernel (2^10 to 2^14) take them the same way: lane b of its team owns
-// column b of the N/32 columns of 32 rows, four rows per load.
+// 2^18 and up: phase 1 by whole CTAs (polaris_wide.cuh), over groups of this many columns (128- or
+// 64-byte slab rows)
+constexpr int kWideMin = 18;
+constexpr int wide_columns(int logn) { return logn == 18 ? 16 : 8; }
+// The sizes that run in one kernel (polaris_fused.cuh), and the columns of their plan (32 rows)
 constexpr int kFusedMin = 10, kFusedMax = 14;
 constexpr bool is_fused(int logn) { return logn >= kFusedMin && logn <= kFusedMax; }
-constexpr int fused_log_b(int logn) { return logn - 5; }  // columns of their plan (32 rows)
-constexpr int kTapsOrderedMin = 13;
+constexpr int fused_log_b(int logn) { return logn - 5; }
+// Order of the window taps in device memory from N = 2^10 up: the order in which the lanes take
+// them.  A lane needs the taps of rows q1 + Q1 t of its column (2^15 to 2^17: lane q1 CW + cw of the
+// warp that owns columns gb CW .. gb CW + CW - 1; above, lane q1 C + cw of the CTA and its group of
+// C columns; below, Q1 = 1 and one lane per column); with four consecutive t of a lane side by side
+// and the lanes after one another, a warp's request is 512 contiguous bytes (one 16-byte load per
+// lane).  In sample order it was one 4-byte load per point over 32 / CW rows of 4 CW bytes: at 2^20
+// (one column per warp) 32 sectors of 32 bytes for 128 bytes used.  Measured with a Hann window,
+// whole passes, before and after: 15 x 2^20 int8 223 -> 160 us, 610 x 2^18 int8 1162 -> 884 us, 1953
+// half-overlapped 2^14 int8 segments of four IFs 379 -> 332 us.  Below 2^10 the taps stay in sample
+// order.
 struct TapOrder {
-  int ln2, lq1, lcw, lt4;  // log2 of the columns, Q1, CW and P1/4 (ln2 < 0: sample order)
+  int ln2, lq1, lcw, lt4;  // log2 of the columns, Q1, lanes along columns and rows per lane / 4 (ln2 < 0: sample order)
   __host__ __device__ constexpr long long slot(long long n) const {
     if (ln2 < 0) return n;
     const long long row = n >> ln2, b = n & ((1LL << ln2) - 1), t = row >> lq1;
@@ -220,8 +240,10 @@ struct TapOrder {
 };
 __host__ __device__ constexpr TapOrder tap_order(int logn) {
   if (is_fused(logn)) return TapOrder{fused_log_b(logn), 0, fused_log_b(logn), logn - fused_log_b(logn) - 2};
-  if (logn < kTapsOrderedMin) return TapOrder{-1, 0, 0, 0};
-  const int ln2 = plan_log_n2(logn), n1 = 1 << (logn - ln2), p1 = plan_p1(logn, n1), lq1 = ct::ilog2(n1 / p1);
+  if (logn < kFusedMin) return TapOrder{-1, 0, 0, 0};
+  const int ln2 = plan_log_n2(logn), n1 = 1 << (logn - ln2);
+  if (logn >= kWideMin) return TapOrder{ln2, ct::ilog2(n1 / 32), ct::ilog2(wide_columns(logn)), 3};
+  const int p1 = plan_p1(logn, n1), lq1 = ct::ilog2(n1 / p1);
   return TapOrder{ln2, lq1, 5 - lq1, ct::ilog2(p1 / 4)};
 }
 // ----------------------------------------------------------------------------------------
@@ -246,9 +268,6 @@ constexpr Ld2 p1_layout(int P, int Q1) {
          : (P == 32 && Q1 == 2)  ? Ld2{16, 512}
          : (P == 32 && Q1 == 4)  ? Ld2{8, 264}
          : (P == 32 && Q1 == 8)  ? Ld2{4, 132}
-         : (P == 32 && Q1 == 16) ? Ld2{2, 66}
-         : (P == 32 && Q1 == 32) ? Ld2{1, 33}
-         : (P == 64 && Q1 == 32) ? Ld2{1, 65}
                                  : Ld2{32 / Q1, P * (32 / Q1)};  // Q1 = 1: no transpose
 }
 constexpr Ld2 p2_layout(int P, int Q2) {
@@ -278,8 +297,9 @@ struct Plan {
   static constexpr int P = plan_p(LOGN);
   static constexpr int N2 = 1 << plan_log_n2(LOGN);
   static constexpr int N1 = N / N2;
+  static constexpr bool WIDE = LOGN >= kWideMin;        // phase 1 by whole CTAs: WidePlan (none of the below)
   static constexpr int P1 = plan_p1(LOGN, N1);          // phase-1 points per lane
-  static constexpr int Q1 = N1 / P1;
+  static constexpr int Q1 = WIDE ? 1 : N1 / P1;
   static constexpr int Q2 = N2 / P;
   static constexpr int UPS = N1 / 2;                   // units (column + mirror) per pair-segment
   static constexpr int NACC = P / 2;                   // accumulator bins per phase-2 lane
@@ -294,7 +314,7 @@ struct Plan {
   static constexpr int LDP1 = L1.a, LDQ1 = L1.b;
   static constexpr int REGION1 = Q1 > 1 ? Q1 * LDQ1 : 0;  // float2 per warp
   static constexpr int TW1 = ((2 * P1 + 15) / 16) * 16;     // tensor-memory columns per lane (W_N1 twiddles)
-  static constexpr int MINB1 = P1 <= 16 ? 3 : (P1 <= 32 ? 2 : 1);  // phase-1 CTAs per SM the registers aim at
+  static constexpr int MINB1 = P1 <= 16 ? 3 : 2;  // phase-1 CTAs per SM the registers aim at
   static constexpr int TCOLS1 = pow2_at_least((WARPS / 4) * TW1, 32);
   // CTA tiles of IPT * WARPS * CW columns inside one segment (Stage1<BITS>): the CTA stages
   // the tile's packed words (both IFs) in shared memory and transposes their codes there;
@@ -302,6 +322,7 @@ struct Plan {
   // two where the tile divides N2 and the staged and the transposed words still leave room for
   // two CTAs per SM (fewer CTA barriers and less staging work per column).  Four measured slower
   // at 2^17: too few tiles per SM to balance.
+  // (2^18 and up, where a warp would hold one or two columns: polaris_wide.cuh)
   static constexpr size_t kSmemPerCta2 = (233472 - MINB1 * 1024) / MINB1;  // MINB1 CTAs per SM
   static constexpr size_t REGIONS1 = sizeof(float2) * (size_t)WARPS * REGION1;
   template <int BITS>
@@ -323,59 +344,25 @@ struct Plan {
     }
     static constexpr size_t raw_bytes(int ipt) { return 2 * (size_t)N1 * tile_of(ipt) * BITS / 8; }
     static constexpr size_t tr_bytes(int ipt) { return 4 * (size_t)Q1 * s_of(ipt) * BR; }
-    static constexpr bool fits(int ipt, bool in_place) {
-      const size_t r = raw_bytes(ipt), t = tr_bytes(ipt);
-      return REGIONS1 + (in_place ? (r > t ? r : t) : r + t) + 32 <= kSmemPerCta2;
-    }
-    // a tile of whole words that divides N2
+    static constexpr bool fits(int ipt) { return REGIONS1 + raw_bytes(ipt) + tr_bytes(ipt) + 32 <= kSmemPerCta2; }
+    // a tile of whole words and 32 or more columns that divides N2
     static constexpr bool aligned(int ipt) {
-      return N2 % tile_of(ipt) == 0 && (tile_of(ipt) * BITS) % 32 == 0 && tile_of(ipt) * BITS >= 32;
+      return N2 % tile_of(ipt) == 0 && (tile_of(ipt) * BITS) % 32 == 0 && tile_of(ipt) % 32 == 0;
     }
-    static constexpr bool ok(int ipt) { return aligned(ipt) && tile_of(ipt) % 32 == 0 && fits(ipt, false); }
-    // Column groups per tile, 0 = not staged; + 10: transposed in place (one buffer, the next
-    // tile in flight only once the last column group has been decoded).  Tiles of 32 or more
-    // columns first; for N1 >= 512 (warps of one or two columns, whose unstaged loads would each
-    // touch 32 sectors) any tile of whole words, with two groups in place before one group apart
-    // at N1 >= 1024 (8-bit: 16 bytes per row and IF instead of 8, half the copies).
-    static constexpr int pick() {
-      return ok(2)                                                                ? 2
-             : (N2 % tile_of(1) == 0 && tile_of(1) % 32 == 0 && fits(1, false))  ? 1
-             : N1 < 512                                                          ? 0
-             : (aligned(2) && fits(2, false))                                    ? 2
-             : (N1 >= 1024 && aligned(2) && fits(2, true))                       ? 12
-             : (aligned(1) && fits(1, false))                                    ? 1
-             : (aligned(2) && fits(2, true))                                     ? 12
-             : (aligned(1) && fits(1, true))                                     ? 11
-                                                                                 : 0;
-    }
-    // (1 bit at 2^19 and 2^20 stays unstaged)
-    static constexpr bool STAGED = pick() > 0 && !(BITS == 1 && LOGN >= 19);
-    static constexpr bool INPLACE = pick() >= 10;
-    static constexpr int IPT = STAGED ? pick() % 10 : 1;
+    static constexpr int pick() { return aligned(2) && fits(2) ? 2 : aligned(1) && fits(1) ? 1 : 0; }  // (0: not staged)
+    static constexpr bool STAGED = !WIDE && pick() > 0;
+    static constexpr int IPT = STAGED ? pick() : 1;
     static constexpr int TILE = IPT * WARPS * CW;
-    static constexpr int WPR = TILE * BITS / 32;  // words per IF per staged row
+    static constexpr int WPR = TILE * BITS / 32, RP = WPR;  // words per IF per staged row, and between rows
     static constexpr int SQ = s_of(IPT);          // vectors between lanes q1
     static constexpr int RAWW = STAGED ? (int)(raw_bytes(IPT) / 4) : 0, TRW = STAGED ? (int)(tr_bytes(IPT) / 4) : 0;
-    static constexpr int TR0 = INPLACE ? 0 : RAWW;  // where the transposed words start
-    static constexpr int WORDS = INPLACE ? (RAWW > TRW ? RAWW : TRW) : RAWW + TRW;
+    static constexpr int WORDS = RAWW + TRW;
     static constexpr int UNITS = WPR * Q1 * (BR / KB);  // transposing work units of a tile
-    static constexpr int VEC = WPR >= 4 ? 4 : WPR;      // words per cp.async of an aligned input
     static_assert(!STAGED || (BR % VL == 0 && VL % KB == 0 && RAWW % 4 == 0 && (WPR & (WPR - 1)) == 0), "staged words");
-    static_assert(!INPLACE || UNITS % THREADS == 0, "whole units per thread");
-    // TMA boxes are at most 256 rows: larger N1 moves by N1 / BOXR boxes per copy
-    static constexpr int BOXR = N1 < 256 ? N1 : 256;
-    // N1 <= 256: the warp's [N1][CW] output block leaves by one TMA store (rows of 32 bytes
-    // or more).  N1 >= 512 (warps of one or two columns): the column group's [N1][WARPS CW]
-    // block is assembled in the CTA's transpose regions, which it fits, and leaves by
-    // N1 / BOXR TMA stores of 64- or 128-byte rows (swizzled in shared memory); per-warp
-    // stores of 8- or 16-byte rows measured several times slower.
-    static constexpr int JC = WARPS * CW;  // columns of the joint block
-    static constexpr bool TMA_OUT = STAGED && Q1 > 1 && N1 <= 256;
-    static constexpr bool JOINT_OUT = STAGED && Q1 > 1 && N1 >= 512 && (JC * 8 == 64 || JC * 8 == 128) &&
-                                      (size_t)N1 * JC * 8 <= REGIONS1;
-    static constexpr int JSW = JC * 8 == 128 ? 7 : 3;  // swizzle mask: 128-byte (SW128) or 64-byte (SW64) rows
+    // the warp's [N1][CW] output block leaves by one TMA store (rows of 32 bytes or more)
+    static constexpr bool TMA_OUT = STAGED && Q1 > 1;
     // the tile's input may be staged by TMA (16-byte box rows, one box of all N1 rows)
-    static constexpr bool TMA_IN = STAGED && (WPR * 4) % 16 == 0 && N1 <= 256;
+    static constexpr bool TMA_IN = STAGED && (WPR * 4) % 16 == 0;
     static constexpr size_t SMEM = REGIONS1 + 4 * (size_t)WORDS + 16 + 16;  // + mbarrier + TMEM slot
   };
 

@@ -83,24 +83,6 @@ __device__ __forceinline__ void team_sync(int team) {
   else asm volatile("bar.sync %0, %1;\n" ::"r"(1 + team), "r"(32 * W) : "memory");
 }
 
-// x e^{-2 pi i J / 64}, J compile-time (the butterflies' cosine-factored form)
-template <int J>
-__device__ __forceinline__ float2 turn64(float2 x) {
-  constexpr ct::CS cs = ct::cossin2pi(J, 64);
-  constexpr double wr = cs.c, wi = -cs.s;
-  if constexpr (J == 0) return x;
-  else if constexpr (J == 16) return make_float2(x.y, -x.x);
-  else if constexpr (ct::dabs(wr) >= ct::dabs(wi)) {
-    constexpr float r = (float)(wi / wr), sc = (float)wr;
-    const float2 u = __ffma2_rn(make_float2(x.y, x.x), make_float2(-r, r), x);
-    return __fmul2_rn(u, make_float2(sc, sc));
-  } else {
-    constexpr float r = (float)(wr / wi), sc = (float)wi;
-    const float2 v = __ffma2_rn(x, make_float2(-r, r), make_float2(x.y, x.x));
-    return __fmul2_rn(v, make_float2(-sc, sc));
-  }
-}
-
 template <int LOGN, int BITS>
 __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MINB) k_fused(BatchArgs a) {
   using PL = FusedPlan<LOGN>;

@@ -112,8 +112,6 @@ __device__ __forceinline__ long long seg_word0(const SegSrc& in, int s) {
 // Tensor maps of the packed input for phase 1's TMA staging: m[0][i] views IF i's staged
 // segments [0, n0) and m[1][i] its segments from n0 on, each as words x rows x segments.
 // use = 0: the kernel stages with 4-byte cp.async instead (layouts a tensor map cannot describe).
-// Where phase 1 has no tensor-map path (N1 >= 512), use = 1 says that rows are aligned for its
-// widest cp.async and no map is encoded.
 struct InMaps {
   CUtensorMap m[2][kMaxIF];
   int use;
@@ -349,26 +347,13 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
   using ST = typename PL::template Stage1<BITS>;
   constexpr bool STAGED = ST::STAGED;
   constexpr int TILE = ST::TILE, IPT = ST::IPT, WPR = STAGED ? ST::WPR : 1;  // words per IF per tile row
-  // the warp's [N1][CW] output block leaves by one TMA store (TMA_OUT), or the column
-  // group's [N1][JC] block, assembled over all warps' regions, by N1 / BOXR (JOINT)
-  constexpr bool TMA_OUT = ST::TMA_OUT, JOINT = ST::JOINT_OUT;
-  constexpr int BOXR = ST::BOXR, JC = ST::JC;
-  static_assert(!TMA_OUT || (Q1 > 1 && N1 == BOXR && (CW * 8) % 16 == 0 && N1 * CW <= PL::REGION1 &&
+  constexpr bool TMA_OUT = ST::TMA_OUT;  // the warp's [N1][CW] output block leaves by one TMA store
+  static_assert(!TMA_OUT || (Q1 > 1 && N1 <= 256 && (CW * 8) % 16 == 0 && N1 * CW <= PL::REGION1 &&
                              (PL::REGION1 * 8) % 128 == 0),
                 "TMA output tile");
-  static_assert(!JOINT || (N1 % BOXR == 0 && (BOXR * JC * 8) % 1024 == 0 && (size_t)N1 * JC * 8 <= PL::REGIONS1),
-                "joint output block");
   extern __shared__ __align__(1024) float2 sm1[];
   // (warp index and tensor-memory base broadcast from lane 0: uniform registers, as in phase 2)
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
-  if constexpr (JOINT) {
-    // the swizzled joint block needs a 1024-byte aligned base (the declaration asks for it);
-    // should that ever not hold, report and leave the work undone rather than misplace data
-    if ((smem_addr(sm1) & 1023u) != 0) {
-      if (tid == 0 && a.err) atomicExch(a.err, 1);
-      return;
-    }
-  }
   const int q1 = lane / CW, cw = lane % CW;
   float2* region = sm1 + warp * PL::REGION1;
   uint32_t* stage = reinterpret_cast<uint32_t*>(sm1 + PL::WARPS * PL::REGION1);  // staged, transposed words
@@ -377,7 +362,7 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
   // TMA staging of the input: possible for this plan (16-byte box rows) and chosen by the host
   // for this launch
   constexpr bool TIN = ST::TMA_IN;
-  static_assert(!TIN || (N1 % BOXR == 0 && (BOXR * WPR * 4) % 128 == 0), "TMA input boxes");
+  static_assert(!TIN || (N1 * WPR * 4) % 128 == 0, "TMA input boxes");
   const bool tin = TIN && in_maps.use != 0;
   if (TIN && tin && tid == 0) {
     mbar_init(bar0, 1);
@@ -429,57 +414,12 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
         bulk_wait_read();  // the previous output tile has left the region
         __syncwarp();
       }
-      if constexpr (JOINT) {
-        if (tid == 0) bulk_wait_read();  // the previous joint block has left the regions
-        __syncthreads();
-      }
       sfor<0, P>([&](auto p_) {
         constexpr int p = decltype(p_)::value;
         region[q1 * LDQ + p * LDP + cw] = v[p];
       });
       __syncwarp();
-      if constexpr (JOINT) {
-        sfor<0, PQ>([&](auto r_) {
-          constexpr int r = decltype(r_)::value;
-          const int p = r * Q1 + q1;
-          sfor<0, Q1>([&](auto q_) {
-            constexpr int q = decltype(q_)::value;
-            v[r * Q1 + ct::bitrev(q, Q1)] = region[q * LDQ + p * LDP + cw];
-          });
-          dit<Q1, r * Q1, 1>(v);
-        });
-        __syncthreads();  // every warp has read its transpose: the regions take the joint block
-        // joint block [c][JC] of 8-byte values, JC * 8 = 64 or 128 bytes per row, with the
-        // TMA swizzle of that row width: 16-byte chunk k of row c sits at chunk k ^ (row
-        // bits of the byte offset), so the 16 or 32 rows one store instruction writes fall
-        // on distinct chunks
-        // Row c = C0 + q1 with C0 = r Q1 + P m a multiple of 8: the row bits the swizzle
-        // takes (bits 7-9 of the offset for 128-byte rows, 7-8 for 64-byte rows) are those
-        // of the lane's own first row, and C0's part of the offset has no bits below the
-        // ninth, so the swizzled offset is the lane's swizzled base plus C0's part.
-        static_assert(Q1 % 8 == 0 && P % 8 == 0, "joint block swizzle per lane");
-        char* jb = reinterpret_cast<char*>(sm1);
-        const uint32_t jl = (uint32_t)((q1 * JC + warp * CW + cw) * 8);
-        char* jlane = jb + (jl ^ (((jl >> 7) & (uint32_t)ST::JSW) << 4));
-        sfor<0, PQ>([&](auto r_) {
-          constexpr int r = decltype(r_)::value;
-          sfor<0, Q1>([&](auto m_) {
-            constexpr int m = decltype(m_)::value;
-            *reinterpret_cast<float2*>(jlane + (r * Q1 + P * m) * JC * 8) =
-                slab_val(v[r * Q1 + m], r * Q1 + q1 + P * m);
-          });
-        });
-        fence_async_shared();
-        __syncthreads();
-        if (tid == 0 && act) {  // xcol of warp 0 = the column group's first column
-          sfor<0, N1 / BOXR>([&](auto h_) {
-            constexpr int h = decltype(h_)::value;
-            tma_store_2d(&slab_map, smem_addr(jb + h * BOXR * JC * 8), xcol, (int)(g * N1 + h * BOXR),
-                         l2_evict_last());
-          });
-          bulk_commit();
-        }
-      } else if constexpr (TMA_OUT) {
+      if constexpr (TMA_OUT) {
         sfor<0, PQ>([&](auto r_) {
           constexpr int r = decltype(r_)::value;
           const int p = r * Q1 + q1;
@@ -556,16 +496,15 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
     // before; the CTA transposes their codes (polaris_codes.cuh), and every lane then takes its
     // rows with a few vector loads.  (Decoding from the staged words themselves, a 4-byte load,
     // a funnel shift and a logic operation per sample, bound this kernel: shared-memory pipe 77%
-    // busy at 2^14 and 8 bits, the loads up to four-way bank-conflicted; at N1 >= 512 the words
-    // came in 4-byte copies.  Kernel times before and after, beside the others of a pass: 15 x 2^20
+    // busy at 2^14 and 8 bits, the loads up to four-way bank-conflicted; at 2^18 and up, where it
+    // measured most, the words came in 4-byte copies.  Kernel times before and after, beside the others of a pass: 15 x 2^20
     // int8 Hann 113 -> 68 us, 122 x 2^18 int8 Hann 172 -> 109 us (of which the taps' order 27 us),
     // 122 x 2^17 4-bit 30.2 -> 27.3 us; 2^17 2-bit unchanged alone, 1% in a three-handle pipeline.)
     const long long n_tiles = total_cols / TILE;
-    uint32_t* tr = stage + ST::TR0;
+    uint32_t* tr = stage + ST::RAWW;
     const uint32_t raw_a = smem_addr(stage);
     constexpr int ROWW = N2 * BITS / 32;  // words per row of a segment
-    auto issue_words = [&](long long tile, auto vec_) {
-      constexpr int V = decltype(vec_)::value;  // words per copy
+    auto issue = [&](long long tile) {  // (inputs that a tensor map cannot describe)
       const int g = (int)(tile / (N2 / TILE)), b0 = (int)(tile % (N2 / TILE)) * TILE;
       const int s_local = g / a.n_fpair, f = g - s_local * a.n_fpair;
       const int sg = a.seg0 + s_local;
@@ -574,20 +513,15 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
       const uint32_t* pb = ib >= 0 ? seg_ptr(a.in, ib, sg) + (b0 * BITS) / 32 : pa;
       const long long w0 = seg_word0(a.in, sg) + (b0 * BITS) / 32;
       const long long wext = sg < a.in.n0 ? a.in.in_words0 : a.in.in_words1;
-      constexpr int K = N1 * WPR / V;  // copies per IF
 #pragma unroll 4
-      for (int k = tid; k < K; k += PL::THREADS) {
-        const uint32_t so = (uint32_t)((k / (WPR / V)) * ROWW + (k % (WPR / V)) * V);
-        if (in_bounds(a.err, w0 + so + V - 1, wext)) {
-          cp_async<4 * V>(raw_a + 4u * (uint32_t)(k * V), pa + so);
-          cp_async<4 * V>(raw_a + 4u * (uint32_t)(N1 * WPR + k * V), pb + so);  // (IF a again without an IF b)
+      for (int k = tid; k < N1 * WPR; k += PL::THREADS) {
+        const uint32_t so = (uint32_t)((k / WPR) * ROWW + k % WPR);
+        if (in_bounds(a.err, w0 + so, wext)) {
+          cp_async4(raw_a + 4u * (uint32_t)k, pa + so);
+          cp_async4(raw_a + 4u * (uint32_t)(N1 * WPR + k), pb + so);  // (IF a again without an IF b)
         }
       }
       cp_async_commit();
-    };
-    auto issue = [&](long long tile) {
-      if (ST::VEC > 1 && !TIN && in_maps.use) issue_words(tile, std::integral_constant<int, ST::VEC>{});
-      else issue_words(tile, std::integral_constant<int, 1>{});
     };
     // TMA staging: one thread loads the tile's words of each IF (N1 rows x WPR words) and the
     // CTA waits on the mbarrier (bounded)
@@ -653,27 +587,14 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
       // this tile's words are staged; every warp has decoded the tile before
       if (__syncthreads_or(timed_out)) break;
       const long long next = unit + G;
-      if constexpr (ST::INPLACE) {
-        constexpr int UPT = ST::UNITS / PL::THREADS;
-        uint32_t x[UPT][ST::KB][32 / BITS];
-        sfor<0, UPT>([&](auto i_) {
-          p1_unit_load<PL, ST, BITS>(stage, tid + decltype(i_)::value * PL::THREADS, x[decltype(i_)::value]);
-        });
-        __syncthreads();
-        sfor<0, UPT>([&](auto i_) {
-          p1_unit_store<PL, ST, BITS>(tr, tid + decltype(i_)::value * PL::THREADS, x[decltype(i_)::value]);
-        });
-        __syncthreads();
-      } else {
 #pragma unroll 1
-        for (int u = tid; u < ST::UNITS; u += PL::THREADS) {
-          uint32_t x[ST::KB][32 / BITS];
-          p1_unit_load<PL, ST, BITS>(stage, u, x);
-          p1_unit_store<PL, ST, BITS>(tr, u, x);
-        }
-        __syncthreads();
-        if (next < n_units) issue_next(unit_tile(next));
+      for (int u = tid; u < ST::UNITS; u += PL::THREADS) {
+        uint32_t x[ST::KB][32 / BITS];
+        p1_unit_load<PL, ST, BITS>(stage, u, x);
+        p1_unit_store<PL, ST, BITS>(tr, u, x);
       }
+      __syncthreads();
+      if (next < n_units) issue_next(unit_tile(next));
       if (next >= n_units) pdl_trigger();  // this CTA's last unit: phase 2 may be scheduled
       const int g = (int)(tile / (N2 / TILE)), b0 = (int)(tile % (N2 / TILE)) * TILE;
       const int f = g % a.n_fpair;
@@ -713,18 +634,12 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
           if (has_b) decode(T_{}, F_{});
           else decode(F_{}, F_{});
         }
-        if constexpr (ST::INPLACE) {
-          if (it == it_end - 1) {
-            __syncthreads();  // every warp has decoded the tile: the buffer is free
-            if (next < n_units) issue_next(unit_tile(next));
-          }
-        }
         finish(v, true, g, b, b0 + (it * PL::WARPS + warp) * CW);
       }
     }
     cp_async_wait_all();
   }
-  if constexpr (TMA_OUT || JOINT) {
+  if constexpr (TMA_OUT) {
     bulk_wait_all();  // output tiles written before the CTA's shared memory goes
   }
   if constexpr (Q1 > 1) cta_tmem_end<PL::TCOLS1>(tbase, warp);
@@ -865,6 +780,8 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, 2) k_phase2(BatchArgs a, 
     tmem_wait_st();
     if (!waited) {
       pdl_wait();
+      // (phase 1 of 2^18 and up writes the slab by ordinary stores, the copy engine reads it)
+      asm volatile("fence.proxy.async.global;\n" ::: "memory");
       waited = true;
     }
     float extra[4] = {0.f, 0.f, 0.f, 0.f};
@@ -1126,10 +1043,8 @@ static int ctas_per_sm(K kernel, int threads, size_t smem, int tmem_cols) {
 }
 
 // Tensor map over the slab of one batch, rows (pair-segment, c) x columns b of 8-byte
-// complex values; box = box_cols columns x box_rows rows of an output block, laid out in
-// shared memory with the given swizzle.
-static cudaError_t encode_slab_map(CUtensorMap* map, float2* slab, long long rows, int n2, int box_cols, int box_rows,
-                                   CUtensorMapSwizzle swizzle) {
+// complex values; box = box_cols columns x box_rows rows of an output block.
+static cudaError_t encode_slab_map(CUtensorMap* map, float2* slab, long long rows, int n2, int box_cols, int box_rows) {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
     cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
@@ -1144,16 +1059,16 @@ static cudaError_t encode_slab_map(CUtensorMap* map, float2* slab, long long row
   const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
   const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, slab, dims, strides, box, estr,
-                            CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 // Tensor map over one IF's packed input: 32-bit words x rows (row_bytes apart) x segments
-// (seg_bytes apart); box = one tile's words of box_rows rows of one segment.  Fails (and
+// (seg_bytes apart); box = box_words words of box_rows rows of one segment.  Fails (and
 // phase 1 then stages with cp.async) for an address that is not 16-byte aligned.
-static cudaError_t encode_input_map(CUtensorMap* map, const uint32_t* base, int words_per_row, int rows, int box_rows,
-                                    long long segs, long long row_bytes, long long seg_bytes, int box_words) {
+static cudaError_t encode_input_map(CUtensorMap* map, const uint32_t* base, int words_per_row, int rows, long long segs,
+                                    long long row_bytes, long long seg_bytes, int box_words, int box_rows) {
   if ((reinterpret_cast<uintptr_t>(base) & 15) != 0) return cudaErrorMisalignedAddress;
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   if (!encode) {
@@ -1173,6 +1088,10 @@ static cudaError_t encode_input_map(CUtensorMap* map, const uint32_t* base, int 
                             CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
+
+}  // namespace polaris
+#include "polaris_wide.cuh"
+namespace polaris {
 
 template <int LOGN, int BITS>
 static cudaError_t launch_phase1(const BatchArgs& a, cudaStream_t st, bool pdl) {
@@ -1228,13 +1147,9 @@ static cudaError_t launch_phase1(const BatchArgs& a, cudaStream_t st, bool pdl) 
     cache_next = (cache_next + 1) % 8;
     ms->valid = false;
     memset(&ms->slab, 0, sizeof ms->slab);
-    if constexpr (ST::TMA_OUT || ST::JOINT_OUT) {  // the kernel's TMA output paths
+    if constexpr (ST::TMA_OUT) {
       if ((reinterpret_cast<uintptr_t>(a.scratch) & 15) != 0) return cudaErrorMisalignedAddress;
-      const cudaError_t e =
-          ST::TMA_OUT ? encode_slab_map(&ms->slab, a.scratch, key.slab_rows, PL::N2, PL::CW, PL::N1,
-                                        CU_TENSOR_MAP_SWIZZLE_NONE)
-                      : encode_slab_map(&ms->slab, a.scratch, key.slab_rows, PL::N2, ST::JC, ST::BOXR,
-                                        ST::JSW == 7 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
+      const cudaError_t e = encode_slab_map(&ms->slab, a.scratch, key.slab_rows, PL::N2, PL::CW, PL::N1);
       if (e != cudaSuccess) return e;
     }
     // input maps for TMA staging (else the kernel stages with cp.async)
@@ -1250,21 +1165,9 @@ static cudaError_t launch_phase1(const BatchArgs& a, cudaStream_t st, bool pdl) 
             const long long nseg_src = key.nsrc[src][ifx];
             if (nseg_src <= 0) continue;
             const uint32_t* base = src == 0 ? a.in.src0[ifx] : a.in.src1[ifx];
-            ok = encode_input_map(&ms->in.m[src][ifx], base, PL::N2 * BITS / 32, PL::N1, ST::BOXR, nseg_src,
-                                  row_bytes, seg_bytes, ST::WPR) == cudaSuccess;
+            ok = encode_input_map(&ms->in.m[src][ifx], base, PL::N2 * BITS / 32, PL::N1, nseg_src,
+                                  row_bytes, seg_bytes, ST::WPR, PL::N1) == cudaSuccess;
           }
-        }
-      ms->in.use = ok ? 1 : 0;
-    } else if constexpr (ST::STAGED && ST::VEC > 1) {
-      // rows of VEC words aligned for the widest cp.async?
-      constexpr uintptr_t m = 4 * ST::VEC - 1;
-      bool ok = (a.in.hop_w * 4 & (long long)m) == 0;
-      for (int f = 0; f < a.n_fpair && ok; ++f)
-        for (int k = 0; k < 2 && ok; ++k) {
-          const int ifx = k == 0 ? a.fa[f] : a.fb[f];
-          if (ifx < 0) continue;
-          if (key.nsrc[0][ifx] > 0) ok = (reinterpret_cast<uintptr_t>(a.in.src0[ifx]) & m) == 0;
-          if (key.nsrc[1][ifx] > 0) ok = ok && (reinterpret_cast<uintptr_t>(a.in.src1[ifx]) & m) == 0;
         }
       ms->in.use = ok ? 1 : 0;
     }
@@ -1291,14 +1194,19 @@ static cudaError_t launch_phase1(const BatchArgs& a, cudaStream_t st, bool pdl) 
 }
 
 // phase 1 of one batch
+template <int LOGN, int BITS>
+static cudaError_t launch_phase1_any(const BatchArgs& a, cudaStream_t st, bool pdl) {
+  if constexpr (Plan<LOGN>::WIDE) return launch_phase1w<LOGN, BITS>(a, st, pdl);
+  else return launch_phase1<LOGN, BITS>(a, st, pdl);
+}
 template <int LOGN>
 cudaError_t run_phase1(const BatchArgs& a, cudaStream_t st, bool pdl) {
   if (a.nseg <= 0) return cudaSuccess;
   switch (a.bits) {
-    case 1: return launch_phase1<LOGN, 1>(a, st, pdl);
-    case 2: return launch_phase1<LOGN, 2>(a, st, pdl);
-    case 4: return launch_phase1<LOGN, 4>(a, st, pdl);
-    case 8: return launch_phase1<LOGN, 8>(a, st, pdl);
+    case 1: return launch_phase1_any<LOGN, 1>(a, st, pdl);
+    case 2: return launch_phase1_any<LOGN, 2>(a, st, pdl);
+    case 4: return launch_phase1_any<LOGN, 4>(a, st, pdl);
+    case 8: return launch_phase1_any<LOGN, 8>(a, st, pdl);
     default: return cudaErrorInvalidValue;
   }
 }
