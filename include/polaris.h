@@ -340,7 +340,7 @@ const char* polaris_adj_last_error(const polaris_adj* h);
  * Twiddles and DFT matrices are FP64-computed; integration accumulators are FP64.
  * polaris_tc_create: n_fft 4096 (= 64^2) or 262144 (= 64^3); bits 1/2/4/8; window
  *   POLARIS_WIN_* (taps: n_fft floats for POLARIS_WIN_CUSTOM, copied); on `device`.
- *   Holds about 85 MB of device memory (two pass buffers of 40 MB).
+ *   Holds about 70 MB of device memory (two 32 MB pass buffers).
  * polaris_tc_feed: packed[2] are DEVICE pointers to the two IFs' packed streams (layout as
  *   spectrometer_feed), n_samples each, a multiple of n_fft (whole segments, hop = n_fft);
  *   queued on cuda_stream (NULL = legacy stream); accumulates.

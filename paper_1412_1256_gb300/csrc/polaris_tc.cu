@@ -40,13 +40,10 @@ namespace polaris {
 namespace tc {
 
 constexpr int kR = 64;             // radix of a pass
-constexpr int kRows = 128;         // GEMM M: vectors per tile, kHalves threads each
-constexpr int kHalves = 2;         // a vector's threads: 32 of its 64 points each (16 warps of 128 registers per SM;
-                                   // with one thread and 255 registers per vector, 8 warps kept too few loads in flight)
-constexpr int kPts = kR / kHalves;
+constexpr int kRows = 128;         // GEMM M: vectors per tile, one per thread
 constexpr int kK = 2 * kR;         // GEMM K and N in reals
 constexpr int kGroups = 2;         // independent tile groups per CTA (their latencies overlap)
-constexpr int kGroupThreads = kRows * kHalves;
+constexpr int kGroupThreads = kRows;
 constexpr int kThreads = kGroups * kGroupThreads;
 constexpr uint32_t kOpBytes = kRows * kK * 2;      // one 16-bit operand tile: 32 KB
 constexpr uint32_t kLBO = 128;                     // core matrices (8 rows x 16 B) along K
@@ -58,8 +55,7 @@ constexpr uint32_t kOffAh = 0, kOffAl = kOpBytes;
 constexpr uint32_t kStageBytes = kRows * kStagePitch * 8;
 constexpr uint32_t kGroupBytes = (kStageBytes + 127) / 128 * 128;
 constexpr uint32_t kOffBh = kGroups * kGroupBytes, kOffBl = kOffBh + kOpBytes;
-constexpr uint32_t kOffMax = kOffBl + kOpBytes;    // largest value per vector half (fp16 scaling): [group][half][row]
-constexpr uint32_t kOffBar = kOffMax + 4 * kGroups * kHalves * kRows, kOffSlot = kOffBar + 8 * kGroups;
+constexpr uint32_t kOffBar = kOffBl + kOpBytes, kOffSlot = kOffBar + 8 * kGroups;
 constexpr uint32_t kSmemBytes = kOffSlot + 8;
 constexpr uint32_t kTmemCols = 128 * kGroups;      // group g accumulates in columns [128 g, 128 g + 128)
 constexpr uint32_t kWaitAfter = 1u << 24;
@@ -97,7 +93,7 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t ad, uint64_t bd,
       : "memory");
 }
 
-// barrier over the threads of tile group g (named barrier 1 + g)
+// barrier over the 128 threads of tile group g (named barrier 1 + g)
 __device__ __forceinline__ void group_sync(int g) {
   asm volatile("bar.sync %0, %1;\n" ::"r"(1 + g), "r"(kGroupThreads) : "memory");
 }
@@ -160,22 +156,20 @@ __device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& lo) {
 }
 
 // One radix-64 pass over all vectors of a batch (BITS > 0: the first pass, from the packed
-// samples).  Persistent CTAs of two tile groups of 256 threads; tiles of 128 consecutive
+// samples).  Persistent CTAs of two tile groups of 128 threads; tiles of 128 consecutive
 // vectors (global vector v = segment * m + j) go round robin to the groups of all CTAs.
-// Threads t and 128 + t of a group own vector tile * 128 + t, its inputs r < 32 and r >= 32 and then its
-// outputs q likewise (TMEM lane t of the group's columns).
+// Thread t of a group owns vector tile * 128 + t and TMEM lane t of the group's columns.
 template <int PREC, int BITS>
 __global__ void __launch_bounds__(kThreads, 1) k_tc_pass(PassArgs a) {
   extern __shared__ __align__(128) uint8_t sm[];
-  const int gr = threadIdx.x / kGroupThreads, gt = threadIdx.x % kGroupThreads;
-  const int t = gt % kRows, half = gt / kRows, w = t >> 5, r0 = half * kPts;  // row, half (the same for a warp)
+  const int gr = threadIdx.x / kGroupThreads, t = threadIdx.x % kGroupThreads, w = t >> 5;
   uint8_t* sg = sm + gr * kGroupBytes;
   const uint32_t bar = saddr(sm + kOffBar + 8 * gr);
   uint32_t* slot = reinterpret_cast<uint32_t*>(sm + kOffSlot);
   constexpr int NPROD = PREC == POLARIS_TC_BF16X1 ? 1 : 3;
   constexpr int NB = (PREC == POLARIS_TC_BF16X1 ? 1 : 2) * (int)kOpBytes / 16;
   for (int i = threadIdx.x; i < NB; i += kThreads) reinterpret_cast<uint4*>(sm + kOffBh)[i] = __ldg(a.bmat + i);
-  if (gt == 0) {
+  if (t == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -203,62 +197,54 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_pass(PassArgs a) {
     const bool valid = g < rows;
     const long long gv = valid ? g : 0;
     const int s = (int)(gv / a.m), j = (int)(gv - (long long)s * a.m);
-    float v[2 * kPts];  // this half's real parts, then its imaginary parts
+    float v[kK];
     if constexpr (BITS > 0) {
-      const int j0 = j + r0 * a.m;
-      const long long base = a.sample0 + (long long)s * a.N + j0;
+      const long long base = a.sample0 + (long long)s * a.N + j;
 #pragma unroll
-      for (int r = 0; r < kPts; ++r) {
-        const float wn = __ldg(a.window + j0 + r * a.m);
+      for (int r = 0; r < kR; ++r) {
+        const float wn = __ldg(a.window + j + r * a.m);
         v[r] = wn * tc_level<BITS>(a.in[0], base + (long long)r * a.m);
-        v[kPts + r] = wn * tc_level<BITS>(a.in[1], base + (long long)r * a.m);
+        v[kR + r] = wn * tc_level<BITS>(a.in[1], base + (long long)r * a.m);
       }
     } else {
-      const float2* src = a.src + (long long)s * a.N + j + (long long)r0 * a.m;
-      const float2* tw = a.tw + (r0 * a.Ns + (j & (a.Ns - 1)) - 1);
+      const float2* src = a.src + (long long)s * a.N + j;
+      const int k = j & (a.Ns - 1);
 #pragma unroll
-      for (int r = 0; r < kPts; ++r) {
+      for (int r = 0; r < kR; ++r) {
         float2 z = __ldcg(src + (long long)r * a.m);
-        if (r > 0 || half > 0) z = cmul(z, __ldg(tw + r * a.Ns));
+        if (r > 0) z = cmul(z, __ldg(a.tw + (r * a.Ns + k - 1)));
         v[r] = z.x;
-        v[kPts + r] = z.y;
+        v[kR + r] = z.y;
       }
     }
     float inv_scale = 1.f;
     if constexpr (PREC == POLARIS_TC_FP16X3) {
       float amax = 0.f;
 #pragma unroll
-      for (int i = 0; i < 2 * kPts; ++i) amax = fmaxf(amax, fabsf(v[i]));
-      // the vector's largest value, over both halves (the barriers at the end of the loop and below keep
-      // tiles apart)
-      float* most = reinterpret_cast<float*>(sm + kOffMax) + gr * kHalves * kRows;
-      most[half * kRows + t] = amax;
-      group_sync(gr);
-      amax = fmaxf(most[t], most[kRows + t]);
+      for (int i = 0; i < kK; ++i) amax = fmaxf(amax, fabsf(v[i]));
       int e = 0;
       frexpf(amax, &e);  // amax = f 2^e, f in [0.5, 1); zero gives e = 0
       const float sc = ldexpf(1.f, 15 - e);
       inv_scale = ldexpf(1.f, e - 15);
 #pragma unroll
-      for (int i = 0; i < 2 * kPts; ++i) v[i] *= sc;
+      for (int i = 0; i < kK; ++i) v[i] *= sc;
     }
     if (!valid) {
 #pragma unroll
-      for (int i = 0; i < 2 * kPts; ++i) v[i] = 0.f;
+      for (int i = 0; i < kK; ++i) v[i] = 0.f;
     }
 #pragma unroll
-    for (int kc = 0; kc < 2 * kPts / 8; ++kc) {
+    for (int kc = 0; kc < kK / 8; ++kc) {
       uint4 hi, lo;
       split8<PREC>(v + 8 * kc, hi, lo);
-      const int k = (kc < kPts / 8 ? 8 * kc : kR + 8 * (kc - kPts / 8)) + r0;  // [Re | Im] of all 64 inputs
-      *reinterpret_cast<uint4*>(sg + kOffAh + op_off(t, k)) = hi;
-      if constexpr (NPROD == 3) *reinterpret_cast<uint4*>(sg + kOffAl + op_off(t, k)) = lo;
+      *reinterpret_cast<uint4*>(sg + kOffAh + op_off(t, 8 * kc)) = hi;
+      if constexpr (NPROD == 3) *reinterpret_cast<uint4*>(sg + kOffAl + op_off(t, 8 * kc)) = lo;
     }
     // operands visible to the tensor cores; the previous tile's TMEM reads are complete
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     group_sync(gr);
-    if (gt == 0) {
+    if (t == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
       const uint32_t ah = saddr(sg + kOffAh), al = saddr(sg + kOffAl);
       const uint32_t bh = saddr(sm + kOffBh), bl = saddr(sm + kOffBl);
@@ -277,20 +263,20 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_pass(PassArgs a) {
     // one decision for the whole group (every thread leaves the loop at the same tile)
     if (group_any(gr, !wait_parity(bar, parity, a.wait_limit))) {
       failed = true;
-      if (gt == 0 && a.err) atomicOr(a.err, 1);
+      if (t == 0 && a.err) atomicOr(a.err, 1);
       wait_parity(bar, parity, kWaitAfter);  // the products in flight land before the exit
     }
     parity ^= 1u;
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    // row t of D: Re b_q in columns q, Im b_q in columns 64 + q; this half's 32 q of each
+    // row t of D: Re b_q in columns q, Im b_q in columns 64 + q
 #pragma unroll
-    for (int c = 0; c < 2 * kPts; c += 16) {
+    for (int c = 0; c < kK; c += 16) {
       uint32_t u[16];
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
           : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
             "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
-          : "r"(tmem + ((uint32_t)(32 * w) << 16) + (uint32_t)(r0 + (c < kPts ? c : c - kPts + kR)))
+          : "r"(tmem + ((uint32_t)(32 * w) << 16) + (uint32_t)c)
           : "memory");
 #pragma unroll
       for (int i = 0; i < 16; ++i) v[c + i] = __uint_as_float(u[i]) * inv_scale;
@@ -298,19 +284,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_pass(PassArgs a) {
     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
     if constexpr (BITS > 0) {
       // output row g = 64 consecutive values at 64 g: through shared memory (pitch 65
-      // float2), then the group writes the tile's 64 KB contiguously
+      // float2), then 128 threads write the tile's 64 KB contiguously
       float2* stage = reinterpret_cast<float2*>(sg);
 #pragma unroll
-      for (int q = 0; q < kPts; ++q) stage[t * kStagePitch + r0 + q] = make_float2(v[q], v[kPts + q]);
+      for (int q = 0; q < kR; ++q) stage[t * kStagePitch + q] = make_float2(v[q], v[kR + q]);
       group_sync(gr);
       const long long out0 = (long long)tile * kRows * kR;
       const int nvals = (int)(min((long long)kRows, rows - (long long)tile * kRows) * kR);
-      for (int e = gt; e < nvals; e += kGroupThreads) __stcg(a.dst + out0 + e, stage[(e / kR) * kStagePitch + (e % kR)]);
+      for (int e = t; e < nvals; e += kGroupThreads) __stcg(a.dst + out0 + e, stage[(e / kR) * kStagePitch + (e % kR)]);
     } else if (valid) {
       const int k = j & (a.Ns - 1);
-      float2* dst = a.dst + (long long)s * a.N + (long long)(j - k) * kR + k + (long long)r0 * a.Ns;
+      float2* dst = a.dst + (long long)s * a.N + (long long)(j - k) * kR + k;
 #pragma unroll
-      for (int q = 0; q < kPts; ++q) __stcg(dst + (long long)q * a.Ns, make_float2(v[q], v[kPts + q]));
+      for (int q = 0; q < kR; ++q) __stcg(dst + (long long)q * a.Ns, make_float2(v[q], v[kR + q]));
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     group_sync(gr);  // stage reads and TMEM reads done before the next tile's operands
@@ -338,7 +324,7 @@ __global__ void __launch_bounds__(256) k_tc_correlate(const float2* __restrict__
   if (k >= nbin) return;
   const int km = (N - k) & (N - 1);
   float sm[4] = {0.f, 0.f, 0.f, 0.f}, cp[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
+#pragma unroll 4
   for (int s = 0; s < nseg; ++s) {
     const float2 a = __ldcg(Z + (long long)s * N + k), b = __ldcg(Z + (long long)s * N + km);
     const float xr = 0.5f * (a.x + b.x), xi = 0.5f * (a.y - b.y);
@@ -495,6 +481,7 @@ extern "C" int polaris_tc_create(int64_t n_fft, int bits, int window, const floa
   h->prec = precision;
   h->device = device;
   h->nbin = h->N / 2 + 1;
+  h->batch = (int)std::max<int64_t>(2, (int64_t)(32u << 20) / ((int64_t)h->N * 8));  // 32 MB per buffer
   int prev = 0;
   cudaGetDevice(&prev);
   cudaSetDevice(device);
@@ -513,10 +500,7 @@ extern "C" int polaris_tc_create(int64_t n_fft, int bits, int window, const floa
     delete h;
     return tc_err(nullptr, POLARIS_ECUDA, std::string("tensor-core kernels cannot be launched: ") + cudaGetErrorString(e));
   }
-  h->grid = nsm;  // one CTA (two tile groups, 196 KB) per SM
-  // segments per batch: two whole rounds of tiles over the CTAs' groups (19 at 2^18 on 152 SMs, 40 MB per
-  // pass buffer; 16 filled 84% of two rounds), so that both buffers stay in L2
-  h->batch = std::max(2, 2 * nsm * kGroups * kRows / h->m);
+  h->grid = nsm;  // one CTA (two tile groups, 194 KB) per SM
   // window taps (FP64-computed, rounded once)
   std::vector<float> win(h->N);
   for (int n = 0; n < h->N; ++n) {
