@@ -53,6 +53,7 @@
 
 #include "../../include/polaris.h"
 #include "polaris_adjoint.cuh"
+#include "polaris_kernels.cuh"  // dependent launch
 
 namespace polaris {
 
@@ -167,11 +168,8 @@ __device__ __forceinline__ void adj_window_segment(const AdjArgs& a, float2* z, 
   for (int k = threadIdx.x; k < nbin; k += a.threads) {
     const int km = (N - k) & (N - 1);
     const float2 Zk = z[apad(k)], Zm = c_conj(z[apad(km)]);
-    const float2 X = make_float2(0.5f * (Zk.x + Zm.x), 0.5f * (Zk.y + Zm.y));
-    const float2 Y = make_float2(0.5f * (Zk.y - Zm.y), -0.5f * (Zk.x - Zm.x));
-    const float4 r0 = __ldg(a.mat + 2 * k), r1 = __ldg(a.mat + 2 * k + 1);
-    const float2 GX = c_add(cmul(make_float2(r0.x, r0.y), X), cmul(make_float2(r0.z, r0.w), Y));
-    const float2 GY = c_add(cmul(make_float2(r1.x, r1.y), X), cmul(make_float2(r1.z, r1.w), Y));
+    float2 GX, GY;
+    adj_bin_gradient(__ldg(a.mat + k), Zk, Zm, GX, GY);
     if (k == 0 || 2 * k == N) {
       z[apad(k)] = make_float2(GX.x, -GY.x);  // H = Re G_X + i Re G_Y
     } else {
@@ -226,37 +224,54 @@ struct BinArgs {
 };
 
 // A block covers kBinsPerBlock bins; its kSlices warps sum the per-CTA partials of the
-// segment kernel (one 16-byte load per CTA and bin) over interleaved slices of CTAs in fp32
-// (many loads in flight), the slice sums are added in fp64 in slice order, then one warp
+// segment kernel (one 16-byte load per CTA and bin) over interleaved slices of CTAs in fp32, the
+// slice sums are added in fp64 in slice order (one warp per quantity), then one warp
 // evaluates the model per bin: the sums, Stokes and loss in fp64, the gradients and the
 // window-adjoint matrix in fp32.
-constexpr int kBinsPerBlock = 32, kSlices = 8;
+// Bound by the latency of the loads: kInFlight of them per thread are started together, which
+// holds a slice of a grid of one CTA per SM (152 / 8 = 19) in one round.
+constexpr int kBinsPerBlock = 32, kSlices = 8, kInFlight = 20;
 
-__global__ void __launch_bounds__(kBinsPerBlock * kSlices) k_adj_bins(BinArgs a) {
+__global__ void __launch_bounds__(kBinsPerBlock * kSlices, 2) k_adj_bins(BinArgs a) {
   __shared__ float red[kSlices][4][kBinsPerBlock];
+  __shared__ double tot[5][kBinsPerBlock];
   const int nbin = a.nbin;
   const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
   const int k = blockIdx.x * kBinsPerBlock + lane;
   float s4[4] = {0.f, 0.f, 0.f, 0.f};
+  pdl_wait();  // the segment kernel's partials (dependent launch)
   if (k < nbin) {
-#pragma unroll 8
-    for (int g = sl; g < a.grid; g += kSlices) {
-      const float4 v = __ldcg(a.part + (size_t)g * nbin + k);
-      s4[0] += v.x;
-      s4[1] += v.y;
-      s4[2] += v.z;
-      s4[3] += v.w;
+#pragma unroll 1
+    for (int g0 = sl; g0 < a.grid; g0 += kSlices * kInFlight) {
+      float4 v[kInFlight];
+#pragma unroll
+      for (int i = 0; i < kInFlight; ++i) {
+        const int g = g0 + i * kSlices;
+        if (g < a.grid) v[i] = __ldcg(a.part + (size_t)g * nbin + k);
+      }
+#pragma unroll
+      for (int i = 0; i < kInFlight; ++i)
+        if (g0 + i * kSlices < a.grid) {
+          s4[0] += v[i].x;
+          s4[1] += v[i].y;
+          s4[2] += v[i].z;
+          s4[3] += v[i].w;
+        }
     }
   }
+  pdl_trigger();
 #pragma unroll
   for (int q = 0; q < 4; ++q) red[sl][q][lane] = s4[q];
   __syncthreads();
-  if (sl != 0) return;
+  if (sl < 4) {
+    double t = 0.0;
+    for (int w = 0; w < kSlices; ++w) t += (double)red[w][sl][lane];
+    tot[sl][lane] = t;
+  }
+  __syncthreads();
   double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  if (k < nbin) {
-    double t4[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int w = 0; w < kSlices; ++w)
-      for (int q = 0; q < 4; ++q) t4[q] += (double)red[w][q][lane];
+  if (sl == 0 && k < nbin) {
+    const double t4[4] = {tot[0][lane], tot[1][lane], tot[2][lane], tot[3][lane]};
     const double A = t4[0], B = t4[1];
     const dc C = {t4[2], t4[3]};
     const dc gR = {a.gains[0], a.gains[1]}, gL = {a.gains[2], a.gains[3]};
@@ -299,25 +314,28 @@ __global__ void __launch_bounds__(kBinsPerBlock * kSlices) k_adj_bins(BinArgs a)
         a.grad_leak[2 * (nbin + k)] = gDL.x;
         a.grad_leak[2 * (nbin + k) + 1] = gDL.y;
         // G_Xt = al1 X + be1 Y, G_Yt = al2 X + be2 Y; G_X = conj(gR) G_Xt + conj(gL DL) G_Yt,
-        // G_Y = conj(gR DR) G_Xt + conj(gL) G_Yt
+        // G_Y = conj(gR DR) G_Xt + conj(gL) G_Yt: a Hermitian matrix (the loss is a real function
+        // of |X|^2, |Y|^2 and X conj(Y)), kept as its two real entries and m12
         const float2 gLDL = cmul(fgL, fDL), gRDR = cmul(fgR, fDR);
         const float2 al1 = c_add(fscale(fgR, 2.f * ca), cmul(c, gLDL));
         const float2 be1 = c_add(fscale(gRDR, 2.f * ca), cmul(c, fgL));
         const float2 al2 = c_add(fscale(gLDL, 2.f * cb), cmul(cc, fgR));
         const float2 be2 = c_add(fscale(fgL, 2.f * cb), cmul(cc, gRDR));
         const float2 m11 = c_add(cmulc(fgR, al1), cmulc(gLDL, al2)), m12 = c_add(cmulc(fgR, be1), cmulc(gLDL, be2));
-        const float2 m21 = c_add(cmulc(gRDR, al1), cmulc(fgL, al2)), m22 = c_add(cmulc(gRDR, be1), cmulc(fgL, be2));
-        a.mat[2 * k] = make_float4(m11.x, m11.y, m12.x, m12.y);
-        a.mat[2 * k + 1] = make_float4(m21.x, m21.y, m22.x, m22.y);
+        const float2 m22 = c_add(cmulc(gRDR, be1), cmulc(fgL, be2));
+        a.mat[k] = make_float4(m11.x, m22.x, m12.x, m12.y);
       }
     }
   }
-  if (a.bpart) {
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      double v = acc[q];
+  if (a.bpart) {  // (uniform)
+    __syncthreads();  // tot has been read
+    if (sl == 0)
+      for (int q = 0; q < 5; ++q) tot[q][lane] = acc[q];
+    __syncthreads();
+    if (sl < 5) {  // one warp per quantity
+      double v = tot[sl][lane];
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) a.bpart[5 * blockIdx.x + q] = v;
+      if (lane == 0) a.bpart[5 * blockIdx.x + sl] = v;
     }
   }
 }
@@ -325,9 +343,11 @@ __global__ void __launch_bounds__(kBinsPerBlock * kSlices) k_adj_bins(BinArgs a)
 // five warps, one per quantity: block partials summed lane-strided, then across the warp
 // (the last block of k_adj_bins to finish doing this instead, elected by an atomic ticket
 // after a memory fence, measured slower: 20.6 us against 13.4 + 3.7 us)
-__global__ void __launch_bounds__(160) k_adj_finish(const double* bpart, int blocks, double* loss, float* grad_gains) {
+__device__ __forceinline__ void adj_finish(const double* bpart, int blocks, double* loss, float* grad_gains) {
   const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (q >= 5) return;
   double t = 0.0;
+#pragma unroll 4
   for (int b = lane; b < blocks; b += 32) t += bpart[5 * b + q];
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   if (lane == 0) {
@@ -338,19 +358,42 @@ __global__ void __launch_bounds__(160) k_adj_finish(const double* bpart, int blo
     }
   }
 }
+// (without gradients; with them k_adj_wsum's last block does it)
+__global__ void __launch_bounds__(160) k_adj_finish(const double* bpart, int blocks, double* loss) {
+  pdl_wait();
+  pdl_trigger();
+  adj_finish(bpart, blocks, loss, nullptr);
+}
 
-// window-gradient partials summed per tap: 32 taps per block, kSlices warps over the CTAs
-// (four taps per lane with one 16-byte load per CTA ran slower: 9.7 against 7.4 us, a
-// quarter of the blocks)
-__global__ void __launch_bounds__(kBinsPerBlock * kSlices) k_adj_wsum(const float* gpart, int grid, int N,
-                                                                      float* grad_w) {
+// window-gradient partials summed per tap: 32 taps per block, kSlices warps over the CTAs,
+// kInFlight loads started together (four taps per lane with one 16-byte load per CTA ran slower:
+// 9.7 against 7.4 us, a quarter of the blocks); one more block sums the loss and gain gradients
+__global__ void __launch_bounds__(kBinsPerBlock * kSlices) k_adj_wsum(const float* gpart, int grid, int N, float* grad_w,
+                                                                      const double* bpart, int bin_blocks, double* loss,
+                                                                      float* grad_gains) {
   __shared__ float red[kSlices][kBinsPerBlock];
   const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
   const int n = blockIdx.x * kBinsPerBlock + lane;
+  pdl_wait();  // the window pass's partials; k_adj_bins, which that kernel waited for, is complete too
+  pdl_trigger();
+  if (blockIdx.x == gridDim.x - 1) {
+    adj_finish(bpart, bin_blocks, loss, grad_gains);
+    return;
+  }
   float t = 0.f;
   if (n < N) {
-#pragma unroll 4
-    for (int g = sl; g < grid; g += kSlices) t += __ldcg(gpart + (size_t)g * N + n);
+#pragma unroll 1
+    for (int g0 = sl; g0 < grid; g0 += kSlices * kInFlight) {
+      float v[kInFlight];
+#pragma unroll
+      for (int i = 0; i < kInFlight; ++i) {
+        const int g = g0 + i * kSlices;
+        if (g < grid) v[i] = __ldcg(gpart + (size_t)g * N + n);
+      }
+#pragma unroll
+      for (int i = 0; i < kInFlight; ++i)
+        if (g0 + i * kSlices < grid) t += v[i];
+    }
   }
   red[sl][lane] = t;
   __syncthreads();
@@ -372,7 +415,7 @@ struct polaris_adj {
   float2* d_tw = nullptr;
   float4* d_part = nullptr;  // [grid_max][nbin]
   float* d_gpart = nullptr;  // [grid_max][N]
-  float4* d_mat = nullptr;   // [nbin][2]
+  float4* d_mat = nullptr;   // [nbin]
   double* d_bpart = nullptr; // [bin_blocks][5]
   std::string err;
 };
@@ -473,7 +516,7 @@ extern "C" int polaris_adj_create(int64_t n_fft, int bits, int device, polaris_a
   bool ok = cudaMalloc((void**)&h->d_tw, tw.size() * sizeof(float2)) == cudaSuccess &&
             cudaMalloc((void**)&h->d_part, (size_t)h->grid_max * h->nbin * sizeof(float4)) == cudaSuccess &&
             cudaMalloc((void**)&h->d_gpart, (size_t)h->grid_max * h->N * sizeof(float)) == cudaSuccess &&
-            cudaMalloc((void**)&h->d_mat, (size_t)h->nbin * 2 * sizeof(float4)) == cudaSuccess &&
+            cudaMalloc((void**)&h->d_mat, (size_t)h->nbin * sizeof(float4)) == cudaSuccess &&
             cudaMalloc((void**)&h->d_bpart, (size_t)h->bin_blocks * 5 * sizeof(double)) == cudaSuccess &&
             cudaMemcpy(h->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess;
   if (!ok) {
@@ -569,19 +612,15 @@ extern "C" int polaris_adj_run(polaris_adj* h, const void* const* packed, int64_
     b.grad_leak = grads ? grad_leak : nullptr;
     b.mat = grads ? h->d_mat : nullptr;
     b.bpart = (loss || grads) ? h->d_bpart : nullptr;
-    k_adj_bins<<<h->bin_blocks, kBinsPerBlock * kSlices, 0, st>>>(b);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess && (loss || grads)) {
-    k_adj_finish<<<1, 160, 0, st>>>(h->d_bpart, h->bin_blocks, loss, grads ? grad_gains : nullptr);
-    e = cudaGetLastError();
+    e = adj_launch(k_adj_bins, h->bin_blocks, kBinsPerBlock * kSlices, 0, st, b);
   }
   if (e == cudaSuccess && grads) {
     e = adj_segments_bits(h->bits, a, h->smem, true, sized, st);
-    if (e == cudaSuccess) {
-      k_adj_wsum<<<(h->N + kBinsPerBlock - 1) / kBinsPerBlock, kBinsPerBlock * kSlices, 0, st>>>(h->d_gpart, a.grid, h->N, grad_window);
-      e = cudaGetLastError();
-    }
+    if (e == cudaSuccess)
+      e = adj_launch(k_adj_wsum, (h->N + kBinsPerBlock - 1) / kBinsPerBlock + 1, kBinsPerBlock * kSlices, 0, st, h->d_gpart,
+                     a.grid, h->N, grad_window, h->d_bpart, h->bin_blocks, loss, grad_gains);
+  } else if (e == cudaSuccess && loss) {
+    e = adj_launch(k_adj_finish, 1, 160, 0, st, h->d_bpart, h->bin_blocks, loss);
   }
   cudaSetDevice(prev);
   if (e != cudaSuccess) return adj_err(h, POLARIS_ECUDA, "CUDA: ", cudaGetErrorString(e));

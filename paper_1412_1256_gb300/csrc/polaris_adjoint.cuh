@@ -18,7 +18,7 @@ struct AdjArgs {
   const float2* tw;       // per-pass twiddles: tw[r Ns + k - 1] = W_{Ns R}^{r k} (N - 1 entries)
   const float* window;    // N
   float4* part;           // [grid][nbin]: (|X|^2, |Y|^2, Re X conj(Y), Im X conj(Y)) per bin
-  const float4* mat;      // per bin (m11, m12), (m21, m22)
+  const float4* mat;      // per bin the Hermitian matrix of the spectral gradients: (m11, m22, Re m12, Im m12)
   float* gpart;           // [grid][N] window-gradient partials
 };
 
@@ -29,6 +29,33 @@ __host__ __device__ constexpr int adj_smem_points(int N) { return N + N / 16; }
 
 __device__ __forceinline__ float2 c_add(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 c_conj(float2 a) { return make_float2(a.x, -a.y); }
+
+// spectral gradients of bin k, G_X = m11 X + m12 Y, G_Y = conj(m12) X + m22 Y, with
+// X = (Z[k] + Zm) / 2, Y = (Z[k] - Zm) / 2i, Zm = conj Z[N-k]
+__device__ __forceinline__ void adj_bin_gradient(float4 m, float2 Zk, float2 Zm, float2& GX, float2& GY) {
+  const float2 X = make_float2(0.5f * (Zk.x + Zm.x), 0.5f * (Zk.y + Zm.y));
+  const float2 Y = make_float2(0.5f * (Zk.y - Zm.y), -0.5f * (Zk.x - Zm.x));
+  GX = c_add(make_float2(m.x * X.x, m.x * X.y), cmul(make_float2(m.z, m.w), Y));
+  GY = c_add(make_float2(m.y * Y.x, m.y * Y.y), cmul(make_float2(m.z, -m.w), X));
+}
+
+// One launch with programmatic stream serialisation: the kernel may be scheduled while its
+// predecessor ends, and waits for it (griddepcontrol.wait) before it touches what that one, or
+// the caller's earlier work, wrote.
+template <typename... P, typename... Q>
+static cudaError_t adj_launch(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, Q... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
 
 // level of sample idx of one IF
 template <int BITS>

@@ -40,13 +40,21 @@ struct AdjPlan {
   static constexpr int FCOLS = 16 * ((4 * BPT + 15) / 16), WCOLS = PPT;
   static constexpr int TCOLS_F = pow2_at_least(SLOTS * FCOLS, 32), TCOLS_W = pow2_at_least(SLOTS * WCOLS, 32);
   static constexpr size_t SMEM = (size_t)(DATA + NTAB) * sizeof(float2) + 16;
+  // CTAs that may share an SM by shared memory (228 KB, 1 KB of it per CTA the system's) and tensor
+  // memory, eight at most: the kernels' registers are held to that many
+  static constexpr int TCOLS_MAX = TCOLS_F > TCOLS_W ? TCOLS_F : TCOLS_W;
+  static constexpr int CTAS_SMEM = (int)((228 << 10) / (SMEM + 1024)), CTAS_TMEM = 512 / TCOLS_MAX;
+  static constexpr int CTAS_MEM = CTAS_SMEM < CTAS_TMEM ? CTAS_SMEM : CTAS_TMEM;
+  static constexpr int CTAS = CTAS_MEM < 8 ? CTAS_MEM : 8;
   static_assert(T % 32 == 0 && (N / 2) / T == PPT / 2, "whole warps, PPT/2 bins per thread below N/2");
   static_assert(TCOLS_F <= 512 && TCOLS_W <= 512, "tensor memory");
 };
 
-// One Stockham pass of radix R with Ns = NS points already combined: every j < N/R reads
-// z[j + r N/R] (r < R), multiplies by W_{NS R}^{r (j mod NS)}, takes an R-point DFT and writes
-// output r to z[(j / NS) NS R + r NS + j mod NS].  All reads come before any write.
+// One Stockham pass of radix R with Ns = NS points already combined: every j < N/R reads point
+// j + r N/R (r < R), multiplies by W_{NS R}^{r (j mod NS)}, takes an R-point DFT and output r is
+// point (j / NS) NS R + r NS + j mod NS.  A thread takes j = t + q T, so the first pass reads, and
+// the last one writes, the points t + T i (i < PPT) of thread t: those stay in its registers (u[i]),
+// and only the passes between exchange through z.  All of a pass's reads of z come before any write.
 // Every compile-time part of the indices below (q T, r M, r NS) is a multiple of 16, so
 // apad(x + c) = apad(x) + c + c/16: one padded base per lane and j, compile-time offsets.
 template <int C>
@@ -55,10 +63,11 @@ __device__ __forceinline__ constexpr int apad_c() {
   return C + C / 16;
 }
 template <int LOGN, int R, int NS>
-__device__ __forceinline__ void adjs_pass(float2* z, const float2* __restrict__ tws,
+__device__ __forceinline__ void adjs_pass(float2 (&u)[AdjPlan<LOGN>::PPT], float2* z, const float2* __restrict__ tws,
                                           const float2 (&wt)[AdjPlan<LOGN>::RW], int tid) {
   using PL = AdjPlan<LOGN>;
   constexpr int T = PL::T, JPT = PL::PPT / R, M = PL::N / R;
+  constexpr bool FIRST = NS == 1, LAST = NS * R == PL::N;
   float2 v[JPT][R];
   const float2* zt = z + apad(tid);
   sfor<0, JPT>([&](auto q_) {
@@ -67,7 +76,9 @@ __device__ __forceinline__ void adjs_pass(float2* z, const float2* __restrict__ 
     const int k = j & (NS - 1);
     sfor<0, R>([&](auto r_) {
       constexpr int r = decltype(r_)::value;
-      float2 x = zt[apad_c<q * T + r * M>()];  // z[apad(j + r M)]
+      float2 x;
+      if constexpr (FIRST) x = u[q + r * JPT];  // point j + r M = t + T (q + r JPT)
+      else x = zt[apad_c<q * T + r * M>()];
       if constexpr (NS > 1 && r > 0) {
         if constexpr (NS <= 256) {
           x = cmul(x, tws[r * NS + k - 1]);
@@ -84,15 +95,21 @@ __device__ __forceinline__ void adjs_pass(float2* z, const float2* __restrict__ 
       v[q][ct::bitrev(r, R)] = x;
     });
   });
-  __syncthreads();
+  if constexpr (FIRST) sfor<0, JPT>([&](auto q_) { dit<R>(v[decltype(q_)::value]); });
+  if constexpr (!LAST) __syncthreads();  // (first pass: z's readers before this transform are done)
   sfor<0, JPT>([&](auto q_) {
     constexpr int q = decltype(q_)::value;
     const int j = tid + q * T;
-    dit<R>(v[q]);
-    if constexpr (NS == 1) {  // base = 16 j, outputs r < 16: apad(16 j + r) = 17 j + r
+    if constexpr (!FIRST) dit<R>(v[q]);
+    if constexpr (FIRST) {  // base = 16 j, outputs r < 16: apad(16 j + r) = 17 j + r
       sfor<0, R>([&](auto r_) {
         constexpr int r = decltype(r_)::value;
         z[17 * j + r] = v[q][r];
+      });
+    } else if constexpr (LAST) {  // point j + r NS = t + T (q + r JPT)
+      sfor<0, R>([&](auto r_) {
+        constexpr int r = decltype(r_)::value;
+        u[q + r * JPT] = v[q][r];
       });
     } else {
       const int k = j & (NS - 1);
@@ -103,73 +120,74 @@ __device__ __forceinline__ void adjs_pass(float2* z, const float2* __restrict__ 
       });
     }
   });
+  if constexpr (!LAST) __syncthreads();
+}
+
+// forward DFT of the N points u[i] = point t + T i of the CTA's threads t, in place; a barrier
+// before the first write of z, none after the last read of it
+template <int LOGN>
+__device__ __forceinline__ void adjs_fft(float2 (&u)[AdjPlan<LOGN>::PPT], float2* z, const float2* __restrict__ tws,
+                                         const float2 (&wt)[AdjPlan<LOGN>::RW], int tid) {
+  using PL = AdjPlan<LOGN>;
+  sfor<0, PL::F>([&](auto p_) { adjs_pass<LOGN, 16, (1 << (4 * decltype(p_)::value))>(u, z, tws, wt, tid); });
+  if constexpr (PL::REM > 0) adjs_pass<LOGN, (1 << PL::REM), PL::NS_LAST>(u, z, tws, wt, tid);
+}
+
+// Points t + T i and N - (t + T i), i < PPT/2, meet in thread t: every thread puts its upper half
+// (i >= PPT/2) into z, where mirror point i of thread t is zm[-apad_c<T i>()], zm = z + apad(N - t)
+// (only thread 0's i = 0 is its own mirror).  Barriers before and after.
+template <int LOGN>
+__device__ __forceinline__ void adjs_store_upper(const float2 (&u)[AdjPlan<LOGN>::PPT], float2* z, int tid) {
+  using PL = AdjPlan<LOGN>;
+  float2* zt = z + apad(tid);
+  __syncthreads();  // the last pass's reads of z
+  sfor<PL::PPT / 2, PL::PPT>([&](auto i_) {
+    constexpr int i = decltype(i_)::value;
+    zt[apad_c<PL::T * i>()] = u[i];
+  });
   __syncthreads();
 }
 
-// forward DFT of the N points in z (natural order in and out); callers sync before
-template <int LOGN>
-__device__ __forceinline__ void adjs_fft(float2* z, const float2* __restrict__ tws,
-                                         const float2 (&wt)[AdjPlan<LOGN>::RW], int tid) {
-  using PL = AdjPlan<LOGN>;
-  sfor<0, PL::F>([&](auto p_) { adjs_pass<LOGN, 16, (1 << (4 * decltype(p_)::value))>(z, tws, wt, tid); });
-  if constexpr (PL::REM > 0) adjs_pass<LOGN, (1 << PL::REM), PL::NS_LAST>(z, tws, wt, tid);
-}
-
-// The levels of the 16 consecutive samples 16 g .. 16 g + 15 of segment s of one IF, from
-// one vector load (16 B at 8 bits, 8 B at 4, 4 B at 2, 2 B at 1 bit; the caller guarantees
-// 16-byte aligned inputs).  Sample i of a word sits at bits i BITS .. (i + 1) BITS - 1.
+// A thread's samples t + T i of one segment (first = s N + t): a warp's loads are 32 consecutive
+// codes.  Codes below 8 bits sit at the same place of every word the thread reads (T is a
+// multiple of the samples per word): the word is rotated so that the code starts at bit 1.
+// (Ordinary loads, here and of the window and the matrix: a read-only one could be moved up
+// over the wait for the kernel before.)
 template <int LOGN, int BITS>
-__device__ __forceinline__ void adjs_group_levels(const uint32_t* in, long long s, int g, float (&x)[16]) {
-  const long long first = s * (1LL << LOGN) + 16LL * g;  // a multiple of 16 samples
-  if constexpr (BITS == 8) {
-    const int4 v = __ldg(reinterpret_cast<const int4*>(reinterpret_cast<const signed char*>(in) + first));
-    const int w[4] = {v.x, v.y, v.z, v.w};
-    sfor<0, 16>([&](auto i_) {
-      constexpr int i = decltype(i_)::value;
-      x[i] = (float)((w[i / 4] << (24 - 8 * (i % 4))) >> 24);  // the byte, sign-extended
-    });
-  } else if constexpr (BITS == 4) {
-    const uint2 v = __ldg(reinterpret_cast<const uint2*>(in) + first / 16);
-    sfor<0, 16>([&](auto i_) {
-      constexpr int i = decltype(i_)::value;
-      x[i] = decode_level<4>(i < 8 ? v.x : v.y, (uint32_t)(i % 8) * 4);
-    });
-  } else if constexpr (BITS == 2) {
-    const uint32_t v = __ldg(in + first / 16);
-    sfor<0, 16>([&](auto i_) {
-      constexpr int i = decltype(i_)::value;
-      x[i] = decode_level<2>(v, (uint32_t)i * 2);
-    });
-  } else {
-    const uint32_t v = __ldg(reinterpret_cast<const unsigned short*>(in) + first / 16);
-    sfor<0, 16>([&](auto i_) {
-      constexpr int i = decltype(i_)::value;
-      x[i] = decode_level<1>(v, (uint32_t)i);
-    });
+struct AdjSamples {
+  static constexpr int SPW = 32 / BITS;
+  const uint32_t* p;
+  uint32_t rot;
+  __device__ __forceinline__ AdjSamples(const uint32_t* in, long long first) {
+    if constexpr (BITS == 8) p = reinterpret_cast<const uint32_t*>(reinterpret_cast<const unsigned char*>(in) + first);
+    else p = in + first / SPW;
+    rot = (uint32_t)(first % SPW) * BITS - 1u;
   }
-}
+  template <int I>
+  __device__ __forceinline__ float level() const {
+    constexpr int off = AdjPlan<LOGN>::T * I;
+    static_assert(off % SPW == 0, "whole words");
+    if constexpr (BITS == 8) {  // 2^23 + (c ^ 0x80) - 2^23 - 128
+      const uint32_t c = reinterpret_cast<const unsigned char*>(p)[off];
+      return __uint_as_float(c ^ 0x4B000080u) - 8388736.0f;
+    } else {  // (2^23 + 2c) - (2^23 + 2^b - 1)
+      const uint32_t w = p[off / SPW];
+      return __uint_as_float(and_or(__funnelshift_r(w, w, rot), ((1u << BITS) - 1u) << 1, 0x4B000000u)) -
+             (8388608.0f + (float)((1 << BITS) - 1));
+    }
+  }
+};
 
-// z[n] = w[n] (x[n] + i y[n]) for segment s: thread t fills the groups g = t + T h (h <
-// PPT/16) of 16 consecutive samples; apad(16 g + j) = 17 g + j, so the 16 lanes of a
-// half-warp write distinct bank pairs
+// u[i] = w[n] (x[n] + i y[n]), n = t + T i, of segment s
 template <int LOGN, int BITS>
-__device__ __forceinline__ void adjs_load(const AdjArgs& a, float2* z, long long s, int tid) {
+__device__ __forceinline__ void adjs_load(const AdjArgs& a, float2 (&u)[AdjPlan<LOGN>::PPT], long long s, int tid) {
   using PL = AdjPlan<LOGN>;
-  sfor<0, PL::PPT / 16>([&](auto h_) {
-    const int g = tid + decltype(h_)::value * PL::T;
-    float x[16], y[16];
-    adjs_group_levels<LOGN, BITS>(a.in[0], s, g, x);
-    adjs_group_levels<LOGN, BITS>(a.in[1], s, g, y);
-    const float4* wp = reinterpret_cast<const float4*>(a.window) + 4 * g;
-    sfor<0, 4>([&](auto c_) {
-      constexpr int c = decltype(c_)::value;
-      const float4 w4 = __ldg(wp + c);
-      const float w[4] = {w4.x, w4.y, w4.z, w4.w};
-      sfor<0, 4>([&](auto i_) {
-        constexpr int j = 4 * c + decltype(i_)::value;
-        z[17 * g + j] = make_float2(w[j % 4] * x[j], w[j % 4] * y[j]);
-      });
-    });
+  const AdjSamples<LOGN, BITS> xs(a.in[0], s * PL::N + tid), ys(a.in[1], s * PL::N + tid);
+  const float* wp = a.window + tid;
+  sfor<0, PL::PPT>([&](auto i_) {
+    constexpr int i = decltype(i_)::value;
+    const float w = wp[PL::T * i], x = xs.template level<i>(), y = ys.template level<i>();
+    u[i] = make_float2(w * x, w * y);
   });
 }
 
@@ -196,7 +214,7 @@ __device__ __forceinline__ uint32_t adjs_setup(const AdjArgs& a, float2* tws, ui
 }
 
 template <int LOGN, int BITS>
-__global__ void __launch_bounds__(AdjPlan<LOGN>::T) k_adjs_forward(AdjArgs a) {
+__global__ void __launch_bounds__(AdjPlan<LOGN>::T, AdjPlan<LOGN>::CTAS) k_adjs_forward(AdjArgs a) {
   using PL = AdjPlan<LOGN>;
   constexpr int N = PL::N, T = PL::T;
   extern __shared__ __align__(16) float2 zs[];
@@ -207,11 +225,14 @@ __global__ void __launch_bounds__(AdjPlan<LOGN>::T) k_adjs_forward(AdjArgs a) {
   float2 wt[PL::RW];
   uint32_t tbase;
   const uint32_t tacc = adjs_setup<LOGN, PL::TCOLS_F, PL::FCOLS>(a, tws, tslot, wt, tbase, tid);
+  pdl_wait();  // (dependent launch: the inputs and the partials may be touched from here on)
 #pragma unroll 1
   for (long long s = blockIdx.x; s < a.nseg; s += a.grid) {
-    adjs_load<LOGN, BITS>(a, z, s, tid);
-    __syncthreads();
-    adjs_fft<LOGN>(z, tws, wt, tid);
+    float2 u[PL::PPT];
+    adjs_load<LOGN, BITS>(a, u, s, tid);
+    adjs_fft<LOGN>(u, z, tws, wt, tid);
+    adjs_store_upper<LOGN>(u, z, tid);
+    const float2* zm = z + apad(N - tid);
     // X = (Z[k] + conj Z[N-k]) / 2, Y = (Z[k] - conj Z[N-k]) / 2i; the sums of bin i of this
     // thread at columns 4 i .. 4 i + 3
     sfor<0, PL::FCOLS / 16>([&](auto c_) {
@@ -222,9 +243,12 @@ __global__ void __launch_bounds__(AdjPlan<LOGN>::T) k_adjs_forward(AdjArgs a) {
       sfor<0, 4>([&](auto i_) {
         constexpr int i = 4 * cc + decltype(i_)::value;
         if constexpr (i < PL::BPT) {
-          if (i < PL::BPT - 1 || tid == 0) {
-            const int k = i < PL::BPT - 1 ? tid + T * i : N / 2;
-            const float2 Zk = z[apad(k)], Zm = c_conj(z[apad((N - k) & (N - 1))]);
+          if (i < PL::BPT - 1 || tid == 0) {  // (i = BPT - 1: bin N/2, its own mirror)
+            const float2 Zk = u[i];
+            float2 Zm;
+            if constexpr (i == PL::BPT - 1) Zm = c_conj(Zk);
+            else if constexpr (i == 0) Zm = c_conj(tid == 0 ? Zk : zm[0]);
+            else Zm = c_conj(zm[-apad_c<T * i>()]);
             const float2 X = make_float2(0.5f * (Zk.x + Zm.x), 0.5f * (Zk.y + Zm.y));
             const float2 Y = make_float2(0.5f * (Zk.y - Zm.y), -0.5f * (Zk.x - Zm.x));
             constexpr int o = 4 * (i - 4 * cc);
@@ -238,8 +262,8 @@ __global__ void __launch_bounds__(AdjPlan<LOGN>::T) k_adjs_forward(AdjArgs a) {
       tmem_st16(tacc + 16 * cc, acc);
     });
     tmem_wait_st();
-    __syncthreads();  // z is refilled by the next segment
   }
+  pdl_trigger();
   float4* part = a.part + (size_t)blockIdx.x * PL::NBIN;
   sfor<0, PL::FCOLS / 16>([&](auto c_) {
     constexpr int cc = decltype(c_)::value;
@@ -261,7 +285,7 @@ __global__ void __launch_bounds__(AdjPlan<LOGN>::T) k_adjs_forward(AdjArgs a) {
 }
 
 template <int LOGN, int BITS>
-__global__ void __launch_bounds__(AdjPlan<LOGN>::T) k_adjs_window(AdjArgs a) {
+__global__ void __launch_bounds__(AdjPlan<LOGN>::T, AdjPlan<LOGN>::CTAS) k_adjs_window(AdjArgs a) {
   using PL = AdjPlan<LOGN>;
   constexpr int N = PL::N, T = PL::T;
   extern __shared__ __align__(16) float2 zs[];
@@ -272,66 +296,76 @@ __global__ void __launch_bounds__(AdjPlan<LOGN>::T) k_adjs_window(AdjArgs a) {
   float2 wt[PL::RW];
   uint32_t tbase;
   const uint32_t tacc = adjs_setup<LOGN, PL::TCOLS_W, PL::WCOLS>(a, tws, tslot, wt, tbase, tid);
+  // (dependent launch: the inputs, read before k_adj_bins started, are complete; its matrix is
+  // not before the wait below)
 #pragma unroll 1
   for (long long s = blockIdx.x; s < a.nseg; s += a.grid) {
-    adjs_load<LOGN, BITS>(a, z, s, tid);
-    __syncthreads();
-    adjs_fft<LOGN>(z, tws, wt, tid);
-    // G_X, G_Y per bin pair; conj of the Hermitian extension of G_X + i G_Y goes back into z
-    // (the inverse transform is conj(DFT(conj H))).  This thread owns slots k and N - k.
-#pragma unroll 1
-    for (int k = tid; k < PL::NBIN; k += T) {  // (rolled: unrolled, its loads crowd the registers)
-      {
-        const int km = (N - k) & (N - 1);
-        const float2 Zk = z[apad(k)], Zm = c_conj(z[apad(km)]);
-        const float2 X = make_float2(0.5f * (Zk.x + Zm.x), 0.5f * (Zk.y + Zm.y));
-        const float2 Y = make_float2(0.5f * (Zk.y - Zm.y), -0.5f * (Zk.x - Zm.x));
-        const float4 r0 = __ldg(a.mat + 2 * k), r1 = __ldg(a.mat + 2 * k + 1);
-        const float2 GX = c_add(cmul(make_float2(r0.x, r0.y), X), cmul(make_float2(r0.z, r0.w), Y));
-        const float2 GY = c_add(cmul(make_float2(r1.x, r1.y), X), cmul(make_float2(r1.z, r1.w), Y));
-        if (k == 0 || 2 * k == N) {
-          z[apad(k)] = make_float2(GX.x, -GY.x);  // H = Re G_X + i Re G_Y
-        } else {
-          const float2 hx = make_float2(0.5f * GX.x, 0.5f * GX.y), hy = make_float2(0.5f * GY.x, 0.5f * GY.y);
-          // H[k] = hx + i hy, H[N-k] = conj(hx) + i conj(hy); store their conjugates
-          z[apad(k)] = make_float2(hx.x - hy.y, -(hx.y + hy.x));
-          z[apad(km)] = make_float2(hx.x + hy.y, hx.y - hy.x);
-        }
+    float2 u[PL::PPT];
+    adjs_load<LOGN, BITS>(a, u, s, tid);
+    adjs_fft<LOGN>(u, z, tws, wt, tid);
+    adjs_store_upper<LOGN>(u, z, tid);
+    if (s == blockIdx.x) pdl_wait();
+    // G_X, G_Y per bin pair; u and z become conj of the Hermitian extension H of G_X + i G_Y
+    // (the inverse transform is conj(DFT(conj H))).  Thread t owns bins k = t + T i and the slots
+    // of their mirrors, so these are read and overwritten without a barrier.
+    float2* zm = z + apad(N - tid);
+    sfor<0, PL::PPT / 2>([&](auto i_) {
+      constexpr int i = decltype(i_)::value;
+      const float2 Zk = u[i];
+      float2 Zm;
+      if constexpr (i == 0) Zm = c_conj(tid == 0 ? Zk : zm[0]);
+      else Zm = c_conj(zm[-apad_c<T * i>()]);
+      float2 GX, GY;
+      adj_bin_gradient(a.mat[tid + T * i], Zk, Zm, GX, GY);
+      const float2 hx = make_float2(0.5f * GX.x, 0.5f * GX.y), hy = make_float2(0.5f * GY.x, 0.5f * GY.y);
+      // H[k] = hx + i hy, H[N-k] = conj(hx) + i conj(hy); store their conjugates
+      u[i] = make_float2(hx.x - hy.y, -(hx.y + hy.x));
+      const float2 hm = make_float2(hx.x + hy.y, hx.y - hy.x);
+      if constexpr (i == 0) {
+        if (tid == 0) u[0] = make_float2(GX.x, -GY.x);  // H = Re G_X + i Re G_Y (likewise at N/2)
+        else zm[0] = hm;
+      } else {
+        zm[-apad_c<T * i>()] = hm;
       }
+    });
+    if (tid == 0) {
+      const float2 Zk = u[PL::PPT / 2];
+      float2 GX, GY;
+      adj_bin_gradient(a.mat[N / 2], Zk, c_conj(Zk), GX, GY);
+      z[apad(N / 2)] = make_float2(GX.x, -GY.x);
     }
     __syncthreads();
-    adjs_fft<LOGN>(z, tws, wt, tid);
-    // h = conj(F): dL/dw[n] += x[n] Re h[n] + y[n] Im h[n] = x F.x - y F.y
-    // (this thread's taps are the samples of its groups: column 16 h + j holds n = 16 g + j)
+    const float2* zt = z + apad(tid);
+    sfor<PL::PPT / 2, PL::PPT>([&](auto i_) {
+      constexpr int i = decltype(i_)::value;
+      u[i] = zt[apad_c<T * i>()];
+    });
+    adjs_fft<LOGN>(u, z, tws, wt, tid);
+    // h = conj(F): dL/dw[n] += x[n] Re h[n] + y[n] Im h[n] = x F.x - y F.y (column i: n = t + T i)
+    const AdjSamples<LOGN, BITS> xs(a.in[0], s * N + tid), ys(a.in[1], s * N + tid);
     sfor<0, PL::PPT / 16>([&](auto h_) {
       constexpr int h = decltype(h_)::value;
-      const int g = tid + h * T;
-      float x[16], y[16];
-      adjs_group_levels<LOGN, BITS>(a.in[0], s, g, x);
-      adjs_group_levels<LOGN, BITS>(a.in[1], s, g, y);
       float acc[16];
       tmem_ld16(tacc + 16 * h, acc);
       tmem_wait_ld();
       sfor<0, 16>([&](auto j_) {
-        constexpr int j = decltype(j_)::value;
-        const float2 F = z[17 * g + j];
-        acc[j] += fmaf(x[j], F.x, -y[j] * F.y);
+        constexpr int j = decltype(j_)::value, i = 16 * h + j;
+        acc[j] += fmaf(xs.template level<i>(), u[i].x, -ys.template level<i>() * u[i].y);
       });
       tmem_st16(tacc + 16 * h, acc);
     });
     tmem_wait_st();
-    __syncthreads();
   }
-  float* gpart = a.gpart + (size_t)blockIdx.x * N;
+  pdl_trigger();
+  float* gpart = a.gpart + (size_t)blockIdx.x * N + tid;
   sfor<0, PL::PPT / 16>([&](auto h_) {
     constexpr int h = decltype(h_)::value;
-    const int g = tid + h * T;
     float acc[16];
     tmem_ld16(tacc + 16 * h, acc);
     tmem_wait_ld();
-    sfor<0, 4>([&](auto c_) {
-      constexpr int c = decltype(c_)::value;
-      reinterpret_cast<float4*>(gpart + 16 * g)[c] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
+    sfor<0, 16>([&](auto j_) {
+      constexpr int j = decltype(j_)::value;
+      gpart[T * (16 * h + j)] = acc[j];
     });
   });
   cta_tmem_end<PL::TCOLS_W>(tbase, tid >> 5);
@@ -358,9 +392,7 @@ static cudaError_t adjs_prepare(int* ctas_per_sm) {
 template <int LOGN, int BITS>
 static cudaError_t adjs_launch(bool window_pass, const AdjArgs& a, cudaStream_t st) {
   using PL = AdjPlan<LOGN>;
-  if (!window_pass) k_adjs_forward<LOGN, BITS><<<a.grid, PL::T, PL::SMEM, st>>>(a);
-  else k_adjs_window<LOGN, BITS><<<a.grid, PL::T, PL::SMEM, st>>>(a);
-  return cudaGetLastError();
+  return adj_launch(window_pass ? k_adjs_window<LOGN, BITS> : k_adjs_forward<LOGN, BITS>, a.grid, PL::T, PL::SMEM, st, a);
 }
 
 template <int LOGN>
