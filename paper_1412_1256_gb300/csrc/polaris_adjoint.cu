@@ -37,10 +37,12 @@
 //   k_adj_bins     per bin: partials summed (fp32 slices, added in fp64), the model,
 //                  Stokes and loss in fp64, the gain and leakage gradients and the
 //                  window-adjoint matrix in fp32
-//   k_adj_finish   block partials of the loss and gain gradients summed in order
 //   k_adj_window   per segment again: forward transform, G_X and G_Y, inverse transform,
 //                  per-CTA partials of the window gradient
-//   k_adj_wsum     the window-gradient partials summed per tap
+//   k_adj_wsum     the window-gradient partials summed per tap, and the block partials of the
+//                  loss and gain gradients in order (k_adj_finish: those alone, without gradients)
+// The launches are programmatic dependent ones (but for the kernels for any N): each kernel's
+// set-up, and the window pass's first transform, run while the one before ends.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -225,16 +227,19 @@ struct BinArgs {
 
 // A block covers kBinsPerBlock bins; its kSlices warps sum the per-CTA partials of the
 // segment kernel (one 16-byte load per CTA and bin) over interleaved slices of CTAs in fp32, the
-// slice sums are added in fp64 in slice order (one warp per quantity), then one warp
-// evaluates the model per bin: the sums, Stokes and loss in fp64, the gradients and the
-// window-adjoint matrix in fp32.
-// Bound by the latency of the loads: kInFlight of them per thread are started together, which
-// holds a slice of a grid of one CTA per SM (152 / 8 = 19) in one round.
+// slice sums are added in fp64 in slice order (one warp per quantity), then the model per bin:
+// the sums, Stokes and loss in fp64, the gradients and the window-adjoint matrix in fp32.
+// Bound by the latency of the loads, of which kInFlight per thread are started together (a slice
+// of a grid of one CTA per SM, 152 / 8 = 19, in one round), and by the fp64 arithmetic, at 64
+// cycles per warp and instruction and scheduler: four warps share it, one expression each.
 constexpr int kBinsPerBlock = 32, kSlices = 8, kInFlight = 20;
 
 __global__ void __launch_bounds__(kBinsPerBlock * kSlices, 2) k_adj_bins(BinArgs a) {
   __shared__ float red[kSlices][4][kBinsPerBlock];
-  __shared__ double tot[5][kBinsPerBlock];
+  __shared__ double tot[5][kBinsPerBlock];  // A, B, C of a bin, then its loss and gain gradients
+  __shared__ double mod[6][kBinsPerBlock];  // RR, LL, Qm, gR conj(gL)
+  __shared__ double dif[4][kBinsPerBlock];  // Stokes minus target
+  __shared__ float fmd[4][kBinsPerBlock];  // P_R, P_L, Qm
   const int nbin = a.nbin;
   const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
   const int k = blockIdx.x * kBinsPerBlock + lane;
@@ -269,38 +274,64 @@ __global__ void __launch_bounds__(kBinsPerBlock * kSlices, 2) k_adj_bins(BinArgs
     tot[sl][lane] = t;
   }
   __syncthreads();
+  const int kk = k < nbin ? k : 0;
+  const double A = tot[0][lane], B = tot[1][lane];
+  const dc C = {tot[2][lane], tot[3][lane]};
+  const float2 fgR = make_float2(a.gains[0], a.gains[1]), fgL = make_float2(a.gains[2], a.gains[3]);
+  const float2 fDR = make_float2(a.leak[2 * kk], a.leak[2 * kk + 1]);
+  const float2 fDL = make_float2(a.leak[2 * (nbin + kk)], a.leak[2 * (nbin + kk) + 1]);
+  if (sl == 0) {
+    const dc gR = {fgR.x, fgR.y}, DR = {fDR.x, fDR.y};
+    const double PR = A + dnorm(DR) * B + 2.0 * dmul(dconj(DR), C).x;
+    mod[0][lane] = dnorm(gR) * PR;
+    fmd[0][lane] = (float)PR;
+  } else if (sl == 1) {
+    const dc gL = {fgL.x, fgL.y}, DL = {fDL.x, fDL.y};
+    const double PL = B + dnorm(DL) * A + 2.0 * dmul(DL, C).x;
+    mod[1][lane] = dnorm(gL) * PL;
+    fmd[1][lane] = (float)PL;
+  } else if (sl == 2) {
+    const dc DR = {fDR.x, fDR.y}, DL = {fDL.x, fDL.y};
+    const dc Qm = dadd(dadd(C, dscale(dconj(DL), A)), dadd(dscale(DR, B), dmul(dmul(DR, dconj(DL)), dconj(C))));
+    mod[2][lane] = Qm.x;
+    mod[3][lane] = Qm.y;
+    fmd[2][lane] = (float)Qm.x;
+    fmd[3][lane] = (float)Qm.y;
+  } else if (sl == 3) {
+    const dc gR = {fgR.x, fgR.y}, gL = {fgL.x, fgL.y};
+    const dc g = dmul(gR, dconj(gL));
+    mod[4][lane] = g.x;
+    mod[5][lane] = g.y;
+  }
+  __syncthreads();
+  if (sl < 4) {  // warp q: Stokes parameter q (I, Q, U, V)
+    const double RR = mod[0][lane], LL = mod[1][lane];
+    const dc Qm = {mod[2][lane], mod[3][lane]}, g = {mod[4][lane], mod[5][lane]};
+    double S;
+    if (sl == 0) S = 0.5 * (RR + LL);
+    else if (sl == 1) S = dmul(g, Qm).x;
+    else if (sl == 2) S = dmul(g, Qm).y;
+    else S = 0.5 * (RR - LL);
+    if (k < nbin && a.stokes) a.stokes[sl * nbin + k] = (float)S;
+    dif[sl][lane] = a.target ? S - (double)a.target[sl * nbin + kk] : 0.0;
+  }
+  __syncthreads();
   double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   if (sl == 0 && k < nbin) {
-    const double t4[4] = {tot[0][lane], tot[1][lane], tot[2][lane], tot[3][lane]};
-    const double A = t4[0], B = t4[1];
-    const dc C = {t4[2], t4[3]};
-    const dc gR = {a.gains[0], a.gains[1]}, gL = {a.gains[2], a.gains[3]};
-    const dc DR = {a.leak[2 * k], a.leak[2 * k + 1]};
-    const dc DL = {a.leak[2 * (nbin + k)], a.leak[2 * (nbin + k) + 1]};
-    const double PR = A + dnorm(DR) * B + 2.0 * dmul(dconj(DR), C).x;
-    const double PL = B + dnorm(DL) * A + 2.0 * dmul(DL, C).x;
-    const dc Qm = dadd(dadd(C, dscale(dconj(DL), A)), dadd(dscale(DR, B), dmul(dmul(DR, dconj(DL)), dconj(C))));
-    const double RR = dnorm(gR) * PR, LL = dnorm(gL) * PL;
-    const dc RL = dmul(dmul(gR, dconj(gL)), Qm);
-    const double S[4] = {0.5 * (RR + LL), RL.x, RL.y, 0.5 * (RR - LL)};
-    if (a.stokes)
-      for (int q = 0; q < 4; ++q) a.stokes[q * nbin + k] = (float)S[q];
     if (a.target) {
       float r[4];
       for (int q = 0; q < 4; ++q) {
-        const double d = S[q] - (double)a.target[q * nbin + k];
+        const double d = dif[q][lane];
         acc[0] += d * d;
         r[q] = (float)(2.0 * d);
       }
       if (a.mat) {
         const float ca = 0.5f * (r[0] + r[3]), cb = 0.5f * (r[0] - r[3]);
         const float2 c = make_float2(r[1], r[2]), cc = c_conj(c);
-        const float2 fgR = make_float2(a.gains[0], a.gains[1]), fgL = make_float2(a.gains[2], a.gains[3]);
-        const float2 fDR = make_float2((float)DR.x, (float)DR.y), fDL = make_float2((float)DL.x, (float)DL.y);
-        const float2 fC = make_float2((float)C.x, (float)C.y), fQ = make_float2((float)Qm.x, (float)Qm.y);
+        const float2 fC = make_float2((float)C.x, (float)C.y), fQ = make_float2(fmd[2][lane], fmd[3][lane]);
         const float fA = (float)A, fB = (float)B;
-        const float2 ggR = c_add(fscale(fgR, 2.f * ca * (float)PR), cmul(cmul(c, fgL), c_conj(fQ)));
-        const float2 ggL = c_add(fscale(fgL, 2.f * cb * (float)PL), cmul(cmul(cc, fgR), fQ));
+        const float2 ggR = c_add(fscale(fgR, 2.f * ca * fmd[0][lane]), cmul(cmul(c, fgL), c_conj(fQ)));
+        const float2 ggL = c_add(fscale(fgL, 2.f * cb * fmd[1][lane]), cmul(cmul(cc, fgR), fQ));
         acc[1] = ggR.x;
         acc[2] = ggR.y;
         acc[3] = ggL.x;
@@ -409,12 +440,12 @@ __global__ void __launch_bounds__(kBinsPerBlock * kSlices) k_adj_wsum(const floa
 using namespace polaris;
 
 struct polaris_adj {
-  int N = 0, log2n = 0, nbin = 0, bits = 0, device = 0, threads = 0, grid_max = 0, bin_blocks = 0;
+  int N = 0, log2n = 0, nbin = 0, bits = 0, device = 0, threads = 0, grid_max = 0, grid_window = 0, bin_blocks = 0;
   bool sized = false;  // the size-specialised segment kernels (polaris_adjoint_sized.cu)
   size_t smem = 0;
   float2* d_tw = nullptr;
   float4* d_part = nullptr;  // [grid_max][nbin]
-  float* d_gpart = nullptr;  // [grid_max][N]
+  float* d_gpart = nullptr;  // [grid_window][N]
   float4* d_mat = nullptr;   // [nbin]
   double* d_bpart = nullptr; // [bin_blocks][5]
   std::string err;
@@ -478,7 +509,7 @@ extern "C" int polaris_adj_create(int64_t n_fft, int bits, int device, polaris_a
   int nsm = 0, occ = 0;
   cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
   // the kernels for any N always (they also take calls whose buffers are not 16-byte
-  // aligned), the size-specialised ones where they exist; both run on the same grid
+  // aligned), the size-specialised ones where they exist; both forward kernels run on the same grid
   if (e == cudaSuccess) {
     switch (bits) {
       case 1: e = adj_prepare<1>(h, &occ); break;
@@ -487,10 +518,10 @@ extern "C" int polaris_adj_create(int64_t n_fft, int bits, int device, polaris_a
       default: e = adj_prepare<8>(h, &occ); break;
     }
   }
+  int window_ctas = 0;
   if (e == cudaSuccess && h->sized) {
-    int occ_sized = 0;
-    e = adj_sized_prepare(h->log2n, bits, &occ_sized);
-    occ = std::min(occ, occ_sized);
+    e = adj_sized_prepare(h->log2n, bits, &window_ctas);
+    occ = std::min(occ, 1);
   }
   if (e != cudaSuccess || occ < 1) {
     cudaGetLastError();
@@ -500,6 +531,7 @@ extern "C" int polaris_adj_create(int64_t n_fft, int bits, int device, polaris_a
                    e != cudaSuccess ? cudaGetErrorString(e) : "zero occupancy");
   }
   h->grid_max = nsm * std::min(occ, kMaxCtasPerSm);
+  h->grid_window = std::max(h->grid_max, nsm * window_ctas);
   // per-pass twiddles of the Stockham passes (radix 16, then 2, 4 or 8): pass with Ns
   // points done and radix R keeps W_{Ns R}^{r k} at r Ns + k - 1 (1 <= r < R, k < Ns); the
   // offsets Ns - 1 telescope, so the N - 1 entries tile [0, N - 1) exactly
@@ -515,7 +547,7 @@ extern "C" int polaris_adj_create(int64_t n_fft, int bits, int device, polaris_a
   }
   bool ok = cudaMalloc((void**)&h->d_tw, tw.size() * sizeof(float2)) == cudaSuccess &&
             cudaMalloc((void**)&h->d_part, (size_t)h->grid_max * h->nbin * sizeof(float4)) == cudaSuccess &&
-            cudaMalloc((void**)&h->d_gpart, (size_t)h->grid_max * h->N * sizeof(float)) == cudaSuccess &&
+            cudaMalloc((void**)&h->d_gpart, (size_t)h->grid_window * h->N * sizeof(float)) == cudaSuccess &&
             cudaMalloc((void**)&h->d_mat, (size_t)h->nbin * sizeof(float4)) == cudaSuccess &&
             cudaMalloc((void**)&h->d_bpart, (size_t)h->bin_blocks * 5 * sizeof(double)) == cudaSuccess &&
             cudaMemcpy(h->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess;
@@ -615,6 +647,7 @@ extern "C" int polaris_adj_run(polaris_adj* h, const void* const* packed, int64_
     e = adj_launch(k_adj_bins, h->bin_blocks, kBinsPerBlock * kSlices, 0, st, b);
   }
   if (e == cudaSuccess && grads) {
+    if (sized) a.grid = std::min(a.nseg, h->grid_window);
     e = adj_segments_bits(h->bits, a, h->smem, true, sized, st);
     if (e == cudaSuccess)
       e = adj_launch(k_adj_wsum, (h->N + kBinsPerBlock - 1) / kBinsPerBlock + 1, kBinsPerBlock * kSlices, 0, st, h->d_gpart,

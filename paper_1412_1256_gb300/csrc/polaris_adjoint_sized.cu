@@ -1,13 +1,16 @@
 // Leakage calibration: the segment kernels of the forward and window passes specialised per
 // transform size N = 2^LOGN, kAdjSizedMin <= LOGN <= kAdjSizedMax, so that every index, pass
 // and radix is a compile-time constant.  They compute what k_adj_forward and k_adj_window
-// (polaris_adjoint.cu) compute, with the same per-CTA order of summation:
+// (polaris_adjoint.cu) compute (the forward pass with the same order of summation):
 //   - one CTA of T = N/PPT threads per segment at a time, PPT points per thread (16; 32 at
 //     N = 2^14, so that 512 threads of 128 registers hold them), radix-16 Stockham passes and
-//     one pass of radix 2^(LOGN mod 4), in shared memory;
-//   - the samples and window taps arrive by vector loads of 16 consecutive samples per
-//     thread (inputs and window 16-byte aligned: the host routes other calls to the kernels
-//     for any N);
+//     one pass of radix 2^(LOGN mod 4).  Thread t's points before the first and after the last
+//     pass are t + T i, in registers: shared memory holds only what the passes between exchange
+//     and the upper half of the spectrum (the mirror bins), 14 instead of 20 times the segment in
+//     the window pass;
+//   - samples and window taps are read as a warp's 32 consecutive ones; the forward kernel
+//     copies the next segment's words to shared memory meanwhile (inputs and window 16-byte
+//     aligned: the host routes other calls to the kernels for any N);
 //   - the per-CTA partial sums over the CTA's segments (per bin in the forward pass, per tap
 //     in the window pass) stay in tensor memory, used as per-thread storage, and reach global
 //     memory once, at the end (instead of a read and a write per segment);
@@ -15,6 +18,11 @@
 //     (exact FP64 values rounded once); the last pass of N >= 2^13 (Ns = 4096) forms
 //     W_N^{r j}, j = t + q T, as W_N^{r t} (from the table, once per thread) times the
 //     constant W_PPT^{r q}: one rounding of two correctly rounded factors.
+// What bounds them: latency.  At 2^14 (one CTA of 16 warps per SM) a third of the shared-memory
+// and a quarter of the issue slots are used, the warps wait for the window's and the samples'
+// loads, the exchanges and the barriers; 256 segments on 152 SMs are two rounds, the second two
+// thirds full.  Whole steps, before and after (8-bit): 256 x 2^14 94.7 -> 67.0 us, 700 x 2^13
+// 112 -> 83, 5000 x 2^10 177 -> 81; 2000 x 2^12 (1 bit) 148 -> 104, 20000 x 2^9 (2 bit) 463 -> 200.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,10 +48,11 @@ struct AdjPlan {
   static constexpr int FCOLS = 16 * ((4 * BPT + 15) / 16), WCOLS = PPT;
   static constexpr int TCOLS_F = pow2_at_least(SLOTS * FCOLS, 32), TCOLS_W = pow2_at_least(SLOTS * WCOLS, 32);
   static constexpr size_t SMEM = (size_t)(DATA + NTAB) * sizeof(float2) + 16;
-  // CTAs that may share an SM by shared memory (228 KB, 1 KB of it per CTA the system's) and tensor
-  // memory, eight at most: the kernels' registers are held to that many
-  static constexpr int TCOLS_MAX = TCOLS_F > TCOLS_W ? TCOLS_F : TCOLS_W;
-  static constexpr int CTAS_SMEM = (int)((228 << 10) / (SMEM + 1024)), CTAS_TMEM = 512 / TCOLS_MAX;
+  // the forward kernel also holds a segment's words of both IFs
+  static constexpr size_t smem_forward(int bits) { return SMEM + (size_t)2 * N * bits / 8 + sizeof(float2); }
+  // window kernel: CTAs that may share an SM by shared memory (228 KB, 1 KB of it per CTA the
+  // system's) and tensor memory, eight at most: its registers are held to that many
+  static constexpr int CTAS_SMEM = (int)((228 << 10) / (SMEM + 1024)), CTAS_TMEM = 512 / TCOLS_W;
   static constexpr int CTAS_MEM = CTAS_SMEM < CTAS_TMEM ? CTAS_SMEM : CTAS_TMEM;
   static constexpr int CTAS = CTAS_MEM < 8 ? CTAS_MEM : 8;
   static_assert(T % 32 == 0 && (N / 2) / T == PPT / 2, "whole warps, PPT/2 bins per thread below N/2");
@@ -148,20 +157,20 @@ __device__ __forceinline__ void adjs_store_upper(const float2 (&u)[AdjPlan<LOGN>
   __syncthreads();
 }
 
-// A thread's samples t + T i of one segment (first = s N + t): a warp's loads are 32 consecutive
-// codes.  Codes below 8 bits sit at the same place of every word the thread reads (T is a
-// multiple of the samples per word): the word is rotated so that the code starts at bit 1.
-// (Ordinary loads, here and of the window and the matrix: a read-only one could be moved up
-// over the wait for the kernel before.)
+// A thread's samples t + T i of one segment, from global or shared memory (seg: the segment's
+// words): a warp's loads are 32 consecutive codes.  Codes below 8 bits sit at the same place of
+// every word the thread reads (T is a multiple of the samples per word): the word is rotated so
+// that the code starts at bit 1.  (Ordinary loads, here and of the window and the matrix: a
+// read-only one could be moved up over the wait for the kernel before.)
 template <int LOGN, int BITS>
 struct AdjSamples {
   static constexpr int SPW = 32 / BITS;
   const uint32_t* p;
   uint32_t rot;
-  __device__ __forceinline__ AdjSamples(const uint32_t* in, long long first) {
-    if constexpr (BITS == 8) p = reinterpret_cast<const uint32_t*>(reinterpret_cast<const unsigned char*>(in) + first);
-    else p = in + first / SPW;
-    rot = (uint32_t)(first % SPW) * BITS - 1u;
+  __device__ __forceinline__ AdjSamples(const uint32_t* seg, int tid) {
+    if constexpr (BITS == 8) p = reinterpret_cast<const uint32_t*>(reinterpret_cast<const unsigned char*>(seg) + tid);
+    else p = seg + tid / SPW;
+    rot = (uint32_t)(tid % SPW) * BITS - 1u;
   }
   template <int I>
   __device__ __forceinline__ float level() const {
@@ -178,17 +187,35 @@ struct AdjSamples {
   }
 };
 
-// u[i] = w[n] (x[n] + i y[n]), n = t + T i, of segment s
+// words of a segment of one IF
 template <int LOGN, int BITS>
-__device__ __forceinline__ void adjs_load(const AdjArgs& a, float2 (&u)[AdjPlan<LOGN>::PPT], long long s, int tid) {
+__device__ __forceinline__ constexpr int adjs_words() { return (1 << LOGN) * BITS / 32; }
+
+// u[i] = w[n] (x[n] + i y[n]), n = t + T i, of the segment whose words are at x and y
+template <int LOGN, int BITS>
+__device__ __forceinline__ void adjs_load(const float* window, const uint32_t* x, const uint32_t* y,
+                                          float2 (&u)[AdjPlan<LOGN>::PPT], int tid) {
   using PL = AdjPlan<LOGN>;
-  const AdjSamples<LOGN, BITS> xs(a.in[0], s * PL::N + tid), ys(a.in[1], s * PL::N + tid);
-  const float* wp = a.window + tid;
+  const AdjSamples<LOGN, BITS> xs(x, tid), ys(y, tid);
+  const float* wp = window + tid;
   sfor<0, PL::PPT>([&](auto i_) {
     constexpr int i = decltype(i_)::value;
-    const float w = wp[PL::T * i], x = xs.template level<i>(), y = ys.template level<i>();
-    u[i] = make_float2(w * x, w * y);
+    const float w = wp[PL::T * i];
+    u[i] = make_float2(w * xs.template level<i>(), w * ys.template level<i>());
   });
+}
+
+// both IFs' words of segment s into shared memory ([IF][words], 16-byte chunks; one copy group)
+template <int LOGN, int BITS>
+__device__ __forceinline__ void adjs_fetch(const AdjArgs& a, uint32_t* raw, long long s, int tid) {
+  constexpr int W = adjs_words<LOGN, BITS>();
+  static_assert(W % 4 == 0, "whole chunks");
+  const uint32_t dst = smem_addr(raw);
+  for (int c = tid; c < 2 * (W / 4); c += AdjPlan<LOGN>::T) {
+    const int f = c >= W / 4;
+    cp_async<16>(dst + 16u * (uint32_t)c, a.in[f] + s * W + 4 * (c - f * (W / 4)));
+  }
+  cp_async_commit();
 }
 
 // the set-up both kernels share: the twiddle table in shared memory, this thread's W_N^{r t}
@@ -214,23 +241,28 @@ __device__ __forceinline__ uint32_t adjs_setup(const AdjArgs& a, float2* tws, ui
 }
 
 template <int LOGN, int BITS>
-__global__ void __launch_bounds__(AdjPlan<LOGN>::T, AdjPlan<LOGN>::CTAS) k_adjs_forward(AdjArgs a) {
+__global__ void __launch_bounds__(AdjPlan<LOGN>::T) k_adjs_forward(AdjArgs a) {
   using PL = AdjPlan<LOGN>;
-  constexpr int N = PL::N, T = PL::T;
+  constexpr int N = PL::N, T = PL::T, W = adjs_words<LOGN, BITS>();
   extern __shared__ __align__(16) float2 zs[];
   float2* z = zs;
   float2* tws = zs + PL::DATA;
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(tws + PL::NTAB);
+  uint32_t* raw = reinterpret_cast<uint32_t*>(tws + PL::NTAB + 1);  // (NTAB is odd)
+  uint32_t* tslot = raw + 2 * W;
   const int tid = threadIdx.x;
   float2 wt[PL::RW];
   uint32_t tbase;
   const uint32_t tacc = adjs_setup<LOGN, PL::TCOLS_F, PL::FCOLS>(a, tws, tslot, wt, tbase, tid);
   pdl_wait();  // (dependent launch: the inputs and the partials may be touched from here on)
+  adjs_fetch<LOGN, BITS>(a, raw, blockIdx.x, tid);  // (a.grid <= a.nseg)
 #pragma unroll 1
   for (long long s = blockIdx.x; s < a.nseg; s += a.grid) {
     float2 u[PL::PPT];
-    adjs_load<LOGN, BITS>(a, u, s, tid);
-    adjs_fft<LOGN>(u, z, tws, wt, tid);
+    cp_async_wait_all();
+    __syncthreads();
+    adjs_load<LOGN, BITS>(a.window, raw, raw + W, u, tid);
+    adjs_fft<LOGN>(u, z, tws, wt, tid);  // (its first barrier: all have read the words)
+    if (s + a.grid < a.nseg) adjs_fetch<LOGN, BITS>(a, raw, s + a.grid, tid);
     adjs_store_upper<LOGN>(u, z, tid);
     const float2* zm = z + apad(N - tid);
     // X = (Z[k] + conj Z[N-k]) / 2, Y = (Z[k] - conj Z[N-k]) / 2i; the sums of bin i of this
@@ -287,7 +319,7 @@ __global__ void __launch_bounds__(AdjPlan<LOGN>::T, AdjPlan<LOGN>::CTAS) k_adjs_
 template <int LOGN, int BITS>
 __global__ void __launch_bounds__(AdjPlan<LOGN>::T, AdjPlan<LOGN>::CTAS) k_adjs_window(AdjArgs a) {
   using PL = AdjPlan<LOGN>;
-  constexpr int N = PL::N, T = PL::T;
+  constexpr int N = PL::N, T = PL::T, W = adjs_words<LOGN, BITS>();
   extern __shared__ __align__(16) float2 zs[];
   float2* z = zs;
   float2* tws = zs + PL::DATA;
@@ -301,7 +333,8 @@ __global__ void __launch_bounds__(AdjPlan<LOGN>::T, AdjPlan<LOGN>::CTAS) k_adjs_
 #pragma unroll 1
   for (long long s = blockIdx.x; s < a.nseg; s += a.grid) {
     float2 u[PL::PPT];
-    adjs_load<LOGN, BITS>(a, u, s, tid);
+    const uint32_t *x = a.in[0] + s * W, *y = a.in[1] + s * W;
+    adjs_load<LOGN, BITS>(a.window, x, y, u, tid);
     adjs_fft<LOGN>(u, z, tws, wt, tid);
     adjs_store_upper<LOGN>(u, z, tid);
     if (s == blockIdx.x) pdl_wait();
@@ -342,7 +375,7 @@ __global__ void __launch_bounds__(AdjPlan<LOGN>::T, AdjPlan<LOGN>::CTAS) k_adjs_
     });
     adjs_fft<LOGN>(u, z, tws, wt, tid);
     // h = conj(F): dL/dw[n] += x[n] Re h[n] + y[n] Im h[n] = x F.x - y F.y (column i: n = t + T i)
-    const AdjSamples<LOGN, BITS> xs(a.in[0], s * N + tid), ys(a.in[1], s * N + tid);
+    const AdjSamples<LOGN, BITS> xs(x, tid), ys(y, tid);
     sfor<0, PL::PPT / 16>([&](auto h_) {
       constexpr int h = decltype(h_)::value;
       float acc[16];
@@ -374,25 +407,26 @@ __global__ void __launch_bounds__(AdjPlan<LOGN>::T, AdjPlan<LOGN>::CTAS) k_adjs_
 // ------------------------------------------------------------------------------------------
 // host side
 // ------------------------------------------------------------------------------------------
+// Forward pass: one CTA per SM, because its grid sets the order in which a bin's segments are
+// added.  (The runtime's occupancy query says one for any kernel that allocates tensor memory.)
+// Window pass: as many as share an SM; at one, the sizes below 2^13 left most of it idle: 64
+// threads at 1024 points.
 template <int LOGN, int BITS>
-static cudaError_t adjs_prepare(int* ctas_per_sm) {
+static cudaError_t adjs_prepare(int* window_ctas) {
   using PL = AdjPlan<LOGN>;
-  const int smem = (int)PL::SMEM;
-  cudaError_t e = cudaFuncSetAttribute(k_adjs_forward<LOGN, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  *window_ctas = PL::CTAS;
+  cudaError_t e = cudaFuncSetAttribute(k_adjs_forward<LOGN, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)PL::smem_forward(BITS));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_adjs_window<LOGN, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  int o1 = 0, o2 = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_adjs_forward<LOGN, BITS>, PL::T, PL::SMEM);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o2, k_adjs_window<LOGN, BITS>, PL::T, PL::SMEM);
-  // CTAs that share an SM must find their tensor memory free (512 columns per SM)
-  *ctas_per_sm = std::min(std::min(o1, o2), 512 / std::max(PL::TCOLS_F, PL::TCOLS_W));
+    e = cudaFuncSetAttribute(k_adjs_window<LOGN, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::SMEM);
   return e;
 }
 
 template <int LOGN, int BITS>
 static cudaError_t adjs_launch(bool window_pass, const AdjArgs& a, cudaStream_t st) {
   using PL = AdjPlan<LOGN>;
-  return adj_launch(window_pass ? k_adjs_window<LOGN, BITS> : k_adjs_forward<LOGN, BITS>, a.grid, PL::T, PL::SMEM, st, a);
+  if (window_pass) return adj_launch(k_adjs_window<LOGN, BITS>, a.grid, PL::T, PL::SMEM, st, a);
+  return adj_launch(k_adjs_forward<LOGN, BITS>, a.grid, PL::T, PL::smem_forward(BITS), st, a);
 }
 
 template <int LOGN>
@@ -419,8 +453,8 @@ static cudaError_t adjs_any(int log2n, int bits, bool prepare, int* occ, bool wi
   }
 }
 
-cudaError_t adj_sized_prepare(int log2n, int bits, int* ctas_per_sm) {
-  return adjs_any(log2n, bits, true, ctas_per_sm, false, nullptr, nullptr);
+cudaError_t adj_sized_prepare(int log2n, int bits, int* window_ctas) {
+  return adjs_any(log2n, bits, true, window_ctas, false, nullptr, nullptr);
 }
 
 cudaError_t adj_sized_launch(int log2n, int bits, bool window_pass, const AdjArgs& a, cudaStream_t st) {

@@ -450,15 +450,6 @@ class Adjoint:
     def run(self, packed, n_samples: int, window, gains, leak, target=None, grads: bool = False, stream=None):
         """dict(stokes [4, nb], loss (float64, 1 element) and, with grads=True, grad_window [N],
         grad_gains [4], grad_leak [2, nb, 2]).  packed: two CUDA tensors of packed words."""
-        return self._run(packed, n_samples, window, gains, leak, target, grads, stream)[0]
-
-    def _split(self, flat):
-        """grad_window, grad_gains and grad_leak as they lie in one buffer."""
-        n, nb = self.n_fft, self.n_bins
-        return flat[:n], flat[n:n + 4], flat[n + 4:].view(2, nb, 2)
-
-    def _run(self, packed, n_samples: int, window, gains, leak, target, grads: bool, stream):
-        """run()'s outputs, and the buffer that holds the three gradients."""
         import torch
 
         dev = window.device
@@ -466,22 +457,30 @@ class Adjoint:
         out = {"stokes": torch.empty((4, nb), dtype=torch.float32, device=dev)}
         if target is not None:
             out["loss"] = torch.empty((1,), dtype=torch.float64, device=dev)
-        flat = None
+        at = (None, None, None)
         if grads:
-            flat = torch.empty((self.n_fft + 4 + 4 * nb,), dtype=torch.float32, device=dev)
-            out["grad_window"], out["grad_gains"], out["grad_leak"] = self._split(flat)
+            out["grad_window"] = torch.empty((self.n_fft,), dtype=torch.float32, device=dev)
+            out["grad_gains"] = torch.empty((4,), dtype=torch.float32, device=dev)
+            out["grad_leak"] = torch.empty((2, nb, 2), dtype=torch.float32, device=dev)
+            at = (_ptr(out["grad_window"]), _ptr(out["grad_gains"]), _ptr(out["grad_leak"]))
+        self._call(packed, n_samples, window, gains, leak, target, out["stokes"], out.get("loss"), at, stream)
+        return out
+
+    def _call(self, packed, n_samples, window, gains, leak, target, stokes, loss, grads, stream):
+        """polaris_adj_run; grads: the addresses of the three gradients (or None)."""
         arr = (ctypes.c_void_p * 2)(*[_ptr(p) for p in packed])
         ins = [t.contiguous() for t in (window, gains, leak)]
         tgt = None if target is None else target.contiguous()
         rc = load().polaris_adj_run(self._h, arr, int(n_samples), _ptr(ins[0]), _ptr(ins[1]), _ptr(ins[2]),
-                                    None if tgt is None else _ptr(tgt), _ptr(out["stokes"]),
-                                    _ptr(out["loss"]) if "loss" in out else None,
-                                    _ptr(out["grad_window"]) if grads else None,
-                                    _ptr(out["grad_gains"]) if grads else None,
-                                    _ptr(out["grad_leak"]) if grads else None, _stream_ptr(stream))
+                                    None if tgt is None else _ptr(tgt), None if stokes is None else _ptr(stokes),
+                                    None if loss is None else _ptr(loss), *grads, _stream_ptr(stream))
         if rc != OK:
             raise PolarisError(rc, load().polaris_adj_last_error(self._h).decode())
-        return out, flat
+
+    def _split(self, flat):
+        """grad_window, grad_gains and grad_leak as they lie in one buffer."""
+        n, nb = self.n_fft, self.n_bins
+        return flat[:n], flat[n:n + 4], flat[n + 4:].view(2, nb, 2)
 
 
 @functools.lru_cache(maxsize=None)
@@ -493,13 +492,17 @@ def _leakage_function():
         @staticmethod
         def forward(ctx, w, g, d, data):
             adj, packed, n_samples, target = data  # (in a tuple: not part of the graph)
-            need = any(ctx.needs_input_grad)
-            r, flat = adj._run(packed, n_samples, w.detach(), g.detach(), d.detach(), target, need,
-                               torch.cuda.current_stream(w.device))
-            if need:
+            n, nb = adj.n_fft, adj.n_bins
+            loss = torch.empty((1,), dtype=torch.float64, device=w.device)
+            flat, at = None, (None, None, None)
+            if any(ctx.needs_input_grad):  # the three gradients in one buffer
+                flat = torch.empty((n + 4 + 4 * nb,), dtype=torch.float32, device=w.device)
+                at = tuple(flat.data_ptr() + 4 * o for o in (0, n, n + 4))
                 ctx.adj = adj
                 ctx.save_for_backward(flat)
-            return r["loss"][0]
+            adj._call(packed, n_samples, w.detach(), g.detach(), d.detach(), target, None, loss, at,
+                      torch.cuda.current_stream(w.device))
+            return loss[0]
 
         @staticmethod
         def backward(ctx, gout):
