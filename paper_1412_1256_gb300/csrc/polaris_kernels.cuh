@@ -1,4 +1,5 @@
-// Hot-path kernels (sm_103a), templated on log2(N):
+// Hot-path kernels (sm_103a), templated on log2(N), of the sizes that take two kernels (N = 2^4..2^9
+// and 2^15 up; 2^10..2^14 run in one, polaris_fused.cuh, and phase 1 of 2^18 up in polaris_wide.cuh):
 //
 //   k_phase1  data translation (codes -> levels, Fig. 2 caption), window (Sec. 3.1),
 //             first half of the segment FFT: for every column b of n = N2 a + b a DFT of
@@ -285,9 +286,10 @@ __device__ __forceinline__ void p1_load(const BatchArgs& a, int g, int b, int q1
       word_i = (n * BITS) >> 5;
       shift = (n * BITS) & 31u;
     }
+    // (ordinary loads: a read-only one could be moved up over the wait for the kernel before)
     const bool ok = in_bounds(a.err, w0 + word_i, wext);
-    float x = decode_level<BITS>(ok ? __ldg(pa + word_i) : 0u, shift);
-    float y = pb ? decode_level<BITS>(ok ? __ldg(pb + word_i) : 0u, shift) : 0.0f;
+    float x = decode_level<BITS>(ok ? pa[word_i] : 0u, shift);
+    float y = pb ? decode_level<BITS>(ok ? pb[word_i] : 0u, shift) : 0.0f;
     if (taps) {
       const float wv = __ldg(taps + tap_order(LOGN).slot(n));
       x *= wv;
