@@ -315,7 +315,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_pass(PassArgs a) {
 // few threads: one thread per bin, which loaded as well, kept 9 blocks busy.  A block takes 32 bins;
 // its eight warps form the products of kCorrChunk segments (all loads in flight), then four warps,
 // one per quantity, add them in order, so a sum stays one chain per bin, to the bit.  A feed of
-// 8192 segments of 4096 points: 1771 us before, 685 now; 2000: 408, 178; 61 of 2^18: no slower.
+// 8192 segments of 4096 points: 1771 us before, 685, and 571 with the next chunk's loads in flight
+// during the sums; 2000: 408, 178, 149; 61 of 2^18: no slower.
 __device__ __forceinline__ void kahan_add(float& sum, float& comp, float x) {
   const float y = x - comp;
   const float t = sum + y;
@@ -330,15 +331,18 @@ __global__ void __launch_bounds__(32 * kCorrWarps) k_tc_correlate(const float2* 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = blockIdx.x * kCorrBins + lane;
   const int kk = k < nbin ? k : 0, km = (N - kk) & (N - 1);
   float sum = 0.f, comp = 0.f;  // (warps 0 to 3: quantity `warp` of bin k)
-#pragma unroll 1
-  for (int s0 = 0; s0 < nseg; s0 += kCorrChunk) {
-    float2 a[kCorrLoads], b[kCorrLoads];
+  float2 a[kCorrLoads], b[kCorrLoads];
+  auto load = [&](int s0) {  // this warp's segments of the chunk at s0 (past the end: the last one, unused)
 #pragma unroll
     for (int i = 0; i < kCorrLoads; ++i) {
       const float2* z = Z + (long long)min(s0 + warp + i * kCorrWarps, nseg - 1) * N;
       a[i] = __ldcg(z + kk);
       b[i] = __ldcg(z + km);
     }
+  };
+  load(0);
+#pragma unroll 1
+  for (int s0 = 0; s0 < nseg; s0 += kCorrChunk) {
     __syncthreads();  // the last chunk's products have been added
 #pragma unroll
     for (int i = 0; i < kCorrLoads; ++i) {
@@ -350,6 +354,7 @@ __global__ void __launch_bounds__(32 * kCorrWarps) k_tc_correlate(const float2* 
       p[2][lane] = fmaf(xr, yr, xi * yi);
       p[3][lane] = fmaf(xi, yr, -xr * yi);
     }
+    if (s0 + kCorrChunk < nseg) load(s0 + kCorrChunk);  // in flight during the sums
     __syncthreads();
     if (warp < 4) {
       const int n = min(kCorrChunk, nseg - s0);
