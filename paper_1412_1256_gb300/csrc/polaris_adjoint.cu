@@ -443,6 +443,7 @@ struct polaris_adj {
   int N = 0, log2n = 0, nbin = 0, bits = 0, device = 0, threads = 0, grid_max = 0, grid_window = 0, bin_blocks = 0;
   bool sized = false;  // the size-specialised segment kernels (polaris_adjoint_sized.cu)
   size_t smem = 0;
+  unsigned char* d_all = nullptr;  // the device memory of the five below
   float2* d_tw = nullptr;
   float4* d_part = nullptr;  // [grid_max][nbin]
   float* d_gpart = nullptr;  // [grid_window][N]
@@ -473,13 +474,7 @@ static cudaError_t adj_prepare(polaris_adj* h, int* ctas_per_sm) {
   return e;
 }
 
-static void adj_free(polaris_adj* h) {
-  cudaFree(h->d_tw);
-  cudaFree(h->d_part);
-  cudaFree(h->d_gpart);
-  cudaFree(h->d_mat);
-  cudaFree(h->d_bpart);
-}
+static void adj_free(polaris_adj* h) { cudaFree(h->d_all); }
 
 extern "C" int polaris_adj_create(int64_t n_fft, int bits, int device, polaris_adj** out) {
   if (!out) return POLARIS_EINVAL;
@@ -545,12 +540,27 @@ extern "C" int polaris_adj_create(int64_t n_fft, int bits, int device, polaris_a
       }
     Ns *= R;
   }
-  bool ok = cudaMalloc((void**)&h->d_tw, tw.size() * sizeof(float2)) == cudaSuccess &&
-            cudaMalloc((void**)&h->d_part, (size_t)h->grid_max * h->nbin * sizeof(float4)) == cudaSuccess &&
-            cudaMalloc((void**)&h->d_gpart, (size_t)h->grid_window * h->N * sizeof(float)) == cudaSuccess &&
-            cudaMalloc((void**)&h->d_mat, (size_t)h->nbin * sizeof(float4)) == cudaSuccess &&
-            cudaMalloc((void**)&h->d_bpart, (size_t)h->bin_blocks * 5 * sizeof(double)) == cudaSuccess &&
-            cudaMemcpy(h->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess;
+  // one allocation for all of them (each costs the caller's program tens of microseconds)
+  size_t total = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = total;
+    total += (bytes + 255) & ~(size_t)255;
+    return at;
+  };
+  const size_t at_part = take((size_t)h->grid_max * h->nbin * sizeof(float4));
+  const size_t at_gpart = take((size_t)h->grid_window * h->N * sizeof(float));
+  const size_t at_mat = take((size_t)h->nbin * sizeof(float4));
+  const size_t at_bpart = take((size_t)h->bin_blocks * 5 * sizeof(double));
+  const size_t at_tw = take(tw.size() * sizeof(float2));
+  bool ok = cudaMalloc((void**)&h->d_all, total) == cudaSuccess;
+  if (ok) {
+    h->d_part = reinterpret_cast<float4*>(h->d_all + at_part);
+    h->d_gpart = reinterpret_cast<float*>(h->d_all + at_gpart);
+    h->d_mat = reinterpret_cast<float4*>(h->d_all + at_mat);
+    h->d_bpart = reinterpret_cast<double*>(h->d_all + at_bpart);
+    h->d_tw = reinterpret_cast<float2*>(h->d_all + at_tw);
+    ok = cudaMemcpy(h->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess;
+  }
   if (!ok) {
     cudaGetLastError();
     adj_free(h);
