@@ -654,16 +654,16 @@ extern "C" int polaris_adj_run(polaris_adj* h, const void* const* packed, int64_
     b.grad_leak = grads ? grad_leak : nullptr;
     b.mat = grads ? h->d_mat : nullptr;
     b.bpart = (loss || grads) ? h->d_bpart : nullptr;
-    e = adj_launch(k_adj_bins, h->bin_blocks, kBinsPerBlock * kSlices, 0, st, b);
+    e = launch_dependent(k_adj_bins, h->bin_blocks, kBinsPerBlock * kSlices, 0, st, b);
   }
   if (e == cudaSuccess && grads) {
     if (sized) a.grid = std::min(a.nseg, h->grid_window);
     e = adj_segments_bits(h->bits, a, h->smem, true, sized, st);
     if (e == cudaSuccess)
-      e = adj_launch(k_adj_wsum, (h->N + kBinsPerBlock - 1) / kBinsPerBlock + 1, kBinsPerBlock * kSlices, 0, st, h->d_gpart,
+      e = launch_dependent(k_adj_wsum, (h->N + kBinsPerBlock - 1) / kBinsPerBlock + 1, kBinsPerBlock * kSlices, 0, st, h->d_gpart,
                      a.grid, h->N, grad_window, h->d_bpart, h->bin_blocks, loss, grad_gains);
   } else if (e == cudaSuccess && loss) {
-    e = adj_launch(k_adj_finish, 1, 160, 0, st, h->d_bpart, h->bin_blocks, loss);
+    e = launch_dependent(k_adj_finish, 1, 160, 0, st, h->d_bpart, h->bin_blocks, loss);
   }
   cudaSetDevice(prev);
   if (e != cudaSuccess) return adj_err(h, POLARIS_ECUDA, "CUDA: ", cudaGetErrorString(e));

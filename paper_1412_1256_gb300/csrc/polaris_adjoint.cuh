@@ -9,6 +9,7 @@
 #include <cstdint>
 
 #include "polaris_device.cuh"
+#include "polaris_launch.cuh"
 
 namespace polaris {
 
@@ -37,24 +38,6 @@ __device__ __forceinline__ void adj_bin_gradient(float4 m, float2 Zk, float2 Zm,
   const float2 Y = make_float2(0.5f * (Zk.y - Zm.y), -0.5f * (Zk.x - Zm.x));
   GX = c_add(make_float2(m.x * X.x, m.x * X.y), cmul(make_float2(m.z, m.w), Y));
   GY = c_add(make_float2(m.y * Y.x, m.y * Y.y), cmul(make_float2(m.z, -m.w), X));
-}
-
-// One launch with programmatic stream serialisation: the kernel may be scheduled while its
-// predecessor ends, and waits for it (griddepcontrol.wait) before it touches what that one, or
-// the caller's earlier work, wrote.
-template <typename... P, typename... Q>
-static cudaError_t adj_launch(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, Q... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 // level of sample idx of one IF

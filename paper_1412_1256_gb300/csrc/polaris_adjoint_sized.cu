@@ -425,8 +425,8 @@ static cudaError_t adjs_prepare(int* window_ctas) {
 template <int LOGN, int BITS>
 static cudaError_t adjs_launch(bool window_pass, const AdjArgs& a, cudaStream_t st) {
   using PL = AdjPlan<LOGN>;
-  if (window_pass) return adj_launch(k_adjs_window<LOGN, BITS>, a.grid, PL::T, PL::SMEM, st, a);
-  return adj_launch(k_adjs_forward<LOGN, BITS>, a.grid, PL::T, PL::smem_forward(BITS), st, a);
+  if (window_pass) return launch_dependent(k_adjs_window<LOGN, BITS>, a.grid, PL::T, PL::SMEM, st, a);
+  return launch_dependent(k_adjs_forward<LOGN, BITS>, a.grid, PL::T, PL::smem_forward(BITS), st, a);
 }
 
 template <int LOGN>

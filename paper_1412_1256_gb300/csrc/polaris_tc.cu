@@ -35,6 +35,8 @@
 
 #include "../../include/polaris.h"
 #include "polaris_device.cuh"
+#include "polaris_kernels.cuh"  // dependent launch
+#include "polaris_launch.cuh"
 
 namespace polaris {
 namespace tc {
@@ -121,13 +123,14 @@ __device__ __forceinline__ bool wait_parity(uint32_t bar, uint32_t parity, uint3
   return false;
 }
 
+// (ordinary loads: a read-only one could be moved up over the wait for the kernel before)
 template <int BITS>
-__device__ __forceinline__ float tc_level(const uint32_t* __restrict__ in, long long idx) {
+__device__ __forceinline__ float tc_level(const uint32_t* in, long long idx) {
   if constexpr (BITS == 8) {
-    return (float)(int)__ldg(reinterpret_cast<const signed char*>(in) + idx);
+    return (float)(int)reinterpret_cast<const signed char*>(in)[idx];
   } else {
     constexpr int SPW = 32 / BITS;
-    return decode_level<BITS>(__ldg(in + idx / SPW), (uint32_t)(idx % SPW) * BITS);
+    return decode_level<BITS>(in[idx / SPW], (uint32_t)(idx % SPW) * BITS);
   }
 }
 
@@ -183,6 +186,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_pass(PassArgs a) {
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tbase = *slot, tmem = tbase + 128u * gr;
+  pdl_wait();     // the kernel before has written the source and read the destination (dependent launch)
+  // The next pass sets up on each SM as this one's CTA leaves it.  The correlation comes after the
+  // whole grid instead: its blocks (65 at 4096 points) would pile up, eight an SM, on the first SMs
+  // that are left (8192 segments: 824 us; 571 without dependent launches, 482 so; 61 of 2^18 355, 293).
+  if (a.Ns * kR < a.N) pdl_trigger();
   // D f32, A and B bf16 (1) or f16 (0), both K-major, N = 128, M = 128
   constexpr uint32_t fmt = PREC == POLARIS_TC_FP16X3 ? 0u : 1u;
   constexpr uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(kK >> 3) << 17) |
@@ -315,8 +323,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_pass(PassArgs a) {
 // few threads: one thread per bin, which loaded as well, kept 9 blocks busy.  A block takes 32 bins;
 // its eight warps form the products of kCorrChunk segments (all loads in flight), then four warps,
 // one per quantity, add them in order, so a sum stays one chain per bin, to the bit.  A feed of
-// 8192 segments of 4096 points: 1771 us before, 685, and 571 with the next chunk's loads in flight
-// during the sums; 2000: 408, 178, 149; 61 of 2^18: no slower.
+// 8192 segments of 4096 points took 1771 us before, 685, and 571 with the next chunk's loads in flight
+// during the sums (before the launches became dependent ones); 61 of 2^18: no slower.
 __device__ __forceinline__ void kahan_add(float& sum, float& comp, float x) {
   const float y = x - comp;
   const float t = sum + y;
@@ -331,6 +339,8 @@ __global__ void __launch_bounds__(32 * kCorrWarps) k_tc_correlate(const float2* 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = blockIdx.x * kCorrBins + lane;
   const int kk = k < nbin ? k : 0, km = (N - kk) & (N - 1);
   float sum = 0.f, comp = 0.f;  // (warps 0 to 3: quantity `warp` of bin k)
+  pdl_wait();
+  pdl_trigger();
   float2 a[kCorrLoads], b[kCorrLoads];
   auto load = [&](int s0) {  // this warp's segments of the chunk at s0 (past the end: the last one, unused)
 #pragma unroll
@@ -463,15 +473,14 @@ template <int PREC>
 static cudaError_t tc_launch_pass(int bits, const PassArgs& a, int grid, cudaStream_t st) {
   if (a.Ns == 1) {
     switch (bits) {
-      case 1: k_tc_pass<PREC, 1><<<grid, kThreads, kSmemBytes, st>>>(a); break;
-      case 2: k_tc_pass<PREC, 2><<<grid, kThreads, kSmemBytes, st>>>(a); break;
-      case 4: k_tc_pass<PREC, 4><<<grid, kThreads, kSmemBytes, st>>>(a); break;
-      default: k_tc_pass<PREC, 8><<<grid, kThreads, kSmemBytes, st>>>(a); break;
+      case 1: return launch_dependent(k_tc_pass<PREC, 1>, grid, kThreads, kSmemBytes, st, a);
+      case 2: return launch_dependent(k_tc_pass<PREC, 2>, grid, kThreads, kSmemBytes, st, a);
+      case 4: return launch_dependent(k_tc_pass<PREC, 4>, grid, kThreads, kSmemBytes, st, a);
+      default: return launch_dependent(k_tc_pass<PREC, 8>, grid, kThreads, kSmemBytes, st, a);
     }
   } else {
-    k_tc_pass<PREC, 0><<<grid, kThreads, kSmemBytes, st>>>(a);
+    return launch_dependent(k_tc_pass<PREC, 0>, grid, kThreads, kSmemBytes, st, a);
   }
-  return cudaGetLastError();
 }
 
 static void tc_free(polaris_tc* h) {
@@ -646,11 +655,9 @@ extern "C" int polaris_tc_feed(polaris_tc* h, const void* const* packed, int64_t
       }
       cur ^= 1;
     }
-    if (e == cudaSuccess) {
-      k_tc_correlate<<<(h->nbin + kCorrBins - 1) / kCorrBins, 32 * kCorrWarps, 0, st>>>(h->d_buf[cur ^ 1], h->N, h->nbin,
-                                                                                       nb, h->d_acc);
-      e = cudaGetLastError();
-    }
+    if (e == cudaSuccess)
+      e = launch_dependent(k_tc_correlate, (h->nbin + kCorrBins - 1) / kCorrBins, 32 * kCorrWarps, 0, st, h->d_buf[cur ^ 1],
+                           h->N, h->nbin, nb, h->d_acc);
   }
   cudaSetDevice(prev);
   if (e != cudaSuccess) return tc_err(h, POLARIS_ECUDA, std::string("CUDA: ") + cudaGetErrorString(e));
