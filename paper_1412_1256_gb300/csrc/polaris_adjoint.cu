@@ -29,7 +29,8 @@
 // adjoint pass, not stored.
 //
 // Kernels (no atomics; every sum has a fixed order, so runs are bitwise reproducible):
-//   k_adj_forward  a grid of G CTAs, each over segments b, b + G, ...: decode, window, a
+//   k_adj_forward  (2^5 .. 2^8: k_adjm_forward and k_adjm_window, many segments per CTA)
+//                  a grid of G CTAs, each over segments b, b + G, ...: decode, window, a
 //                  radix-16 Stockham transform of the pair x + i y in shared memory, split
 //                  into X and Y, per-CTA partial sums of |X|^2, |Y|^2, X conj(Y)
 //                  (N = 2^9 .. 2^14: k_adjs_forward, the same per size at compile time,
@@ -41,7 +42,7 @@
 //                  per-CTA partials of the window gradient
 //   k_adj_wsum     the window-gradient partials summed per tap, and the block partials of the
 //                  loss and gain gradients in order (k_adj_finish: those alone, without gradients)
-// The launches are programmatic dependent ones (but for the kernels for any N): each kernel's
+// The launches are programmatic dependent ones (but for k_adj_forward and k_adj_window): each kernel's
 // set-up, and the window pass's first transform, run while the one before ends.
 #include <cuda_runtime.h>
 
@@ -69,13 +70,13 @@ constexpr int kMaxCtasPerSm = 8;
 // holds 16 points: one j for R = 16, j = t, t + T, ... for smaller radices, always < N/R
 // (a bounds test here would push the point arrays into local memory).
 template <int R>
-__device__ __forceinline__ void stockham_pass(float2* z, int N, int Ns, const float2* __restrict__ tw, int T) {
+__device__ __forceinline__ void stockham_pass(float2* z, int N, int Ns, const float2* __restrict__ tw, int T, int t) {
   constexpr int JPT = 16 / R;
   const int m = N / R;
   float2 v[JPT][R];
 #pragma unroll
   for (int q = 0; q < JPT; ++q) {
-    const int j = threadIdx.x + q * T;
+    const int j = t + q * T;
     const int k = j & (Ns - 1);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -87,7 +88,7 @@ __device__ __forceinline__ void stockham_pass(float2* z, int N, int Ns, const fl
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < JPT; ++q) {
-    const int j = threadIdx.x + q * T;
+    const int j = t + q * T;
     dit<R>(v[q]);
     const int k = j & (Ns - 1);
     const int base = (j - k) * R + k;
@@ -98,14 +99,14 @@ __device__ __forceinline__ void stockham_pass(float2* z, int N, int Ns, const fl
 }
 
 // forward DFT of the N points in z (natural order in and out); callers sync before
-__device__ __forceinline__ void adj_fft(float2* z, int N, int log2n, const float2* __restrict__ tw, int T) {
+__device__ __forceinline__ void adj_fft(float2* z, int N, int log2n, const float2* __restrict__ tw, int T, int t) {
   int Ns = 1;
 #pragma unroll 1
-  for (int p = 0; p < (log2n >> 2); ++p, Ns <<= 4) stockham_pass<16>(z, N, Ns, tw, T);
+  for (int p = 0; p < (log2n >> 2); ++p, Ns <<= 4) stockham_pass<16>(z, N, Ns, tw, T, t);
   switch (log2n & 3) {
-    case 1: stockham_pass<2>(z, N, Ns, tw, T); break;
-    case 2: stockham_pass<4>(z, N, Ns, tw, T); break;
-    case 3: stockham_pass<8>(z, N, Ns, tw, T); break;
+    case 1: stockham_pass<2>(z, N, Ns, tw, T, t); break;
+    case 2: stockham_pass<4>(z, N, Ns, tw, T, t); break;
+    case 3: stockham_pass<8>(z, N, Ns, tw, T, t); break;
     default: break;
   }
 }
@@ -113,13 +114,39 @@ __device__ __forceinline__ void adj_fft(float2* z, int N, int log2n, const float
 // z[n] = w[n] (x[n] + i y[n]) for segment s; thread t fills n = t + T e, e < 16, so that
 // every load is coalesced and the stores are conflict-free
 template <int BITS>
-__device__ __forceinline__ void adj_load_segment(const AdjArgs& a, float2* z, long long s) {
+__device__ __forceinline__ void adj_load_segment(const AdjArgs& a, float2* z, long long s, int t) {
   const long long base = s * a.N;
 #pragma unroll 8
   for (int e = 0; e < 16; ++e) {
-    const int n = threadIdx.x + e * a.threads;
-    const float w = __ldg(a.window + n);
+    const int n = t + e * a.threads;
+    const float w = a.window[n];
     z[apad(n)] = make_float2(w * adj_level<BITS>(a.in[0], base + n), w * adj_level<BITS>(a.in[1], base + n));
+  }
+}
+
+// |X|^2, |Y|^2, Re and Im X conj(Y) of bin k: X = (Z[k] + conj Z[N-k]) / 2, Y = (Z[k] - conj Z[N-k]) / 2i
+__device__ __forceinline__ float4 adj_products(const float2* z, int N, int k) {
+  const float2 Zk = z[apad(k)], Zm = c_conj(z[apad((N - k) & (N - 1))]);
+  const float2 X = make_float2(0.5f * (Zk.x + Zm.x), 0.5f * (Zk.y + Zm.y));
+  const float2 Y = make_float2(0.5f * (Zk.y - Zm.y), -0.5f * (Zk.x - Zm.x));
+  return make_float4(fmaf(X.x, X.x, X.y * X.y), fmaf(Y.x, Y.x, Y.y * Y.y), fmaf(X.x, Y.x, X.y * Y.y),
+                     fmaf(X.y, Y.x, -X.x * Y.y));
+}
+
+// G_X and G_Y of bin k; conj of the Hermitian extension of G_X + i G_Y goes back into slots k and N - k
+// (the inverse transform is conj(DFT(conj H)))
+__device__ __forceinline__ void adj_pull_back(float2* z, int N, int k, float4 m) {
+  const int km = (N - k) & (N - 1);
+  const float2 Zk = z[apad(k)], Zm = c_conj(z[apad(km)]);
+  float2 GX, GY;
+  adj_bin_gradient(m, Zk, Zm, GX, GY);
+  if (k == 0 || 2 * k == N) {
+    z[apad(k)] = make_float2(GX.x, -GY.x);  // H = Re G_X + i Re G_Y
+  } else {
+    const float2 hx = make_float2(0.5f * GX.x, 0.5f * GX.y), hy = make_float2(0.5f * GY.x, 0.5f * GY.y);
+    // H[k] = hx + i hy, H[N-k] = conj(hx) + i conj(hy); store their conjugates
+    z[apad(k)] = make_float2(hx.x - hy.y, -(hx.y + hy.x));
+    z[apad(km)] = make_float2(hx.x + hy.y, hx.y - hy.x);
   }
 }
 
@@ -128,17 +155,12 @@ template <int BITS>
 __device__ __forceinline__ void adj_forward_segment(const AdjArgs& a, float2* z, long long s, bool first) {
   const int N = a.N, nbin = a.nbin;
   float4* part = a.part + (size_t)blockIdx.x * nbin;
-  adj_load_segment<BITS>(a, z, s);
+  adj_load_segment<BITS>(a, z, s, threadIdx.x);
   __syncthreads();
-  adj_fft(z, N, a.log2n, a.tw, a.threads);
-  // X = (Z[k] + conj Z[N-k]) / 2, Y = (Z[k] - conj Z[N-k]) / 2i
+  adj_fft(z, N, a.log2n, a.tw, a.threads, threadIdx.x);
 #pragma unroll 1
   for (int k = threadIdx.x; k < nbin; k += a.threads) {
-    const float2 Zk = z[apad(k)], Zm = c_conj(z[apad((N - k) & (N - 1))]);
-    const float2 X = make_float2(0.5f * (Zk.x + Zm.x), 0.5f * (Zk.y + Zm.y));
-    const float2 Y = make_float2(0.5f * (Zk.y - Zm.y), -0.5f * (Zk.x - Zm.x));
-    const float4 v = make_float4(fmaf(X.x, X.x, X.y * X.y), fmaf(Y.x, Y.x, Y.y * Y.y), fmaf(X.x, Y.x, X.y * Y.y),
-                                fmaf(X.y, Y.x, -X.x * Y.y));
+    const float4 v = adj_products(z, N, k);
     if (first) {
       part[k] = v;
     } else {
@@ -161,28 +183,14 @@ template <int BITS>
 __device__ __forceinline__ void adj_window_segment(const AdjArgs& a, float2* z, long long s, bool first) {
   const int N = a.N, nbin = a.nbin;
   float* gpart = a.gpart + (size_t)blockIdx.x * N;
-  adj_load_segment<BITS>(a, z, s);
+  adj_load_segment<BITS>(a, z, s, threadIdx.x);
   __syncthreads();
-  adj_fft(z, N, a.log2n, a.tw, a.threads);
-  // G_X, G_Y per bin pair; conj of the Hermitian extension of G_X + i G_Y goes back into z
-  // (the inverse transform is conj(DFT(conj H))).  Thread k owns slots k and N - k.
+  adj_fft(z, N, a.log2n, a.tw, a.threads, threadIdx.x);
+  // thread k owns slots k and N - k
 #pragma unroll 1
-  for (int k = threadIdx.x; k < nbin; k += a.threads) {
-    const int km = (N - k) & (N - 1);
-    const float2 Zk = z[apad(k)], Zm = c_conj(z[apad(km)]);
-    float2 GX, GY;
-    adj_bin_gradient(__ldg(a.mat + k), Zk, Zm, GX, GY);
-    if (k == 0 || 2 * k == N) {
-      z[apad(k)] = make_float2(GX.x, -GY.x);  // H = Re G_X + i Re G_Y
-    } else {
-      const float2 hx = make_float2(0.5f * GX.x, 0.5f * GX.y), hy = make_float2(0.5f * GY.x, 0.5f * GY.y);
-      // H[k] = hx + i hy, H[N-k] = conj(hx) + i conj(hy); store their conjugates
-      z[apad(k)] = make_float2(hx.x - hy.y, -(hx.y + hy.x));
-      z[apad(km)] = make_float2(hx.x + hy.y, hx.y - hy.x);
-    }
-  }
+  for (int k = threadIdx.x; k < nbin; k += a.threads) adj_pull_back(z, N, k, a.mat[k]);
   __syncthreads();
-  adj_fft(z, N, a.log2n, a.tw, a.threads);
+  adj_fft(z, N, a.log2n, a.tw, a.threads, threadIdx.x);
   // h = conj(F): dL/dw[n] += x[n] Re h[n] + y[n] Im h[n] = x F.x - y F.y
   const long long base = s * N;
 #pragma unroll 8
@@ -200,6 +208,106 @@ __global__ void __launch_bounds__(1024) k_adj_window(AdjArgs a) {
   extern __shared__ float2 z[];
 #pragma unroll 1
   for (long long s = blockIdx.x; s < a.nseg; s += a.grid) adj_window_segment<BITS>(a, z, s, s == blockIdx.x);
+}
+
+// ------------------------------------------------------------------------------------------
+// N = 2^5 to 2^8, where one segment's N/16 threads are a fraction of a warp: a CTA takes many segments at
+// once, one per team of N/16 threads.
+//   - Forward: the CTA's group is the segments b, b + G, ... that one small CTA took in turn before, its
+//     teams taking consecutive ones.  The products go to shared memory and are added in that order, one
+//     chain per bin and quantity, so the partial sums are the same to the bit.
+//   - Window pass: every team adds its segments' taps in registers; the CTA adds its teams at the end.
+// Bound by latency (loads, and barriers of two or four warps).  Whole steps of 4 M int8 samples with
+// one segment per CTA at a time, eight CTAs of 4 to 16 threads per SM, and now: 2^6 517 -> 79 us, 2^7
+// 301 -> 76, 2^8 (2 bits) 188 -> 85.
+// ------------------------------------------------------------------------------------------
+template <int LOGN, int THREADS>
+struct AdjSmall {
+  static constexpr int N = 1 << LOGN, T = N / 16, TEAMS = THREADS / T, NBIN = N / 2 + 1, POINTS = adj_smem_points(N);
+};
+constexpr int kSmallForward = 64, kSmallWindow = 128, kSmallWindowCtas = 6;  // threads; window CTAs per SM
+
+template <int LOGN, int BITS>
+__global__ void __launch_bounds__(kSmallForward) k_adjm_forward(AdjArgs a) {
+  using S = AdjSmall<LOGN, kSmallForward>;
+  constexpr int NC = 4 * S::NBIN, CH = (NC + kSmallForward - 1) / kSmallForward;  // chains of a bin and quantity
+  __shared__ float2 zs[S::TEAMS][S::POINTS];
+  __shared__ __align__(16) float prod[S::TEAMS][NC];
+  const int team = threadIdx.x / S::T, t = threadIdx.x % S::T;
+  float2* z = zs[team];
+  float acc[CH];
+#pragma unroll
+  for (int c = 0; c < CH; ++c) acc[c] = 0.f;
+  pdl_wait();  // (dependent launch: the inputs and the partials may be touched from here on)
+#pragma unroll 1
+  for (long long s0 = blockIdx.x; s0 < a.nseg; s0 += (long long)S::TEAMS * a.grid) {
+    const long long left = (a.nseg - 1 - s0) / a.grid + 1;  // segments of the group from s0 on
+    const int n = left < S::TEAMS ? (int)left : S::TEAMS;
+    adj_load_segment<BITS>(a, z, s0 + (long long)(team < n ? team : 0) * a.grid, t);  // (idle teams: the first one again)
+    __syncthreads();
+    adj_fft(z, S::N, LOGN, a.tw, S::T, t);
+#pragma unroll 1
+    for (int k = t; k < S::NBIN; k += S::T) reinterpret_cast<float4*>(prod[team])[k] = adj_products(z, S::N, k);
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+      const int i = threadIdx.x + c * kSmallForward;
+      if (i < NC) {
+#pragma unroll 4
+        for (int j = 0; j < n; ++j) acc[c] += prod[j][i];
+      }
+    }
+  }
+  float* part = reinterpret_cast<float*>(a.part + (size_t)blockIdx.x * S::NBIN);
+#pragma unroll
+  for (int c = 0; c < CH; ++c) {
+    const int i = threadIdx.x + c * kSmallForward;
+    if (i < NC) part[i] = acc[c];
+  }
+}
+
+template <int LOGN, int BITS>
+__global__ void __launch_bounds__(kSmallWindow, kSmallWindowCtas) k_adjm_window(AdjArgs a) {
+  using S = AdjSmall<LOGN, kSmallWindow>;
+  __shared__ float2 zs[S::TEAMS][S::POINTS];
+  const int team = threadIdx.x / S::T, t = threadIdx.x % S::T;
+  float2* z = zs[team];
+  float acc[16];
+#pragma unroll
+  for (int e = 0; e < 16; ++e) acc[e] = 0.f;
+  pdl_wait();
+#pragma unroll 1
+  for (long long s0 = (long long)blockIdx.x * S::TEAMS; s0 < a.nseg; s0 += (long long)S::TEAMS * a.grid) {
+    const bool mine = s0 + team < a.nseg;
+    const long long s = mine ? s0 + team : s0;  // (idle teams: the CTA's first one again)
+    adj_load_segment<BITS>(a, z, s, t);
+    __syncthreads();
+    adj_fft(z, S::N, LOGN, a.tw, S::T, t);
+#pragma unroll 1
+    for (int k = t; k < S::NBIN; k += S::T) adj_pull_back(z, S::N, k, a.mat[k]);
+    __syncthreads();
+    adj_fft(z, S::N, LOGN, a.tw, S::T, t);
+    // h = conj(F): dL/dw[n] += x[n] Re h[n] + y[n] Im h[n] = x F.x - y F.y
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const int n = t + e * S::T;
+      const float2 F = z[apad(n)];
+      const float g = fmaf(adj_level<BITS>(a.in[0], s * S::N + n), F.x, -adj_level<BITS>(a.in[1], s * S::N + n) * F.y);
+      acc[e] += mine ? g : 0.f;
+    }
+    __syncthreads();
+  }
+  // the teams' sums, in order
+  float* sums = reinterpret_cast<float*>(zs[team]);
+#pragma unroll
+  for (int e = 0; e < 16; ++e) sums[t + e * S::T] = acc[e];
+  __syncthreads();
+  for (int n = threadIdx.x; n < S::N; n += kSmallWindow) {
+    float g = 0.f;
+#pragma unroll 4
+    for (int j = 0; j < S::TEAMS; ++j) g += reinterpret_cast<const float*>(zs[j])[n];
+    a.gpart[(size_t)blockIdx.x * S::N + n] = g;
+  }
 }
 
 struct dc {
@@ -440,7 +548,7 @@ __global__ void __launch_bounds__(kBinsPerBlock * kSlices) k_adj_wsum(const floa
 using namespace polaris;
 
 struct polaris_adj {
-  int N = 0, log2n = 0, nbin = 0, bits = 0, device = 0, threads = 0, grid_max = 0, grid_window = 0, bin_blocks = 0;
+  int N = 0, log2n = 0, nbin = 0, bits = 0, device = 0, threads = 0, nsm = 0, grid_max = 0, grid_window = 0, bin_blocks = 0;
   bool sized = false;  // the size-specialised segment kernels (polaris_adjoint_sized.cu)
   size_t smem = 0;
   unsigned char* d_all = nullptr;  // the device memory of the five below
@@ -501,7 +609,7 @@ extern "C" int polaris_adj_create(int64_t n_fft, int bits, int device, polaris_a
   int prev = 0;
   cudaGetDevice(&prev);
   cudaSetDevice(device);
-  int nsm = 0, occ = 0;
+  int &nsm = h->nsm, occ = 0;
   cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
   // the kernels for any N always (they also take calls whose buffers are not 16-byte
   // aligned), the size-specialised ones where they exist; both forward kernels run on the same grid
@@ -526,6 +634,7 @@ extern "C" int polaris_adj_create(int64_t n_fft, int bits, int device, polaris_a
                    e != cudaSuccess ? cudaGetErrorString(e) : "zero occupancy");
   }
   h->grid_max = nsm * std::min(occ, kMaxCtasPerSm);
+  if (h->log2n < kAdjSizedMin) window_ctas = kSmallWindowCtas;
   h->grid_window = std::max(h->grid_max, nsm * window_ctas);
   // per-pass twiddles of the Stockham passes (radix 16, then 2, 4 or 8): pass with Ns
   // points done and radix R keeps W_{Ns R}^{r k} at r Ns + k - 1 (1 <= r < R, k < Ns); the
@@ -594,8 +703,31 @@ static cudaError_t adj_segments(const AdjArgs& a, size_t smem, bool window_pass,
   return cudaGetLastError();
 }
 
+template <int LOGN, int BITS>
+static cudaError_t adj_small(const AdjArgs& a, bool window_pass, cudaStream_t st) {
+  if (window_pass) return launch_dependent(k_adjm_window<LOGN, BITS>, a.grid, kSmallWindow, 0, st, a);
+  return launch_dependent(k_adjm_forward<LOGN, BITS>, a.grid, kSmallForward, 0, st, a);
+}
+template <int BITS>
+static cudaError_t adj_small_any(const AdjArgs& a, bool window_pass, cudaStream_t st) {
+  switch (a.log2n) {
+    case 5: return adj_small<5, BITS>(a, window_pass, st);
+    case 6: return adj_small<6, BITS>(a, window_pass, st);
+    case 7: return adj_small<7, BITS>(a, window_pass, st);
+    default: return adj_small<8, BITS>(a, window_pass, st);
+  }
+}
+
 static cudaError_t adj_segments_bits(int bits, const AdjArgs& a, size_t smem, bool window_pass, bool sized,
                                      cudaStream_t st) {
+  if (a.log2n < kAdjSizedMin) {
+    switch (bits) {
+      case 1: return adj_small_any<1>(a, window_pass, st);
+      case 2: return adj_small_any<2>(a, window_pass, st);
+      case 4: return adj_small_any<4>(a, window_pass, st);
+      default: return adj_small_any<8>(a, window_pass, st);
+    }
+  }
   if (sized) return adj_sized_launch(a.log2n, bits, window_pass, a, st);
   switch (bits) {
     case 1: return adj_segments<1>(a, smem, window_pass, st);
@@ -658,6 +790,10 @@ extern "C" int polaris_adj_run(polaris_adj* h, const void* const* packed, int64_
   }
   if (e == cudaSuccess && grads) {
     if (sized) a.grid = std::min(a.nseg, h->grid_window);
+    if (h->log2n < kAdjSizedMin) {  // a segment per team
+      const int teams = kSmallWindow * 16 / h->N;
+      a.grid = std::min((a.nseg + teams - 1) / teams, h->nsm * kSmallWindowCtas);
+    }
     e = adj_segments_bits(h->bits, a, h->smem, true, sized, st);
     if (e == cudaSuccess)
       e = launch_dependent(k_adj_wsum, (h->N + kBinsPerBlock - 1) / kBinsPerBlock + 1, kBinsPerBlock * kSlices, 0, st, h->d_gpart,

@@ -40,14 +40,15 @@ __device__ __forceinline__ void adj_bin_gradient(float4 m, float2 Zk, float2 Zm,
   GY = c_add(make_float2(m.y * Y.x, m.y * Y.y), cmul(make_float2(m.z, -m.w), X));
 }
 
-// level of sample idx of one IF
+// level of sample idx of one IF (an ordinary load: a read-only one could be moved up over the wait for
+// the kernel before)
 template <int BITS>
-__device__ __forceinline__ float adj_level(const uint32_t* __restrict__ in, long long idx) {
+__device__ __forceinline__ float adj_level(const uint32_t* in, long long idx) {
   if constexpr (BITS == 8) {
-    return (float)(int)__ldg(reinterpret_cast<const signed char*>(in) + idx);
+    return (float)(int)reinterpret_cast<const signed char*>(in)[idx];
   } else {
     constexpr int SPW = 32 / BITS;
-    return decode_level<BITS>(__ldg(in + idx / SPW), (uint32_t)(idx % SPW) * BITS);
+    return decode_level<BITS>(in[idx / SPW], (uint32_t)(idx % SPW) * BITS);
   }
 }
 

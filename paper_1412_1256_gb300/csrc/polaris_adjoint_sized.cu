@@ -21,7 +21,9 @@
 // What bounds them: latency.  At 2^14 (one CTA of 16 warps per SM) a third of the shared-memory
 // and a quarter of the issue slots are used, the warps wait for the window's and the samples'
 // loads, the exchanges and the barriers; 256 segments on 152 SMs are two rounds, the second two
-// thirds full.  Whole steps, before and after (8-bit): 256 x 2^14 94.7 -> 67.0 us, 700 x 2^13
+// thirds full.  Neither kernel releases its successor early: the blocks of k_adj_bins and
+// k_adj_wsum would gather on the SMs that have no second segment (67.1 us a step instead of 66.0).
+// Whole steps, before and after (8-bit): 256 x 2^14 94.7 -> 66.0 us, 700 x 2^13
 // 112 -> 83, 5000 x 2^10 177 -> 81; 2000 x 2^12 (1 bit) 148 -> 104, 20000 x 2^9 (2 bit) 463 -> 200.
 #include <cuda_runtime.h>
 
@@ -295,7 +297,6 @@ __global__ void __launch_bounds__(AdjPlan<LOGN>::T) k_adjs_forward(AdjArgs a) {
     });
     tmem_wait_st();
   }
-  pdl_trigger();
   float4* part = a.part + (size_t)blockIdx.x * PL::NBIN;
   sfor<0, PL::FCOLS / 16>([&](auto c_) {
     constexpr int cc = decltype(c_)::value;
@@ -389,7 +390,6 @@ __global__ void __launch_bounds__(AdjPlan<LOGN>::T, AdjPlan<LOGN>::CTAS) k_adjs_
     });
     tmem_wait_st();
   }
-  pdl_trigger();
   float* gpart = a.gpart + (size_t)blockIdx.x * N + tid;
   sfor<0, PL::PPT / 16>([&](auto h_) {
     constexpr int h = decltype(h_)::value;

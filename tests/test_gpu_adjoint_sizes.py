@@ -42,3 +42,35 @@ def test_sized_kernels_equal_general_ones(logn, bits):
         for key in b:
             x, y = a[key].double(), b[key].double()
             assert float((x - y).norm()) <= 1e-5 * float(y.norm()), (nseg, key)
+
+
+@pytest.mark.parametrize("logn", [5, 6, 7, 8])
+@pytest.mark.parametrize("bits", [1, 2, 4, 8])
+def test_small_sizes_equal_oracle(orc, logn, bits):
+    """N = 2^5 to 2^8 (many segments per CTA) against the FP64 oracle: one segment, a few, one more than the
+    groups of the forward pass (eight per SM), and several rounds of a CTA's teams with a ragged end.
+    The bound is the one above (one side is exact here)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1412_1256_gb300 import polaris
+
+    n_fft, nb = 1 << logn, (1 << logn) // 2 + 1
+    groups = 8 * torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(100 * logn + bits)
+    window = rng.uniform(0.2, 1.0, n_fft).astype(np.float32)
+    gains = np.array([1.1, 0.2, 0.9, -0.3], np.float32)
+    leak = rng.uniform(-0.03, 0.03, (2, nb, 2)).astype(np.float32)
+    target = np.zeros((4, nb), np.float32)
+    dev = [torch.from_numpy(x).cuda() for x in (window, gains, leak, target)]
+    for nseg in (1, 3, groups + 1, 5 * groups + 7):
+        n = nseg * n_fft
+        host = [rng.integers(0, 2**32, n * bits // 32, dtype=np.uint32) for _ in range(2)]
+        st, loss = orc.leak_forward(host, bits, n_fft, n, window, gains, leak, target)
+        gw, gg, gd = orc.leak_grad(host, bits, n_fft, n, window, gains, leak, target)
+        with polaris.Adjoint(n_fft, bits) as adj:
+            r = adj.run([torch.from_numpy(h.view(np.int32)).cuda() for h in host], n, *dev, grads=True)
+            torch.cuda.synchronize()
+        for key, ref in (("stokes", st), ("loss", loss), ("grad_window", gw), ("grad_gains", gg), ("grad_leak", gd)):
+            x, y = r[key].cpu().numpy().astype(np.float64).ravel(), np.asarray(ref, np.float64).ravel()
+            assert np.linalg.norm(x - y) <= 1e-5 * np.linalg.norm(y), (nseg, key)
