@@ -34,7 +34,8 @@
 //                  radix-16 Stockham transform of the pair x + i y in shared memory, split
 //                  into X and Y, per-CTA partial sums of |X|^2, |Y|^2, X conj(Y)
 //                  (N = 2^9 .. 2^14: k_adjs_forward, the same per size at compile time,
-//                  polaris_adjoint_sized.cu; likewise k_adjs_window)
+//                  polaris_adjoint_sized.cu; likewise k_adjs_window; k_adjs_teams,
+//                  polaris_adjoint_teams.cu, where there are more segments than SMs)
 //   k_adj_bins     per bin: partials summed (fp32 slices, added in fp64), the model,
 //                  Stokes and loss in fp64, the gain and leakage gradients and the
 //                  window-adjoint matrix in fp32

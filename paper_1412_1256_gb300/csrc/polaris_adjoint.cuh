@@ -60,5 +60,10 @@ __device__ __forceinline__ float adj_level(const uint32_t* in, long long idx) {
 constexpr int kAdjSizedMin = 9, kAdjSizedMax = 14;
 cudaError_t adj_sized_prepare(int log2n, int bits, int* window_ctas);
 cudaError_t adj_sized_launch(int log2n, int bits, bool window_pass, const AdjArgs& a, cudaStream_t st);
+// the forward kernel for more segments than CTAs (polaris_adjoint_teams.cu), up to 2^kAdjTeamsMax points
+// (above, two teams' points do not fit an SM)
+constexpr int kAdjTeamsMax = 12;
+cudaError_t adj_teams_prepare(int log2n, int bits);
+cudaError_t adj_teams_launch(int log2n, int bits, const AdjArgs& a, cudaStream_t st);
 
 }  // namespace polaris
