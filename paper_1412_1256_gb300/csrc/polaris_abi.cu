@@ -1544,7 +1544,11 @@ extern "C" int spectrometer_run_noalloc(const polaris_config* cfg, const void* c
   for (int64_t s0 = 0; s0 < nseg; s0 += pass) {
     a.seg0 = (int)s0;
     a.nseg = (int)(nseg - s0 < pass ? nseg - s0 : pass);
-    for (int ph = 0; ph < (is_fused(logn) ? 1 : 2) && e == cudaSuccess; ++ph) e = kPhases[logn][ph](a, st, true);
+    // The first kernel is an ordinary launch: the kernels just queued write the twiddles, which it may
+    // read before its wait, and the taps, which it reads by read-only loads.  (A handle's tables are
+    // complete before its first feed.)
+    for (int ph = 0; ph < (is_fused(logn) ? 1 : 2) && e == cudaSuccess; ++ph)
+      e = kPhases[logn][ph](a, st, s0 > 0 || ph > 0);
     if (e != cudaSuccess) return set_err(nullptr, POLARIS_ECUDA, "no-alloc FFT-correlator: %s", cudaGetErrorString(e));
   }
   // readout (same kernel as spectrometer_integrate_device)
