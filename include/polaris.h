@@ -82,7 +82,8 @@ typedef struct polaris_spec polaris_spec; /* opaque, library-owned */
  *   max_batch_segments  segments processed per kernel pass (bounds the device
  *               scratch: 2 * max_batch_segments * n_fft * 8 bytes per pair);
  *               0 selects the default (passes of at least 64 segments).  n_fft of
- *               1024 to 16384 run in one kernel without scratch, whatever the value.
+ *               1024 to 16384 run in one kernel without scratch, whatever the value
+ *               (with FP64 accumulators it adds to them every 14 segments or sooner).
  *   code_stats  1: also count, per IF, how often each b-bit code occurs in the
  *               segments that feed() integrates (the bit distribution used for
  *               total-power measurement, Sec. 2 and Sec. 3.2.2); read with

@@ -16,6 +16,13 @@
 //            component; |X|^2, |Y|^2 and X conj(Y) (as in k_phase2) accumulate in tensor memory
 //            over the range.  At the end the CTA's teams are summed in shared memory and added
 //            once to the integration accumulators, which hold the bins in natural order.
+//            FP64 accumulators: every `flush` segments instead, the teams summed in twice FP32's
+//            precision, so that the sums do not lose bits as a feed gets longer.  The lengths are those of
+//            the two-kernel path's ranges (a pass of 4096 segments over its warps).  Passes of four 2-bit IFs
+//            of 8 M samples with one addition at the end and so: 2^10 33.1, 37.5 us; 2^11 40.2, 40.2; 2^12
+//            50.3, 50.7; 2^13 68.2, 51.3; 2^14 81.4, 60.0 (FP32 accumulators: 30.8 to 51.6): the last ones
+//            from consecutive lanes adding consecutive values and from fewer FP64 instructions, which
+//            bound this part (teams summed in FP64: 2^25 samples of one pair at 2^10 314 us, now 157).
 //
 // What bounds it: instruction issue, about 40 to 43 instructions per complex point, of which 14
 // packed FP32, at 45 to 50% of the issue slots with 16 warps per SM (registers), against 64 of the
@@ -48,6 +55,8 @@ struct FusedPlan {
   static constexpr int REGION = R * PITCH;              // float2 per team
   static constexpr int TW2 = THREE ? B : 0;             // W_B^{b0 d1} at 16 d1 + b0
   static constexpr int TCOLS = (WARPS / 4) * 128;       // 64 accumulator and 64 twiddle columns per lane
+  // FP64 accumulators: segments per FFT pair (14 at most) that a team sums in FP32 before it adds to them
+  static constexpr int FLUSH = LOGN == 10 ? 2 : LOGN == 11 ? 4 : LOGN == 12 ? 7 : 14;
   template <int BITS>
   struct In {
     static constexpr int SPW = 32 / BITS;
@@ -77,13 +86,29 @@ struct FusedPlan {
   static_assert(!THREE || (PITCH >= 17 * P1 && (LC == 16 || (PITCH % LC == 0 && PITCH / LC % 2 == 1))), "column rows");
 };
 
+// hi + lo += x, the rounding error of the sum (Knuth's TwoSum) kept in lo
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
+  const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+  hi = s;
+}
+
+// x in FP64, by integer operations: FP64 ones, the conversion among them, take a scheduler 64 cycles a warp
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), e = b & 0x7F800000u;
+  if (e == 0x7F800000u || (e == 0 && x != 0.f)) return (double)x;  // infinite, NaN, denormal
+  const uint32_t h = (b & 0x80000000u) | (x != 0.f ? ((b & 0x7FFFFFFFu) >> 3) + 0x38000000u : 0u);
+  return __hiloint2double((int)h, (int)(b << 29));
+}
+
 template <int W>
 __device__ __forceinline__ void team_sync(int team) {
   if constexpr (W == 1) __syncwarp();
   else asm volatile("bar.sync %0, %1;\n" ::"r"(1 + team), "r"(32 * W) : "memory");
 }
 
-template <int LOGN, int BITS>
+// FP64: the integration accumulators are doubles
+template <int LOGN, int BITS, bool FP64>
 __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MINB) k_fused(BatchArgs a) {
   using PL = FusedPlan<LOGN>;
   using IN = typename PL::template In<BITS>;
@@ -192,188 +217,207 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
     team_sync<W>(team);
     if (s_begin + G < s_end) issue(s_begin + G);
   }
-  int g = 0;
+  // rounds: one; with FP64 accumulators as many as keep a team's FP32 sums to `flush` segments
+  const int flush = min(14, PL::FLUSH * a.n_fpair);
+  const int rounds = FP64 ? (int)(((a.nseg + teams - 1) / teams + flush - 1) / flush) : 1;
+  int g = 0, s = s_begin;
 #pragma unroll 1
-  for (int s = s_begin; s < s_end; ++s) {
-    const bool turn = g == G - 1 && s + 1 < s_end;  // the next segment starts a group
-    // step A: decode column tl, window, 32-point DFT
-    float2 v[32];
-    uint32_t cw[IN::VW];
-    const uint32_t* col = tr + g * IN::TR + (tl + tl / IN::PADC) * VL;
-    sfor<0, IN::VW / VL>([&](auto q_) {
-      constexpr int q = decltype(q_)::value;
-      if constexpr (VL == 4) {
-        const uint4 x = *reinterpret_cast<const uint4*>(col + q * IN::SLAB);
-        cw[4 * q] = x.x;
-        cw[4 * q + 1] = x.y;
-        cw[4 * q + 2] = x.z;
-        cw[4 * q + 3] = x.w;
-      } else {
-        const uint2 x = *reinterpret_cast<const uint2*>(col + q * IN::SLAB);
-        cw[2 * q] = x.x;
-        cw[2 * q + 1] = x.y;
-      }
-    });
-    auto rows = [&](auto hb_, auto tp_) {
-      constexpr bool HBP = decltype(hb_)::value, TP = decltype(tp_)::value;
-      [[maybe_unused]] const float4* tp = reinterpret_cast<const float4*>(a.taps) + tl;
-      [[maybe_unused]] float4 w4;
-      sfor<0, 32>([&](auto t_) {
-        constexpr int t = decltype(t_)::value;
-        float2 z = code_pair<BITS, t % SPW>(cw[t / SPW], cw[IN::VW / 2 + t / SPW]);
-        if constexpr (!HBP) z.y = 0.f;
-        if constexpr (TP) {  // (four consecutive t per load: tap_order)
-          if constexpr (t % 4 == 0) w4 = __ldg(tp + (t / 4) * B);
-          const float x = t % 4 == 0 ? w4.x : t % 4 == 1 ? w4.y : t % 4 == 2 ? w4.z : w4.w;
-          z = __fmul2_rn(z, make_float2(x, x));
-        }
-        v[ct::bitrev(t, 32)] = z;
-      });
-    };
-    using T_ = std::true_type;
-    using F_ = std::false_type;
-    if (a.taps) {
-      if (ib >= 0) rows(T_{}, T_{});
-      else rows(F_{}, T_{});
-    } else {
-      if (ib >= 0) rows(T_{}, F_{});
-      else rows(F_{}, F_{});
-    }
-    dit<32>(v);
-    sfor<0, 4>([&](auto c_) {
-      constexpr int cc = decltype(c_)::value;
-      float w16[16];
-      tmem_ld16(t_tw + 16 * cc, w16);
-      tmem_wait_ld();
-      sfor<0, 8>([&](auto k_) {
-        constexpr int k = decltype(k_)::value, i = 8 * cc + k;
-        if constexpr (i > 0) v[i] = cmul(v[i], make_float2(w16[2 * k], w16[2 * k + 1]));
-      });
-    });
-    if (turn) cp_async_wait_all();
-    team_sync<W>(team);  // the previous exchange and this group's codes have been read; the next group is staged
-    sfor<0, 32>([&](auto i_) {
-      constexpr int i = decltype(i_)::value;
-      region[i * PITCH + tl] = v[i];
-    });
-    if (turn) transpose(min(G, s_end - s - 1));
-    team_sync<W>(team);
-    if (turn && s + 1 + G < s_end) issue(s + 1 + G);
-    // B-point DFT of column cb
-    float2* row = region + cb * PITCH;
-    if constexpr (THREE) {
-      sfor<0, 32 / P1>([&](auto j_) {
-        constexpr int j = decltype(j_)::value;
-        sfor<0, P1>([&](auto i_) {
-          constexpr int i = decltype(i_)::value;
-          v[j * P1 + ct::bitrev(i, P1)] = row[16 * i + l + LC * j];
-        });
-        dit<P1, j * P1>(v);
-        sfor<1, P1>([&](auto i_) {
-          constexpr int i = decltype(i_)::value;
-          v[j * P1 + i] = cmul(v[j * P1 + i], tw2[16 * i + l + LC * j]);
-        });
-      });
-      __syncwarp();  // the column's row has been read
-      sfor<0, 32>([&](auto i_) {
-        constexpr int i = decltype(i_)::value;
-        row[17 * (i % P1) + l + LC * (i / P1)] = v[i];
-      });
-      __syncwarp();
-      sfor<0, 2>([&](auto s_) {
-        constexpr int sl = decltype(s_)::value;
-        const float2* src = row + 17 * (sl ? P1 - 1 - l : l);
-        sfor<0, 16>([&](auto i_) {
-          constexpr int i = decltype(i_)::value;
-          v[16 * sl + ct::bitrev(i, 16)] = src[i];
-        });
-        dit<16, 16 * sl>(v);
-      });
-    } else {
-      sfor<0, 32>([&](auto i_) {
-        constexpr int i = decltype(i_)::value;
-        if constexpr (HB == 1) {
-          v[ct::bitrev(i, 32)] = row[i];
+  for (int left = rounds; left > 0; --left) {
+    const int s_stop = FP64 && left > 1 ? min(s + flush, s_end) : s_end;
+#pragma unroll 1
+    for (; s < s_stop; ++s) {
+      const bool turn = g == G - 1 && s + 1 < s_end;  // the next segment starts a group
+      // step A: decode column tl, window, 32-point DFT
+      float2 v[32];
+      uint32_t cw[IN::VW];
+      const uint32_t* col = tr + g * IN::TR + (tl + tl / IN::PADC) * VL;
+      sfor<0, IN::VW / VL>([&](auto q_) {
+        constexpr int q = decltype(q_)::value;
+        if constexpr (VL == 4) {
+          const uint4 x = *reinterpret_cast<const uint4*>(col + q * IN::SLAB);
+          cw[4 * q] = x.x;
+          cw[4 * q + 1] = x.y;
+          cw[4 * q + 2] = x.z;
+          cw[4 * q + 3] = x.w;
         } else {
-          float2 z = __ffma2_rn(row[i + 32], make_float2(sgn_b, sgn_b), row[i]);
-          const float2 zt = turn64<i>(z);
-          z.x = hb ? zt.x : z.x;
-          z.y = hb ? zt.y : z.y;
-          v[ct::bitrev(i, 32)] = z;
+          const uint2 x = *reinterpret_cast<const uint2*>(col + q * IN::SLAB);
+          cw[2 * q] = x.x;
+          cw[2 * q + 1] = x.y;
         }
       });
+      auto rows = [&](auto hb_, auto tp_) {
+        constexpr bool HBP = decltype(hb_)::value, TP = decltype(tp_)::value;
+        [[maybe_unused]] const float4* tp = reinterpret_cast<const float4*>(a.taps) + tl;
+        [[maybe_unused]] float4 w4;
+        sfor<0, 32>([&](auto t_) {
+          constexpr int t = decltype(t_)::value;
+          float2 z = code_pair<BITS, t % SPW>(cw[t / SPW], cw[IN::VW / 2 + t / SPW]);
+          if constexpr (!HBP) z.y = 0.f;
+          if constexpr (TP) {  // (four consecutive t per load: tap_order)
+            if constexpr (t % 4 == 0) w4 = __ldg(tp + (t / 4) * B);
+            const float x = t % 4 == 0 ? w4.x : t % 4 == 1 ? w4.y : t % 4 == 2 ? w4.z : w4.w;
+            z = __fmul2_rn(z, make_float2(x, x));
+          }
+          v[ct::bitrev(t, 32)] = z;
+        });
+      };
+      using T_ = std::true_type;
+      using F_ = std::false_type;
+      if (a.taps) {
+        if (ib >= 0) rows(T_{}, T_{});
+        else rows(F_{}, T_{});
+      } else {
+        if (ib >= 0) rows(T_{}, F_{});
+        else rows(F_{}, F_{});
+      }
       dit<32>(v);
-    }
-    // correlate this lane's 16 bins k < N/2: k = cb + 32 d, d = HB i + hb, i < 16, or
-    // d = d1 + P1 d0, d0 < 8, for the lane's two d1 (i = 8 slot + d0)
-    auto correlate = [&](auto sp_) {
-      constexpr bool SP = decltype(sp_)::value;  // the warp holds column 0
       sfor<0, 4>([&](auto c_) {
         constexpr int cc = decltype(c_)::value;
-        float a16[16];
-        tmem_ld16(t_acc + 16 * cc, a16);
+        float w16[16];
+        tmem_ld16(t_tw + 16 * cc, w16);
         tmem_wait_ld();
-        sfor<0, 4>([&](auto k_) {
-          constexpr int k = decltype(k_)::value, i = 4 * cc + k;
-          constexpr int sl = THREE ? i / 8 : 0, d0 = i % 8;
-          constexpr int own = THREE ? 16 * sl + d0 : i, far = THREE ? 16 * (sl ^ 1) + 15 - d0 : 31 - i;
-          const int from = !THREE ? partner : sl ? partner1 : partner0;
-          float2 z = make_float2(__shfl_sync(0xffffffffu, v[far].x, from), __shfl_sync(0xffffffffu, v[far].y, from));
-          if constexpr (SP) {  // the bins that mirror onto their own lane's outputs
-            constexpr int near = THREE ? (sl ? 16 + 15 - d0 : (16 - d0) % 16) : (32 - i) % 32;
-            const bool me = sl ? self1 : self;
-            z.x = me ? v[near].x : z.x;
-            z.y = me ? v[near].y : z.y;
-          }
-          float(&q)[4] = *reinterpret_cast<float(*)[4]>(a16 + 4 * k);
-          corr_acc(q, v[own], make_float2(z.x, -z.y));
+        sfor<0, 8>([&](auto k_) {
+          constexpr int k = decltype(k_)::value, i = 8 * cc + k;
+          if constexpr (i > 0) v[i] = cmul(v[i], make_float2(w16[2 * k], w16[2 * k + 1]));
         });
-        tmem_st16(t_acc + 16 * cc, a16);
       });
-    };
-    if (W == 1 || wt == 0) correlate(std::true_type{});
-    else correlate(std::false_type{});
-    tmem_wait_st();
-    if (self) {  // bin N/2, its own mirror
-      constexpr int i = THREE ? 8 : 16;
-      corr_acc(extra, v[i], make_float2(v[i].x, -v[i].y));
+      if (turn) cp_async_wait_all();
+      team_sync<W>(team);  // the previous exchange and this group's codes have been read; the next group is staged
+      sfor<0, 32>([&](auto i_) {
+        constexpr int i = decltype(i_)::value;
+        region[i * PITCH + tl] = v[i];
+      });
+      if (turn) transpose(min(G, s_end - s - 1));
+      team_sync<W>(team);
+      if (turn && s + 1 + G < s_end) issue(s + 1 + G);
+      // B-point DFT of column cb
+      float2* row = region + cb * PITCH;
+      if constexpr (THREE) {
+        sfor<0, 32 / P1>([&](auto j_) {
+          constexpr int j = decltype(j_)::value;
+          sfor<0, P1>([&](auto i_) {
+            constexpr int i = decltype(i_)::value;
+            v[j * P1 + ct::bitrev(i, P1)] = row[16 * i + l + LC * j];
+          });
+          dit<P1, j * P1>(v);
+          sfor<1, P1>([&](auto i_) {
+            constexpr int i = decltype(i_)::value;
+            v[j * P1 + i] = cmul(v[j * P1 + i], tw2[16 * i + l + LC * j]);
+          });
+        });
+        __syncwarp();  // the column's row has been read
+        sfor<0, 32>([&](auto i_) {
+          constexpr int i = decltype(i_)::value;
+          row[17 * (i % P1) + l + LC * (i / P1)] = v[i];
+        });
+        __syncwarp();
+        sfor<0, 2>([&](auto s_) {
+          constexpr int sl = decltype(s_)::value;
+          const float2* src = row + 17 * (sl ? P1 - 1 - l : l);
+          sfor<0, 16>([&](auto i_) {
+            constexpr int i = decltype(i_)::value;
+            v[16 * sl + ct::bitrev(i, 16)] = src[i];
+          });
+          dit<16, 16 * sl>(v);
+        });
+      } else {
+        sfor<0, 32>([&](auto i_) {
+          constexpr int i = decltype(i_)::value;
+          if constexpr (HB == 1) {
+            v[ct::bitrev(i, 32)] = row[i];
+          } else {
+            float2 z = __ffma2_rn(row[i + 32], make_float2(sgn_b, sgn_b), row[i]);
+            const float2 zt = turn64<i>(z);
+            z.x = hb ? zt.x : z.x;
+            z.y = hb ? zt.y : z.y;
+            v[ct::bitrev(i, 32)] = z;
+          }
+        });
+        dit<32>(v);
+      }
+      // correlate this lane's 16 bins k < N/2: k = cb + 32 d, d = HB i + hb, i < 16, or
+      // d = d1 + P1 d0, d0 < 8, for the lane's two d1 (i = 8 slot + d0)
+      auto correlate = [&](auto sp_) {
+        constexpr bool SP = decltype(sp_)::value;  // the warp holds column 0
+        sfor<0, 4>([&](auto c_) {
+          constexpr int cc = decltype(c_)::value;
+          float a16[16];
+          tmem_ld16(t_acc + 16 * cc, a16);
+          tmem_wait_ld();
+          sfor<0, 4>([&](auto k_) {
+            constexpr int k = decltype(k_)::value, i = 4 * cc + k;
+            constexpr int sl = THREE ? i / 8 : 0, d0 = i % 8;
+            constexpr int own = THREE ? 16 * sl + d0 : i, far = THREE ? 16 * (sl ^ 1) + 15 - d0 : 31 - i;
+            const int from = !THREE ? partner : sl ? partner1 : partner0;
+            float2 z = make_float2(__shfl_sync(0xffffffffu, v[far].x, from), __shfl_sync(0xffffffffu, v[far].y, from));
+            if constexpr (SP) {  // the bins that mirror onto their own lane's outputs
+              constexpr int near = THREE ? (sl ? 16 + 15 - d0 : (16 - d0) % 16) : (32 - i) % 32;
+              const bool me = sl ? self1 : self;
+              z.x = me ? v[near].x : z.x;
+              z.y = me ? v[near].y : z.y;
+            }
+            float(&q)[4] = *reinterpret_cast<float(*)[4]>(a16 + 4 * k);
+            corr_acc(q, v[own], make_float2(z.x, -z.y));
+          });
+          tmem_st16(t_acc + 16 * cc, a16);
+        });
+      };
+      if (W == 1 || wt == 0) correlate(std::true_type{});
+      else correlate(std::false_type{});
+      tmem_wait_st();
+      if (self) {  // bin N/2, its own mirror
+        constexpr int i = THREE ? 8 : 16;
+        corr_acc(extra, v[i], make_float2(v[i].x, -v[i].y));
+      }
+      g = turn ? 0 : g + 1;
     }
-    g = turn ? 0 : g + 1;
-  }
-  pdl_trigger();
-  // the CTA's teams summed in shared memory, then one add per bin (natural order; copy by CTA)
-  team_sync<W>(team);
-  float4* sums = reinterpret_cast<float4*>(region);
-  sfor<0, 4>([&](auto c_) {
-    constexpr int cc = decltype(c_)::value;
-    float a16[16];
-    tmem_ld16(t_acc + 16 * cc, a16);
-    tmem_wait_ld();
-    sfor<0, 4>([&](auto k_) {
-      constexpr int k = decltype(k_)::value, i = 4 * cc + k;
-      const int d = THREE ? (i / 8 ? P1 - 1 - l : l) + P1 * (i % 8) : HB * i + hb;
-      sums[cb + 32 * d] = make_float4(a16[4 * k], a16[4 * k + 1], a16[4 * k + 2], a16[4 * k + 3]);
+    if (!FP64 || left == 1) pdl_trigger();
+    // the CTA's teams summed in shared memory, then one add per bin (natural order; copy by CTA)
+    team_sync<W>(team);
+    float4* sums = reinterpret_cast<float4*>(region);
+    sfor<0, 4>([&](auto c_) {
+      constexpr int cc = decltype(c_)::value;
+      float a16[16];
+      tmem_ld16(t_acc + 16 * cc, a16);
+      tmem_wait_ld();
+      sfor<0, 4>([&](auto k_) {
+        constexpr int k = decltype(k_)::value, i = 4 * cc + k;
+        const int d = THREE ? (i / 8 ? P1 - 1 - l : l) + P1 * (i % 8) : HB * i + hb;
+        sums[cb + 32 * d] = make_float4(a16[4 * k], a16[4 * k + 1], a16[4 * k + 2], a16[4 * k + 3]);
+      });
+      if (FP64 && left > 1) {
+        sfor<0, 16>([&](auto i_) { a16[decltype(i_)::value] = 0.f; });
+        tmem_st16(t_acc + 16 * cc, a16);
+      }
     });
-  });
-  if (self) xbin[team] = make_float4(extra[0], extra[1], extra[2], extra[3]);
-  __syncthreads();
-  const size_t base = ((size_t)(a.acc_copies > 1 ? slot % a.acc_copies : 0) * a.n_fpair + f) * (PL::N / 2 + 1);
-  for (int k = tid; k <= PL::N / 2; k += PL::THREADS) {
-    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int q = 0; q < T; ++q) {
-      const float4 x = k == PL::N / 2 ? xbin[q] : reinterpret_cast<const float4*>(smf + q * IN::TEAM)[k];
-      t = make_float4(t.x + x.x, t.y + x.y, t.z + x.z, t.w + x.w);
+    if (self) xbin[team] = make_float4(extra[0], extra[1], extra[2], extra[3]);
+    __syncthreads();
+    const size_t base = ((size_t)(a.acc_copies > 1 ? slot % a.acc_copies : 0) * a.n_fpair + f) * (PL::N / 2 + 1);
+    if constexpr (!FP64) {
+      for (int k = tid; k <= PL::N / 2; k += PL::THREADS) {
+        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int q = 0; q < T; ++q) {
+          const float4 x = k == PL::N / 2 ? xbin[q] : reinterpret_cast<const float4*>(smf + q * IN::TEAM)[k];
+          t = make_float4(t.x + x.x, t.y + x.y, t.z + x.z, t.w + x.w);
+        }
+        const size_t o = base + k;
+        if (in_bounds(a.err, (long long)o, a.acc_slots)) atomicAdd(reinterpret_cast<float4*>(a.acc) + o, t);
+      }
+    } else {  // consecutive lanes take consecutive values
+      double* op = reinterpret_cast<double*>(a.acc) + 4 * base;
+      for (int k = tid; k < 4 * (PL::N / 2 + 1); k += PL::THREADS) {
+        float hi = 0.f, lo = 0.f;  // their sum, to twice 24 bits
+        for (int q = 0; q < T; ++q)
+          two_sum(hi, lo, k >= 2 * PL::N ? reinterpret_cast<const float*>(xbin + q)[k - 2 * PL::N]
+                                         : reinterpret_cast<const float*>(smf + q * IN::TEAM)[k]);
+        const double t = T == 1 || lo != lo ? widen(hi) : widen(hi) + widen(lo);  // (lo: NaN where hi is infinite)
+        if (in_bounds(a.err, (long long)base + k / 4, a.acc_slots)) atomicAdd(op + k, t);
+      }
     }
-    const size_t o = base + k;
-    if (!in_bounds(a.err, (long long)o, a.acc_slots)) continue;
-    if (!a.fp64) {
-      atomicAdd(reinterpret_cast<float4*>(a.acc) + o, t);
-    } else {
-      double* op = reinterpret_cast<double*>(a.acc) + 4 * o;
-      atomicAdd(op + 0, (double)t.x);
-      atomicAdd(op + 1, (double)t.y);
-      atomicAdd(op + 2, (double)t.z);
-      atomicAdd(op + 3, (double)t.w);
+    if (FP64 && left > 1) {
+      for (int i = 0; i < 4; ++i) extra[i] = 0.f;
+      tmem_wait_st();
+      __syncthreads();  // the sums have been read: the teams' regions take the next exchange
     }
   }
   cta_tmem_end<PL::TCOLS>(tbase, warp);
@@ -381,8 +425,8 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
 
 // One launch per feed: CTAs in equal numbers per FFT pair, as many as fit and have a segment per
 // team.
-template <int LOGN, int BITS>
-static cudaError_t launch_fused(const BatchArgs& a, cudaStream_t st, bool pdl) {
+template <int LOGN, int BITS, bool FP64>
+static cudaError_t launch_fused_acc(const BatchArgs& a, cudaStream_t st, bool pdl) {
   using PL = FusedPlan<LOGN>;
   constexpr size_t smem = PL::template In<BITS>::SMEM;
   static int attr_dev = -1, per_sm = 1;
@@ -390,9 +434,9 @@ static cudaError_t launch_fused(const BatchArgs& a, cudaStream_t st, bool pdl) {
   cudaGetDevice(&dev);
   if (attr_dev != dev) {
     const cudaError_t e =
-        cudaFuncSetAttribute(k_fused<LOGN, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_fused<LOGN, BITS, FP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    per_sm = ctas_per_sm(k_fused<LOGN, BITS>, PL::THREADS, smem, PL::TCOLS);
+    per_sm = ctas_per_sm(k_fused<LOGN, BITS, FP64>, PL::THREADS, smem, PL::TCOLS);
     attr_dev = dev;
   }
   int eff = per_sm;
@@ -412,7 +456,12 @@ static cudaError_t launch_fused(const BatchArgs& a, cudaStream_t st, bool pdl) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_fused<LOGN, BITS>, a);
+  return cudaLaunchKernelEx(&cfg, k_fused<LOGN, BITS, FP64>, a);
+}
+
+template <int LOGN, int BITS>
+static cudaError_t launch_fused(const BatchArgs& a, cudaStream_t st, bool pdl) {
+  return a.fp64 ? launch_fused_acc<LOGN, BITS, true>(a, st, pdl) : launch_fused_acc<LOGN, BITS, false>(a, st, pdl);
 }
 
 template <int LOGN>
