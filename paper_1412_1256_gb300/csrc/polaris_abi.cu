@@ -359,6 +359,10 @@ static int host_plan_n2(int logn) { return 1 << (is_fused(logn) ? fused_log_b(lo
 // entries of the twiddle table W_N^{b u}, b < N2: u <= N1/2 (the units of phase 2), or, where one
 // kernel does both phases, every u < N1
 static int host_tw_rows(int logn, int n1) { return is_fused(logn) ? n1 : n1 / 2 + 1; }
+// Rows u > N1/2 of the table (one kernel): what k_fused multiplies the conjugated column u by, the twiddles
+// of its mirror, W_N^{b (N1 - u)}, negated at odd b
+__host__ __device__ static int tw_unit(int u, int n1) { return u > n1 / 2 ? n1 - u : u; }
+__host__ __device__ static double tw_sign(int b, int u, int n1) { return u > n1 / 2 && (b & 1) ? -1.0 : 1.0; }
 // Accumulator copies K.  At small N many warps (or, in the one-kernel path, CTAs) add into the
 // same few slots, and adds to one address are served one after another: each adds into copy
 // (its range or CTA) mod K instead, about 64 adds per copy, and the readout sums the copies.
@@ -725,9 +729,9 @@ extern "C" int spectrometer_create(const polaris_config* cfg, polaris_spec** out
   std::vector<float2> tw((size_t)s->N2 * host_tw_rows(logn, s->N1));
   for (int b = 0; b < s->N2; ++b)
     for (int u = 0; u < host_tw_rows(logn, s->N1); ++u) {
-      const int64_t e = ((int64_t)b * u) % N;
-      const double ang = -2.0 * M_PI * (double)e / (double)N;
-      tw[(size_t)u * s->N2 + b] = make_float2((float)std::cos(ang), (float)std::sin(ang));
+      const int64_t e = ((int64_t)b * tw_unit(u, s->N1)) % N;
+      const double ang = -2.0 * M_PI * (double)e / (double)N, sg = tw_sign(b, u, s->N1);
+      tw[(size_t)u * s->N2 + b] = make_float2((float)(sg * std::cos(ang)), (float)(sg * std::sin(ang)));
     }
   cudaError_t e = cudaMemcpy(s->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice);
   if (e == cudaSuccess && c.window != POLARIS_WIN_RECT) {
@@ -1336,16 +1340,17 @@ static const int kNoallocMaxDevices = 64;
 static void* g_noalloc_ptr[kNoallocMaxDevices] = {nullptr};
 static std::mutex g_noalloc_mu;
 
-// twiddles W_N^{b u} (b < N2, u < rows) in FP64, rounded once to f32, unit-major ([u][b])
+// twiddles W_N^{b u} (b < N2, u < rows; tw_unit, tw_sign) in FP64, rounded once to f32, unit-major ([u][b])
 __global__ void k_noalloc_twiddles(float2* tw, int N2, int rows, long long N) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long total = (long long)N2 * rows;
   if (i >= total) return;
-  const long long u = i / N2, b = i % N2;
-  const long long e = (b * u) % N;
+  const int u = (int)(i / N2), b = (int)(i % N2), n1 = (int)(N / N2);
+  const long long e = ((long long)b * tw_unit(u, n1)) % N;
+  const double sg = tw_sign(b, u, n1);
   double s, c;
   sincospi(-2.0 * (double)e / (double)N, &s, &c);
-  tw[i] = make_float2((float)c, (float)s);
+  tw[i] = make_float2((float)(sg * c), (float)(sg * s));
 }
 
 // periodic Hann taps 0.5 - 0.5 cos(2 pi n / N), in tap_order

@@ -12,10 +12,11 @@
 //                    the odd half turned by W_64^i)
 //              2^12+ B = 16 P1: P1-point DFTs over b1 (b = 16 b1 + b0), W_B^{b0 d1}, an exchange
 //                    among the P1/2 lanes of the column, 16-point DFTs over b0 (d = d1 + P1 d0)
-//            A bin and its mirror (column 32 - c, in the same warp) meet by one shuffle per
-//            component; |X|^2, |Y|^2 and X conj(Y) (as in k_phase2) accumulate in tensor memory
-//            over the range.  At the end the CTA's teams are summed in shared memory and added
-//            once to the integration accumulators, which hold the bins in natural order.
+//            A bin and its mirror (column 32 - c, in the same warp, conjugated and taken through
+//            column c's own twiddles) meet by one shuffle per component; |X|^2, |Y|^2 and X conj(Y)
+//            (as in k_phase2) accumulate in tensor memory over the range.  At the end the CTA's teams
+//            are summed in shared memory and added once to the integration accumulators, which hold
+//            the bins in natural order.
 //            FP64 accumulators: every `flush` segments instead, the teams summed in twice FP32's
 //            precision, so that the sums do not lose bits as a feed gets longer.  The lengths are those of
 //            the two-kernel path's ranges (a pass of 4096 segments over its warps).  Passes of four 2-bit IFs
@@ -133,14 +134,21 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
   const int hb = HB == 2 ? (lane >> 3) & 1 : 0, l = THREE ? lane % LC : 0;
   const int u = THREE ? (16 / LC) * wt + (lane & 15) / LC : HB == 2 ? 8 * wt + (lane & 7) : lane & 15;
   const int cb = u == 0 ? (mir ? 16 : 0) : (mir ? 32 - u : u);
-  // the lanes that hold this lane's mirror bins.  Two steps: output 31 - i of `partner` mirrors output
+  // Columns u and 32 - u, 0 < u < 16: column 32 - u goes conjugated through column u's twiddles and
+  // transform, its odd b negated, so that its output d is conj Z[N - k] of bin k = u + 32 (d + B/2 mod B): a
+  // lane and its `partner` hold bins and mirrors at d and d + B/2, and each two of them have had the same
+  // operations.  Both columns by their own twiddles leaked the rounding of the transform's constants
+  // from X into Y: cross spectra of 2^25 samples 1.5e-8 to 2.1e-8 rms off, of sqrt(A_x A_y), 4.5e-9 to
+  // 6.0e-9 so; time within 2%, 2^10 4 bits 3%.
+  // Columns 0 and 16 hold their own mirrors.  Two steps: output 31 - i of `partner` mirrors output
   // i; column 0's even outputs mirror onto themselves (output (32 - i) mod 32 of the lane itself).
   // Three: a lane holds d1 = l (slot 0) and P1 - 1 - l (slot 1); the mirror of (slot, d0) is the other
-  // slot's 15 - d0 in the same lane of column 32 - c; in column 0 it is slot 1 of lane l - 1 (for slot
-  // 0) and slot 0 of lane l + 1 (for slot 1), except d1 = 0 and P1/2, which mirror onto themselves
-  const int partner = u == 0 ? (THREE || HB == 1 || mir == 0 ? lane : lane ^ 8) : (HB == 2 ? lane ^ 24 : lane ^ 16);
+  // slot's 15 - d0, in column 0 in slot 1 of lane l - 1 (for slot 0) and slot 0 of lane l + 1 (for slot
+  // 1), except d1 = 0 and P1/2, which mirror onto themselves
+  const int partner = u != 0 ? lane ^ 16 : (THREE || HB == 1 || mir == 0) ? lane : lane ^ 8;
   const int partner0 = THREE && cb == 0 && l > 0 ? lane - 1 : partner;
   const int partner1 = THREE && cb == 0 && l < LC - 1 ? lane + 1 : partner;
+  const bool conjg = mir && u != 0;
   const bool self = cb == 0 && hb == 0 && l == 0, self1 = THREE && cb == 0 && l == LC - 1;
 
   if constexpr (THREE) {
@@ -278,7 +286,9 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
         tmem_wait_ld();
         sfor<0, 8>([&](auto k_) {
           constexpr int k = decltype(k_)::value, i = 8 * cc + k;
-          if constexpr (i > 0) v[i] = cmul(v[i], make_float2(w16[2 * k], w16[2 * k + 1]));
+          const float2 w = make_float2(w16[2 * k], w16[2 * k + 1]);
+        if constexpr (i > 16) v[i] = cmulc(v[i], w);  // conjugated: mirrors of column 32 - i
+        else if constexpr (i > 0) v[i] = cmul(v[i], w);
         });
       });
       if (turn) cp_async_wait_all();
@@ -335,7 +345,7 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
         });
         dit<32>(v);
       }
-      // correlate this lane's 16 bins k < N/2: k = cb + 32 d, d = HB i + hb, i < 16, or
+      // correlate this lane's 16 bins below N/2, by its outputs d = HB i + hb, i < 16, or
       // d = d1 + P1 d0, d0 < 8, for the lane's two d1 (i = 8 slot + d0)
       auto correlate = [&](auto sp_) {
         constexpr bool SP = decltype(sp_)::value;  // the warp holds column 0
@@ -347,17 +357,23 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
           sfor<0, 4>([&](auto k_) {
             constexpr int k = decltype(k_)::value, i = 4 * cc + k;
             constexpr int sl = THREE ? i / 8 : 0, d0 = i % 8;
-            constexpr int own = THREE ? 16 * sl + d0 : i, far = THREE ? 16 * (sl ^ 1) + 15 - d0 : 31 - i;
+            constexpr int own = THREE ? 16 * sl + d0 : i, far = own + (THREE ? 8 : 16);
             const int from = !THREE ? partner : sl ? partner1 : partner0;
-            float2 z = make_float2(__shfl_sync(0xffffffffu, v[far].x, from), __shfl_sync(0xffffffffu, v[far].y, from));
+            float2 z = v[far];
+            if constexpr (SP) {  // columns 0 and 16
+              constexpr int far0 = THREE ? 16 * (sl ^ 1) + 15 - d0 : 31 - i;
+              z.x = u == 0 ? v[far0].x : z.x;
+              z.y = u == 0 ? -v[far0].y : z.y;
+            }
+            z = make_float2(__shfl_sync(0xffffffffu, z.x, from), __shfl_sync(0xffffffffu, z.y, from));
             if constexpr (SP) {  // the bins that mirror onto their own lane's outputs
               constexpr int near = THREE ? (sl ? 16 + 15 - d0 : (16 - d0) % 16) : (32 - i) % 32;
               const bool me = sl ? self1 : self;
               z.x = me ? v[near].x : z.x;
-              z.y = me ? v[near].y : z.y;
+              z.y = me ? -v[near].y : z.y;
             }
             float(&q)[4] = *reinterpret_cast<float(*)[4]>(a16 + 4 * k);
-            corr_acc(q, v[own], make_float2(z.x, -z.y));
+            corr_acc(q, v[own], z);
           });
           tmem_st16(t_acc + 16 * cc, a16);
         });
@@ -383,7 +399,9 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
       sfor<0, 4>([&](auto k_) {
         constexpr int k = decltype(k_)::value, i = 4 * cc + k;
         const int d = THREE ? (i / 8 ? P1 - 1 - l : l) + P1 * (i % 8) : HB * i + hb;
-        sums[cb + 32 * d] = make_float4(a16[4 * k], a16[4 * k + 1], a16[4 * k + 2], a16[4 * k + 3]);
+        // (conjugated columns: bin N/2 - u - 32 d, and X conj(Y) came out as its negative conjugate)
+        sums[conjg ? PL::N / 2 - u - 32 * d : cb + 32 * d] =
+            make_float4(a16[4 * k], a16[4 * k + 1], conjg ? -a16[4 * k + 2] : a16[4 * k + 2], a16[4 * k + 3]);
       });
       if (FP64 && left > 1) {
         sfor<0, 16>([&](auto i_) { a16[decltype(i_)::value] = 0.f; });
