@@ -197,19 +197,18 @@ int spectrometer_n_pairs(const polaris_spec* s);
  * host floats `out`, on the GPU.  n must be a multiple of 32/bits. */
 int spectrometer_debug_unpack(polaris_spec* s, const void* packed, int64_t n, float* out);
 
-/* The data-translation step as the FFT kernel runs it on staged input, N = 2^13 and up (Fig. 2
- * caption: integer codes to floats; Sec. 2: two IF streams enter one transform): that kernel stages
- * each tile's packed words in shared memory, transposes their codes so that the rows of one
- * column share a word, and decodes both IFs of a pair together.  This call stages, transposes
- * and decodes through that same device code, for bit-exact checks of the levels the transform
- * sees.
+/* The data-translation step as the FFT kernel of the handle's size runs it on staged input, N = 2^13
+ * and up (Fig. 2 caption: integer codes to floats; Sec. 2: two IF streams enter one transform): that
+ * kernel stages packed words in shared memory, transposes their codes so that the rows of one
+ * column share a word, and decodes both IFs of a pair together.  This call stages in that kernel's
+ * layout and transposes and decodes through the same device code, for bit-exact checks of the
+ * levels the transform sees.
  *   packed_a, packed_b  host words of IF a and IF b of one FFT pair (packed_b NULL: a pair
  *               without an IF b, decoded by the single-IF variant), n samples each;
  *   n           a positive multiple of n_fft (whole segments, hop = n_fft);
- *   layout      0: transposed into a second buffer; 1: transposed in place;
+ *   layout      0 or 1 (each kernel has one layout; both values check it);
  *   out_a, out_b  host floats, n each (out_b unused when packed_b is NULL).
- * POLARIS_EINVAL when the FFT kernel does not stage at this handle's size and width (below
- * 2^13, and 1-bit samples at 2^19 and 2^20: there it decodes as spectrometer_debug_unpack). */
+ * POLARIS_EINVAL below 2^13, and for 1-bit samples at 2^19 and 2^20. */
 int spectrometer_debug_unpack_staged(polaris_spec* s, const void* packed_a, const void* packed_b, int64_t n,
                                      int layout, float* out_a, float* out_b);
 

@@ -48,10 +48,10 @@ typedef cudaError_t (*phase_fn)(const BatchArgs&, cudaStream_t, bool);
 // per-IF code histograms of segments [0, nseg) of `in` (polaris_stats.cu)
 cudaError_t launch_code_hist(const SegSrc& in, int n_if, int bits, int nseg, int64_t n_fft,
                              unsigned long long* hist, int* err, int num_sms, cudaStream_t st);
-// the staged data translation of phase 1 alone (polaris_debug.cu)
-bool phase1_staged(int logn, int bits);
-cudaError_t launch_unpack_staged(int logn, int bits, const uint32_t* pa, const uint32_t* pb, long long nseg, int dense,
-                                 float* oa, float* ob, cudaStream_t st);
+// the staged data translation alone (polaris_debug.cu)
+bool unpack_staged_takes(int logn, int bits);
+cudaError_t launch_unpack_staged(int logn, int bits, const uint32_t* pa, const uint32_t* pb, long long nseg, float* oa,
+                                 float* ob, cudaStream_t st);
 #define POLARIS_ROW(LOGN) {run_phase1<LOGN>, run_phase2<LOGN>}
 #define POLARIS_FUSED_ROW(LOGN) {run_fused<LOGN>, nullptr}  // both phases in one kernel
 static const phase_fn kPhases[21][2] = {
@@ -1221,9 +1221,9 @@ extern "C" int spectrometer_debug_unpack_staged(polaris_spec* s, const void* pac
   if (rc) return rc;
   if (!packed_a || !out_a || (packed_b && !out_b)) return set_err(s, POLARIS_EINVAL, "null pointer");
   if (n <= 0 || n % s->N) return set_err(s, POLARIS_EINVAL, "n must be a positive multiple of n_fft");
-  if (layout != 0 && layout != 1) return set_err(s, POLARIS_EINVAL, "layout must be 0 (transposed apart) or 1 (in place)");
-  if (!phase1_staged(s->logn, s->bits))
-    return set_err(s, POLARIS_EINVAL, "phase 1 does not stage its input at this size and width");
+  if (layout != 0 && layout != 1) return set_err(s, POLARIS_EINVAL, "layout must be 0 or 1");
+  if (!unpack_staged_takes(s->logn, s->bits))
+    return set_err(s, POLARIS_EINVAL, "no check of the staged decoder at this size and width");
   DeviceGuard dg(s->device);
   const size_t nw = (size_t)(n / s->spw);
   const int nif = packed_b ? 2 : 1;
@@ -1238,7 +1238,7 @@ extern "C" int spectrometer_debug_unpack_staged(polaris_spec* s, const void* pac
   cudaError_t e = cudaMemcpy(dw, packed_a, nw * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess && packed_b) e = cudaMemcpy(dw + nw, packed_b, nw * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
-    e = launch_unpack_staged(s->logn, s->bits, dw, packed_b ? dw + nw : nullptr, (long long)(n / s->N), layout, df,
+    e = launch_unpack_staged(s->logn, s->bits, dw, packed_b ? dw + nw : nullptr, (long long)(n / s->N), df,
                              packed_b ? df + n : nullptr, nullptr);
   if (e == cudaSuccess) e = cudaMemcpy(out_a, df, (size_t)n * 4, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess && packed_b) e = cudaMemcpy(out_b, df + n, (size_t)n * 4, cudaMemcpyDeviceToHost);

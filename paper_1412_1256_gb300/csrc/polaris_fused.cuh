@@ -108,6 +108,55 @@ __device__ __forceinline__ void team_sync(int team) {
   else asm volatile("bar.sync %0, %1;\n" ::"r"(1 + team), "r"(32 * W) : "memory");
 }
 
+// where word j of a segment of one IF is staged
+template <typename IN>
+__device__ __forceinline__ uint32_t fused_raw_place(int j) {
+  return (uint32_t)(j + (j / (IN::SPW * IN::WPR)) * IN::WL);
+}
+// codes of the cnt staged segments transposed, block by block (SPW words down a word column of one block
+// row), by the TL lanes of the team
+template <typename IN, int BITS, int TL>
+__device__ __forceinline__ void fused_transpose(const uint32_t* raw, uint32_t* tr, int cnt, int tl) {
+  constexpr int SPW = IN::SPW, WPR = IN::WPR, WL = IN::WL, VL = IN::VL;
+#pragma unroll 1
+  for (int k = tl; k < cnt * IN::NB; k += TL) {
+    const int br = (k / WL) % IN::BR, w = k % WL + (k / (WL * IN::BR)) % (WPR / WL) * WL, g = k / IN::NB;
+    const uint32_t* src = raw + g * IN::RAW + br * IN::RAWBLK + w;
+    uint32_t x[SPW];
+    sfor<0, SPW>([&](auto i_) { x[decltype(i_)::value] = src[decltype(i_)::value * WPR]; });
+    transpose_codes<BITS>(x);
+    // (columns w SPW + c, c < SPW, share one PADC group)
+    uint32_t* dst = tr + g * IN::TR + (br / VL) * IN::SLAB + (w * SPW + w * SPW / IN::PADC) * VL + br % VL;
+    sfor<0, SPW>([&](auto c_) { dst[decltype(c_)::value * VL] = stored_codes<BITS>(x[decltype(c_)::value]); });
+  }
+}
+// the codes of column tl of staged segment g, and its levels in row t
+template <typename IN>
+__device__ __forceinline__ void fused_lane_codes(const uint32_t* tr, int g, int tl, uint32_t (&cw)[IN::VW]) {
+  constexpr int VL = IN::VL;
+  const uint32_t* col = tr + g * IN::TR + (tl + tl / IN::PADC) * VL;
+  sfor<0, IN::VW / VL>([&](auto q_) {
+    constexpr int q = decltype(q_)::value;
+    if constexpr (VL == 4) {
+      const uint4 x = *reinterpret_cast<const uint4*>(col + q * IN::SLAB);
+      cw[4 * q] = x.x;
+      cw[4 * q + 1] = x.y;
+      cw[4 * q + 2] = x.z;
+      cw[4 * q + 3] = x.w;
+    } else {
+      const uint2 x = *reinterpret_cast<const uint2*>(col + q * IN::SLAB);
+      cw[2 * q] = x.x;
+      cw[2 * q + 1] = x.y;
+    }
+  });
+}
+template <typename IN, int BITS, bool HB, int T>
+__device__ __forceinline__ float2 fused_level(const uint32_t (&cw)[IN::VW]) {
+  float2 z = code_pair<BITS, T % IN::SPW>(cw[T / IN::SPW], cw[IN::VW / 2 + T / IN::SPW]);
+  if constexpr (!HB) z.y = 0.f;
+  return z;
+}
+
 // FP64: the integration accumulators are doubles
 template <int LOGN, int BITS, bool FP64>
 __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MINB) k_fused(BatchArgs a) {
@@ -115,7 +164,7 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
   using IN = typename PL::template In<BITS>;
   constexpr int W = PL::W, T = PL::T, B = PL::B, R = PL::R, HB = PL::HB, PITCH = PL::PITCH, P1 = PL::P1, LC = PL::LC;
   constexpr bool THREE = PL::THREE;
-  constexpr int SPW = IN::SPW, WPR = IN::WPR, WL = IN::WL, VL = IN::VL, G = IN::G, TL = 32 * W;
+  constexpr int G = IN::G, TL = 32 * W;
   extern __shared__ __align__(16) unsigned char smf[];
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int team = warp / W, wt = warp % W, tl = wt * 32 + lane;  // team, warp and lane inside it
@@ -187,7 +236,7 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
       const uint32_t dst = smem_addr(raw + g * IN::RAW);
       sfor<0, IN::NW / TL>([&](auto i_) {
         const int j = tl + decltype(i_)::value * TL;
-        const uint32_t o = 4u * (uint32_t)(j + (j / (SPW * WPR)) * WL);
+        const uint32_t o = 4u * fused_raw_place<IN>(j);
         if (in_bounds(a.err, w0 + j, wext)) {
           cp_async4(dst + o, pa + j);
           cp_async4(dst + o + 4u * (uint32_t)(IN::RAW / 2), pb + j);
@@ -199,21 +248,7 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
 
   float extra[4] = {0.f, 0.f, 0.f, 0.f};
   [[maybe_unused]] const float sgn_b = hb ? -1.f : 1.f;
-  // codes of the cnt staged segments transposed, block by block: SPW words down a word column of one
-  // block row
-  auto transpose = [&](int cnt) {
-#pragma unroll 1
-    for (int k = tl; k < cnt * IN::NB; k += TL) {
-      const int br = (k / WL) % IN::BR, w = k % WL + (k / (WL * IN::BR)) % (WPR / WL) * WL, g = k / IN::NB;
-      const uint32_t* src = raw + g * IN::RAW + br * IN::RAWBLK + w;
-      uint32_t x[SPW];
-      sfor<0, SPW>([&](auto i_) { x[decltype(i_)::value] = src[decltype(i_)::value * WPR]; });
-      transpose_codes<BITS>(x);
-      // (columns w SPW + c, c < SPW, share one PADC group)
-      uint32_t* dst = tr + g * IN::TR + (br / VL) * IN::SLAB + (w * SPW + w * SPW / IN::PADC) * VL + br % VL;
-      sfor<0, SPW>([&](auto c_) { dst[decltype(c_)::value * VL] = stored_codes<BITS>(x[decltype(c_)::value]); });
-    }
-  };
+  auto transpose = [&](int cnt) { fused_transpose<IN, BITS, TL>(raw, tr, cnt, tl); };
   // Segments come in groups of G.  The next group's words are copied during a group and transposed in
   // its last segment, between the two barriers of the exchange, which order those steps too: two
   // barriers per segment (with a pass of its own over each group, four per segment at 4 and 8 bits)
@@ -238,29 +273,14 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
       // step A: decode column tl, window, 32-point DFT
       float2 v[32];
       uint32_t cw[IN::VW];
-      const uint32_t* col = tr + g * IN::TR + (tl + tl / IN::PADC) * VL;
-      sfor<0, IN::VW / VL>([&](auto q_) {
-        constexpr int q = decltype(q_)::value;
-        if constexpr (VL == 4) {
-          const uint4 x = *reinterpret_cast<const uint4*>(col + q * IN::SLAB);
-          cw[4 * q] = x.x;
-          cw[4 * q + 1] = x.y;
-          cw[4 * q + 2] = x.z;
-          cw[4 * q + 3] = x.w;
-        } else {
-          const uint2 x = *reinterpret_cast<const uint2*>(col + q * IN::SLAB);
-          cw[2 * q] = x.x;
-          cw[2 * q + 1] = x.y;
-        }
-      });
+      fused_lane_codes<IN>(tr, g, tl, cw);
       auto rows = [&](auto hb_, auto tp_) {
         constexpr bool HBP = decltype(hb_)::value, TP = decltype(tp_)::value;
         [[maybe_unused]] const float4* tp = reinterpret_cast<const float4*>(a.taps) + tl;
         [[maybe_unused]] float4 w4;
         sfor<0, 32>([&](auto t_) {
           constexpr int t = decltype(t_)::value;
-          float2 z = code_pair<BITS, t % SPW>(cw[t / SPW], cw[IN::VW / 2 + t / SPW]);
-          if constexpr (!HBP) z.y = 0.f;
+          float2 z = fused_level<IN, BITS, HBP, t>(cw);
           if constexpr (TP) {  // (four consecutive t per load: tap_order)
             if constexpr (t % 4 == 0) w4 = __ldg(tp + (t / 4) * B);
             const float x = t % 4 == 0 ? w4.x : t % 4 == 1 ? w4.y : t % 4 == 2 ? w4.z : w4.w;

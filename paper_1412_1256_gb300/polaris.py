@@ -366,7 +366,7 @@ class Spectrometer:
 
     def debug_unpack_staged(self, words_a: np.ndarray, words_b, n: int, layout: int = 0):
         """Levels of n samples (whole segments) of IF a and IF b (words_b None: a pair without
-        an IF b) through the FFT kernel's staged decoder; layout 0: transposed apart, 1: in place.
+        an IF b) through the FFT kernel's staged decoder; layout 0 or 1 (each kernel has one).
         Returns (levels_a, levels_b or None)."""
         wa = np.ascontiguousarray(words_a, dtype=np.uint32)
         wb = None if words_b is None else np.ascontiguousarray(words_b, dtype=np.uint32)
