@@ -347,8 +347,7 @@ static cudaError_t launch_readout(const ReadoutArgs& r, int n_fpair, cudaStream_
 #define POLARIS_RO(LN1)                                       \
   case 1 << LN1:                                              \
     return cudaLaunchKernelEx(&cfg, k_readout<LN1>, r);
-    POLARIS_RO(1) POLARIS_RO(2) POLARIS_RO(3) POLARIS_RO(4) POLARIS_RO(5) POLARIS_RO(6) POLARIS_RO(7)
-    POLARIS_RO(8) POLARIS_RO(9) POLARIS_RO(10) POLARIS_RO(11)
+    POLARIS_RO(2) POLARIS_RO(3) POLARIS_RO(4) POLARIS_RO(7) POLARIS_RO(8) POLARIS_RO(9) POLARIS_RO(10) POLARIS_RO(11)
 #undef POLARIS_RO
     default: return cudaErrorInvalidValue;
   }

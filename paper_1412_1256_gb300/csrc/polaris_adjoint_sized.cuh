@@ -190,7 +190,7 @@ __device__ __forceinline__ void adjs_fetch(const AdjArgs& a, uint32_t* raw, long
   const uint32_t dst = smem_addr(raw);
   for (int c = tid; c < 2 * (W / 4); c += AdjPlan<LOGN>::T) {
     const int f = c >= W / 4;
-    cp_async<16>(dst + 16u * (uint32_t)c, a.in[f] + s * W + 4 * (c - f * (W / 4)));
+    cp_async16(dst + 16u * (uint32_t)c, a.in[f] + s * W + 4 * (c - f * (W / 4)));
   }
   cp_async_commit();
 }

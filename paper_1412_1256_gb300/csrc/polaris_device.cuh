@@ -208,7 +208,7 @@ constexpr int plan_p(int logn) { return logn >= 10 ? 32 : (logn >= 8 ? 16 : (log
 // that measured slower than 32 points per lane at two CTAs per SM.
 constexpr int plan_p1(int logn, int n1) { return n1 == 128 ? 16 : plan_p(logn); }
 constexpr int plan_log_n2(int logn) {
-  // 4:2 5:3 6:3 7:4 8:4 9:5 10:5 11:6 12:6 13:7 14:7 15:8 16:8 17:9 18:9 19:9 20:9
+  // 4:2 5:3 6:3 7:4 8:4 9:5 (2^10 to 2^14: fused_log_b) 15:8 16:8 17:9 18:9 19:9 20:9
   return logn >= 17 ? 9 : (logn + 1) / 2;
 }
 // 2^18 and up: phase 1 by whole CTAs (polaris_wide.cuh), over groups of this many columns (128- or
@@ -262,20 +262,13 @@ struct Ld2 {
   int a, b;
 };
 constexpr Ld2 p1_layout(int P, int Q1) {
-  return (P == 16 && Q1 == 4)    ? Ld2{8, 136}
-         : (P == 16 && Q1 == 8)  ? Ld2{4, 68}
-         : (P == 16 && Q1 == 16) ? Ld2{2, 34}
-         : (P == 32 && Q1 == 2)  ? Ld2{16, 512}
-         : (P == 32 && Q1 == 4)  ? Ld2{8, 264}
-         : (P == 32 && Q1 == 8)  ? Ld2{4, 132}
-                                 : Ld2{32 / Q1, P * (32 / Q1)};  // Q1 = 1: no transpose
+  return (P == 16 && Q1 == 8)   ? Ld2{4, 68}
+         : (P == 32 && Q1 == 8) ? Ld2{4, 132}
+                                : Ld2{32 / Q1, P * (32 / Q1)};  // Q1 = 1: no transpose
 }
 constexpr Ld2 p2_layout(int P, int Q2) {
   return (P == 32 && Q2 == 16)  ? Ld2{17, 544}
          : (P == 32 && Q2 == 8) ? Ld2{9, 296}
-         : (P == 32 && Q2 == 4) ? Ld2{5, 163}
-         : (P == 32 && Q2 == 2) ? Ld2{3, 95}
-         : (P == 32 && Q2 == 1) ? Ld2{1, 33}
          : (P == 16 && Q2 == 2) ? Ld2{2, 33}
          : (P == 16 && Q2 == 1) ? Ld2{1, 17}
          : (P == 8 && Q2 == 2)  ? Ld2{3, 26}
@@ -293,6 +286,7 @@ constexpr int pow2_at_least(int v, int lo) {
 
 template <int LOGN>
 struct Plan {
+  static_assert(!is_fused(LOGN), "2^10 to 2^14: FusedPlan");
   static constexpr int N = 1 << LOGN;
   static constexpr int P = plan_p(LOGN);
   static constexpr int N2 = 1 << plan_log_n2(LOGN);

@@ -76,7 +76,10 @@ struct BatchArgs {
   int nseg;             // segments in this batch
   const float* taps;    // window taps (N, in tap_order) or nullptr for the rectangular window
   float2* scratch;      // slab [nseg * n_fpair][N1][N2]: row c (phase-1 output index), b contiguous
-  const float2* tw;     // [UPS + 1][N2]: W_N^{b u} (unit-major)
+  // [UPS + 1][N2]: W_N^{b u} (unit-major); one kernel: [N1][N2], rows above N1/2 as tw_unit and tw_sign
+  // say.  Read before the wait for the kernel before, and like the taps by read-only loads: both
+  // tables are complete when a dependent launch is queued
+  const float2* tw;
   void* acc;            // native accumulators [acc_copies][n_fpair][N/2 + 1] of float4 (double4 if fp64)
   int acc_copies;       // 1, or K: segment range r of a (pair, unit group) adds into copy r % K
   int fp64;
@@ -126,10 +129,8 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
 }
-template <int BYTES>  // 4, 8 or 16, both addresses aligned to it
-__device__ __forceinline__ void cp_async(uint32_t dst, const void* src) {
-  if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-  else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(dst), "l"(src), "n"(BYTES) : "memory");
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {  // both addresses aligned to 16 bytes
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
@@ -156,14 +157,6 @@ __device__ __forceinline__ void tma_store_2d_elect(const CUtensorMap* map, const
       "r"(smem_addr(src)), "r"(x), "r"(y), "l"(policy)
       : "memory");
 }
-// TMA store of a 2-D box by the calling thread alone (the caller commits the group)
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int x, int y, uint64_t policy) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group.L2::cache_hint [%0, {%2, %3}], [%1], %4;\n" ::"l"(
-                   map),
-               "r"(src), "r"(x), "r"(y), "l"(policy)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;\n" ::: "memory"); }
 // wait until this thread's bulk groups have finished reading shared memory (a lane that
 // issued none returns at once)
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
@@ -291,7 +284,7 @@ __device__ __forceinline__ void p1_load(const BatchArgs& a, int g, int b, int q1
     float x = decode_level<BITS>(ok ? pa[word_i] : 0u, shift);
     float y = pb ? decode_level<BITS>(ok ? pb[word_i] : 0u, shift) : 0.0f;
     if (taps) {
-      const float wv = __ldg(taps + tap_order(LOGN).slot(n));
+      const float wv = __ldg(taps + n);
       x *= wv;
       y *= wv;
     }
@@ -349,7 +342,9 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
   using ST = typename PL::template Stage1<BITS>;
   constexpr bool STAGED = ST::STAGED;
   constexpr int TILE = ST::TILE, IPT = ST::IPT, WPR = STAGED ? ST::WPR : 1;  // words per IF per tile row
-  constexpr bool TMA_OUT = ST::TMA_OUT;  // the warp's [N1][CW] output block leaves by one TMA store
+  // staged: the warp's [N1][CW] output block leaves by one TMA store; else one lane holds a whole column
+  constexpr bool TMA_OUT = ST::TMA_OUT;
+  static_assert(TMA_OUT == (Q1 > 1), "a lane's column leaves from its registers, or a warp's block by TMA");
   static_assert(!TMA_OUT || (Q1 > 1 && N1 <= 256 && (CW * 8) % 16 == 0 && N1 * CW <= PL::REGION1 &&
                              (PL::REGION1 * 8) % 128 == 0),
                 "TMA output tile");
@@ -412,57 +407,33 @@ __global__ void __launch_bounds__(Plan<LOGN>::THREADS, Plan<LOGN>::MINB1)
           if constexpr (p > 0) v[p] = cmul(v[p], make_float2(w16[2 * k], w16[2 * k + 1]));
         });
       });
-      if constexpr (TMA_OUT) {
-        bulk_wait_read();  // the previous output tile has left the region
-        __syncwarp();
-      }
+      bulk_wait_read();  // the previous output tile has left the region
+      __syncwarp();
       sfor<0, P>([&](auto p_) {
         constexpr int p = decltype(p_)::value;
         region[q1 * LDQ + p * LDP + cw] = v[p];
       });
       __syncwarp();
-      if constexpr (TMA_OUT) {
-        sfor<0, PQ>([&](auto r_) {
-          constexpr int r = decltype(r_)::value;
-          const int p = r * Q1 + q1;
-          sfor<0, Q1>([&](auto q_) {
-            constexpr int q = decltype(q_)::value;
-            v[r * Q1 + ct::bitrev(q, Q1)] = region[q * LDQ + p * LDP + cw];
-          });
+      sfor<0, PQ>([&](auto r_) {
+        constexpr int r = decltype(r_)::value;
+        const int p = r * Q1 + q1;
+        sfor<0, Q1>([&](auto q_) {
+          constexpr int q = decltype(q_)::value;
+          v[r * Q1 + ct::bitrev(q, Q1)] = region[q * LDQ + p * LDP + cw];
         });
-        __syncwarp();  // region consumed: it now takes the output tile [c][cw]
-        sfor<0, PQ>([&](auto r_) {
-          constexpr int r = decltype(r_)::value;
-          dit<Q1, r * Q1, 1>(v);
-          sfor<0, Q1>([&](auto m_) {
-            constexpr int m = decltype(m_)::value;
-            region[(r * Q1 + q1 + P * m) * CW + cw] = slab_val(v[r * Q1 + m], r * Q1 + q1 + P * m);
-          });
+      });
+      __syncwarp();  // region consumed: it now takes the output tile [c][cw]
+      sfor<0, PQ>([&](auto r_) {
+        constexpr int r = decltype(r_)::value;
+        dit<Q1, r * Q1, 1>(v);
+        sfor<0, Q1>([&](auto m_) {
+          constexpr int m = decltype(m_)::value;
+          region[(r * Q1 + q1 + P * m) * CW + cw] = slab_val(v[r * Q1 + m], r * Q1 + q1 + P * m);
         });
-        fence_async_shared();
-        __syncwarp();
-        if (act) tma_store_2d_elect(&slab_map, region, xcol, (int)(g * N1), l2_evict_last());
-      } else {
-        sfor<0, PQ>([&](auto r_) {
-          constexpr int r = decltype(r_)::value;
-          const int p = r * Q1 + q1;
-          float2 u[Q1];
-          sfor<0, Q1>([&](auto q_) {
-            constexpr int q = decltype(q_)::value;
-            u[ct::bitrev(q, Q1)] = region[q * LDQ + p * LDP + cw];
-          });
-          dit<Q1>(u);
-          if (act) {
-            float2* dst = a.scratch + ((size_t)g * N1 + p) * N2 + b;
-            sfor<0, Q1>([&](auto m_) {
-              constexpr int m = decltype(m_)::value;
-              if (in_bounds(a.err, ((long long)g * N1 + p + (long long)m * P) * N2 + b, a.slab_elems))
-                dst[(size_t)m * P * N2] = slab_val(u[m], p + m * P);
-            });
-          }
-        });
-        __syncwarp();  // region free for the next item
-      }
+      });
+      fence_async_shared();
+      __syncwarp();
+      if (act) tma_store_2d_elect(&slab_map, region, xcol, (int)(g * N1), l2_evict_last());
     } else {
       if (act) {
         float2* dst = a.scratch + (size_t)g * N1 * N2 + b;
