@@ -804,7 +804,9 @@ static int check_device_status(polaris_spec* s, int st) {
 // four IFs (copy in, kernels, spectra back) with one / two / three / four pieces: 122 x 2^17 int8
 // (64 MB) 488 / 435 / 422 / 416 us, 976 x 2^14 int8 Hann (64 MB) 473 / 419 / 407 / 400 us; 61 x
 // 2^17 4-bit with code statistics (16 MB) 243 / 227 / 246 / 246 us (each piece costs about 20 us of
-// host time in launches); 8 MB and less: no gain.
+// host time in launches); 8 MB and less: no gain.  Only where nothing is carried into the feed (the
+// segments that start in carried samples are assembled from the whole input first) and one pass takes
+// it: an overlapped stream's later feeds, and ragged ones, are copied whole before their first kernel.
 constexpr int64_t kPieceBytes = 8 << 20;
 constexpr int kMaxPieces = 4;
 

@@ -1,7 +1,8 @@
 // Leakage calibration (forward model and adjoint): what the segment kernels share.  The
 // model, its gradients and the kernel sequence are described in polaris_adjoint.cu; the
-// transforms of N = 2^9 .. 2^14 run in size-specialised kernels (polaris_adjoint_sized.cu),
-// the smaller ones in polaris_adjoint.cu's kernels for any N.
+// transforms of N = 2^9 .. 2^14 run in size-specialised kernels (polaris_adjoint_sized.cu,
+// polaris_adjoint_teams.cu), those of buffers that are not 16-byte aligned in polaris_adjoint.cu's
+// kernels for any N, the smaller sizes in that file's kernels of many segments per CTA.
 #pragma once
 
 #include <cuda_runtime.h>

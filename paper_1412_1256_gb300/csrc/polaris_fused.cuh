@@ -20,17 +20,17 @@
 //            FP64 accumulators: every `flush` segments instead, the teams summed in twice FP32's
 //            precision, so that the sums do not lose bits as a feed gets longer.  The lengths are those of
 //            the two-kernel path's ranges (a pass of 4096 segments over its warps).  Passes of four 2-bit IFs
-//            of 8 M samples with one addition at the end and so: 2^10 33.1, 37.5 us; 2^11 40.2, 40.2; 2^12
-//            50.3, 50.7; 2^13 68.2, 51.3; 2^14 81.4, 60.0 (FP32 accumulators: 30.8 to 51.6): the last ones
+//            of 8 M samples with one addition at the end and so: 2^10 33.1, 38.4 us; 2^11 40.2, 41.9; 2^12
+//            50.3, 52.2; 2^13 68.2, 52.2; 2^14 81.4, 61.4 (FP32 accumulators: 31.0 to 51.4): the last ones
 //            from consecutive lanes adding consecutive values and from fewer FP64 instructions, which
-//            bound this part (teams summed in FP64: 2^25 samples of one pair at 2^10 314 us, now 157).
+//            bound this part (teams summed in FP64: 2^25 samples of one pair at 2^10 314 us, now 162).
 //
-// What bounds it: instruction issue, about 40 to 43 instructions per complex point, of which 14
-// packed FP32, at 45 to 50% of the issue slots with 16 warps per SM (registers), against 64 of the
-// two-phase path of the larger sizes, which these sizes took before and which sends every point
+// What bounds it: instruction issue, 47 instructions per complex point (2^14, 1024 segments of two
+// pairs, set-up included) at 43 to 51% of the issue slots with 16 warps per SM (registers), against 64 of
+// the two-phase path of the larger sizes, which these sizes took before and which sends every point
 // through a slab in L2.  Measured against that path (GB300, four 2-bit IFs of 8 M samples, whole
-// passes, Msample/s before and after): 2^10 313k, 1114k; 2^11 435k, 926k; 2^12 393k, 770k; 2^13
-// 480k, 697k; 2^14 478k, 638k; 64 int8 Hann segments of 1024 points 28.7 and 13.2 us (host-bound);
+// passes, Msample/s before and after): 2^10 313k, 1082k; 2^11 435k, 912k; 2^12 393k, 788k; 2^13
+// 480k, 706k; 2^14 478k, 653k; 64 int8 Hann segments of 1024 points 28.7 and 13.4 us (host-bound);
 // one 2^14 segment 23 and 17 us.  (2^12 with both transforms split by parity like 2^11's second one,
 // 64 x 64 points, ran at 727k.)  The line: 2^15 points do not fit an SM's registers, and below 2^10
 // a warp would hold several segments.
@@ -462,7 +462,9 @@ __global__ void __launch_bounds__(FusedPlan<LOGN>::THREADS, FusedPlan<LOGN>::MIN
 }
 
 // One launch per feed: CTAs in equal numbers per FFT pair, as many as fit and have a segment per
-// team.
+// team.  Either of the caller's caps holds (this kernel is both phases): with three handles and phase 1
+// capped, six passes of four 2-bit IFs of 16 M samples took, uncapped and capped, 306, 295 us at 2^10,
+// 368, 354 at 2^11, 404, 397 at 2^12, 465, 433 at 2^13; on one handle 339, 476; 402, 571; 439, 506; 501, 671.
 template <int LOGN, int BITS, bool FP64>
 static cudaError_t launch_fused_acc(const BatchArgs& a, cudaStream_t st, bool pdl) {
   using PL = FusedPlan<LOGN>;
